@@ -45,7 +45,7 @@ WORKLOAD_NAMES = {
 }
 CELL = {"treernn": "rnn", "treelstm": "lstm"}
 KERNEL_SOURCES = ["rdf_device.cuh", "rdf_exec.cu", "rdf_exec.h", "rdf_grad.cu", "rdf_internal.h", "rdf_lists.cuh", "rdf_lstm.cuh",
-                  "rdf_tc.cuh", "rdf_tc_dw.cuh"]
+                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh"]
 
 
 def fib_iter(n):
@@ -492,7 +492,7 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
                      "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak if peak else None, "peak_source": src,
                      "traffic": traffic.get((kernel, workload))})
 
-    add("rdf_scheduler_kernel", "schedule", "hbm", 128.0 * N,
+    add("rdf_scheduler_kernel" if case.cfg["kind"] in ("fib", "topdown") else "rdf_fold_kernel", "schedule", "hbm", 128.0 * N,
         "128 B per invocation: call token write+read, return token / store slot write+read, frame record")
     if case.cfg["kind"] == "fib":
         return rows
@@ -506,11 +506,8 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     Hp = 64 * ((H + 63) // 64)
     lstm = case.cell == "lstm"
     mm = "tensor" if case.use_tc else "alu"
-    if case.use_tc:       # tensor-core path: the cells listed by call depth (the same lists serve the gradient pass)
-        add("rdf_list_count/scan/fill/ends/compact/zdst_kernel", "group", "hbm", N * 32.0 + C * 24.0,
-            "operand ids and frame records read (two passes), cell lists and operand-row destinations written")
-    else:
-        add("rdf_height_count/scan/scatter_kernel", "group", "hbm", 48.0 * C, "16 B cell record read twice and written once")
+    if not case.use_tc and not lstm:
+        add("rdf_group_count/scan/scatter_kernel", "group", "hbm", 48.0 * C, "16 B cell record read twice and written once")
     add("rdf_operator_kernel", "operators", mm, case.flops_fwd(),
         "cell contraction 2*2H*H per cell" + (" (x5 gates) + leaf projection 2*D*3H per leaf" if lstm else ""))
     add("rdf_gather_roots_kernel", "roots", "hbm", tb.B * H * (4.0 + (2 if case.use_tc and not lstm else 4)), "root rows read and written")

@@ -50,7 +50,7 @@ static const uint64_t SLOT_EMPTY = ~0ull;     // depth field 63: never a tag
 
 struct __align__(16) CellItem {               // one ready cell: state of `out` from states of l, r
     uint32_t out, l, r;
-    uint32_t height;                          // 1 + the larger height of its operands (leaves: 0)
+    uint32_t valid;
 };
 struct __align__(8) LeafItem {
     uint32_t slot;
@@ -78,15 +78,16 @@ struct Control {
     uint32_t all_cells;           // backward: cells seen so far (length of the all-cells list)
     uint32_t all_leaves;          // backward: leaves seen so far
     uint32_t resume_wave;         // wave index at which the grid carries on after a stretch of narrow waves
-    uint32_t max_height;          // largest height of a cell of this call (operator waves run height by height)
-    uint32_t h_split;             // clustered fp32 path: heights up to here are wide and fired by the whole grid, the rest cluster by cluster
-    uint32_t d_split;             // clustered gradient pass: call depths (scheduler wave + 1) up to here are wide and run by the whole grid
+    uint32_t d_split;             // clustered fp32 path: call depths (scheduler wave + 1) up to here are wide and run by the whole grid,
+                                  // the deeper ones cluster by cluster
+    uint32_t call_waves;          // one past the last scheduler wave that made calls
     uint32_t n_depth_waves;       // scheduler waves that made calls = call depths of the run (length of the compacted wave_marks)
     unsigned long long invocations, tokens, store_inserts, store_matches, store_probes, cells, leaves;
     unsigned long long trace_count;
     unsigned long long cyc[6];    // block 0: forward schedule / batch / barrier, backward frames / batch / barrier
     float    loss;
     int32_t  forward_status;      // status word at the end of the forward pass and the loss head
+    uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
 };
 static_assert(sizeof(Control) <= 4096, "the control block is 4 KB");
 
@@ -108,6 +109,10 @@ struct DevCtx {
     // wave queues
     Token*   q[2];
     uint32_t qcap;
+    // structural recursion (rdf_fold.cuh)
+    int       fold_label[3], fold_right[2];
+    uint32_t* level_counts;       // [3][level_cap]: cells per chunk of a level, three levels in turn
+    uint32_t  level_cap;
     // frames (frame-form tags)
     Frame*    frames;
     uint32_t* finst;              // [frame_cap] fp32 tree networks: the instance (tree) an invocation belongs to, handed down
@@ -129,11 +134,9 @@ struct DevCtx {
     Slot*     table;
     uint64_t  table_cap;          // slots per match node, power of two
     // batched operators
-    CellItem* cell_items;         // every cell in the order it became ready (wave after wave); the operator kernel
-                                  // gets the copy sorted by height here
-    CellItem* cell_sorted;        // the cells grouped by height: the operands of a cell of height k have heights < k, so
-                                  // all cells of one height fire together whatever wave the scheduler found them in
-    uint32_t* height_ends;        // [wave_cap + 2]: cells per height, then (after the scatter) the end of each group
+    CellItem* cell_items;         // every cell in the order it became ready (general scheduler)
+    CellItem* cell_sorted;        // clustered fp32 path: the cells grouped by (cluster of their instance, call depth)
+    uint32_t* group_ends;         // [wave_cap + 2]: cells per group, then (after the scatter) the end of each group
     LeafItem* leaf_items;         // every leaf in the order it was reached
     uint32_t  work_cap;
     uint32_t* op_l;               // per frame: operand frames of the operator that made its state
@@ -204,25 +207,16 @@ struct DevCtx {
 
 static const uint32_t LEAF_MARK = 0xFFFFFFFFu;
 
-// How many groups the ready cells are sorted into (by instance, then by height): the clusters of the clustered
-// operator kernel when the (group, height) table fits the space of the height table, else one group (all cells
-// by height, fired by the whole grid).  Every kernel of a call computes the same answer from the same words.
-// Shallow batches stay with the grid-wide kernel: a few dozen waves are too few for the second kernel to pay.
-static const uint32_t CLUSTER_MIN_HEIGHT = 64;
-__device__ __forceinline__ uint32_t cell_groups(const DevCtx& c) {
-    const uint64_t stride = (uint64_t)min(c.ctl->max_height, c.wave_cap) + 1u;
-    return c.n_groups > 1 && stride > CLUSTER_MIN_HEIGHT && (uint64_t)c.n_groups * stride <= (uint64_t)c.wave_cap + 2u
-               ? (uint32_t)c.n_groups : 1u;
-}
-// The same for the gradient pass, whose waves go by call depth (the scheduler wave that created the frame): cells grouped
-// by (cluster of their instance, scheduler wave + 1).
+// How many groups the cells are sorted into (by instance, then by call depth): the clusters of the clustered kernels when
+// the (group, depth) table fits its space, else one group (everything is fired by the whole grid).  Every kernel of a call
+// computes the same answer from the same words.
+// Shallow batches stay with the grid-wide kernels: a few dozen waves are too few for the second kernel to pay.
+static const uint32_t CLUSTER_MIN_DEPTH = 64;
+__device__ __forceinline__ uint32_t depth_stride(const DevCtx& c) { return min(c.ctl->call_waves, c.wave_cap) + 1u; }
 __device__ __forceinline__ uint32_t depth_groups(const DevCtx& c) {
-    const uint64_t stride = (uint64_t)min(c.ctl->waves, c.wave_cap) + 1u;
-    return cell_groups(c) > 1u && (uint64_t)c.n_groups * stride <= (uint64_t)c.wave_cap + 2u ? (uint32_t)c.n_groups : 1u;
-}
-__device__ __forceinline__ uint32_t bucket_groups(const DevCtx& c, int by_depth) { return by_depth ? depth_groups(c) : cell_groups(c); }
-__device__ __forceinline__ uint32_t bucket_stride(const DevCtx& c, int by_depth) {
-    return min(by_depth ? c.ctl->waves : c.ctl->max_height, c.wave_cap) + 1u;
+    const uint64_t stride = depth_stride(c);
+    return c.n_groups > 1 && stride > CLUSTER_MIN_DEPTH && (uint64_t)c.n_groups * stride <= (uint64_t)c.wave_cap + 2u
+               ? (uint32_t)c.n_groups : 1u;
 }
 static const uint32_t NO_ZDST = 0xFFFFFFFFu;
 

@@ -4,11 +4,11 @@
 //      push / pop, Switch, token-store insert or match) and emits the next
 //      wave's tokens.  A vector value travels by reference (the frame that
 //      holds it), so a ready leaf / cell operator is queued, not computed: the
-//      kernel leaves behind the lists of ready operators, each cell with the
-//      height of the operator tree below it.
+//      kernel leaves behind the lists of ready operators.  (Structural recursion
+//      over the input trees has a scheduler of its own, rdf_fold.cuh.)
 //   Operator kernel: fires the ready operators as batches, the leaves first and
-//      then the cells height by height (grouped by three small kernels between
-//      the two): operands before results, in as few dependent waves as possible.
+//      then the cells call depth by call depth, deepest first: operands before
+//      results, in as few dependent waves as possible.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -17,6 +17,7 @@
 
 #include "rdf_exec.h"
 #include "rdf_lists.cuh"
+#include "rdf_fold.cuh"
 #include "rdf_lstm.cuh"
 #include "rdf_tc.cuh"
 
@@ -31,7 +32,7 @@ struct SharedProgram {
 };
 
 struct ThreadStats {
-    uint32_t invocations = 0, tokens = 0, cells = 0, leaves = 0, max_depth = 0, max_height = 0;
+    uint32_t invocations = 0, tokens = 0, cells = 0, leaves = 0, max_depth = 0;
     StoreCounters sc;
 };
 
@@ -55,19 +56,16 @@ __device__ __forceinline__ void fire_cell(const DevCtx& c, const LocalQ* lq, con
         set_status(c, RDF_ERR_QUEUE_FULL);
         return;
     }
-    // A vector value travels as the frame that holds it (low half of the datum) and the height of the
-    // operator tree below it (high half): leaves 0, a cell one more than the higher of its operands.
+    // A vector value travels as the frame that holds it.
     CellItem it;
     it.out = (uint32_t)tag; it.l = (uint32_t)regs[0]; it.r = (uint32_t)regs[1];
-    it.height = max((uint32_t)((uint64_t)regs[0] >> 32), (uint32_t)((uint64_t)regs[1] >> 32)) + 1u;
+    it.valid = 1u;
     c.cell_items[i] = it;
-    st.max_height = max(st.max_height, it.height);
     c.op_l[tag] = it.l;
     c.op_r[tag] = it.r;
     ++st.cells;
-    const int64_t datum = (int64_t)(((uint64_t)it.height << 32) | (uint32_t)tag);
-    if (lq) push_token(c, lq, wave, tag, datum, (uint32_t)M.cont_pc);
-    else store_token(&c.q[(wave + 1) & 1][slot], tag, datum, (uint32_t)M.cont_pc);
+    if (lq) push_token(c, lq, wave, tag, (int64_t)(uint32_t)tag, (uint32_t)M.cont_pc);
+    else store_token(&c.q[(wave + 1) & 1][slot], tag, (int64_t)(uint32_t)tag, (uint32_t)M.cont_pc);
 }
 
 // Runs one token through its segment and on through every continuation it
@@ -310,13 +308,12 @@ __device__ void run_token(const DevCtx& c, const SharedProgram& sp, const LocalQ
                 }
                 CellItem it;
                 it.out = (uint32_t)tag; it.l = (uint32_t)r[in.a]; it.r = in.dst ? CHILD_R_MARK : CHILD_L_MARK;
-                it.height = (uint32_t)((uint64_t)r[in.a] >> 32) + 1u;
+                it.valid = 1u;
                 c.cell_items[i] = it;
-                st.max_height = max(st.max_height, it.height);
                 c.op_l[tag] = it.l;
                 c.op_r[tag] = it.r;
                 ++st.cells;
-                store_token(&c.q[(wave + 1) & 1][slot], tag, (int64_t)(((uint64_t)it.height << 32) | (uint32_t)tag), (uint32_t)in.imm);
+                store_token(&c.q[(wave + 1) & 1][slot], tag, (int64_t)(uint32_t)tag, (uint32_t)in.imm);
                 break;
             }
             default:   // VM_HALT
@@ -447,8 +444,10 @@ __device__ void rnn_cell_thin(const DevCtx& c, float* xs, const float4* wres, ui
     }
 }
 
-__device__ void rnn_leaf_rows(const DevCtx& c, uint32_t n_items) {
-    // one warp per leaf: state(slot) = E[tok]
+// fp32 TreeRNN leaves, one warp per leaf: state(slot) = E[tok]
+__global__ void __launch_bounds__(256) rdf_leaf_rows_kernel(const DevCtx c) {
+    if (c.ctl->forward_status != 0) return;                          // the scheduler failed: the lists are not to be trusted
+    const uint32_t n_items = min(c.ctl->leaf_count.v, c.work_cap);
     const int H = c.H;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
     const int n_warps = gridDim.x * blockDim.x / 32;
@@ -466,13 +465,12 @@ __device__ void rnn_leaf_rows(const DevCtx& c, uint32_t n_items) {
 // per-thread counters -> one set of atomics per warp
 __device__ __forceinline__ void flush_stats(const DevCtx& c, const ThreadStats& st) {
     unsigned long long v[7] = {st.invocations, st.tokens, st.cells, st.leaves, st.sc.inserts, st.sc.matches, st.sc.probes};
-    uint32_t mp = st.sc.max_probe, md = st.max_depth, mh = st.max_height;
+    uint32_t mp = st.sc.max_probe, md = st.max_depth;
     for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
         for (int k = 0; k < 7; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
         mp = max(mp, __shfl_xor_sync(0xffffffffu, mp, o));
         md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
-        mh = max(mh, __shfl_xor_sync(0xffffffffu, mh, o));
     }
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(&c.ctl->invocations, v[0]); atomicAdd(&c.ctl->tokens, v[1]); atomicAdd(&c.ctl->cells, v[2]);
@@ -480,7 +478,6 @@ __device__ __forceinline__ void flush_stats(const DevCtx& c, const ThreadStats& 
         atomicAdd(&c.ctl->store_probes, v[6]);
         atomicMax(&c.ctl->max_probe, mp);
         atomicMax(&c.ctl->max_depth, md);
-        if (mh) atomicMax(&c.ctl->max_height, mh);        // (the operator waves run height by height)
     }
 }
 
@@ -766,8 +763,8 @@ __global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
 }
 
 // The operator kernel: the leaves first (they wait for nothing), then the cells in waves whose operands are complete;
-// a grid barrier separates the waves.  fp32 FMA tiles: height by height (a cell reads states of smaller heights).
-// TC: bf16 operands on the tensor cores (the tile pipeline of rdf_tc.cuh), depth by depth from the deepest cells up.
+// a grid barrier separates the waves: depth by depth from the deepest cells up.  TC: bf16 operands on the tensor cores
+// (the tile pipeline of rdf_tc.cuh); else fp32 FMA tiles.
 // RNN32: the fp32 TreeRNN alone (no TreeLSTM code in the kernel): few enough registers for two blocks per SM, which is what
 // the FFMA tiles need to hide their shared-memory and barrier latencies.
 template <bool TC, bool RNN32 = false>
@@ -803,7 +800,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
         acc += now - t_mark;
         t_mark = now;
     };
-    const uint32_t n_leaf = min(c.ctl->leaf_count.v, c.work_cap);
+    const uint32_t n_leaf = RNN32 ? 0u : min(c.ctl->leaf_count.v, c.work_cap);     // (fp32 TreeRNN: rdf_leaf_rows_kernel wrote them)
     bool alive = true;
     if (n_leaf) {
         if constexpr (TC) {
@@ -813,11 +810,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
                 asm volatile("fence.proxy.async;" ::: "memory");      // the operand rows it wrote are read by tile copies after the barrier
             }
         } else {
-            if constexpr (RNN32) rnn_leaf_rows(c, n_leaf);
-            else {
-                if (lstm) lstm_forward_tiles<3>(c, smem, 0, n_leaf);
-                else rnn_leaf_rows(c, n_leaf);
-            }
+            if constexpr (!RNN32) lstm_forward_tiles<3>(c, smem, 0, n_leaf);
         }
         __syncthreads();
         lap(cyc_c);
@@ -843,34 +836,34 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
             lap(cyc_b);
         }
     } else {
-        // fp32 path: height by height (cell_items is the sorted list here: the launch passes cell_sorted in its place).
-        // With the clustered path the list is sorted by (group of instances, height): this kernel fires the wide heights
-        // (1 .. h_split: every group's cells of the height, then one barrier) and leaves the rest to the clusters.
-        const uint32_t groups = cell_groups(c), stride = min(c.ctl->max_height, c.wave_cap) + 1u;
-        const uint32_t top = groups > 1u ? min(c.ctl->h_split, stride - 1u) : stride - 1u;
-        for (uint32_t w = 1; w <= top && alive; ++w) {
-            bool any = false;
-            for (uint32_t gq = 0; gq < groups; ++gq) {
-                const uint32_t first = min(c.height_ends[(size_t)gq * stride + w - 1], c.work_cap);
-                const uint32_t end = min(c.height_ends[(size_t)gq * stride + w], c.work_cap);
-                if (end <= first) continue;                              // (no cell of this height in the group)
-                const uint32_t nc = end - first;
-                any = true;
-                bool done = false;
-                if constexpr (!RNN32) {
-                    if (lstm) {
-                        lstm_forward_tiles<5>(c, smem, first, nc);
-                        done = true;
-                    }
-                }
-                // thin patches while they fit in two rounds over the grid, tiles for wide waves
-                if (done) {
-                } else if (c.H <= 384 && ((nc + 7) / 8) * ((c.H + 15) / 16) <= 2 * gridDim.x)
-                    rnn_cell_thin(c, reinterpret_cast<float*>(&smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
-                else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, nc);
-                __syncthreads();
+        // fp32 path: the same order.  With the clustered path this kernel fires the wide depths (scheduler waves below
+        // d_split) and the clusters have fired the deeper ones before it.
+        uint32_t nw = min(c.ctl->n_depth_waves, c.wave_cap);
+        if (RNN32 && depth_groups(c) > 1u) {
+            uint32_t lo = 0, hi = nw;                                   // depths [0, lo) are this kernel's
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) / 2;
+                if ((__ldcg(&c.frames[c.wave_marks[mid].x].label) >> FRAME_WAVE_SHIFT) + 1u <= c.ctl->d_split) lo = mid + 1; else hi = mid;
             }
-            if (!any) continue;
+            nw = lo;
+        }
+        uint4 wv = nw ? c.wave_marks[nw - 1] : make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t k = nw; k-- > 0 && alive;) {
+            const uint4 cur = wv;
+            if (k > 0) wv = c.wave_marks[k - 1];                         // in flight during this wave
+            if (cur.w <= cur.z) continue;
+            const uint32_t first = min(cur.z, c.work_cap), nc = min(cur.w, c.work_cap) - first;
+            bool done = false;
+            if constexpr (!RNN32) {
+                lstm_forward_tiles<5>(c, smem, first, nc);
+                done = true;
+            }
+            // thin patches while they fit in two rounds over the grid, tiles for wide waves
+            if (done) {
+            } else if (c.H <= 384 && ((nc + 7) / 8) * ((c.H + 15) / 16) <= 2 * gridDim.x)
+                rnn_cell_thin(c, reinterpret_cast<float*>(&smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
+            else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, nc);
+            __syncthreads();
             lap(cyc_c);
             alive = grid_barrier(c, &c.ctl->bar_ops.v, generation);
             lap(cyc_b);
@@ -887,9 +880,9 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
 // fp32 TreeRNN cells without a grid barrier: one thread-block cluster per group of instances
 // ===========================================================================
 // Tokens of different instances never meet (matching needs equal tags, and a tag belongs to one instance), so the cells
-// of different instances do not depend on one another.  The ready cells are sorted by (group of their instance,
-// height); a cluster of CLUSTER_CTAS blocks fires the cells of its group height by height and synchronises with the
-// hardware cluster barrier only -- a deep, thin recursion (a wave of a few dozen cells, thousands of waves) pays about
+// of different instances do not depend on one another.  The cells are sorted by (group of their instance, call
+// depth); a cluster of CLUSTER_CTAS blocks fires the cells of its group depth by depth, deepest first, and synchronises
+// with the hardware cluster barrier only -- a deep, thin recursion (a wave of a few dozen cells, thousands of waves) pays about
 // a microsecond per wave instead of a barrier over the whole grid.  The blocks of a cluster split the columns of W
 // (kept in shared memory for the whole kernel); a block step computes `cells_per_step` cells x its columns, thread =
 // (cell, column), operand rows staged in shared memory.  States travel between the blocks through global memory
@@ -903,7 +896,7 @@ __global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __gr
     constexpr int CS = 256 / CPC;              // cells per step = slices of k
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     // every block of the grid takes the same decision from the same words: no block of a cluster is left waiting
-    if (c.ctl->forward_status != 0 || cell_groups(c) <= 1u) return;
+    if (c.ctl->forward_status != 0 || c.ctl->status != 0 || depth_groups(c) <= 1u) return;
     const int H = c.H, K2 = 2 * c.H;
     const int rank = blockIdx.x % CLUSTER_CTAS, group = blockIdx.x / CLUSTER_CTAS;
     const int j0 = rank * CPC;
@@ -916,8 +909,8 @@ __global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __gr
         wres[q] = j0 + jj < H ? __ldg(&c.W[(size_t)(j0 + jj) * K2 + k]) : 0.f;
     }
     __syncthreads();
-    const uint32_t stride = min(c.ctl->max_height, c.wave_cap) + 1u, top = stride - 1u;
-    const uint32_t* ends = c.height_ends + (size_t)group * stride;      // ends[h]: end of (group, h); ends[0]: start of the group
+    const uint32_t stride = depth_stride(c), top = stride - 1u;
+    const uint32_t* ends = c.group_ends + (size_t)group * stride;       // ends[d]: end of (group, depth d); ends[0]: start of the group
     const int jj = threadIdx.x % CPC, ks = threadIdx.x / CPC;           // column; slice of k (contraction) / cell (reduction)
     const bool active = ks < CS;
     const int klen = ((K2 + CS - 1) / CS + 3) & ~3, k_begin = ks * klen, k_end = min(K2, k_begin + klen);
@@ -932,28 +925,28 @@ __global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __gr
             const int r = p / (K2 / 4), k = (p % (K2 / 4)) * 4;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if ((uint32_t)r < n) {
-                const uint4 it = pre && p == (int)threadIdx.x ? *pre : __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + r]));   // {out, l, r, height}
+                const uint4 it = pre && p == (int)threadIdx.x ? *pre : __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + r]));   // {out, l, r, valid}
                 v = k < H ? ldcg4(c.arena + (size_t)it.y * H + k) : ldcg4(c.arena + (size_t)it.z * H + (k - H));
                 if (k == 0) s_out[buf * CS + r] = it.x;
             }
             *reinterpret_cast<float4*>(dst + (size_t)r * K2 + k) = v;
         }
     };
-    const uint32_t h0 = min(c.ctl->h_split, top);                     // (the grid-wide kernel fired heights 1 .. h0)
-    uint32_t begin = min(ends[h0], c.work_cap);
-    uint32_t end_next = top > h0 ? min(ends[h0 + 1], c.work_cap) : begin;
+    const uint32_t d0 = min(c.ctl->d_split, top);                      // (the grid-wide kernel fires depths d0 .. 1 afterwards)
+    uint32_t begin_next = top > d0 ? min(ends[top - 1], c.work_cap) : 0u, end_next = top > d0 ? min(ends[top], c.work_cap) : 0u;
     // the list is complete before the kernel starts: the record this thread needs first in the next wave is fetched a wave ahead
     const int my_row = threadIdx.x / (K2 / 4);
     uint4 rec_next = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x < pieces && begin + my_row < end_next) rec_next = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[begin + my_row]));
-    for (uint32_t h = h0 + 1; h <= top; ++h) {
-        const uint32_t end = end_next;
-        if (h < top) end_next = min(ends[h + 1], c.work_cap);           // in flight during this wave
-        // the cells of (group, h), CS at a time; the next step's rows are fetched while this one computes
+    if (threadIdx.x < pieces && begin_next + my_row < end_next) rec_next = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[begin_next + my_row]));
+    for (uint32_t d = top; d > d0; --d) {
+        const uint32_t begin = begin_next, end = end_next;
+        end_next = begin;
+        if (d - 1 > d0) begin_next = min(ends[d - 2], c.work_cap);      // in flight during this wave
+        // the cells of (group, d), CS at a time; the next step's rows are fetched while this one computes
         int buf = 0;
         const uint4 rec = rec_next;
         if (end > begin) stage(0, begin, min((uint32_t)CS, end - begin), &rec);
-        if (threadIdx.x < pieces && end + my_row < end_next) rec_next = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[end + my_row]));
+        if (threadIdx.x < pieces && begin_next + my_row < end_next) rec_next = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[begin_next + my_row]));
         for (uint32_t first = begin; first < end; first += CS) {
             const uint32_t n = min((uint32_t)CS, end - first);
             __syncthreads();                                            // rows of this step are in place, `part` is free
@@ -984,9 +977,8 @@ __global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __gr
             }
             buf ^= 1;
         }
-        begin = end;
         __syncthreads();
-        cluster_sync_all();                                             // the states of height h are complete for the whole cluster
+        cluster_sync_all();                                             // the states of depth d are complete for the whole cluster
     }
 }
 
@@ -997,43 +989,40 @@ inline size_t cluster_smem_bytes(int H) {
 }
 static const int CLUSTER_MAX_H = 384;
 
-// ---- cells grouped by height (between the scheduler and the operator kernel)
-// The scheduler finds a cell ready in the wave in which its second operand returns, which depends on how deep the
-// whole tree below it reaches; what the arithmetic needs is only that operands come first.  Grouping the cells by
-// height gives the smallest number of dependent operator waves (the largest height instead of about twice the depth).
-// (With the clustered operator kernel the cells are grouped by (cluster of their instance, height): bucket index
-// group * (max height + 1) + height; one group otherwise.  The largest height is known from the scheduler.)
-__device__ __forceinline__ uint32_t cell_bucket(const DevCtx& c, const CellItem& it, uint32_t groups, uint32_t stride, int by_depth) {
-    if (it.height == 0u) return 0u;                                                  // (0: not a cell)
-    // by_depth (gradient pass): the scheduler wave that created the cell's frame, + 1
-    const uint32_t h = min(by_depth ? (__ldcg(&c.frames[it.out].label) >> FRAME_WAVE_SHIFT) + 1u : it.height, stride - 1u);
-    return (groups > 1u ? __ldcg(&c.finst[it.out]) % groups : 0u) * stride + h;
+// ---- cells grouped for the clustered kernels: bucket (cluster of their instance) * stride + call depth
+__device__ __forceinline__ uint32_t cell_bucket(const DevCtx& c, const uint4& it, uint32_t groups, uint32_t stride) {    // {cell, left, right, valid}
+    if (it.w == 0u) return 0u;
+    // call depth: the scheduler wave that created the cell's frame, + 1
+    const uint32_t d = min((__ldcg(&c.frames[it.x].label) >> FRAME_WAVE_SHIFT) + 1u, stride - 1u);
+    return (__ldcg(&c.finst[it.x]) % groups) * stride + d;
 }
 
-__global__ void __launch_bounds__(256) rdf_height_count_kernel(const DevCtx c, int by_depth) {
+__global__ void __launch_bounds__(256) rdf_group_count_kernel(const DevCtx c) {
     if (c.ctl->status != 0) return;
-    const uint32_t n = min(c.ctl->cell_count.v, c.work_cap), lane = threadIdx.x % 32;
-    const uint32_t groups = bucket_groups(c, by_depth), stride = bucket_stride(c, by_depth);
+    const uint32_t n = min(c.ctl->all_cells, c.work_cap), lane = threadIdx.x % 32;
+    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
+    if (groups <= 1u) return;
     for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * blockDim.x) {
         const uint32_t i = i0 + lane;
-        const uint32_t k = i < n ? cell_bucket(c, c.cell_items[i], groups, stride, by_depth) : 0u;
+        const uint32_t k = i < n ? cell_bucket(c, c.cell_ops[i], groups, stride) : 0u;
         const unsigned peers = __match_any_sync(0xffffffffu, k);                      // one atomic per bucket and warp
-        if (k && (uint32_t)(__ffs(peers) - 1) == lane) atomicAdd(&c.height_ends[k], (uint32_t)__popc(peers));
+        if (k && (uint32_t)(__ffs(peers) - 1) == lane) atomicAdd(&c.group_ends[k], (uint32_t)__popc(peers));
     }
 }
 
-// counts -> first position of each bucket (one block; buckets 1 .. groups * (max height + 1) - 1)
-__global__ void __launch_bounds__(1024) rdf_height_scan_kernel(const DevCtx c, int by_depth) {
+// counts -> first position of each bucket (one block; buckets 1 .. groups * stride - 1)
+__global__ void __launch_bounds__(1024) rdf_group_scan_kernel(const DevCtx c) {
     __shared__ uint32_t warp_sum[32];
     __shared__ uint32_t carry;
     if (c.ctl->status != 0) return;
-    const uint32_t top = bucket_groups(c, by_depth) * bucket_stride(c, by_depth) - 1u;
+    if (depth_groups(c) <= 1u) return;
+    const uint32_t top = depth_groups(c) * depth_stride(c) - 1u;
     const uint32_t lane = threadIdx.x % 32, warp = threadIdx.x / 32;
     if (threadIdx.x == 0) carry = 0;
     __syncthreads();
     for (uint32_t h0 = 1; h0 <= top; h0 += 1024) {
         const uint32_t h = h0 + threadIdx.x;
-        const uint32_t v = h <= top ? c.height_ends[h] : 0u;
+        const uint32_t v = h <= top ? c.group_ends[h] : 0u;
         uint32_t x = v;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -1051,42 +1040,43 @@ __global__ void __launch_bounds__(1024) rdf_height_scan_kernel(const DevCtx c, i
         }
         __syncthreads();
         const uint32_t before = carry + (warp ? warp_sum[warp - 1] : 0u) + x - v;
-        if (h <= top) c.height_ends[h] = before;
+        if (h <= top) c.group_ends[h] = before;
         __syncthreads();
         if (threadIdx.x == 1023) carry = before + v;
         __syncthreads();
     }
 }
 
-// every cell to its bucket; afterwards height_ends[k] is where bucket k ends (it starts where bucket k - 1 ends;
+// every cell to its bucket; afterwards group_ends[k] is where bucket k ends (it starts where bucket k - 1 ends;
 // bucket group * stride + 0 is empty, so it ends where the previous group ends)
-__global__ void __launch_bounds__(256) rdf_height_scatter_kernel(const DevCtx c, int by_depth) {
+__global__ void __launch_bounds__(256) rdf_group_scatter_kernel(const DevCtx c) {
     if (c.ctl->status != 0) return;
-    const uint32_t n = min(c.ctl->cell_count.v, c.work_cap), lane = threadIdx.x % 32;
-    const uint32_t groups = bucket_groups(c, by_depth), stride = bucket_stride(c, by_depth);
+    const uint32_t n = min(c.ctl->all_cells, c.work_cap), lane = threadIdx.x % 32;
+    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
+    if (groups <= 1u) return;
     for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * blockDim.x) {
         const uint32_t i = i0 + lane;
-        CellItem it = i < n ? c.cell_items[i] : CellItem{0u, 0u, 0u, 0u};
-        const uint32_t k = cell_bucket(c, it, groups, stride, by_depth);
+        const uint4 it = i < n ? c.cell_ops[i] : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t k = cell_bucket(c, it, groups, stride);
         const unsigned peers = __match_any_sync(0xffffffffu, k);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (k && (uint32_t)leader == lane) base = atomicAdd(&c.height_ends[k], (uint32_t)__popc(peers));
+        if (k && (uint32_t)leader == lane) base = atomicAdd(&c.group_ends[k], (uint32_t)__popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
-        if (k) c.cell_sorted[min(base + (uint32_t)__popc(peers & ((1u << lane) - 1u)), c.work_cap - 1u)] = it;
+        if (k) reinterpret_cast<uint4*>(c.cell_sorted)[min(base + (uint32_t)__popc(peers & ((1u << lane) - 1u)), c.work_cap - 1u)] = it;
     }
 }
 
-// Which heights are wide enough for the whole grid (clustered path): the last height that has more than `threshold` cells
-// over all groups; the heights above it are left to the clusters.
-__global__ void __launch_bounds__(256) rdf_height_split_kernel(const DevCtx c, uint32_t threshold, int by_depth) {
+// Which depths are wide enough for the whole grid (clustered path): up to the last one that has more than `threshold` cells
+// over all groups; the deeper ones are left to the clusters.
+__global__ void __launch_bounds__(256) rdf_group_split_kernel(const DevCtx c, uint32_t threshold) {
     if (c.ctl->status != 0) return;
-    const uint32_t groups = bucket_groups(c, by_depth), stride = bucket_stride(c, by_depth);
+    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
     if (groups <= 1u) return;
     for (uint32_t h = 1 + blockIdx.x * blockDim.x + threadIdx.x; h < stride; h += gridDim.x * blockDim.x) {
         uint32_t total = 0;
-        for (uint32_t gq = 0; gq < groups; ++gq) total += c.height_ends[(size_t)gq * stride + h] - c.height_ends[(size_t)gq * stride + h - 1];
-        if (total > threshold) atomicMax(by_depth ? &c.ctl->d_split : &c.ctl->h_split, h);
+        for (uint32_t gq = 0; gq < groups; ++gq) total += c.group_ends[(size_t)gq * stride + h] - c.group_ends[(size_t)gq * stride + h - 1];
+        if (total > threshold) atomicMax(&c.ctl->d_split, h);
     }
 }
 
@@ -1171,7 +1161,7 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.table = P.take<char>(L.table_bytes);
     L.cell_items = P.take<CellItem>(L.work_cap);
     L.leaf_items = P.take<LeafItem>(L.work_cap);
-    L.cell_sorted = P.take<CellItem>(g->has_vector_ops ? L.work_cap : 0);
+    L.cell_sorted = P.take<CellItem>(L.clustered ? L.work_cap : 0);
     const size_t vf = g->has_vector_ops ? L.frame_cap : 0;
     L.op_l = P.take<uint32_t>(vf);
     L.op_r = P.take<uint32_t>(vf);
@@ -1205,12 +1195,14 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     // every wave of a vector program holds at least one token of an invocation on its way down or up
     L.wave_cap = g->has_vector_ops ? (uint32_t)std::min<long long>(2 * (long long)L.frame_cap + 64, 1ll << 24) : 0;
     L.wave_marks = P.take<uint4>(L.wave_cap);
-    L.height_ends = P.take<uint32_t>(L.wave_cap ? (size_t)L.wave_cap + 2 : 0);
-    // the lists over the frames: the gradient pass needs them, and so do the tensor-core operator waves
-    const size_t lf = want_grad || L.use_tc ? L.frame_cap : 0;
+    L.group_ends = P.take<uint32_t>(L.clustered ? (size_t)L.wave_cap + 2 : 0);
+    L.level_cap = g->fold ? L.frame_cap / FS_CHUNK + 2 : 0;
+    L.level_counts = P.take<uint32_t>((size_t)3 * L.level_cap);
+    // the lists over the frames (the interleaved execution fires its operators as it finds them)
+    const size_t lf = g->has_vector_ops && !g->interleaved ? L.frame_cap : 0;
     L.list_seg = P.take<uint2>(lf ? (size_t)in->max_invocations / LIST_SEG + 2 : 0);
     L.all_cells = P.take<uint32_t>(lf);
-    L.cell_ops = P.take<uint4>(L.use_tc ? lf : 0);
+    L.cell_ops = P.take<uint4>(lf);
     L.leaf_ops = P.take<uint4>(tcl ? gf : 0);
     L.all_leaves = P.take<uint32_t>(g->has_lstm ? lf : gf);
     L.loss_partial = P.take<float>(want_grad ? 4096 : 0);
@@ -1299,6 +1291,10 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
     c.n_ports_total = g->n_ports_total; c.K = g->max_calls_per_body;
     c.finst = L.clustered ? reinterpret_cast<uint32_t*>(ws + L.finst) : nullptr;
     c.n_groups = L.clustered && S->n_clusters > 1 ? S->n_clusters : 0;
+    for (int k = 0; k < 3; ++k) c.fold_label[k] = g->fold_label[k];
+    for (int k = 0; k < 2; ++k) c.fold_right[k] = g->fold_right[k];
+    c.level_counts = reinterpret_cast<uint32_t*>(ws + L.level_counts);
+    c.level_cap = L.level_cap;
     c.has_loops = g->has_loops ? 1 : 0;
     c.frame_ptag = g->has_loops ? reinterpret_cast<uint64_t*>(ws + L.frame_ptag) : nullptr;
     c.B = in->B; c.N = in->N; c.x = in->x;
@@ -1315,7 +1311,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
     c.table_cap = L.table_cap;
     c.cell_items = reinterpret_cast<CellItem*>(ws + L.cell_items);
     c.cell_sorted = reinterpret_cast<CellItem*>(ws + L.cell_sorted);
-    c.height_ends = reinterpret_cast<uint32_t*>(ws + L.height_ends);
+    c.group_ends = reinterpret_cast<uint32_t*>(ws + L.group_ends);
     c.leaf_items = reinterpret_cast<LeafItem*>(ws + L.leaf_items);
     c.work_cap = L.work_cap;
     c.op_l = reinterpret_cast<uint32_t*>(ws + L.op_l);
@@ -1353,7 +1349,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
     c.wave_marks = L.wave_cap ? reinterpret_cast<uint4*>(ws + L.wave_marks) : nullptr;
     c.wave_cap = L.wave_cap;
     c.all_cells = reinterpret_cast<uint32_t*>(ws + L.all_cells);
-    c.cell_ops = L.use_tc ? reinterpret_cast<uint4*>(ws + L.cell_ops) : nullptr;
+    c.cell_ops = g->has_vector_ops ? reinterpret_cast<uint4*>(ws + L.cell_ops) : nullptr;
     c.leaf_ops = L.use_tc && g->has_lstm && L.want_grad ? reinterpret_cast<uint4*>(ws + L.leaf_ops) : nullptr;
     c.all_leaves = reinterpret_cast<uint32_t*>(ws + L.all_leaves);
     c.loss_partial = reinterpret_cast<float*>(ws + L.loss_partial);
@@ -1399,14 +1395,19 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     rdf_mark(S, 0, stream);
     S->launches = 0;
     CUDA_OK(cudaMemsetAsync(ws + L.ctl, 0, 4096, stream));
-    if (L.wave_cap) CUDA_OK(cudaMemsetAsync(ws + L.height_ends, 0, ((size_t)L.wave_cap + 2) * sizeof(uint32_t), stream));
-    if (g->tag_mode == RDF_TAGS_FRAME) {
+    // Structural recursion over the input trees has its own scheduler; a traced call records every firing of the graph and
+    // goes through the general one.
+    const bool fold = g->fold && !out->trace;
+    if (fold) {
+        CUDA_OK(cudaMemsetAsync(ws + L.level_counts, 0, (size_t)3 * L.level_cap * sizeof(uint32_t), stream));
+    } else if (g->tag_mode == RDF_TAGS_FRAME) {
         bool wide = false;                        // an operator with more than two tagged inputs
         for (const MatchNode& m : g->match) wide = wide || m.n_ports > 2;
         if (L.pair_bytes) CUDA_OK(cudaMemsetAsync(ws + L.pair_slots, 0, L.pair_bytes, stream));
         if (wide && L.arrived_bytes) CUDA_OK(cudaMemsetAsync(ws + L.arrived, 0, L.arrived_bytes, stream));
     }
     if (L.table_bytes) CUDA_OK(cudaMemsetAsync(ws + L.table, 0xFF, L.table_bytes, stream));
+    if (!fold)
     {
         // the four program tables sit next to each other in the workspace (code first, constants last): one copy
         const size_t bytes = L.consts + g->consts.size() * sizeof(int64_t) - L.code;
@@ -1431,7 +1432,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         }
         CUDA_OK(cudaMemcpyAsync(ws + L.code, S->tables, bytes, cudaMemcpyHostToDevice, stream));
     }
-    RDF_KERNEL(S, rdf_seed_kernel<<<(unsigned)((in->B + 255) / 256), 256, 0, stream>>>(c));
+    if (!fold) RDF_KERNEL(S, rdf_seed_kernel<<<(unsigned)((in->B + 255) / 256), 256, 0, stream>>>(c));
     CUDA_OK(cudaGetLastError());
     if (c.use_tc) {
         if (c.lstm) {
@@ -1444,7 +1445,11 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     }
     rdf_mark(S, 1, stream);
     void* args[] = {(void*)&c};
-    if (g->interleaved)
+    if (fold) {
+        // a run of a few chunks: one block, no grid to wait for
+        const int blocks = L.frame_cap <= FS_ONE_BLOCK ? 1 : S->grid;
+        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_fold_kernel, dim3(blocks), dim3(FS_CHUNK), args, 0, stream)));
+    } else if (g->interleaved)
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel, dim3(S->grid), dim3(1024), args,
                                             (size_t)interleaved_smem_bytes(c.H), stream)));
     else
@@ -1461,48 +1466,51 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         void* oargs[] = {(void*)&c};
         DevCtx co = c;
         if (c.use_tc) {
-            // the cells listed by call depth, with the operand row that every invocation's state goes to
             int rc = encode_row_tiles(&c.tmap_z128, c.z_bf, c.cells_cap, (uint64_t)2 * c.Hp, 128);
             if (rc == RDF_OK) rc = encode_row_tiles(&c.tmap_z64, c.z_bf, c.cells_cap, (uint64_t)2 * c.Hp, 64);
-            if (rc == RDF_OK) rc = rdf_launch_lists(in, ws, L, S, c, stream);
             if (rc != RDF_OK) return rc;
+        }
+        if (!fold) {                              // the cells listed by call depth (the tree scheduler made the lists itself)
+            const int rc = rdf_launch_lists(in, ws, L, S, c, stream);
+            if (rc != RDF_OK) return rc;
+        }
+        if (c.use_tc) {
             rdf_mark(S, 3, stream);
             RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<true>, dim3(S->grid), dim3(TC_THREADS), oargs,
                                                 (size_t)L.tc_smem_fwd, stream)));
         } else {
-            // the cells grouped by height; the operator kernel reads the grouped list in place of the scheduler's
-            RDF_KERNEL(S, rdf_height_count_kernel<<<2 * S->grid, 256, 0, stream>>>(c, 0));
-            RDF_KERNEL(S, rdf_height_scan_kernel<<<1, 1024, 0, stream>>>(c, 0));
-            RDF_KERNEL(S, rdf_height_scatter_kernel<<<2 * S->grid, 256, 0, stream>>>(c, 0));
-            CUDA_OK(cudaGetLastError());
+            const int rc = rdf_launch_depth_groups(ws, L, S, c, stream);
+            if (rc != RDF_OK) return rc;
             rdf_mark(S, 3, stream);
-            co.cell_items = c.cell_sorted;
-            oargs[0] = (void*)&co;
             S->last_clusters = c.n_groups > 1 ? c.n_groups : 0;
-            if (c.n_groups > 1) RDF_KERNEL(S, rdf_height_split_kernel<<<S->grid, 256, 0, stream>>>(c, 40u * (uint32_t)c.n_groups, 0));
-            // the leaves and the wide heights with the whole grid ...
+            co.cell_items = reinterpret_cast<CellItem*>(c.cell_ops);          // the operator kernels read the cells in depth order
+            oargs[0] = (void*)&co;
             if (c.lstm)
-                RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false>, dim3(S->grid), dim3(256), oargs,
-                                                    thin_resident_bytes(c.lstm, c.H), stream)));
-            else
+                RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false>, dim3(S->grid), dim3(256), oargs, 0, stream)));
+            else {
+                RDF_KERNEL(S, rdf_leaf_rows_kernel<<<8 * S->grid, 256, 0, stream>>>(c));
+                if (c.n_groups > 1) {
+                    // the narrow depths cluster by cluster of instances, deepest first (the kernel leaves at once when the
+                    // recursion is shallow or the grouped table did not fit) ...
+                    DevCtx cs = c;
+                    cs.cell_items = c.cell_sorted;
+                    cudaLaunchConfig_t cfg = {};
+                    cudaLaunchAttribute at[1];
+                    at[0].id = cudaLaunchAttributeClusterDimension;
+                    at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+                    cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.blockDim = dim3(256);
+                    cfg.dynamicSmemBytes = cluster_smem_bytes(c.H); cfg.stream = stream;
+                    cfg.attrs = at; cfg.numAttrs = 1;
+                    switch (cluster_cols_per_block(c.H)) {
+                        case 8: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<8>, cs))); break;
+                        case 16: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<16>, cs))); break;
+                        case 32: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<32>, cs))); break;
+                        default: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<48>, cs))); break;
+                    }
+                }
+                // ... the wide ones with the whole grid
                 RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false, true>, dim3(S->grid * S->rnn32_per_sm),
                                                     dim3(256), oargs, thin_resident_bytes(0, c.H), stream)));
-            if (c.n_groups > 1) {
-                // ... the narrow ones cluster by cluster of instances (the kernel leaves at once when the grouped table
-                // did not fit and the grid-wide kernel did all the work)
-                cudaLaunchConfig_t cfg = {};
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeClusterDimension;
-                at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-                cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.blockDim = dim3(256);
-                cfg.dynamicSmemBytes = cluster_smem_bytes(c.H); cfg.stream = stream;
-                cfg.attrs = at; cfg.numAttrs = 1;
-                switch (cluster_cols_per_block(c.H)) {
-                    case 8: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<8>, co))); break;
-                    case 16: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<16>, co))); break;
-                    case 32: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<32>, co))); break;
-                    default: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<48>, co))); break;
-                }
             }
         }
         rdf_mark(S, 4, stream);
@@ -1549,15 +1557,14 @@ int rdf_launch_lists(const rdf_batch* in, char* ws, const Layout& L, ExecState* 
     return RDF_OK;
 }
 
-// The cells grouped again for the clustered gradient pass: by (cluster of their instance, call depth).  Reuses the
-// grouped list and the bucket table of the forward pass, which is over.
+// The cells grouped by (cluster of their instance, call depth) for the clustered fp32 kernels, forward and gradient.
 int rdf_launch_depth_groups(char* ws, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream) {
     if (c.n_groups <= 1) return RDF_OK;
-    CUDA_OK(cudaMemsetAsync(ws + L.height_ends, 0, ((size_t)L.wave_cap + 2) * sizeof(uint32_t), stream));
-    RDF_KERNEL(S, rdf_height_count_kernel<<<2 * S->grid, 256, 0, stream>>>(c, 1));
-    RDF_KERNEL(S, rdf_height_scan_kernel<<<1, 1024, 0, stream>>>(c, 1));
-    RDF_KERNEL(S, rdf_height_scatter_kernel<<<2 * S->grid, 256, 0, stream>>>(c, 1));
-    RDF_KERNEL(S, rdf_height_split_kernel<<<S->grid, 256, 0, stream>>>(c, 40u * (uint32_t)c.n_groups, 1));
+    CUDA_OK(cudaMemsetAsync(ws + L.group_ends, 0, ((size_t)L.wave_cap + 2) * sizeof(uint32_t), stream));
+    RDF_KERNEL(S, rdf_group_count_kernel<<<2 * S->grid, 256, 0, stream>>>(c));
+    RDF_KERNEL(S, rdf_group_scan_kernel<<<1, 1024, 0, stream>>>(c));
+    RDF_KERNEL(S, rdf_group_scatter_kernel<<<2 * S->grid, 256, 0, stream>>>(c));
+    RDF_KERNEL(S, rdf_group_split_kernel<<<S->grid, 256, 0, stream>>>(c, 40u * (uint32_t)c.n_groups));
     CUDA_OK(cudaGetLastError());
     return RDF_OK;
 }

@@ -82,8 +82,8 @@ inline void rdf_mark(ExecState* S, int k, cudaStream_t stream) {
 
 struct Layout {
     size_t ctl, code, match, labels, consts, q0, q1, frames, frame_args, frame_ptag, finst, pair_slots, port_val, arrived, table, cell_items,
-        leaf_items, cell_sorted, height_ends, op_l, op_r, arena, gates, arena_bf, wp, wtp, dz_bf, z_bf, zdst, cell_pos, wxp, wxtp, e_bf, dg_bf, ybuf, dhp, dlog, wave_marks, list_seg, all_cells, cell_ops, leaf_ops, all_leaves, loss_partial, dw_partial, de_fix, head_fix, rank_tmp, node_info, canon_hist, total;
-    uint32_t qcap, frame_cap, work_cap, wave_cap, cells_cap, canon_cap;
+        leaf_items, cell_sorted, group_ends, level_counts, op_l, op_r, arena, gates, arena_bf, wp, wtp, dz_bf, z_bf, zdst, cell_pos, wxp, wxtp, e_bf, dg_bf, ybuf, dhp, dlog, wave_marks, list_seg, all_cells, cell_ops, leaf_ops, all_leaves, loss_partial, dw_partial, de_fix, head_fix, rank_tmp, node_info, canon_hist, total;
+    uint32_t qcap, frame_cap, work_cap, wave_cap, cells_cap, canon_cap, level_cap;
     int use_tc, Hp, tc_smem_fwd, tc_smem_bwd, want_grad, repro, clustered;
     uint64_t table_cap;
     size_t arrived_bytes, table_bytes, pair_bytes;
@@ -110,7 +110,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
 int rdf_check_common(rdf_graph* g, const rdf_batch* in, const rdf_params* params, rdf_outputs* out, void* ws);
 // a row-major bf16 matrix [rows, cols] as a 2D tensor map for tile copies: boxes of box_rows x 64 columns, 128-byte swizzle
 int encode_row_tiles(TensorMap* out, void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-// the lists over the frames (cells in depth order, waves, operand-row destinations); TC path: part of the forward pass
+// the lists over the frames (cells in depth order, waves, operand-row destinations)
 int rdf_launch_depth_groups(char* ws, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream);
 int rdf_launch_lists(const rdf_batch* in, char* ws, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream);
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,

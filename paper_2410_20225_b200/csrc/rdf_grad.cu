@@ -1026,8 +1026,8 @@ __global__ void __launch_bounds__(BWD_CLUSTER_THREADS, 1) rdf_backward_cluster_k
         wres[q] = j0 + jj < K2 ? __ldg(&c.W[(size_t)j * K2 + j0 + jj]) : 0.f;
     }
     __syncthreads();
-    const uint32_t stride = bucket_stride(c, 1), top = stride - 1u;
-    const uint32_t* ends = c.height_ends + (size_t)group * stride;     // ends[d]: end of (group, depth d); ends[0]: start of the group
+    const uint32_t stride = depth_stride(c), top = stride - 1u;
+    const uint32_t* ends = c.group_ends + (size_t)group * stride;     // ends[d]: end of (group, depth d); ends[0]: start of the group
     const int jj = threadIdx.x % CPC, ks = threadIdx.x / CPC;          // column; slice of the contraction (then: cell)
     const bool active = ks < CS;
     const int col = j0 + jj, cc = col < H ? col : col - H;
@@ -1399,12 +1399,7 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         if (!c.repro) RDF_KERNEL(S, rdf_loss_final_kernel<<<1, 256, 0, stream>>>(c, loss_blocks));
     }
     rdf_mark(S, 6, stream);
-    // lists of the gradient pass (cells in frame order, the waves that made calls); the tensor-core forward pass made them already
-    if (!c.use_tc) {
-        rc = rdf_launch_lists(in, ws, L, S, c, stream);
-        if (rc != RDF_OK) return rc;
-    }
-    rdf_mark(S, 7, stream);
+    rdf_mark(S, 7, stream);                // (the lists are those of the forward pass)
     // gradient waves
     CUDA_OK(cudaGetLastError());
     void* args[] = {(void*)&c};
@@ -1413,13 +1408,9 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_backward_kernel<true>, dim3(S->grid), dim3(TC_THREADS), args,
                                             (size_t)L.tc_smem_bwd, stream)));
     } else {
-        // deep recursions: the cells grouped by (cluster of instances, call depth); the grid-wide kernel runs the wide depths,
-        // the clusters the narrow ones after them (both leave at once when there is nothing for them to do)
+        // deep recursions (cells grouped by the forward pass): the grid-wide kernel runs the wide depths, the clusters the
+        // narrow ones after them (both leave at once when there is nothing for them to do)
         const bool clusters = c.n_groups > 1 && !c.lstm && H <= 512;
-        if (clusters) {
-            rc = rdf_launch_depth_groups(ws, L, S, c, stream);
-            if (rc != RDF_OK) return rc;
-        }
         if (c.lstm) {
             CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
             RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_backward_kernel<false>, dim3(S->grid), dim3(256), args,

@@ -980,6 +980,50 @@ struct Lower {
     }
 };
 
+// Is the program a structural recursion over the input trees (see rdf_graph::fold)?
+//   result(v) = f(v)
+//   f(v) = [NODE_LOSS](IF(IS_LEAF v, leaf(TOK v), cell(f(LEFT | RIGHT v), f(LEFT | RIGHT v))), v)
+void detect_fold(const Prog& P, rdf_graph* g) {
+    const rdf_program* p = P.p;
+    if (p->n_functions != 2 || p->tag_mode != RDF_TAGS_FRAME || g->labels.size() != 3 || g->match.size() != 1) return;
+    const int R = p->result, F = 1 - R;
+    if (p->functions[F].kind != RDF_FN_FUNCTION || P.fn(R).n_params != 1 || P.fn(F).n_params != 1) return;
+    auto is_param = [&](int f, int e) { return P.ex(f, e).op == RDF_OP_PARAM; };
+    const rdf_expr& call = P.ex(R, P.fn(R).root);
+    if (call.op != RDF_OP_CALL || call.imm != F || !is_param(R, call.a)) return;
+    int e = P.fn(F).root;
+    if (P.ex(F, e).op == RDF_OP_NODE_LOSS) {
+        if (!is_param(F, P.ex(F, e).b)) return;
+        e = P.ex(F, e).a;
+    }
+    const rdf_expr& branch = P.ex(F, e);
+    if (branch.op != RDF_OP_IF) return;
+    const rdf_expr &cond = P.ex(F, branch.a), &leaf = P.ex(F, branch.b), &cell = P.ex(F, branch.c);
+    if (cond.op != RDF_OP_IS_LEAF || !is_param(F, cond.a)) return;
+    const bool rnn = leaf.op == RDF_OP_EMBED && cell.op == RDF_OP_CELL_RNN, lstm = leaf.op == RDF_OP_LEAF_LSTM && cell.op == RDF_OP_CELL_LSTM;
+    if (!rnn && !lstm) return;
+    if (P.ex(F, leaf.a).op != RDF_OP_TOK || !is_param(F, P.ex(F, leaf.a).a)) return;
+    if (cell.a == cell.b) return;
+    const int calls[2] = {cell.a, cell.b};
+    int32_t right[2], label[3] = {-1, -1, -1};
+    for (int k = 0; k < 2; ++k) {
+        const rdf_expr& x = P.ex(F, calls[k]);
+        if (x.op != RDF_OP_CALL || x.imm != F) return;
+        const rdf_expr& arg = P.ex(F, x.a);
+        if ((arg.op != RDF_OP_LEFT && arg.op != RDF_OP_RIGHT) || !is_param(F, arg.a)) return;
+        right[k] = arg.op == RDF_OP_RIGHT;
+    }
+    for (int i = 0; i < 3; ++i) {                       // the label of the call that feeds each operand port; the third is `result`'s
+        const LabelInfo& L = g->labels[i];
+        const int at = L.k_kind == K_PORT ? L.k_port : 2;
+        if (at < 0 || at > 2 || label[at] >= 0) return;
+        label[at] = i;
+    }
+    for (int k = 0; k < 3; ++k) g->fold_label[k] = label[k];
+    for (int k = 0; k < 2; ++k) g->fold_right[k] = right[k];
+    g->fold = true;
+}
+
 }  // namespace
 
 extern "C" int rdf_graph_build(const rdf_program* prog, rdf_graph** out_graph) {
@@ -995,6 +1039,7 @@ extern "C" int rdf_graph_build(const rdf_program* prog, rdf_graph** out_graph) {
         build_literal(P, g);
         Lower L{P, g};
         L.run();
+        detect_fold(P, g);
     } catch (const Err& e) {
         delete g;
         return e.code;

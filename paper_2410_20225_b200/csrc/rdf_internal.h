@@ -98,6 +98,10 @@ struct rdf_graph {
     bool has_rnn = false, has_lstm = false, has_loss = false;
     bool uses_tree = false;
     bool has_loops = false;
+    // structural recursion over the input trees (rdf_fold.cuh): f(v) = leaf(tok v) or cell(f(child), f(child)), result(v) = f(v)
+    bool fold = false;
+    int32_t fold_label[3] = {0, 0, 0};    // label ids of the calls of operand 0 and operand 1 and of `result`'s call
+    int32_t fold_right[2] = {0, 1};       // the child that operand 0 / 1 descends into: 0 left, 1 right
     bool interleaved = false;     // some Switch reads a vector value: operators run between the token waves
     std::vector<std::string> func_names;
     // per-run state owned by the executor (rdf_exec.cu)

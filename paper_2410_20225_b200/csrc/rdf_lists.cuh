@@ -139,6 +139,22 @@ __global__ void __launch_bounds__(256) rdf_list_fill_kernel(const DevCtx c, cons
     }
 }
 
+// The weight gradient reads dz and the operand rows in whole stages of 64 rows: the rows after the last cell are zero
+// (one block).
+__device__ __forceinline__ void zero_tail_rows(const DevCtx& c, uint32_t n_cells) {
+    const uint32_t n = min(n_cells, c.cells_cap), n_end = min((n + 63u) & ~63u, c.cells_cap);
+    if (c.dz_bf) {
+        const uint32_t per_row = (uint32_t)c.Hp / 8;
+        for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
+            *reinterpret_cast<uint4*>(c.dz_bf + (size_t)(n + q / per_row) * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (c.z_bf) {
+        const uint32_t per_row = (uint32_t)c.Hp / 4;
+        for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
+            *reinterpret_cast<uint4*>(c.z_bf + (size_t)(n + q / per_row) * 2 * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
 // marks[d].w = cells among the frames below marks[d].x: where wave d ends in all_cells.  One warp per wave.
 __global__ void __launch_bounds__(256) rdf_list_ends_kernel(const DevCtx c, const uint2* seg_base) {
     if (c.ctl->status != 0) return;                    // an earlier kernel of this call failed: its lists and rows are not to be trusted
@@ -153,20 +169,7 @@ __global__ void __launch_bounds__(256) rdf_list_ends_kernel(const DevCtx c, cons
         for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         if (lane == 0) c.wave_marks[d].w = seg_base[seg].x + cnt;
     }
-    // the weight gradient reads dz and the operand rows in whole stages of 64 rows: the rows after the last cell are zero
-    if (blockIdx.x == 0) {
-        const uint32_t n = min(c.ctl->all_cells, c.cells_cap), n_end = min((n + 63u) & ~63u, c.cells_cap);
-        if (c.dz_bf) {
-            const uint32_t per_row = (uint32_t)c.Hp / 8;
-            for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
-                *reinterpret_cast<uint4*>(c.dz_bf + (size_t)(n + q / per_row) * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (c.z_bf) {
-            const uint32_t per_row = (uint32_t)c.Hp / 4;
-            for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
-                *reinterpret_cast<uint4*>(c.z_bf + (size_t)(n + q / per_row) * 2 * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
+    if (blockIdx.x == 0) zero_tail_rows(c, c.ctl->all_cells);
 }
 
 // Where an invocation's state goes besides its own row: the operand row of the cell that called it
@@ -361,7 +364,10 @@ __global__ void __launch_bounds__(1024) rdf_wave_compact_kernel(const DevCtx c) 
         if (warp) { p_cnt += w_cnt[warp - 1]; p_f = max(p_f, w_f[warp - 1]); p_c = max(p_c, w_c[warp - 1]); }
         p_cnt += carry_cnt; p_f = max(p_f, carry_f); p_c = max(p_c, carry_c);
         __syncthreads();                                                   // every thread has read its wave and the carries
-        if (has) c.wave_marks[p_cnt] = make_uint4(p_f, m.x, p_c, m.w);
+        if (has) {
+            c.wave_marks[p_cnt] = make_uint4(p_f, m.x, p_c, m.w);
+            atomicMax(&c.ctl->call_waves, d + 1u);
+        }
         if (threadIdx.x == 1023) { carry_cnt = p_cnt + has; carry_f = max(p_f, m.x); carry_c = max(p_c, ce); }
         __syncthreads();
     }

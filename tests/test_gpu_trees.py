@@ -9,6 +9,7 @@ import pytest
 
 import workloads
 import paper_2410_20225_b200 as rdf
+from paper_2410_20225_b200 import binding as bd
 from oracle import direct
 
 torch = pytest.importorskip("torch")
@@ -444,3 +445,38 @@ def test_depth_stress_config5_full_size_gradients():
     st, errs = check_grad(workloads.config(5), rdf.F32, workers=WORKERS)
     print("config 5 errors:", errs)
     assert st["waves_backward"] >= 4096
+
+
+@pytest.mark.parametrize("cell", ["rnn", "lstm"])
+@pytest.mark.parametrize("B,leaves", [(1, 700), (3, 1), (511, 5), (512, 6), (513, 3), (700, 20), (40, 400), (5, 2600)])
+def test_structural_scheduler_matches_the_general_one(cell, B, leaves):
+    """Structural recursion over the input trees is scheduled level by level (512 records per chunk; one block while a
+    level or the whole run is small); a traced call goes through the token scheduler.  Same counts, and the same root
+    states bit for bit (every state is one fixed expression), with levels at the edges of a chunk, levels that grow past
+    a chunk and shrink again, and with the operands descending right child first."""
+    rng = np.random.default_rng(B * 1000 + leaves)
+    shapes = [workloads.random_split_shape(rng, int(rng.integers(max(1, leaves // 2), leaves + 1))) for _ in range(B)]
+    if B == 5:
+        shapes.append(workloads.chain_tree_shape(150))
+    tb = workloads.tree_batch_from_shapes(shapes, 7, vocab=50)
+    p = (workloads.treernn_params if cell == "rnn" else workloads.treelstm_params)(7, 50, 8, 8)
+    dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(p)
+    fs, r = rdf.tree_net_program(cell)
+    for swapped in (False, True):
+        if swapped:
+            ops = fs[1].exprs
+            fs[1].exprs = [(bd.OP_RIGHT if e[0] == bd.OP_LEFT else bd.OP_LEFT if e[0] == bd.OP_RIGHT else e[0],) + tuple(e[1:]) for e in ops]
+        g = rdf.Graph(fs, r, rdf.TAGS_FRAME)
+        h, _ = g.eval_trees(dt, dp)
+        st = g.stats()
+        h2, _ = g.eval_trees(dt, dp, trace_capacity=2 * tb.N)
+        st2 = g.stats()
+        assert torch.equal(h, h2)
+        for k in ("invocations", "cells", "leaves", "waves", "tokens", "store_inserts", "store_matches"):
+            assert st[k] == st2[k], k
+    g.set_limits(wave_limit=st["waves"] - 1)
+    with pytest.raises(rdf.RdfError) as e:
+        g.eval_trees(dt, dp)
+    assert e.value.code == -8                     # RDF_ERR_WAVE_LIMIT, as from the token scheduler
+    g.set_limits(wave_limit=st["waves"])
+    assert torch.equal(g.eval_trees(dt, dp)[0], h)
