@@ -45,7 +45,7 @@ WORKLOAD_NAMES = {
 }
 CELL = {"treernn": "rnn", "treelstm": "lstm"}
 KERNEL_SOURCES = ["rdf_device.cuh", "rdf_exec.cu", "rdf_exec.h", "rdf_grad.cu", "rdf_internal.h", "rdf_lists.cuh", "rdf_lstm.cuh",
-                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh"]
+                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh", "rdf_cluster.cuh"]
 
 
 def fib_iter(n):
@@ -514,9 +514,6 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     if case.grad:
         rowbytes = Hp * 2 if case.use_tc else H * 4 * (2 if lstm else 1)
         add("rdf_loss_heads_kernel", "loss", "hbm", float(N) * (rowbytes + 32), "one state row read + 32 B of dlog written per invocation")
-        if not case.use_tc:
-            add("rdf_list_count/scan/fill/ends/compact_kernel", "lists", "hbm", N * 28.0 + C * 24.0,
-                "operand ids and frame records read (two passes), cell lists written")
         bwd = C * 2.0 * H * (2 * H) * (5 if lstm else 1)
         add("rdf_backward_kernel", "backward", mm, bwd, "operand-gradient contraction W^T dz: 2*H*2H per cell" + (" (x5 gates)" if lstm else ""))
         dw = bwd + (Lf * 2.0 * H * 3 * H if lstm else 0.0)

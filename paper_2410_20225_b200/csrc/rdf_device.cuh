@@ -136,6 +136,7 @@ struct DevCtx {
     // batched operators
     CellItem* cell_items;         // every cell in the order it became ready (general scheduler)
     CellItem* cell_sorted;        // clustered fp32 path: the cells grouped by (cluster of their instance, call depth)
+    uint4*    cell_link;          // [work_cap] per grouped cell: where its operands come from and its state goes (rdf_group_link_kernel)
     uint32_t* group_ends;         // [wave_cap + 2]: cells per group, then (after the scatter) the end of each group
     LeafItem* leaf_items;         // every leaf in the order it was reached
     uint32_t  work_cap;
@@ -150,7 +151,8 @@ struct DevCtx {
     __nv_bfloat16* WTp;           // [2Hp, Hp]   gradient operand
     __nv_bfloat16* dz_bf;         // [frame_cap, Hp] bf16 dz rows of the cells (rdf_grad), row = position of the cell in
                                   // all_cells: the cells of a gradient wave are consecutive rows, read as plain 2D tiles
-    uint32_t* cell_pos;           // per frame: position of a cell in all_cells (written with the lists; leaves: undefined)
+    uint32_t* cell_pos;           // per frame: position of a cell in all_cells (written with the lists; leaves: undefined);
+                                  // clustered fp32 path: in the grouped list
     TensorMap tmap_dz128, tmap_dz64;   // dz_bf as [rows, Hp], 128-byte swizzle, boxes of 128 / 64 rows by 64 columns
     __nv_bfloat16* z_bf;          // [cells_cap, 2Hp] operand rows [h_l ; h_r] of the cells, row = position of the cell in
                                   // all_cells: every invocation writes its state into the half of its caller's row

@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "rdf_exec.h"
+#include "rdf_cluster.cuh"
 #include "rdf_lists.cuh"
 #include "rdf_fold.cuh"
 #include "rdf_lstm.cuh"
@@ -877,22 +878,15 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
 }
 
 // ===========================================================================
-// fp32 TreeRNN cells without a grid barrier: one thread-block cluster per group of instances
+// fp32 TreeRNN cells without a grid barrier, hidden sizes beyond those of rdf_cluster.cuh
 // ===========================================================================
-// Tokens of different instances never meet (matching needs equal tags, and a tag belongs to one instance), so the cells
-// of different instances do not depend on one another.  The cells are sorted by (group of their instance, call
-// depth); a cluster of CLUSTER_CTAS blocks fires the cells of its group depth by depth, deepest first, and synchronises
-// with the hardware cluster barrier only -- a deep, thin recursion (a wave of a few dozen cells, thousands of waves) pays about
-// a microsecond per wave instead of a barrier over the whole grid.  The blocks of a cluster split the columns of W
-// (kept in shared memory for the whole kernel); a block step computes `cells_per_step` cells x its columns, thread =
-// (cell, column), operand rows staged in shared memory.  States travel between the blocks through global memory
-// (L2): the cluster barrier's release / acquire orders them.
-
+// The same split (cells by (group of instances, call depth), a cluster of CLUSTER_CTAS blocks per group), with the weights
+// in shared memory -- 48 columns x 2H do not fit the registers -- and the states travelling through global memory.
 // CPC: columns of W per block (8 blocks x CPC >= H).  A block step fires CS = 256 / CPC cells: thread = (column, slice
 // of the contraction index), CS accumulators per thread -- a weight is read from shared memory once per step and an
 // operand word once per warp; the slices are added up through shared memory by thread = (cell, column).
 template <int CPC>
-__global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __grid_constant__ DevCtx c) {
+__global__ void __launch_bounds__(256, 1) rdf_operator_cluster_wide_kernel(const __grid_constant__ DevCtx c) {
     constexpr int CS = 256 / CPC;              // cells per step = slices of k
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     // every block of the grid takes the same decision from the same words: no block of a cluster is left waiting
@@ -982,9 +976,9 @@ __global__ void __launch_bounds__(256, 1) rdf_operator_cluster_kernel(const __gr
     }
 }
 
-inline int cluster_cols_per_block(int H) { return H <= 64 ? 8 : H <= 128 ? 16 : H <= 256 ? 32 : 48; }
-inline size_t cluster_smem_bytes(int H) {
-    const int CPC = cluster_cols_per_block(H), CS = 256 / CPC, K2 = 2 * H;
+static const int CLUSTER_WIDE_CPC = 48;
+inline size_t cluster_wide_smem_bytes(int H) {
+    const int CPC = CLUSTER_WIDE_CPC, CS = 256 / CPC, K2 = 2 * H;
     return ((size_t)K2 * CPC + (size_t)2 * CS * K2 + (size_t)CS * CS * CPC) * sizeof(float) + 2 * CS * sizeof(uint32_t);
 }
 static const int CLUSTER_MAX_H = 384;
@@ -1063,7 +1057,11 @@ __global__ void __launch_bounds__(256) rdf_group_scatter_kernel(const DevCtx c) 
         uint32_t base = 0;
         if (k && (uint32_t)leader == lane) base = atomicAdd(&c.group_ends[k], (uint32_t)__popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
-        if (k) reinterpret_cast<uint4*>(c.cell_sorted)[min(base + (uint32_t)__popc(peers & ((1u << lane) - 1u)), c.work_cap - 1u)] = it;
+        if (k) {
+            const uint32_t at = min(base + (uint32_t)__popc(peers & ((1u << lane) - 1u)), c.work_cap - 1u);
+            reinterpret_cast<uint4*>(c.cell_sorted)[at] = it;
+            c.cell_pos[it.x] = at;
+        }
     }
 }
 
@@ -1078,6 +1076,48 @@ __global__ void __launch_bounds__(256) rdf_group_split_kernel(const DevCtx c, ui
         for (uint32_t gq = 0; gq < groups; ++gq) total += c.group_ends[(size_t)gq * stride + h] - c.group_ends[(size_t)gq * stride + h - 1];
         if (total > threshold) atomicMax(&c.ctl->d_split, h);
     }
+}
+
+// Per grouped cell below the split, for the clusters that fire it: x, y = its left and right operand: 1 << 31 | token id of a
+// leaf, else the place of that cell among the cells of its (group, depth), at most CL_NO_SLOT; z = the place of the calling
+// cell, | the operand port << 6.  The clusters hand states on from one depth to the next: a program whose operands lie
+// further apart than one call depth (calls that waited for other calls) is left to the grid-wide kernels.
+__global__ void __launch_bounds__(256) rdf_group_link_kernel(const DevCtx c) {
+    if (c.ctl->status != 0) return;
+    const uint32_t groups = depth_groups(c), stride = depth_stride(c), split = c.ctl->d_split;
+    if (groups <= 1u) return;
+    const uint32_t n = min(c.ctl->all_cells, c.work_cap), B = (uint32_t)c.B;
+    auto depth_of = [&](uint32_t f) { return (c.frames[f].label >> FRAME_WAVE_SHIFT) + 1u; };
+    auto place = [&](uint32_t f) {
+        const uint32_t k = cell_bucket(c, make_uint4(f, 0u, 0u, 1u), groups, stride);
+        return min(c.cell_pos[f] - c.group_ends[k - 1u], CL_NO_SLOT);
+    };
+    bool regular = true;
+    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        const uint4 it = reinterpret_cast<const uint4*>(c.cell_sorted)[p];
+        const uint32_t d = depth_of(it.x);
+        uint4 link = make_uint4(CL_NO_SLOT, CL_NO_SLOT, CL_NO_SLOT, 0u);
+        if (d > split) {
+            const uint32_t ch[2] = {it.y, it.z};
+            uint32_t w[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (c.op_l[ch[q]] == LEAF_MARK) w[q] = 0x80000000u | c.op_r[ch[q]];
+                else {
+                    w[q] = place(ch[q]);
+                    regular = regular && depth_of(ch[q]) == d + 1u;
+                }
+            }
+            link.x = w[0]; link.y = w[1];
+            const uint32_t parent = c.frames[it.x].parent;
+            if (parent >= B && parent < c.frame_cap && c.op_l[parent] != LEAF_MARK) {
+                link.z = place(parent) | (c.op_l[parent] == it.x ? 0u : 64u);
+                regular = regular && depth_of(parent) + 1u == d;
+            } else regular = regular && d == 1u;
+        }
+        c.cell_link[p] = link;
+    }
+    if (!regular) atomicMax(&c.ctl->d_split, stride - 1u);
 }
 
 // root states: h_root[b] = state(frame y[b])
@@ -1162,6 +1202,7 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.cell_items = P.take<CellItem>(L.work_cap);
     L.leaf_items = P.take<LeafItem>(L.work_cap);
     L.cell_sorted = P.take<CellItem>(L.clustered ? L.work_cap : 0);
+    L.cell_link = P.take<uint4>(L.clustered ? L.work_cap : 0);
     const size_t vf = g->has_vector_ops ? L.frame_cap : 0;
     L.op_l = P.take<uint32_t>(vf);
     L.op_r = P.take<uint32_t>(vf);
@@ -1181,7 +1222,7 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.dz_bf = P.take<__nv_bfloat16>(tcr && want_grad ? (size_t)L.cells_cap * L.Hp : 0);
     L.z_bf = P.take<__nv_bfloat16>(L.use_tc ? (size_t)L.cells_cap * 2 * L.Hp : 0);
     L.zdst = P.take<uint32_t>(L.use_tc ? vf : 0);
-    L.cell_pos = P.take<uint32_t>(L.use_tc ? vf : 0);
+    L.cell_pos = P.take<uint32_t>(L.use_tc || L.clustered ? vf : 0);
     L.wxp = P.take<__nv_bfloat16>(tcl ? (size_t)3 * L.Hp * L.Hp : 0);
     L.wxtp = P.take<__nv_bfloat16>(tcl ? (size_t)3 * L.Hp * L.Hp : 0);
     L.e_bf = P.take<__nv_bfloat16>(tcl ? (size_t)params->V * L.Hp : 0);
@@ -1258,19 +1299,22 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     // the clustered fp32 operator kernel: how many clusters of CLUSTER_CTAS blocks the device holds at once
     S->n_clusters = 0;
     {
-        const size_t smem = cluster_smem_bytes(CLUSTER_MAX_H);
-        bool ok = cudaFuncSetAttribute(rdf_operator_cluster_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem_bytes(64)) == cudaSuccess &&
-                  cudaFuncSetAttribute(rdf_operator_cluster_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem_bytes(128)) == cudaSuccess &&
-                  cudaFuncSetAttribute(rdf_operator_cluster_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem_bytes(256)) == cudaSuccess &&
-                  cudaFuncSetAttribute(rdf_operator_cluster_kernel<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+        const size_t wide = cluster_wide_smem_bytes(CLUSTER_MAX_H), narrow = cl_smem_bytes<32, 32>(false);
+        bool ok = cudaFuncSetAttribute(rdf_operator_cluster_kernel<16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes<16, 8>(false)) == cudaSuccess &&
+                  cudaFuncSetAttribute(rdf_operator_cluster_kernel<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)narrow) == cudaSuccess &&
+                  cudaFuncSetAttribute(rdf_operator_cluster_wide_kernel<CLUSTER_WIDE_CPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide) == cudaSuccess;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3((sms / CLUSTER_CTAS) * CLUSTER_CTAS); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = smem;
+        cfg.gridDim = dim3((sms / CLUSTER_CTAS) * CLUSTER_CTAS); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = wide;
         cfg.attrs = at; cfg.numAttrs = 1;
-        int n = 0;
-        if (ok && cudaOccupancyMaxActiveClusters(&n, rdf_operator_cluster_kernel<48>, &cfg) == cudaSuccess)
+        int n = 0, m = 0;
+        ok = ok && cudaOccupancyMaxActiveClusters(&n, rdf_operator_cluster_wide_kernel<CLUSTER_WIDE_CPC>, &cfg) == cudaSuccess;
+        cfg.blockDim = dim3(CL_THREADS); cfg.dynamicSmemBytes = narrow;
+        ok = ok && cudaOccupancyMaxActiveClusters(&m, rdf_operator_cluster_kernel<32, 32>, &cfg) == cudaSuccess;
+        n = std::min(n, m);
+        if (ok)
             S->n_clusters = std::min(n, sms / CLUSTER_CTAS);
         else
             cudaGetLastError();            // (no clusters: the grid-wide kernel is used)
@@ -1311,6 +1355,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
     c.table_cap = L.table_cap;
     c.cell_items = reinterpret_cast<CellItem*>(ws + L.cell_items);
     c.cell_sorted = reinterpret_cast<CellItem*>(ws + L.cell_sorted);
+    c.cell_link = reinterpret_cast<uint4*>(ws + L.cell_link);
     c.group_ends = reinterpret_cast<uint32_t*>(ws + L.group_ends);
     c.leaf_items = reinterpret_cast<LeafItem*>(ws + L.leaf_items);
     c.work_cap = L.work_cap;
@@ -1334,7 +1379,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
         c.z_bf = L.use_tc ? reinterpret_cast<__nv_bfloat16*>(ws + L.z_bf) : nullptr;
         c.zdst = L.use_tc ? reinterpret_cast<uint32_t*>(ws + L.zdst) : nullptr;
         c.cells_cap = L.cells_cap;
-        c.cell_pos = L.use_tc ? reinterpret_cast<uint32_t*>(ws + L.cell_pos) : nullptr;
+        c.cell_pos = L.use_tc || L.clustered ? reinterpret_cast<uint32_t*>(ws + L.cell_pos) : nullptr;
         c.Wxp = reinterpret_cast<__nv_bfloat16*>(ws + L.wxp);
         c.WxTp = reinterpret_cast<__nv_bfloat16*>(ws + L.wxtp);
         c.E_bf = reinterpret_cast<__nv_bfloat16*>(ws + L.e_bf);
@@ -1498,14 +1543,18 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                     cudaLaunchAttribute at[1];
                     at[0].id = cudaLaunchAttributeClusterDimension;
                     at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-                    cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.blockDim = dim3(256);
-                    cfg.dynamicSmemBytes = cluster_smem_bytes(c.H); cfg.stream = stream;
-                    cfg.attrs = at; cfg.numAttrs = 1;
-                    switch (cluster_cols_per_block(c.H)) {
-                        case 8: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<8>, cs))); break;
-                        case 16: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<16>, cs))); break;
-                        case 32: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<32>, cs))); break;
-                        default: RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<48>, cs))); break;
+                    cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.blockDim = dim3(CL_THREADS);
+                    cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 1;
+                    if (c.H <= CL_MAX_H / 2) {
+                        cfg.dynamicSmemBytes = cl_smem_bytes<16, 8>(false);
+                        RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<16, 8>, c)));
+                    } else if (c.H <= CL_MAX_H) {
+                        cfg.dynamicSmemBytes = cl_smem_bytes<32, 32>(false);
+                        RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_kernel<32, 32>, c)));
+                    } else {
+                        cfg.blockDim = dim3(256);
+                        cfg.dynamicSmemBytes = cluster_wide_smem_bytes(c.H);
+                        RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_operator_cluster_wide_kernel<CLUSTER_WIDE_CPC>, cs)));
                     }
                 }
                 // ... the wide ones with the whole grid
@@ -1565,6 +1614,7 @@ int rdf_launch_depth_groups(char* ws, const Layout& L, ExecState* S, DevCtx& c, 
     RDF_KERNEL(S, rdf_group_scan_kernel<<<1, 1024, 0, stream>>>(c));
     RDF_KERNEL(S, rdf_group_scatter_kernel<<<2 * S->grid, 256, 0, stream>>>(c));
     RDF_KERNEL(S, rdf_group_split_kernel<<<S->grid, 256, 0, stream>>>(c, 40u * (uint32_t)c.n_groups));
+    RDF_KERNEL(S, rdf_group_link_kernel<<<4 * S->grid, 256, 0, stream>>>(c));
     CUDA_OK(cudaGetLastError());
     return RDF_OK;
 }

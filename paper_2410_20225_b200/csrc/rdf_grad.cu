@@ -11,6 +11,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "rdf_cluster.cuh"
 #include "rdf_exec.h"
 #include "rdf_tc.cuh"
 #include "rdf_tc_dw.cuh"
@@ -999,18 +1000,16 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
 }
 
 // ===========================================================================
-// fp32 TreeRNN gradient waves without a grid barrier: one thread-block cluster per group of instances
+// fp32 TreeRNN gradient waves without a grid barrier, hidden sizes beyond those of rdf_cluster.cuh
 // ===========================================================================
-// The counterpart of rdf_operator_cluster_kernel for the reverse pass.  The cells are grouped by (cluster of their
-// instance, call depth); a cluster runs the depths below the split one after the other for its own instances and
-// meets at the hardware cluster barrier only.  Per cell: [dh_l ; dh_r] = W^T dz; the blocks of a cluster split the 2H
-// output columns (their part of W stays in shared memory), a block step takes CS cells, thread = (column, slice of the
-// contraction index); the thread that adds the slices up finishes the callee of its column (adds W_s^T dlog; a cell
-// callee gets dz = dh (1 - h^2) as its row, a leaf callee adds dh to dE[tok]) -- what it needs of the callee is
-// fetched before the contraction starts.  Rows travel between the blocks through L2, ordered by the barrier.
+// The same split, with the weights in shared memory and the dz rows travelling through global memory.  Per cell:
+// [dh_l ; dh_r] = W^T dz; the blocks of a cluster split the 2H output columns, a block step takes CS cells, thread =
+// (column, slice of the contraction index); the thread that adds the slices up finishes the callee of its column (adds
+// W_s^T dlog; a cell callee gets dz = dh (1 - h^2) as its row, a leaf callee adds dh to dE[tok]) -- what it needs of the
+// callee is fetched before the contraction starts.
 static const int BWD_CLUSTER_THREADS = 512;
 template <int CPC, int CS>                     // columns per block; cells per step = slices of the contraction index (CPC x CS threads work)
-__global__ void __launch_bounds__(BWD_CLUSTER_THREADS, 1) rdf_backward_cluster_kernel(const __grid_constant__ DevCtx c) {
+__global__ void __launch_bounds__(BWD_CLUSTER_THREADS, 1) rdf_backward_cluster_wide_kernel(const __grid_constant__ DevCtx c) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     // every block takes the same decision from the same words (the kernels before this one are complete)
     if (c.ctl->forward_status != 0 || c.ctl->status != 0 || depth_groups(c) <= 1u) return;
@@ -1148,9 +1147,9 @@ __global__ void __launch_bounds__(BWD_CLUSTER_THREADS, 1) rdf_backward_cluster_k
     if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl->waves_backward += top - d0;      // (after the grid-wide kernel's count)
 }
 
-inline int bwd_cluster_cols_per_block(int H) { return H <= 64 ? 16 : H <= 128 ? 32 : H <= 256 ? 64 : 128; }
+static const int BWD_CLUSTER_CPC = 128, BWD_CLUSTER_CS = 4;
 inline size_t bwd_cluster_smem_bytes(int H) {
-    const int CPC = bwd_cluster_cols_per_block(H), CS = CPC <= 64 ? 8 : 4;
+    const int CPC = BWD_CLUSTER_CPC, CS = BWD_CLUSTER_CS;
     return ((size_t)H * CPC + (size_t)2 * CS * H + (size_t)CS * CS * CPC) * sizeof(float) + 5 * CS * sizeof(uint4);
 }
 
@@ -1429,24 +1428,18 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
             at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.blockDim = dim3(BWD_CLUSTER_THREADS);
-            cfg.dynamicSmemBytes = bwd_cluster_smem_bytes(H); cfg.stream = stream;
+            cfg.gridDim = dim3(c.n_groups * CLUSTER_CTAS); cfg.stream = stream;
             cfg.attrs = at; cfg.numAttrs = 1;
-            const int smem = (int)cfg.dynamicSmemBytes;
-            switch (bwd_cluster_cols_per_block(H)) {
-                case 16:
-                    CUDA_OK(cudaFuncSetAttribute(rdf_backward_cluster_kernel<16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-                    RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_backward_cluster_kernel<16, 8>, c))); break;
-                case 32:
-                    CUDA_OK(cudaFuncSetAttribute(rdf_backward_cluster_kernel<32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-                    RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_backward_cluster_kernel<32, 8>, c))); break;
-                case 64:
-                    CUDA_OK(cudaFuncSetAttribute(rdf_backward_cluster_kernel<64, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-                    RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_backward_cluster_kernel<64, 8>, c))); break;
-                default:
-                    CUDA_OK(cudaFuncSetAttribute(rdf_backward_cluster_kernel<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-                    RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_backward_cluster_kernel<128, 4>, c))); break;
-            }
+            auto launch = [&](void (*kernel)(DevCtx), int threads, size_t smem) -> int {
+                cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem;
+                CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, c)));
+                return RDF_OK;
+            };
+            if (H <= CL_MAX_H / 2) rc = launch(rdf_backward_cluster_kernel<32, 8>, CL_THREADS, cl_smem_bytes<32, 8>(true));
+            else if (H <= CL_MAX_H) rc = launch(rdf_backward_cluster_kernel<64, 16>, CL_THREADS, cl_smem_bytes<64, 16>(true));
+            else rc = launch(rdf_backward_cluster_wide_kernel<BWD_CLUSTER_CPC, BWD_CLUSTER_CS>, BWD_CLUSTER_THREADS, bwd_cluster_smem_bytes(H));
+            if (rc != RDF_OK) return rc;
         }
     }
     rdf_mark(S, 8, stream);

@@ -480,3 +480,14 @@ def test_structural_scheduler_matches_the_general_one(cell, B, leaves):
     assert e.value.code == -8                     # RDF_ERR_WAVE_LIMIT, as from the token scheduler
     g.set_limits(wave_limit=st["waves"])
     assert torch.equal(g.eval_trees(dt, dp)[0], h)
+
+
+@pytest.mark.parametrize("H,chains,depth", [(8, 1, 70), (128, 40, 90), (132, 260, 70), (200, 3, 301), (256, 130, 66), (260, 20, 80)])
+def test_clustered_depths(H, chains, depth):
+    """Deep, thin recursions in fp32 are fired by thread-block clusters: hidden sizes on both sides of the 128- and 256-wide
+    variants, fewer instances than clusters, and more cells per depth and cluster than have an operand row in shared
+    memory (16; 260 chains make 18 per cluster)."""
+    cfg = workloads.config(5, chains=chains, chain_depth=depth, perfect=2, perfect_height=6, V=300, H=H)
+    cfg["params"]["b"] = (0.1 * np.random.default_rng(H).standard_normal(H)).astype(np.float32)
+    st, _ = check_grad(cfg, workers=WORKERS)
+    assert st["clusters"] > 1 and st["waves_backward"] >= depth
