@@ -45,7 +45,7 @@ WORKLOAD_NAMES = {
 }
 CELL = {"treernn": "rnn", "treelstm": "lstm"}
 KERNEL_SOURCES = ["rdf_device.cuh", "rdf_exec.cu", "rdf_exec.h", "rdf_grad.cu", "rdf_internal.h", "rdf_lists.cuh", "rdf_lstm.cuh",
-                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh", "rdf_cluster.cuh"]
+                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh", "rdf_cluster.cuh", "rdf_pool.cuh"]
 
 
 def fib_iter(n):
@@ -323,7 +323,7 @@ class Case:
     """One workload set up on the current device: resident inputs, host copies for the end-to-end path, step functions."""
 
     def __init__(self, rdf, torch, cfg, grad, dist=None, store="thread", hash_load=None):
-        self.rdf, self.torch, self.cfg, self.dist = rdf, torch, cfg, dist
+        self.rdf, self.torch, self.cfg, self.dist, self.store = rdf, torch, cfg, dist, store
         self.N = cfg["N"]
         self.grad = bool(grad)
         if cfg["kind"] == "fib":
@@ -492,7 +492,8 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
                      "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak if peak else None, "peak_source": src,
                      "traffic": traffic.get((kernel, workload))})
 
-    add("rdf_scheduler_kernel" if case.cfg["kind"] in ("fib", "topdown") else "rdf_fold_kernel", "schedule", "hbm", 128.0 * N,
+    fib = "rdf_pool_kernel" if getattr(case, "store", "thread") == "thread" else "rdf_scheduler_kernel"
+    add({"fib": fib, "topdown": "rdf_scheduler_kernel"}.get(case.cfg["kind"], "rdf_fold_kernel"), "schedule", "hbm", 128.0 * N,
         "128 B per invocation: call token write+read, return token / store slot write+read, frame record")
     if case.cfg["kind"] == "fib":
         return rows

@@ -87,6 +87,7 @@ struct Control {
     unsigned long long cyc[6];    // block 0: forward schedule / batch / barrier, backward frames / batch / barrier
     float    loss;
     int32_t  forward_status;      // status word at the end of the forward pass and the loss head
+    uint32_t next_chunk, blocks_done, pool_exhausted;   // rdf_pool.cuh
     uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
 };
 static_assert(sizeof(Control) <= 4096, "the control block is 4 KB");
@@ -111,6 +112,7 @@ struct DevCtx {
     uint32_t qcap;
     // structural recursion (rdf_fold.cuh)
     int       fold_label[3], fold_right[2];
+    int       after_pool;         // general scheduler behind the pool kernel: it runs only if a pool was exhausted
     uint32_t* level_counts;       // [3][level_cap]: cells per chunk of a level, three levels in turn
     uint32_t  level_cap;
     // frames (frame-form tags)

@@ -490,6 +490,7 @@ static const uint32_t NARROW_STRETCH = 4096;   // waves block 0 runs alone befor
 __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
     __shared__ uint32_t lq_count[3], lq_ctr[3];
+    if (c.after_pool && !c.ctl->pool_exhausted) return;              // (the pool kernel has run the call)
     extern __shared__ __align__(16) unsigned char lq_smem[];         // local queue of narrow stretches: 2 x LQ_CAP tokens
     LocalQ lq;
     lq.buf[0] = reinterpret_cast<Token*>(lq_smem);
@@ -741,10 +742,8 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
     }
 }
 
-__global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
-    const long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= c.B) return;
-    // one token <[], x_b> per instance enters `result`
+// one token <[], x_b> per instance enters `result`
+__device__ __forceinline__ void seed_instance(const DevCtx& c, long long b) {
     uint64_t tag;
     const int64_t datum = c.x ? c.x[b] : (int64_t)c.tree_root[b];
     if (c.tag_mode == RDF_TAGS_PATH) {
@@ -762,6 +761,12 @@ __global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
         c.ctl->frame_count.v = c.tag_mode == RDF_TAGS_FRAME ? (uint32_t)c.B : 0u;
     }
 }
+__global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
+    const long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < c.B) seed_instance(c, b);
+}
+
+#include "rdf_pool.cuh"
 
 // The operator kernel: the leaves first (they wait for nothing), then the cells in waves whose operands are complete;
 // a grid barrier separates the waves: depth by depth from the deepest cells up.  TC: bf16 operands on the tensor cores
@@ -1273,6 +1278,8 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CUDA_OK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     CUDA_OK(cudaDeviceGetAttribute(&S->clock_khz, cudaDevAttrClockRate, dev));
+    CUDA_OK(cudaDeviceGetAttribute(&S->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
+    CUDA_OK(cudaDeviceGetAttribute(&S->smem_per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (!coop) return RDF_ERR_CUDA;
     const int max_dyn = std::max(tc_smem_bytes(80, 2 * TC_HP_MAX, 48, TC_HP_MAX, TC_STAGES_LSTM_FWD),
                                  tc_smem_bytes(TC_HP_MAX / 4, 2 * TC_HP_MAX, 0, 0, TC_STAGES_RNN_FWD));   // the largest configurations
@@ -1434,6 +1441,35 @@ int rdf_check_common(rdf_graph* g, const rdf_batch* in, const rdf_params* params
     return RDF_OK;
 }
 
+static size_t pool_smem_bytes(const ExecState* S) { return std::min<size_t>(S->smem_per_sm / POOL_PER_SM - 2048, S->smem_per_block - 1024); }
+static uint32_t pool_frames(const PoolProgram& P, const ExecState* S) {
+    const size_t fixed = pool_fixed_bytes(P), smem = pool_smem_bytes(S);
+    return smem <= fixed ? 0u : (uint32_t)std::min<size_t>((smem - fixed) / pool_frame_bytes(P), POOL_MAX_FRAMES) & ~7u;
+}
+// The pool executor: how many frames a block has, and how the instances are dealt out.
+static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream) {
+    const PoolProgram& P = g->pool_prog;
+    const size_t smem = pool_smem_bytes(S);
+    PoolSizes z{};
+    z.cap = pool_frames(P, S);
+    z.max_depth = g->tag_mode == RDF_TAGS_PATH ? (uint32_t)(RDF_PATH_BITS / g->label_bits) : 0xFFFFFFFFu;
+    // frames a token may take in a round, and what depth-first recursion one token at a time needs (rdf_pool.cuh: pool_width)
+    const uint32_t calls = (uint32_t)std::max(1, std::max(P.calls_entry, P.calls_cont));
+    z.div = std::max(4u, calls);
+    z.reserve = std::min(z.cap / 2, ((g->tag_mode == RDF_TAGS_PATH ? z.max_depth : 64u) + 1u) * calls + z.div);
+    z.cont_calls = P.calls_cont > 0;
+    const int grid = (int)std::min<long long>((long long)S->grid * POOL_PER_SM, in->B);
+    z.chunk = (uint32_t)std::max<long long>(1, std::min<long long>(in->B / ((long long)grid * 8), POOL_THREADS / 4));
+    z.refill = in->B >= 16ll * grid ? (uint32_t)POOL_THREADS : 1u;
+    z.max_calls = (unsigned long long)in->max_invocations;
+    z.max_parked = (unsigned long long)L.table_cap * std::max<size_t>(1, g->match.size());
+    rdf_mark(S, 1, stream);
+    CUDA_OK(cudaFuncSetAttribute(rdf_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RDF_KERNEL(S, rdf_pool_kernel<<<grid, POOL_THREADS, smem, stream>>>(c, P, z));
+    CUDA_OK(cudaGetLastError());
+    return RDF_OK;
+}
+
 // zero what must start at zero, upload the program, seed, run all waves
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,
                        DevCtx& c, cudaStream_t stream) {
@@ -1443,7 +1479,25 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     // Structural recursion over the input trees has its own scheduler; a traced call records every firing of the graph and
     // goes through the general one.
     const bool fold = g->fold && !out->trace;
-    if (fold) {
+    // Integer programs run out of shared memory.  The general scheduler has what that executor does not: trace records, a
+    // bound on the width of a wave, the waits and waves that rdf_set_limits limits, and the cooperative probes.
+    const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= 4u * POOL_THREADS && S->wait_cycles == 0 &&
+                      S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
+                      (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B);
+    if (pool) {
+        const int rc = rdf_launch_pool(g, in, L, S, c, stream);
+        if (rc != RDF_OK) return rc;
+        if (g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1) {      // bounded depth, one match per frame: a pool always suffices
+            for (int k = 2; k <= 5; ++k) rdf_mark(S, k, stream);
+            S->last_ctl = c.ctl;
+            S->last_stream = stream;
+            S->ran = true;
+            return RDF_OK;
+        }
+        c.after_pool = 1;
+        RDF_KERNEL(S, rdf_pool_fallback_kernel<<<2 * S->grid, 256, 0, stream>>>(c, L.pair_bytes / sizeof(Slot), L.arrived_bytes / sizeof(uint32_t),
+                                                                               L.table_bytes / sizeof(Slot)));
+    } else if (fold) {
         CUDA_OK(cudaMemsetAsync(ws + L.level_counts, 0, (size_t)3 * L.level_cap * sizeof(uint32_t), stream));
     } else if (g->tag_mode == RDF_TAGS_FRAME) {
         bool wide = false;                        // an operator with more than two tagged inputs
@@ -1451,7 +1505,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         if (L.pair_bytes) CUDA_OK(cudaMemsetAsync(ws + L.pair_slots, 0, L.pair_bytes, stream));
         if (wide && L.arrived_bytes) CUDA_OK(cudaMemsetAsync(ws + L.arrived, 0, L.arrived_bytes, stream));
     }
-    if (L.table_bytes) CUDA_OK(cudaMemsetAsync(ws + L.table, 0xFF, L.table_bytes, stream));
+    if (L.table_bytes && !pool) CUDA_OK(cudaMemsetAsync(ws + L.table, 0xFF, L.table_bytes, stream));
     if (!fold)
     {
         // the four program tables sit next to each other in the workspace (code first, constants last): one copy
@@ -1477,7 +1531,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         }
         CUDA_OK(cudaMemcpyAsync(ws + L.code, S->tables, bytes, cudaMemcpyHostToDevice, stream));
     }
-    if (!fold) RDF_KERNEL(S, rdf_seed_kernel<<<(unsigned)((in->B + 255) / 256), 256, 0, stream>>>(c));
+    if (!fold && !pool) RDF_KERNEL(S, rdf_seed_kernel<<<(unsigned)((in->B + 255) / 256), 256, 0, stream>>>(c));
     CUDA_OK(cudaGetLastError());
     if (c.use_tc) {
         if (c.lstm) {
@@ -1488,7 +1542,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         }
         CUDA_OK(cudaGetLastError());
     }
-    rdf_mark(S, 1, stream);
+    if (!pool) rdf_mark(S, 1, stream);
     void* args[] = {(void*)&c};
     if (fold) {
         // a run of a few chunks: one block, no grid to wait for

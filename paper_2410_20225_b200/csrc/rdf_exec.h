@@ -51,6 +51,7 @@ struct ExecState {
     int rnn32_per_sm = 1;        // blocks per SM of the fp32 TreeRNN operator / gradient kernels
     int n_clusters = 0;          // clusters of the clustered fp32 operator kernel that fit the device at once (0: none)
     int clock_khz = 0;
+    int smem_per_sm = 0, smem_per_block = 0;
     void* last_ctl = nullptr;
     cudaStream_t last_stream = nullptr;
     bool ran = false;

@@ -1024,6 +1024,301 @@ void detect_fold(const Prog& P, rdf_graph* g) {
     g->fold = true;
 }
 
+// ------------------------------------------------- fused program (rdf_pool.cuh)
+// Registers are local to a segment and nearly single-assignment, so constants, copies and additions of constants are not
+// executed: they are folded into the operands (register + immediate) of the instructions that read them.
+struct PoolBuilder {
+    const rdf_graph* g;
+    PoolProgram& out;
+    struct Sym { int base; int64_t imm; bool folded; };       // value of a register: register `base` (-1: none) + imm
+    struct Fail {};
+    static const uint8_t NONE = 255;
+    std::vector<int> new_pc;                     // per old pc
+    std::vector<char> leader;                    // jump target or segment start
+    std::map<int, std::vector<Sym>> saved;       // state at the only branch to a leader
+    Sym sym[RDF_MAX_REGS];
+    int n_consts = 0;
+    bool in_entry = false;
+
+    static void need(bool ok) { if (!ok) throw Fail{}; }
+    int n_args(int label) const { return g->labels[label].n_args; }
+    static bool is_call(uint8_t op) { return op == VM_CALL || op == VM_CALL_A || op == VM_CALL_B; }
+    std::vector<int> reads(const VmInstr& in) const {
+        if (is_call(in.op)) {
+            std::vector<int> r{in.a};
+            if (n_args(in.imm) > 1) r.push_back(in.b);
+            if (n_args(in.imm) > 2) r.push_back(in.dst);
+            return r;
+        }
+        switch (in.op) {
+            case VM_MOV: case VM_ISLEAF: case VM_LEFT: case VM_RIGHT: case VM_TOK: case VM_BRZ: case VM_PORT: case VM_RET: case VM_OUT:
+                return {in.a};
+            case VM_ADD: case VM_SUB: case VM_MUL: case VM_MAX: case VM_LT: case VM_EQ: case VM_REM: return {in.a, in.b};
+            default: return {};
+        }
+    }
+    bool read_later(int reg, int from, int end) const {
+        for (int q = from; q < end; ++q)
+            for (int r : reads(g->code[q]))
+                if (r == reg) return true;
+        return false;
+    }
+    PoolInstr& emit(uint8_t op) {
+        need(out.n_code < POOL_MAX_CODE);
+        PoolInstr& in = out.code[out.n_code++];
+        in = PoolInstr{};
+        in.op = op;
+        in.ra = in.rb = in.rc = NONE;
+        return in;
+    }
+    void operand(int reg, uint8_t& r, int32_t& imm) {
+        const Sym& s = sym[reg];
+        r = s.base < 0 ? NONE : (uint8_t)s.base;
+        imm = (int32_t)s.imm;
+        if (s.base >= 0) out.n_regs = std::max(out.n_regs, s.base + 1);
+    }
+    void written(PoolInstr& in, int reg) {       // `in` puts a value into the register
+        in.dst = (uint8_t)reg;
+        sym[reg] = Sym{reg, 0, false};
+        out.n_regs = std::max(out.n_regs, reg + 1);
+    }
+    void materialize(int reg) {
+        PoolInstr& in = emit(PI_MOV);
+        operand(reg, in.ra, in.ia);
+        written(in, reg);
+    }
+    void define(int reg, int pc, int end) {      // before reg gets a new value: nothing may still be folded onto the old one
+        for (int x = 0; x < RDF_MAX_REGS; ++x)
+            if (x != reg && sym[x].folded && sym[x].base == reg && read_later(x, pc, end)) materialize(x);
+    }
+    void flush(int pc, int end) {                // every folded register that is read from pc on
+        for (int x = 0; x < RDF_MAX_REGS; ++x)
+            if (sym[x].folded && read_later(x, pc, end)) materialize(x);
+    }
+    bool falls_through(int q) const {            // does q - 1 run on into q?
+        const uint8_t op = g->code[q - 1].op;
+        return !(op == VM_JMP || op == VM_RET || op == VM_OUT || op == VM_HALT);
+    }
+    // jump to the target of the branch at q unless (a cmp b); b < 0: compare with zero
+    void branch(int q, int end, int edges, uint8_t cmp, int a, int b) {
+        const int target = g->code[q].imm;
+        // a target that is reached only from here starts with what is folded now; else everything it reads is put in place
+        if (edges == 1 && !falls_through(target)) saved[target] = std::vector<Sym>(sym, sym + RDF_MAX_REGS);
+        else flush(q + 1, end);
+        PoolInstr& in = emit(PI_BR);
+        in.cmp = cmp;
+        operand(a, in.ra, in.ia);
+        if (b >= 0) operand(b, in.rb, in.ib);
+        in.imm = target;
+    }
+    void reset() {
+        for (int x = 0; x < RDF_MAX_REGS; ++x) sym[x] = Sym{x, 0, false};
+    }
+
+    void segment(int begin, int end) {
+        reset();
+        saved.clear();
+        std::vector<int> edges(end - begin, 0);
+        for (int q = begin; q < end; ++q)
+            if (g->code[q].op == VM_BRZ || g->code[q].op == VM_JMP) {
+                const int t = g->code[q].imm;
+                need(t > q && t < end);          // structured forward branches
+                ++edges[t - begin];
+            }
+        for (int q = begin; q < end; ++q) {
+            const VmInstr& v = g->code[q];
+            if (q > begin && edges[q - begin]) {
+                leader[q] = 1;
+                if (saved.count(q)) std::copy(saved[q].begin(), saved[q].end(), sym);
+                else {
+                    if (falls_through(q)) flush(q, end);
+                    reset();
+                }
+            }
+            new_pc[q] = out.n_code;
+            if (is_call(v.op)) {
+                PoolInstr& in = emit(PI_CALL);
+                operand(v.a, in.ra, in.ia);
+                if (n_args(v.imm) > 1) operand(v.b, in.rb, in.ib);
+                if (n_args(v.imm) > 2) operand(v.dst, in.rc, in.ic);
+                in.imm = v.imm;
+                continue;
+            }
+            switch (v.op) {
+                case VM_MOVI: define(v.dst, q + 1, end); sym[v.dst] = Sym{-1, v.imm, true}; break;
+                case VM_MOVC: {
+                    define(v.dst, q + 1, end);
+                    int at = 0;
+                    while (at < n_consts && out.consts[at] != g->consts[v.imm]) ++at;
+                    need(at < POOL_MAX_CONSTS);
+                    out.consts[at] = g->consts[v.imm];
+                    n_consts = std::max(n_consts, at + 1);
+                    PoolInstr& in = emit(PI_CONST);
+                    in.imm = at;
+                    written(in, v.dst);
+                    break;
+                }
+                case VM_MOV: {
+                    const Sym s = sym[v.a];
+                    define(v.dst, q + 1, end);
+                    if (s.base != v.dst) sym[v.dst] = Sym{s.base, s.imm, true};
+                    else if (s.imm == 0) sym[v.dst] = Sym{v.dst, 0, false};
+                    else {                                                 // reg = itself + constant
+                        PoolInstr& in = emit(PI_MOV);
+                        operand(v.a, in.ra, in.ia);
+                        written(in, v.dst);
+                    }
+                    break;
+                }
+                case VM_ADD: case VM_SUB: case VM_MUL: case VM_MAX: case VM_REM: case VM_LT: case VM_EQ: {
+                    const Sym a = sym[v.a], b = sym[v.b];
+                    int base = -2;
+                    int64_t imm = 0;
+                    if (v.op == VM_ADD && a.base < 0) { base = b.base; imm = a.imm + b.imm; }
+                    else if (v.op == VM_ADD && b.base < 0) { base = a.base; imm = a.imm + b.imm; }
+                    else if (v.op == VM_SUB && b.base < 0) { base = a.base; imm = a.imm - b.imm; }
+                    if (base != -2 && base != v.dst && imm >= INT32_MIN && imm <= INT32_MAX) {
+                        define(v.dst, q + 1, end);
+                        sym[v.dst] = Sym{base, imm, true};
+                        break;
+                    }
+                    const bool cmp = v.op == VM_LT || v.op == VM_EQ;
+                    if (cmp && q + 1 < end && !edges[q + 1 - begin] && g->code[q + 1].op == VM_BRZ && g->code[q + 1].a == v.dst &&
+                        !read_later(v.dst, q + 2, end)) {
+                        branch(q + 1, end, edges[g->code[q + 1].imm - begin], v.op == VM_LT ? PC_LT : PC_EQ, v.a, v.b);
+                        new_pc[++q] = out.n_code;
+                        break;
+                    }
+                    define(v.dst, q + 1, end);
+                    PoolInstr& in = emit(cmp ? PI_CMP : v.op == VM_ADD ? PI_ADD : v.op == VM_SUB ? PI_SUB : v.op == VM_MUL ? PI_MUL : v.op == VM_MAX ? PI_MAX : PI_REM);
+                    in.cmp = v.op == VM_LT ? PC_LT : PC_EQ;
+                    operand(v.a, in.ra, in.ia);
+                    operand(v.b, in.rb, in.ib);
+                    written(in, v.dst);
+                    break;
+                }
+                case VM_ISLEAF: case VM_LEFT: case VM_RIGHT: case VM_TOK: {
+                    define(v.dst, q + 1, end);
+                    PoolInstr& in = emit(PI_TREE);
+                    in.cmp = v.op == VM_ISLEAF ? PT_ISLEAF : v.op == VM_LEFT ? PT_LEFT : v.op == VM_RIGHT ? PT_RIGHT : PT_TOK;
+                    operand(v.a, in.ra, in.ia);
+                    written(in, v.dst);
+                    break;
+                }
+                case VM_BRZ: branch(q, end, edges[v.imm - begin], PC_NE, v.a, -1); break;
+                case VM_JMP: flush(v.imm, end); emit(PI_JMP).imm = v.imm; break;
+                case VM_LDARG: {
+                    if (in_entry) { sym[v.dst] = Sym{v.imm, 0, v.dst != v.imm}; break; }      // parameters are in registers 0 ..
+                    define(v.dst, q + 1, end);
+                    PoolInstr& in = emit(PI_ARG);
+                    in.imm = v.imm;
+                    written(in, v.dst);
+                    break;
+                }
+                case VM_PORT: {
+                    PoolInstr& in = emit(PI_PORT);
+                    operand(v.a, in.ra, in.ia);
+                    in.cmp = v.b; in.imm = v.imm;
+                    break;
+                }
+                case VM_RET: case VM_OUT: {
+                    PoolInstr& in = emit(v.op == VM_RET ? PI_RET : PI_OUT);
+                    operand(v.a, in.ra, in.ia);
+                    break;
+                }
+                case VM_HALT: emit(PI_HALT); break;
+                default: need(false);
+            }
+        }
+    }
+
+    // false: not a program for the pool executor
+    bool build() {
+        if (g->has_vector_ops || g->has_loops || g->interleaved) return false;
+        if ((int)g->labels.size() > POOL_MAX_LABELS || (int)g->match.size() > POOL_MAX_MATCH) return false;
+        const int n = (int)g->code.size();
+        leader.assign(n, 0);
+        new_pc.assign(n, 0);
+        std::set<int> entries{g->result_entry_pc};
+        int max_args = 1;
+        for (const LabelInfo& L : g->labels) {
+            entries.insert(L.entry_pc);
+            max_args = std::max(max_args, L.n_args);
+        }
+        std::set<int> starts = entries;
+        for (const LabelInfo& L : g->labels)
+            if (L.k_kind == K_SEG) starts.insert(L.k_pc);
+        for (const MatchNode& M : g->match) starts.insert(M.cont_pc);
+        std::vector<int> seg(starts.begin(), starts.end());
+        seg.push_back(n);
+        bool late_args = false;                  // a parameter is read after the segment that enters the function
+        out = PoolProgram{};
+        out.n_regs = std::max(max_args, 2);      // (a match loads two operands at least)
+        try {
+            for (size_t k = 0; k + 1 < seg.size(); ++k) {
+                in_entry = entries.count(seg[k]) != 0;
+                leader[seg[k]] = 1;
+                for (int q = seg[k]; q < seg[k + 1]; ++q) late_args = late_args || (!in_entry && g->code[q].op == VM_LDARG);
+                segment(seg[k], seg[k + 1]);
+            }
+        } catch (const Fail&) {
+            return false;
+        }
+        for (const MatchNode& M : g->match) {
+            if (M.n_ports < 2) return false;
+            out.n_regs = std::max(out.n_regs, M.n_ports);
+        }
+        std::vector<char> is_leader(out.n_code + 1, 0);
+        for (int q = 0; q < n; ++q)
+            if (leader[q]) is_leader[new_pc[q]] = 1;
+        for (int i = 0; i < out.n_code; ++i) {
+            PoolInstr& in = out.code[i];
+            if (in.op == PI_BR || in.op == PI_JMP) in.imm = new_pc[in.imm];
+            for (uint8_t* r : {&in.ra, &in.rb, &in.rc})
+                if (*r == NONE) *r = (uint8_t)out.n_regs;
+        }
+        auto halts = [&](int i) {                // (every segment ends with a halt, and branches go forward)
+            while (out.code[i].op == PI_JMP) i = out.code[i].imm;
+            return out.code[i].op == PI_HALT;
+        };
+        for (int i = 0; i < out.n_code; ++i)
+            if (out.code[i].op == PI_CALL || out.code[i].op == PI_PORT) out.code[i].last = halts(i + 1);
+        for (int i = 0; i < out.n_code; ++i) {
+            if (out.code[i].op != PI_CALL) continue;
+            int j = i + 1;
+            while (out.code[j].op == PI_CALL && !is_leader[j]) ++j;
+            out.code[i].n_run = (uint8_t)(j - i);
+            if (j == i + 1) out.code[i].tail = out.code[i].last && g->labels[out.code[i].imm].k_kind == K_RET;
+            i = j - 1;
+        }
+        // frames: the arguments share their words with the operands of the match nodes, unless they are read late
+        out.n_labels = (int)g->labels.size(); out.n_match = (int)g->match.size();
+        out.result_entry = new_pc[g->result_entry_pc];
+        const int word0 = late_args ? max_args : 0;
+        out.words = std::max(max_args, word0 + g->n_ports_total);
+        if (out.words > POOL_MAX_WORDS) return false;
+        for (int k = 0; k < out.n_labels; ++k) {
+            const LabelInfo& L = g->labels[k];
+            out.labels[k] = PoolLabel{(int16_t)new_pc[L.entry_pc], (int16_t)(L.k_kind == K_SEG ? new_pc[L.k_pc] : 0), (uint8_t)L.k_kind,
+                                      (uint8_t)(L.k_kind == K_PORT ? L.k_node : 0), (uint8_t)(L.k_kind == K_PORT ? L.k_port : 0), (uint8_t)L.n_args};
+        }
+        for (int k = 0; k < out.n_match; ++k) {
+            const MatchNode& M = g->match[k];
+            const int w = word0 + M.port_base;
+            out.match[k] = PoolMatch{(int16_t)new_pc[M.cont_pc], (uint8_t)M.n_ports, (uint8_t)w, ((1u << M.n_ports) - 1u) << w};
+        }
+        // most frames one segment takes (over its branches: an upper bound)
+        for (size_t k = 0; k + 1 < seg.size(); ++k) {
+            const int end = seg[k + 1] < n ? new_pc[seg[k + 1]] : out.n_code;
+            int calls = 0;
+            for (int i = new_pc[seg[k]]; i < end; ++i) calls += out.code[i].op == PI_CALL && !out.code[i].tail;
+            int& most = entries.count(seg[k]) ? out.calls_entry : out.calls_cont;
+            most = std::max(most, calls);
+        }
+        return true;
+    }
+};
+
 }  // namespace
 
 extern "C" int rdf_graph_build(const rdf_program* prog, rdf_graph** out_graph) {
@@ -1040,6 +1335,8 @@ extern "C" int rdf_graph_build(const rdf_program* prog, rdf_graph** out_graph) {
         Lower L{P, g};
         L.run();
         detect_fold(P, g);
+        PoolBuilder pool{g, g->pool_prog};
+        g->pool = pool.build();
     } catch (const Err& e) {
         delete g;
         return e.code;

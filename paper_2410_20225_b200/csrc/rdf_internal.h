@@ -78,6 +78,46 @@ static const int RDF_PATH_BITS = 38;       // packed path field
 static const int RDF_DEPTH_SHIFT = 38;     // 6-bit depth field above it
 static const int RDF_INST_SHIFT = 44;      // 20-bit instance field
 
+// ---------------------------------------------------------------------------
+// The lowered program of an integer graph once more, fused for the pool executor
+// (rdf_pool.cuh): operands are register + immediate, a comparison branches by
+// itself.  Small programs only; the kernel gets it as a parameter.
+// ---------------------------------------------------------------------------
+enum PoolOp : uint8_t {
+    PI_HALT = 0, PI_BR, PI_RET, PI_CALL, PI_PORT, PI_ADD, PI_SUB, PI_MUL, PI_MAX, PI_REM, PI_CMP, PI_MOV, PI_CONST, PI_ARG, PI_JMP,
+    PI_TREE, PI_OUT
+};
+enum PoolCmp : uint8_t { PC_LT = 0, PC_EQ, PC_NE };
+enum PoolTree : uint8_t { PT_ISLEAF = 0, PT_LEFT, PT_RIGHT, PT_TOK };
+
+struct alignas(16) PoolInstr {
+    uint8_t op, dst, cmp, n_run;     // cmp: PoolCmp / PoolTree / port; n_run: calls that follow one another from here
+    uint8_t ra, rb, rc;              // operand registers (n_regs: the zero register) ...
+    uint8_t last : 1, tail : 1;      // nothing follows in the segment; the call is the caller's own output
+    int32_t ia, ib, ic;              // ... plus immediates
+    int32_t imm;                     // branch target, label, match node, constant, parameter
+    int32_t pad[2];
+};
+struct PoolLabel {
+    int16_t entry, k_pc;
+    uint8_t k_kind, k_node, k_port, n_args;
+};
+struct PoolMatch {
+    int16_t  cont;
+    uint8_t  n_ports, word0;         // its ports are words word0 .. of the frame
+    uint32_t all;                    // bits of its ports
+};
+static const int POOL_MAX_CODE = 48, POOL_MAX_LABELS = 16, POOL_MAX_MATCH = 8, POOL_MAX_CONSTS = 4, POOL_MAX_WORDS = 8;
+struct alignas(16) PoolProgram {
+    int32_t   n_code, n_labels, n_match, result_entry;
+    int32_t   words, n_regs;         // 64-bit words per frame, registers per thread
+    int32_t   calls_entry, calls_cont;   // most frames taken by a segment that enters a function / that carries on after a match
+    PoolInstr code[POOL_MAX_CODE];
+    PoolLabel labels[POOL_MAX_LABELS];
+    PoolMatch match[POOL_MAX_MATCH];
+    int64_t   consts[POOL_MAX_CONSTS];
+};
+
 struct rdf_graph {
     // literal graph (Section 3 transformation), for inspection
     std::vector<rdf_node> nodes;
@@ -102,6 +142,8 @@ struct rdf_graph {
     bool fold = false;
     int32_t fold_label[3] = {0, 0, 0};    // label ids of the calls of operand 0 and operand 1 and of `result`'s call
     int32_t fold_right[2] = {0, 1};       // the child that operand 0 / 1 descends into: 0 left, 1 right
+    bool pool = false;            // an integer program that fits the pool executor
+    PoolProgram pool_prog{};
     bool interleaved = false;     // some Switch reads a vector value: operators run between the token waves
     std::vector<std::string> func_names;
     // per-run state owned by the executor (rdf_exec.cu)

@@ -1,0 +1,377 @@
+// Integer programs run out of shared memory: one pool of tokens per thread block.
+//
+// Tokens of different instances never meet, and inside an instance only the frames of the calls in flight are needed: a
+// block takes instances, keeps their frames, pending tokens and parked operands in its shared memory, and works depth-first
+// -- in rounds of up to one token per thread from the top of a stack -- until they have returned their results; then it
+// takes more.  Nothing of a call goes to global memory but its argument and its result.  (The general scheduler runs all
+// instances in step, breadth-first: its queues, frames and store hold a whole wave, so every token costs about 128 bytes and
+// three or four dependent L2 round trips, and every wave a grid barrier.)
+//
+// A token is a frame that waits to be entered, or a frame whose match node has all its operands and waits to go on; the two
+// kinds have a stack each.  A round: the warps take completed matches first (they give frames back) and the other warps the
+// top of the frames to enter, so that the threads of a warp do the same thing.  A thread runs one segment: new frames for
+// the calls it makes, pushed as tokens; or a value that is returned -- parked in the caller's frame, and if it was the last
+// operand the match becomes a token (carrying on in the same thread instead leaves the warp to a few long chains of returns:
+// 131 072 calls of fib took 13.0 ms with up to three in a row, 24.7 with eight, 7.8 with none).
+// The program is a fused form of the lowered code (PoolBuilder): operands are register + immediate, a comparison branches by
+// itself, consecutive calls reserve their frames together.
+//
+// What bounds it: the latency of a round -- a warp runs some 500 dependent instructions of the interpreter between two block
+// barriers, and the frames that fit the shared memory limit the warps to about 16 per SM.
+// Measured, general scheduler -> this: 131 072 calls of fib(0..18) 36.3 -> 7.8 ms, 1024 calls 0.721 -> 0.321 ms, 8 calls of
+// fib(0..10) 0.137 -> 0.038 ms, 200 calls of tak 1.76 -> 1.19 ms (one block runs the largest instance to its end).
+// (Included by rdf_exec.cu only: it defines kernels.)
+#pragma once
+#include "rdf_exec.h"
+
+static const int POOL_THREADS = 512, POOL_PER_SM = 1;   // threads of a block, blocks per SM
+static const uint32_t POOL_ROOT = 0x80000000u;          // frame word of an instance's `result` context: | instance
+// Frame word of an invocation: parent frame [15:0], label [21:16], depth of the tag [27:22] (path tags)
+
+struct PoolSizes {
+    uint32_t cap;            // frames of a block
+    uint32_t div, reserve;   // pool_width
+    uint32_t cont_calls;     // a completed match may take frames too
+    uint32_t chunk;          // instances a block takes at a time
+    uint32_t refill;         // it takes them when fewer tokens than this are pending
+    uint32_t max_depth;      // path tags: labels that fit the packed tag; frame tags: no limit (0xFFFFFFFF)
+    unsigned long long max_calls;   // frame tags: Call firings the caller allows
+    unsigned long long max_parked;  // path tags: operands the token store of the call holds
+};
+
+struct PoolShared {
+    uint32_t entered[2];     // frames to enter pushed in the round (by parity)
+    uint32_t matched[2];     // completed matches pushed in the round
+    uint32_t taken[2];       // frames taken in the round
+    uint32_t freed[2];       // frames given back in the round
+    uint32_t next_chunk;
+    int      stop;           // 1: an error, 2: the pool is exhausted
+};
+
+inline size_t pool_fixed_bytes(const PoolProgram& P) { return sizeof(PoolProgram) + (size_t)(P.n_regs + 1) * POOL_THREADS * 8; }
+inline size_t pool_frame_bytes(const PoolProgram& P) { return 8 * (size_t)P.words + 4 + 4 + 2 + 2 + 2; }
+static const uint32_t POOL_MAX_FRAMES = 1u << 13;       // a completed match: frame | node << 13
+
+// The pool's arrays in dynamic shared memory
+struct Pool {
+    const PoolProgram* prog;
+    int64_t*  regs;          // [n_regs + 1][T]; the last one is zero
+    int64_t*  words;         // [words][cap]: arguments while the frame waits to be entered, then the operands of its match nodes
+    uint32_t* head;          // [cap] frame word
+    uint32_t* state;         // [cap] waiting to be entered: calls above it; then the operands that have arrived
+    uint16_t* enter;         // [cap] frames to enter, oldest first (a deque)
+    uint16_t* match;         // [cap] stack of completed matches
+    uint16_t* ring;          // [cap] free frames, oldest first
+};
+
+struct PoolThread {
+    static const int T = POOL_THREADS;
+    const DevCtx& c;
+    const PoolSizes& z;
+    const Pool& P;
+    PoolShared& sh;
+    uint32_t tid;
+    uint32_t ring0, avail, ring_tail, enter0, match0, par;  // this round: first free frame, free frames, where frames go back, tops of the stacks
+    uint32_t invocations = 0, inserts = 0, matches = 0, max_depth = 0, max_wave = 0;
+
+    __device__ __forceinline__ int64_t val(uint32_t reg, int32_t imm) const { return P.regs[reg * T + tid] + (int64_t)imm; }
+    __device__ __forceinline__ void set(uint32_t reg, int64_t v) { P.regs[reg * T + tid] = v; }
+    __device__ __forceinline__ uint32_t wrap(uint32_t at) const { return at >= z.cap ? at - z.cap : at; }
+    __device__ __forceinline__ void error(int code) {
+        set_status(c, code);
+        sh.stop = 1;
+    }
+    __device__ __forceinline__ void give_back(uint32_t f) { P.ring[wrap(ring_tail + aggregated_inc(&sh.freed[par]))] = (uint16_t)f; }
+    // k frames for calls that follow one another, and their places on the stack (first of each); false: the pool is exhausted
+    __device__ __forceinline__ bool reserve(uint32_t k, uint32_t& frame_at, uint32_t& slot) {
+        aggregated_inc2n(&sh.taken[par], &sh.entered[par], k, frame_at, slot);
+        if (frame_at + k <= avail) return true;
+        sh.stop = 2;
+        return false;
+    }
+
+    // The operand `v` arrives at port `port` of match node `node` in frame f; the last one makes the match a token.
+    __device__ __forceinline__ void deliver(uint32_t f, uint32_t node, uint32_t port, int64_t v) {
+        const PoolMatch M = P.prog->match[node];
+        P.words[(M.word0 + port) * z.cap + f] = v;
+        __threadfence_block();
+        const uint32_t bit = 1u << (M.word0 + port), before = atomicOr(&P.state[f], bit);
+        if (((before | bit) & M.all) != M.all) {
+            ++inserts;
+            return;
+        }
+        ++matches;
+        const uint32_t at = match0 + aggregated_inc(&sh.matched[par]);
+        if (at < z.cap) P.match[at] = (uint16_t)(f | node << 13);
+        else sh.stop = 2;                                   // (only bodies with several match nodes can have more matches than frames)
+    }
+
+    __device__ __forceinline__ void fill_frame(uint32_t f, int64_t a0, const PoolInstr& in, uint32_t n_args, uint32_t head, uint32_t wave) {
+        P.head[f] = head;
+        P.words[f] = a0;
+        if (n_args > 1) P.words[z.cap + f] = val(in.rb, in.ib);
+        if (n_args > 2) P.words[2 * z.cap + f] = val(in.rc, in.ic);
+        P.state[f] = wave;
+    }
+
+    // Return_i: frame f (its word h) has the value v.  Returns the code to go on with (in frame f, r0 = v), or -1.
+    __device__ __forceinline__ int give_value(uint32_t& f, uint32_t& h, int64_t v) {
+        for (;;) {
+            const PoolLabel L = P.prog->labels[(h >> 16) & 63u];
+            give_back(f);
+            f = h & 0xFFFFu;
+            if (L.k_kind == K_PORT) {
+                deliver(f, L.k_node, L.k_port, v);
+                return -1;
+            }
+            h = P.head[f];
+            if (L.k_kind == K_SEG) {
+                set(0, v);
+                return L.k_pc;
+            }                                               // (K_RET: the call was the caller's own output)
+        }
+    }
+
+    // Token `f`: a frame to enter (node < 0), or the completed match `node` of frame f.
+    __device__ __forceinline__ void run(uint32_t f, int node) {
+        const PoolProgram& prog = *P.prog;
+        uint32_t h = P.head[f], wave = 0;
+        int pc;
+        if (node >= 0) {
+            const PoolMatch M = prog.match[node];
+            const int64_t* w = P.words + M.word0 * z.cap + f;
+            set(0, w[0]); set(1, w[z.cap]);
+            for (uint32_t k = 2; k < M.n_ports; ++k) set(k, w[k * z.cap]);
+            pc = M.cont;
+        } else {
+            uint32_t n_args = 1;
+            pc = prog.result_entry;
+            if (!(h & POOL_ROOT)) {
+                const PoolLabel L = prog.labels[(h >> 16) & 63u];
+                pc = L.entry;
+                n_args = L.n_args;
+            }
+            set(0, P.words[f]);
+            if (n_args > 1) set(1, P.words[z.cap + f]);
+            if (n_args > 2) set(2, P.words[2 * z.cap + f]);
+            wave = P.state[f];
+            P.state[f] = 0u;
+            max_wave = max(max_wave, wave);
+        }
+        uint32_t frame_at = 0, slot = 0, run_left = 0;
+        for (uint32_t step = 0; step < (1u << 22); ++step) {
+            const PoolInstr in = prog.code[pc++];
+            const int64_t a = val(in.ra, in.ia);
+            if (in.op == PI_BR) {                           // carry on when the comparison holds, else go to imm
+                const int64_t b = val(in.rb, in.ib);
+                const bool t = in.cmp == PC_LT ? a < b : (a == b) == (in.cmp == PC_EQ);
+                if (!t) pc = in.imm;
+            } else if (in.op == PI_RET) {
+                pc = give_value(f, h, a);
+                if (pc < 0) return;
+            } else if (in.op == PI_CALL) {
+                const uint32_t label = (uint32_t)in.imm, n_args = prog.labels[label].n_args;
+                uint32_t depth = 0;
+                ++invocations;
+                if (z.max_depth != 0xFFFFFFFFu) {
+                    depth = ((h & POOL_ROOT) ? 0u : (h >> 22) & 63u) + 1u;
+                    if (depth > z.max_depth) {
+                        error(RDF_ERR_TAG_OVERFLOW);
+                        return;
+                    }
+                    max_depth = max(max_depth, depth);
+                }
+                if (in.tail && !(h & POOL_ROOT) && prog.labels[(h >> 16) & 63u].entry == prog.labels[label].entry) {
+                    // the caller's own output, the same function: the callee takes over the frame (and returns to where its
+                    // caller would)
+                    const uint32_t at = wrap(enter0 + aggregated_inc(&sh.entered[par]));
+                    fill_frame(f, a, in, n_args, (h & ~(63u << 22)) | depth << 22, wave + 1u);
+                    P.enter[at] = (uint16_t)f;              // (one token per frame: the deque holds all frames)
+                    return;
+                }
+                if (run_left == 0) {
+                    run_left = in.n_run;
+                    if (!reserve(run_left, frame_at, slot)) return;
+                }
+                --run_left;
+                const uint32_t nf = P.ring[wrap(ring0 + frame_at++)];
+                fill_frame(nf, a, in, n_args, f | label << 16 | depth << 22, wave + 1u);
+                P.enter[wrap(enter0 + slot++)] = (uint16_t)nf;
+                if (in.last) return;
+            } else {
+                const int64_t b = val(in.rb, in.ib);
+                switch (in.op) {
+                    case PI_ADD: set(in.dst, a + b); break;
+                    case PI_SUB: set(in.dst, a - b); break;
+                    case PI_MUL: set(in.dst, a * b); break;
+                    case PI_MAX: set(in.dst, a > b ? a : b); break;
+                    case PI_REM: set(in.dst, b == 0 ? 0 : a % b); break;
+                    case PI_CMP: set(in.dst, in.cmp == PC_LT ? a < b : (a == b) == (in.cmp == PC_EQ)); break;
+                    case PI_MOV: set(in.dst, a); break;
+                    case PI_CONST: set(in.dst, prog.consts[in.imm]); break;
+                    case PI_ARG: set(in.dst, P.words[in.imm * z.cap + f]); break;
+                    case PI_JMP: pc = in.imm; break;
+                    case PI_PORT:
+                        deliver(f, in.imm, in.cmp, a);
+                        if (in.last) return;
+                        break;
+                    case PI_TREE: {
+                        if (a < 0 || a >= c.N) {
+                            error(RDF_ERR_BAD_ARG);
+                            return;
+                        }
+                        const int32_t* src = in.cmp == PT_RIGHT ? c.right : in.cmp == PT_TOK ? c.tok : c.left;
+                        const int32_t x = __ldg(&src[a]);
+                        set(in.dst, in.cmp == PT_ISLEAF ? (int64_t)(x < 0) : (int64_t)x);
+                        break;
+                    }
+                    case PI_OUT: {
+                        const uint32_t inst = h & ~POOL_ROOT;
+                        if (inst < c.B) c.y[inst] = a;
+                        give_back(f);
+                        return;
+                    }
+                    default: return;                        // PI_HALT
+                }
+            }
+        }
+        error(RDF_ERR_WAVE_LIMIT);
+    }
+};
+
+// Frames a round may enter: one per thread while the pool has frames to spare for what they may call (`div` each).  A reserve
+// of (depth + 1) x (calls per body) frames stays untouched by rounds that enter two or more, so that a single frame at a
+// time -- plain depth-first recursion -- always gets through where the depth is bounded.
+__device__ __forceinline__ uint32_t pool_width(const PoolSizes& z, uint32_t avail) {
+    return max(1u, avail > z.reserve ? (avail - z.reserve) / z.div : 0u);
+}
+
+__global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ PoolProgram program,
+                                                                             const __grid_constant__ PoolSizes z) {
+    constexpr uint32_t T = POOL_THREADS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ PoolShared sh;
+    const uint32_t tid = threadIdx.x;
+    Pool P;
+    {
+        unsigned char* p = smem;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(p);
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(&program);
+        for (uint32_t i = tid; i < sizeof(PoolProgram) / 4; i += T) dst[i] = src[i];
+        P.prog = reinterpret_cast<const PoolProgram*>(p);
+        p += sizeof(PoolProgram);
+        P.regs = reinterpret_cast<int64_t*>(p); p += (size_t)(program.n_regs + 1) * T * 8;
+        P.words = reinterpret_cast<int64_t*>(p); p += (size_t)program.words * z.cap * 8;
+        P.head = reinterpret_cast<uint32_t*>(p); p += (size_t)z.cap * 4;
+        P.state = reinterpret_cast<uint32_t*>(p); p += (size_t)z.cap * 4;
+        P.enter = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2;
+        P.match = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2;
+        P.ring = reinterpret_cast<uint16_t*>(p);
+    }
+    for (uint32_t i = tid; i < z.cap; i += T) P.ring[i] = (uint16_t)i;
+    P.regs[program.n_regs * T + tid] = 0ll;
+    if (tid == 0) sh = PoolShared{};
+    const uint32_t B = (uint32_t)c.B, chunks = (B + z.chunk - 1) / z.chunk;
+    uint32_t ib = min(B, blockIdx.x * z.chunk), ie = min(B, ib + z.chunk);       // instances this block has taken and not yet started
+    bool more = blockIdx.x < chunks;
+    PoolThread t{c, z, P, sh, tid};
+    uint32_t ebase = 0, ne = 0, nm = 0, ring0 = 0, avail = z.cap, par = 0, widest = 0;      // frames to enter, completed matches
+    unsigned long long tokens = 0;
+    __syncthreads();
+    for (uint32_t round = 0;; ++round) {
+        // ---- more instances, while few tokens are pending and at most half of the frames are in use
+        if (more && ne + nm < z.refill && avail > z.cap / 2 && ib < ie) {
+            const uint32_t k = min(min(ie - ib, T - min(ne, T)), avail / 4);
+            if (tid < k) {
+                const uint32_t f = P.ring[t.wrap(ring0 + tid)], inst = ib + tid;
+                P.head[f] = POOL_ROOT | inst;
+                P.words[f] = c.x ? c.x[inst] : (int64_t)c.tree_root[inst];
+                P.state[f] = 0u;
+                P.enter[t.wrap(ebase + ne + tid)] = (uint16_t)f;
+            }
+            ib += k; ne += k; avail -= k;
+            ring0 = t.wrap(ring0 + k);
+            if (ib == ie) {
+                if (tid == 0) sh.next_chunk = gridDim.x + atomicAdd(&c.ctl->next_chunk, 1u);
+                __syncthreads();
+                const uint32_t q = sh.next_chunk;
+                more = q < chunks;
+                if (more) { ib = q * z.chunk; ie = min(B, ib + z.chunk); }
+            }
+            __syncthreads();
+        }
+        if (ne + nm == 0) {
+            if (!more) break;
+            continue;
+        }
+        // ---- this round's tokens: completed matches for the first warps, frames to enter for the others
+        const uint32_t width = pool_width(z, avail);
+        const uint32_t mm = min(min(nm, T), z.cont_calls ? width : T), w0 = (mm + 31u) & ~31u;
+        const uint32_t me = min(min(ne, T - w0), z.cont_calls && mm ? (width > mm ? width - mm : 0u) : width);
+        uint32_t f = 0xFFFFFFFFu;
+        int node = -1;
+        if (tid < mm) {
+            const uint32_t v = P.match[nm - 1u - tid];
+            f = v & (POOL_MAX_FRAMES - 1u);
+            node = (int)(v >> 13);
+        } else if (tid >= w0 && tid - w0 < me) f = P.enter[t.wrap(ebase + ne - 1u - (tid - w0))];
+        widest = max(widest, ne + nm);
+        tokens += mm + me;
+        t.ring0 = ring0; t.avail = avail; t.ring_tail = t.wrap(ring0 + avail);
+        t.enter0 = t.wrap(ebase + ne - me); t.match0 = nm - mm; t.par = par;
+        __syncthreads();
+        if (f != 0xFFFFFFFFu) t.run(f, node);
+        if (tid == 0) {
+            sh.entered[par ^ 1u] = 0u; sh.matched[par ^ 1u] = 0u; sh.freed[par ^ 1u] = 0u; sh.taken[par ^ 1u] = 0u;
+            if ((round & 255u) == 255u && ld_volatile_i32(&c.ctl->status) != 0) sh.stop = 1;       // another block failed
+            if (c.tag_mode == RDF_TAGS_FRAME && tokens > 2ull * (z.max_calls + B) + T) {             // more calls than the caller allows
+                set_status(c, RDF_ERR_FRAMES_FULL);
+                sh.stop = 1;
+            }
+        }
+        __syncthreads();
+        ne = ne - me + sh.entered[par];
+        nm = nm - mm + sh.matched[par];
+        ring0 = t.wrap(ring0 + sh.taken[par]);
+        avail = avail - sh.taken[par] + sh.freed[par];
+        if (sh.stop) break;
+        par ^= 1u;
+    }
+    // ---- counters, and (the block that ends last) the verdict on the capacities of the call
+    if (sh.stop == 2 && tid == 0) c.ctl->pool_exhausted = 1;
+    ThreadStats st;
+    st.invocations = t.invocations; st.max_depth = t.max_depth;
+    st.sc.inserts = t.inserts; st.sc.matches = t.matches;
+    flush_stats(c, st);
+    const uint32_t w = __reduce_max_sync(0xffffffffu, t.max_wave);
+    if ((tid & 31u) == 0) atomicMax(&c.ctl->waves, w + 1u);
+    if (tid == 0) atomicMax(&c.ctl->max_wave_tokens, widest);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0 && atomicAdd(&c.ctl->blocks_done, 1u) == gridDim.x - 1u) {
+        __threadfence();
+        volatile Control* k = c.ctl;
+        k->tokens = k->invocations + (unsigned long long)c.B;
+        if (!k->pool_exhausted) {
+            if (c.tag_mode == RDF_TAGS_FRAME && k->invocations > z.max_calls) set_status(c, RDF_ERR_FRAMES_FULL);
+            if (c.tag_mode == RDF_TAGS_PATH && k->store_inserts > z.max_parked) set_status(c, RDF_ERR_STORE_FULL);
+        }
+        k->forward_status = k->status;
+    }
+}
+
+// The call again for the general scheduler, when a block of the pool kernel ran out of frames (recursion deeper than a pool):
+// what that scheduler expects cleared and seeded.
+__global__ void __launch_bounds__(256) rdf_pool_fallback_kernel(const DevCtx c, size_t pair_n, size_t arrived_n, size_t table_n) {
+    if (!c.ctl->pool_exhausted) return;
+    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = i0; i < pair_n; i += stride) reinterpret_cast<uint4*>(c.pair_slots)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = i0; i < arrived_n; i += stride) c.arrived[i] = 0u;
+    for (size_t i = i0; i < table_n; i += stride) reinterpret_cast<uint4*>(c.table)[i] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    for (long long b = (long long)i0; b < c.B; b += (long long)stride) seed_instance(c, b);
+    if (i0 == 0) {
+        Control* k = c.ctl;
+        k->invocations = k->tokens = k->store_inserts = k->store_matches = 0ull;
+        k->status = 0; k->waves = k->max_wave_tokens = k->max_depth = 0u;
+    }
+}

@@ -519,3 +519,123 @@ def test_search_steered_by_a_call_result(threshold):
         mine = {w for w in got if w[0] == b}
         assert len(mine) == len(res.calls) or len(mine) >= len(res.calls)     # (tags of different callees may coincide in the oracle's table)
         assert {(b, t, a[0], res.returns[t]) for t, a in res.calls.items()} <= mine
+
+
+# ------------------------------------------------------------- the pool executor
+def _wrap64(v):
+    return (v + (1 << 63)) % (1 << 64) - (1 << 63)
+
+
+def _random_program(seed):
+    """result(x) = f(x) + const; f(n) = a random call-free expression below 2, else a random combination of calls of f at
+    smaller arguments: value conditionals, shared subexpressions, constants beyond 32 bits, one to three match nodes, calls
+    as arguments of calls."""
+    rng = np.random.default_rng(seed)
+    r = rdf.Function("result", 1)
+    r.ret(r.add(r.call(1, r.param()), r.const([0, 5, 2 ** 40 + 1][rng.integers(3)])))
+    f = rdf.Function("f", 1)
+    n = f.param()
+    pool = [n, f.const(int(rng.integers(-3, 4))), f.const(2 ** 35 + int(rng.integers(9)))]
+
+    def expr(depth):
+        if depth == 0:
+            return pool[rng.integers(len(pool))]
+        k = ["add", "sub", "mul", "max", "lt", "eq", "rem", "if_"][rng.integers(8)]
+        v = getattr(f, k)(*[expr(depth - 1) for _ in range(3 if k == "if_" else 2)])
+        pool.append(v)
+        return v
+
+    base = expr(int(rng.integers(1, 4)))
+    c1, c2 = f.call(1, f.sub(n, f.const(1))), f.call(1, f.sub(n, f.const(int(rng.integers(2, 4)))))
+    comb = f.add(f.mul(c1, f.const(3)), c2) if rng.random() < 0.4 else f.max(f.add(c1, expr(1)), f.sub(c2, n))
+    if rng.random() < 0.3:
+        comb = f.add(comb, f.call(1, f.sub(n, f.const(4))))
+    f.ret(f.if_(f.lt(n, f.const(2)), base, comb))
+    return [r, f]
+
+
+def _evaluate(functions, x):
+    """The program by direct recursion over its expressions: (value, calls)."""
+    calls = [0]
+
+    def call(k, a):
+        fn, memo = functions[k], {}
+
+        def ev(i):
+            if i not in memo:
+                op, p, q, s, imm = fn.exprs[i]
+                if op == bd.OP_PARAM:
+                    memo[i] = a
+                elif op == bd.OP_CONST:
+                    memo[i] = imm
+                elif op == bd.OP_CALL:
+                    calls[0] += 1
+                    memo[i] = call(imm, ev(p))
+                elif op == bd.OP_IF:
+                    memo[i] = ev(q) if ev(p) else ev(s)
+                else:
+                    u, v = ev(p), ev(q)
+                    memo[i] = {bd.OP_ADD: lambda: _wrap64(u + v), bd.OP_SUB: lambda: _wrap64(u - v), bd.OP_MUL: lambda: _wrap64(u * v),
+                               bd.OP_MAX: lambda: max(u, v), bd.OP_LT: lambda: int(u < v), bd.OP_EQ: lambda: int(u == v),
+                               bd.OP_REM: lambda: programs.INT_OPS["%"](u, v)}[op]()
+            return memo[i]
+        return ev(fn.root)
+    return call(0, x), calls[0]
+
+
+def test_pool_executor_runs_random_programs():
+    """Programs fused for the pool executor (constants and copies folded into operands, compare-and-branch, runs of calls,
+    several match nodes in a body) against direct recursion: values and numbers of calls."""
+    xs = list(range(9))
+    x = torch.tensor(xs * 20, dtype=torch.int64, device="cuda")
+    ran = 0
+    for seed in range(60):
+        fs = _random_program(seed)
+        want = [_evaluate(fs, v) for v in xs]
+        try:
+            g = rdf.Graph(fs, 0, rdf.TAGS_FRAME)
+        except rdf.RdfError as e:
+            assert e.code == -11                  # more registers than a segment has
+            continue
+        ran += 1
+        y, _ = g.eval_int(x, max_invocations=20 * sum(w[1] for w in want))
+        assert y.tolist() == [w[0] for w in want] * 20, seed
+        assert g.stats()["invocations"] == 20 * sum(w[1] for w in want), seed
+    assert ran >= 30
+
+
+@pytest.mark.parametrize("mode", [rdf.TAGS_PATH, rdf.TAGS_FRAME])
+@pytest.mark.parametrize("B", [1, 2, 147, 148, 149, 592, 2367, 2368, 5000])
+def test_pool_executor_batch_sizes(B, mode):
+    """Batches around one instance per block, several chunks per block and the switch to early refills; one instance with
+    more calls than a pool has frames among small ones."""
+    x_host = workloads.fib_batch(seed=B, B=B, n_hi=12)
+    x_host[B // 2] = 18
+    n_inv = int(sum(2 * _fib_iter(int(n) + 1) - 1 for n in x_host))
+    g = rdf.Graph(*rdf.fib_program(), mode)
+    for _ in range(2):
+        y, _ = g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=n_inv)
+        assert y.tolist() == [_fib_iter(int(n)) for n in x_host]
+        st = g.stats()
+        assert st["invocations"] == n_inv and st["store_inserts"] == st["store_matches"] == (n_inv - B) // 2
+    if mode == rdf.TAGS_FRAME:                    # one call too many is a status code (no traceback kept: it would hold the workspace)
+        code = 0
+        try:
+            g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=n_inv - 1)
+        except rdf.RdfError as err:
+            code = err.code
+        assert code == -6
+
+
+def test_recursion_deeper_than_a_pool():
+    """More frames alive at a time than a pool holds: the call goes to the general scheduler and ends with the same results."""
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f = rdf.Function("down", 1)
+    n = f.param()
+    f.ret(f.if_(f.lt(n, f.const(1)), f.const(0), f.add(n, f.call(1, f.sub(n, f.const(1))))))
+    g = rdf.Graph([r, f], 0, rdf.TAGS_FRAME)
+    xs = [0, 5, 20000, 300, 8191, 8192]
+    y, _ = g.eval_int(torch.tensor(xs, dtype=torch.int64, device="cuda"), max_invocations=sum(xs) + len(xs))
+    assert y.tolist() == [v * (v + 1) // 2 for v in xs]
+    assert g.stats()["invocations"] == sum(xs) + len(xs) and g.stats()["waves"] >= 20000
