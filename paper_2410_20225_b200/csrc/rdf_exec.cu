@@ -1455,12 +1455,13 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     z.max_depth = g->tag_mode == RDF_TAGS_PATH ? (uint32_t)(RDF_PATH_BITS / g->label_bits) : 0xFFFFFFFFu;
     // frames a token may take in a round, and what depth-first recursion one token at a time needs (rdf_pool.cuh: pool_width)
     const uint32_t calls = (uint32_t)std::max(1, std::max(P.calls_entry, P.calls_cont));
-    z.div = std::max(4u, calls);
-    z.reserve = std::min(z.cap / 2, ((g->tag_mode == RDF_TAGS_PATH ? z.max_depth : 64u) + 1u) * calls + z.div);
+    z.div_shift = 1;
+    while ((1u << z.div_shift) < calls) ++z.div_shift;
+    z.reserve = std::min(z.cap / 2, ((g->tag_mode == RDF_TAGS_PATH ? z.max_depth : 64u) + 1u) * calls + (1u << z.div_shift));
     z.cont_calls = P.calls_cont > 0;
     const int grid = (int)std::min<long long>((long long)S->grid * POOL_PER_SM, in->B);
-    z.chunk = (uint32_t)std::max<long long>(1, std::min<long long>(in->B / ((long long)grid * 8), POOL_THREADS / 4));
-    z.refill = in->B >= 16ll * grid ? (uint32_t)POOL_THREADS : 1u;
+    z.chunk = (uint32_t)std::max<long long>(1, std::min<long long>(in->B / ((long long)grid * 4), POOL_THREADS / 4));
+    z.refill = POOL_THREADS / 3;
     z.max_calls = (unsigned long long)in->max_invocations;
     z.max_parked = (unsigned long long)L.table_cap * std::max<size_t>(1, g->match.size());
     rdf_mark(S, 1, stream);
@@ -1469,6 +1470,11 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     CUDA_OK(cudaGetLastError());
     return RDF_OK;
 }
+
+// One block runs an instance to its end, so a few large instances are better spread over the device wave by wave: one call
+// of fib(18) (8361 calls) takes 0.10 ms in a pool and 0.22 in waves, fib(22) (57 313) 0.36 and 0.30, fib(24) (150 049) 0.87
+// and 0.34, eight of fib(22) 0.36 and 0.34; but 32 of fib(24) 0.90 and 1.58.
+static const long long POOL_CALLS = 40000, POOL_MANY = 32;
 
 // zero what must start at zero, upload the program, seed, run all waves
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,
@@ -1483,7 +1489,8 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     // bound on the width of a wave, the waits and waves that rdf_set_limits limits, and the cooperative probes.
     const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= 4u * POOL_THREADS && S->wait_cycles == 0 &&
                       S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
-                      (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B);
+                      (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B) &&
+                      (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);
     if (pool) {
         const int rc = rdf_launch_pool(g, in, L, S, c, stream);
         if (rc != RDF_OK) return rc;

@@ -1232,6 +1232,96 @@ struct PoolBuilder {
         }
     }
 
+    // ---- shapes that run without the interpreter
+    PoolOperand plain(uint8_t reg, int32_t imm, int n_in) const {       // an operand over the first n_in registers
+        need(reg == out.n_regs || reg < n_in);
+        return PoolOperand{reg == out.n_regs ? 3 : reg, imm};
+    }
+    PoolAction action(int i, int n_in) const {                          // return or calls, and nothing else
+        PoolAction act{};
+        const PoolInstr& in = out.code[i];
+        if (in.op == PI_RET) {
+            act.ops[0] = plain(in.ra, in.ia, n_in);
+            return act;
+        }
+        need(in.op == PI_CALL && in.n_run >= 1 && in.n_run <= 3 && !in.tail);
+        act.n_calls = in.n_run;
+        for (int k = 0; k < in.n_run; ++k) {
+            const PoolInstr& q = out.code[i + k];
+            need(q.op == PI_CALL && (bool)q.last == (k + 1 == in.n_run));
+            const int m = n_args(q.imm);
+            act.labels[k] = q.imm | m << 8;
+            act.ops[3 * k] = plain(q.ra, q.ia, n_in);
+            act.ops[3 * k + 1] = m > 1 ? plain(q.rb, q.ib, n_in) : PoolOperand{3, 0};
+            act.ops[3 * k + 2] = m > 2 ? plain(q.rc, q.ic, n_in) : PoolOperand{3, 0};
+        }
+        return act;
+    }
+    PoolEntry entry_shape(int i, int n_in) const {
+        PoolEntry e{};
+        e.n_args = n_in;
+        while (out.code[i].op == PI_BR) {
+            need(e.n_cond < 2);
+            const PoolInstr& in = out.code[i];
+            e.cmp[e.n_cond] = in.cmp;
+            e.a[e.n_cond] = plain(in.ra, in.ia, n_in);
+            e.b[e.n_cond] = plain(in.rb, in.ib, n_in);
+            e.act[e.n_cond] = action(i + 1, n_in);
+            ++e.n_cond;
+            i = in.imm;
+        }
+        e.act[e.n_cond] = action(i, n_in);
+        return e;
+    }
+    PoolCont cont_shape(int i, int n_in) const {
+        PoolCont q{};
+        const PoolInstr* in = &out.code[i];
+        if (in->op == PI_CALL && in->tail) {
+            q.op = PI_CALL;
+            q.label = in->imm;
+            const int m = n_args(in->imm);
+            q.ops[0] = plain(in->ra, in->ia, n_in);
+            q.ops[1] = m > 1 ? plain(in->rb, in->ib, n_in) : PoolOperand{3, 0};
+            q.ops[2] = m > 2 ? plain(in->rc, in->ic, n_in) : PoolOperand{3, 0};
+            return q;
+        }
+        need(in->op == PI_ADD || in->op == PI_SUB || in->op == PI_MUL || in->op == PI_MAX);
+        need(out.code[i + 1].op == PI_RET && out.code[i + 1].ra == in->dst);
+        q.op = in->op;
+        q.a = plain(in->ra, in->ia, n_in);
+        q.b = plain(in->rb, in->ib, n_in);
+        q.imm = out.code[i + 1].ia;
+        return q;
+    }
+    void find_shapes() {
+        std::map<int, int> of_pc;                // entry -> PoolProgram::entry_of
+        for (int k = 0; k < out.n_labels; ++k) {
+            PoolLabel& L = out.labels[k];
+            L.fast = -1;
+            if (of_pc.count(L.entry)) { L.fast = of_pc[L.entry]; continue; }
+            int at = -1;
+            if ((int)of_pc.size() < POOL_MAX_ENTRY) {
+                try {
+                    const PoolEntry e = entry_shape(L.entry, L.n_args);
+                    at = 0;
+                    for (const auto& q : of_pc) at = std::max(at, q.second + 1);
+                    if (at < POOL_MAX_ENTRY) out.entry_of[at] = e; else at = -1;
+                } catch (const Fail&) {
+                    at = -1;
+                }
+            }
+            of_pc[L.entry] = at;
+            L.fast = at;
+        }
+        for (int k = 0; k < out.n_match && k < POOL_MAX_CONT; ++k) {
+            try {
+                out.cont_of[k] = cont_shape(out.match[k].cont, out.match[k].n_ports);
+            } catch (const Fail&) {
+                out.cont_of[k] = PoolCont{};     // (PI_HALT)
+            }
+        }
+    }
+
     // false: not a program for the pool executor
     bool build() {
         if (g->has_vector_ops || g->has_loops || g->interleaved) return false;
@@ -1300,7 +1390,7 @@ struct PoolBuilder {
         for (int k = 0; k < out.n_labels; ++k) {
             const LabelInfo& L = g->labels[k];
             out.labels[k] = PoolLabel{(int16_t)new_pc[L.entry_pc], (int16_t)(L.k_kind == K_SEG ? new_pc[L.k_pc] : 0), (uint8_t)L.k_kind,
-                                      (uint8_t)(L.k_kind == K_PORT ? L.k_node : 0), (uint8_t)(L.k_kind == K_PORT ? L.k_port : 0), (uint8_t)L.n_args};
+                                      (uint8_t)(L.k_kind == K_PORT ? L.k_node : 0), (uint8_t)(L.k_kind == K_PORT ? L.k_port : 0), (uint8_t)L.n_args, -1, 0};
         }
         for (int k = 0; k < out.n_match; ++k) {
             const MatchNode& M = g->match[k];
@@ -1315,6 +1405,7 @@ struct PoolBuilder {
             int& most = entries.count(seg[k]) ? out.calls_entry : out.calls_cont;
             most = std::max(most, calls);
         }
+        find_shapes();
         return true;
     }
 };

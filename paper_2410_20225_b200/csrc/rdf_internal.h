@@ -98,15 +98,38 @@ struct alignas(16) PoolInstr {
     int32_t imm;                     // branch target, label, match node, constant, parameter
     int32_t pad[2];
 };
-struct PoolLabel {
+struct alignas(16) PoolLabel {
     int16_t entry, k_pc;
     uint8_t k_kind, k_node, k_port, n_args;
+    int32_t fast;                    // PoolProgram::entry_of its callee, -1: run by the interpreter
+    int32_t pad;
 };
 struct PoolMatch {
     int16_t  cont;
     uint8_t  n_ports, word0;         // its ports are words word0 .. of the frame
     uint32_t all;                    // bits of its ports
 };
+// Common shapes of a segment, run without the interpreter, everything in registers (operand registers 0 .. 2: the arguments
+// or the operands of the match; 3: zero).
+struct PoolOperand { int32_t reg, imm; };
+struct alignas(16) PoolAction {                  // return ops[0], or make n_calls calls with 3 operands each
+    int32_t n_calls, labels[3];                  // n_calls 0: return; label | arguments << 8
+    PoolOperand ops[9];
+    int32_t pad[2];
+};
+struct alignas(16) PoolEntry {                   // entering a function: the action of the first condition that holds, else the last one
+    int32_t n_cond, n_args, cmp[2];              // n_cond -1: not of this shape
+    PoolOperand a[2], b[2];
+    PoolAction act[3];
+};
+struct alignas(16) PoolCont {                    // after a match: return `a op b` + imm, or (op PI_CALL) the caller's own output is a call
+    int32_t op, imm;                             // op PI_HALT: not of this shape
+    PoolOperand a, b;
+    PoolOperand ops[3];
+    int32_t label;
+    int32_t pad[3];
+};
+static const int POOL_MAX_ENTRY = 4, POOL_MAX_CONT = 2;
 static const int POOL_MAX_CODE = 48, POOL_MAX_LABELS = 16, POOL_MAX_MATCH = 8, POOL_MAX_CONSTS = 4, POOL_MAX_WORDS = 8;
 struct alignas(16) PoolProgram {
     int32_t   n_code, n_labels, n_match, result_entry;
@@ -116,6 +139,8 @@ struct alignas(16) PoolProgram {
     PoolLabel labels[POOL_MAX_LABELS];
     PoolMatch match[POOL_MAX_MATCH];
     int64_t   consts[POOL_MAX_CONSTS];
+    PoolEntry entry_of[POOL_MAX_ENTRY];
+    PoolCont  cont_of[POOL_MAX_CONT];    // by match node
 };
 
 struct rdf_graph {

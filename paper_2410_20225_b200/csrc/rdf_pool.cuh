@@ -12,25 +12,31 @@
 // top of the frames to enter, so that the threads of a warp do the same thing.  A thread runs one segment: new frames for
 // the calls it makes, pushed as tokens; or a value that is returned -- parked in the caller's frame, and if it was the last
 // operand the match becomes a token (carrying on in the same thread instead leaves the warp to a few long chains of returns:
-// 131 072 calls of fib took 13.0 ms with up to three in a row, 24.7 with eight, 7.8 with none).
+// 131 072 calls of fib took 13.0 ms with up to three in a row, 24.7 with eight, 7.8 with none, before the other measures).
 // The program is a fused form of the lowered code (PoolBuilder): operands are register + immediate, a comparison branches by
 // itself, consecutive calls reserve their frames together.
 //
-// What bounds it: the latency of a round -- a warp runs some 500 dependent instructions of the interpreter between two block
-// barriers, and the frames that fit the shared memory limit the warps to about 16 per SM.
-// Measured, general scheduler -> this: 131 072 calls of fib(0..18) 36.3 -> 7.8 ms, 1024 calls 0.721 -> 0.321 ms, 8 calls of
-// fib(0..10) 0.137 -> 0.038 ms, 200 calls of tak 1.76 -> 1.19 ms (one block runs the largest instance to its end).
+// Segments of the common shapes (a list of conditions that ends in a return or in calls; an operator and a return; a tail
+// call) run without the interpreter, from registers.
+//
+// What bounds it: the latency of a round -- some 400 dependent instructions per warp between two block barriers -- and the
+// frames that fit the shared memory, which limit the tokens of a round.
+// Measured, general scheduler -> this: 131 072 calls of fib(0..18) 36.3 -> 5.5 ms, 1024 calls 0.721 -> 0.17 ms, 8 calls of
+// fib(0..10) 0.137 -> 0.036 ms, 200 calls of tak 1.76 -> 0.75 ms (limited by the depth of the largest instance).
+// Handing calls of a busy block to idle ones through global memory was built and dropped: 200 calls of tak 0.90 -> 0.83 ms,
+// but 1024 calls of fib 0.23 -> 0.31 ms.
 // (Included by rdf_exec.cu only: it defines kernels.)
 #pragma once
 #include "rdf_exec.h"
 
-static const int POOL_THREADS = 512, POOL_PER_SM = 1;   // threads of a block, blocks per SM
+static const int POOL_THREADS = 768, POOL_PER_SM = 1;   // threads of a block, blocks per SM (131 072 calls of fib: 512 threads 6.7 ms, 768 5.5,
+                                                        // 1024 6.2, two blocks of 256 6.7: more threads leave each fewer frames)
 static const uint32_t POOL_ROOT = 0x80000000u;          // frame word of an instance's `result` context: | instance
 // Frame word of an invocation: parent frame [15:0], label [21:16], depth of the tag [27:22] (path tags)
 
 struct PoolSizes {
     uint32_t cap;            // frames of a block
-    uint32_t div, reserve;   // pool_width
+    uint32_t div_shift, reserve;   // pool_width
     uint32_t cont_calls;     // a completed match may take frames too
     uint32_t chunk;          // instances a block takes at a time
     uint32_t refill;         // it takes them when fewer tokens than this are pending
@@ -64,6 +70,14 @@ struct Pool {
     uint16_t* ring;          // [cap] free frames, oldest first
 };
 
+// k consecutive places on a shared counter for every thread that gets here together: one atomic per group
+__device__ __forceinline__ uint32_t pool_take(uint32_t* counter, uint32_t k) {
+    const uint32_t group = __activemask(), lane = threadIdx.x & 31u, leader = __ffs(group) - 1;
+    uint32_t base = 0;
+    if (lane == leader) base = atomicAdd(counter, k * __popc(group));
+    return __shfl_sync(group, base, leader) + k * __popc(group & ((1u << lane) - 1u));
+}
+
 struct PoolThread {
     static const int T = POOL_THREADS;
     const DevCtx& c;
@@ -81,10 +95,11 @@ struct PoolThread {
         set_status(c, code);
         sh.stop = 1;
     }
-    __device__ __forceinline__ void give_back(uint32_t f) { P.ring[wrap(ring_tail + aggregated_inc(&sh.freed[par]))] = (uint16_t)f; }
+    __device__ __forceinline__ void give_back(uint32_t f) { P.ring[wrap(ring_tail + pool_take(&sh.freed[par], 1u))] = (uint16_t)f; }
     // k frames for calls that follow one another, and their places on the stack (first of each); false: the pool is exhausted
     __device__ __forceinline__ bool reserve(uint32_t k, uint32_t& frame_at, uint32_t& slot) {
-        aggregated_inc2n(&sh.taken[par], &sh.entered[par], k, frame_at, slot);
+        frame_at = pool_take(&sh.taken[par], k);
+        slot = pool_take(&sh.entered[par], k);
         if (frame_at + k <= avail) return true;
         sh.stop = 2;
         return false;
@@ -101,17 +116,69 @@ struct PoolThread {
             return;
         }
         ++matches;
-        const uint32_t at = match0 + aggregated_inc(&sh.matched[par]);
+        const uint32_t at = match0 + pool_take(&sh.matched[par], 1u);
         if (at < z.cap) P.match[at] = (uint16_t)(f | node << 13);
         else sh.stop = 2;                                   // (only bodies with several match nodes can have more matches than frames)
     }
 
-    __device__ __forceinline__ void fill_frame(uint32_t f, int64_t a0, const PoolInstr& in, uint32_t n_args, uint32_t head, uint32_t wave) {
+    // a frame that waits to be entered
+    __device__ __forceinline__ void fill_frame(uint32_t f, uint32_t n_args, int64_t a0, int64_t a1, int64_t a2, uint32_t head, uint32_t wave) {
         P.head[f] = head;
         P.words[f] = a0;
-        if (n_args > 1) P.words[z.cap + f] = val(in.rb, in.ib);
-        if (n_args > 2) P.words[2 * z.cap + f] = val(in.rc, in.ic);
+        if (n_args > 1) P.words[z.cap + f] = a1;
+        if (n_args > 2) P.words[2 * z.cap + f] = a2;
         P.state[f] = wave;
+    }
+    // Call_i under the tag of frame word h: the depth of the new tag.  False (status set) when it does not fit.
+    __device__ __forceinline__ bool push_tag(uint32_t h, uint32_t& depth) {
+        depth = 0;
+        if (z.max_depth == 0xFFFFFFFFu) return true;
+        depth = ((h & POOL_ROOT) ? 0u : (h >> 22) & 63u) + 1u;
+        if (depth > z.max_depth) {
+            error(RDF_ERR_TAG_OVERFLOW);
+            return false;
+        }
+        max_depth = max(max_depth, depth);
+        return true;
+    }
+    // The call is frame f's own output and enters the same function: the callee takes over the frame (and returns to where its
+    // caller would).
+    __device__ __forceinline__ bool same_function(uint32_t h, uint32_t label) const {
+        return !(h & POOL_ROOT) && P.prog->labels[(h >> 16) & 63u].entry == P.prog->labels[label].entry;
+    }
+    __device__ __forceinline__ void tail_call(uint32_t f, uint32_t h, uint32_t label, int64_t a0, int64_t a1, int64_t a2, uint32_t depth, uint32_t wave) {
+        fill_frame(f, P.prog->labels[label].n_args, a0, a1, a2, (h & ~(63u << 22)) | depth << 22, wave);
+        P.enter[wrap(enter0 + pool_take(&sh.entered[par], 1u))] = (uint16_t)f;      // (one token per frame: the deque holds all frames)
+    }
+    __device__ __forceinline__ static int64_t pick(const PoolOperand& o, int64_t a0, int64_t a1, int64_t a2) {
+        return (o.reg == 0 ? a0 : o.reg == 1 ? a1 : o.reg == 2 ? a2 : 0ll) + (int64_t)o.imm;
+    }
+    __device__ __forceinline__ static bool holds(int cmp, int64_t a, int64_t b) { return cmp == PC_LT ? a < b : (a == b) == (cmp == PC_EQ); }
+
+    // Entering a function of the common shape.
+    __device__ __forceinline__ int enter_fast(uint32_t& f, uint32_t& h, const PoolEntry& e, uint32_t wave) {
+        const int64_t a0 = P.words[f], a1 = e.n_args > 1 ? P.words[z.cap + f] : 0ll, a2 = e.n_args > 2 ? P.words[2 * z.cap + f] : 0ll;
+        int which = e.n_cond;
+        if (e.n_cond > 1 && holds(e.cmp[1], pick(e.a[1], a0, a1, a2), pick(e.b[1], a0, a1, a2))) which = 1;
+        if (e.n_cond > 0 && holds(e.cmp[0], pick(e.a[0], a0, a1, a2), pick(e.b[0], a0, a1, a2))) which = 0;
+        const PoolAction& act = e.act[which];
+        if (act.n_calls == 0) return give_value(f, h, pick(act.ops[0], a0, a1, a2));
+        const uint32_t k = act.n_calls;
+        uint32_t depth, frame_at, slot;
+        invocations += k;
+        if (!push_tag(h, depth) || !reserve(k, frame_at, slot)) return -1;
+#pragma unroll
+        for (uint32_t q = 0; q < 3; ++q)
+            if (q < k) {
+                const uint32_t nf = P.ring[wrap(ring0 + frame_at + q)], label = act.labels[q] & 0xFFu, n_args = act.labels[q] >> 8;
+                P.enter[wrap(enter0 + slot + q)] = (uint16_t)nf;
+                P.head[nf] = f | label << 16 | depth << 22;
+                P.state[nf] = wave + 1u;
+                P.words[nf] = pick(act.ops[3 * q], a0, a1, a2);
+                if (n_args > 1) P.words[z.cap + nf] = pick(act.ops[3 * q + 1], a0, a1, a2);
+                if (n_args > 2) P.words[2 * z.cap + nf] = pick(act.ops[3 * q + 2], a0, a1, a2);
+            }
+        return -1;
     }
 
     // Return_i: frame f (its word h) has the value v.  Returns the code to go on with (in frame f, r0 = v), or -1.
@@ -140,23 +207,46 @@ struct PoolThread {
         if (node >= 0) {
             const PoolMatch M = prog.match[node];
             const int64_t* w = P.words + M.word0 * z.cap + f;
-            set(0, w[0]); set(1, w[z.cap]);
-            for (uint32_t k = 2; k < M.n_ports; ++k) set(k, w[k * z.cap]);
-            pc = M.cont;
+            const int64_t p0 = w[0], p1 = w[z.cap], p2 = M.n_ports > 2 ? w[2 * z.cap] : 0ll;
+            const PoolCont& q = prog.cont_of[min(node, POOL_MAX_CONT - 1)];
+            if (node < POOL_MAX_CONT && q.op == PI_CALL && same_function(h, q.label)) {
+                uint32_t depth;
+                ++invocations;
+                if (push_tag(h, depth))
+                    tail_call(f, h, q.label, pick(q.ops[0], p0, p1, p2), pick(q.ops[1], p0, p1, p2), pick(q.ops[2], p0, p1, p2), depth, 1u);
+                return;
+            }
+            if (node < POOL_MAX_CONT && q.op >= PI_ADD && q.op <= PI_MAX) {
+                const int64_t a = pick(q.a, p0, p1, p2), b = pick(q.b, p0, p1, p2);
+                const int64_t r = q.op == PI_ADD ? a + b : q.op == PI_SUB ? a - b : q.op == PI_MUL ? a * b : a > b ? a : b;
+                pc = give_value(f, h, r + (int64_t)q.imm);
+                if (pc < 0) return;
+            } else {
+                set(0, p0); set(1, p1);
+                for (uint32_t k = 2; k < M.n_ports; ++k) set(k, w[k * z.cap]);
+                pc = M.cont;
+            }
         } else {
             uint32_t n_args = 1;
+            int fast = -1;
             pc = prog.result_entry;
             if (!(h & POOL_ROOT)) {
                 const PoolLabel L = prog.labels[(h >> 16) & 63u];
                 pc = L.entry;
                 n_args = L.n_args;
+                fast = L.fast;
             }
-            set(0, P.words[f]);
-            if (n_args > 1) set(1, P.words[z.cap + f]);
-            if (n_args > 2) set(2, P.words[2 * z.cap + f]);
             wave = P.state[f];
             P.state[f] = 0u;
             max_wave = max(max_wave, wave);
+            if (fast >= 0) {
+                pc = enter_fast(f, h, prog.entry_of[fast], wave);
+                if (pc < 0) return;
+            } else {
+                set(0, P.words[f]);
+                if (n_args > 1) set(1, P.words[z.cap + f]);
+                if (n_args > 2) set(2, P.words[2 * z.cap + f]);
+            }
         }
         uint32_t frame_at = 0, slot = 0, run_left = 0;
         for (uint32_t step = 0; step < (1u << 22); ++step) {
@@ -164,29 +254,18 @@ struct PoolThread {
             const int64_t a = val(in.ra, in.ia);
             if (in.op == PI_BR) {                           // carry on when the comparison holds, else go to imm
                 const int64_t b = val(in.rb, in.ib);
-                const bool t = in.cmp == PC_LT ? a < b : (a == b) == (in.cmp == PC_EQ);
-                if (!t) pc = in.imm;
+                if (!holds(in.cmp, a, b)) pc = in.imm;
             } else if (in.op == PI_RET) {
                 pc = give_value(f, h, a);
                 if (pc < 0) return;
             } else if (in.op == PI_CALL) {
                 const uint32_t label = (uint32_t)in.imm, n_args = prog.labels[label].n_args;
-                uint32_t depth = 0;
+                uint32_t depth;
                 ++invocations;
-                if (z.max_depth != 0xFFFFFFFFu) {
-                    depth = ((h & POOL_ROOT) ? 0u : (h >> 22) & 63u) + 1u;
-                    if (depth > z.max_depth) {
-                        error(RDF_ERR_TAG_OVERFLOW);
-                        return;
-                    }
-                    max_depth = max(max_depth, depth);
-                }
-                if (in.tail && !(h & POOL_ROOT) && prog.labels[(h >> 16) & 63u].entry == prog.labels[label].entry) {
-                    // the caller's own output, the same function: the callee takes over the frame (and returns to where its
-                    // caller would)
-                    const uint32_t at = wrap(enter0 + aggregated_inc(&sh.entered[par]));
-                    fill_frame(f, a, in, n_args, (h & ~(63u << 22)) | depth << 22, wave + 1u);
-                    P.enter[at] = (uint16_t)f;              // (one token per frame: the deque holds all frames)
+                if (!push_tag(h, depth)) return;
+                const int64_t a1 = n_args > 1 ? val(in.rb, in.ib) : 0ll, a2 = n_args > 2 ? val(in.rc, in.ic) : 0ll;
+                if (in.tail && same_function(h, label)) {
+                    tail_call(f, h, label, a, a1, a2, depth, wave + 1u);
                     return;
                 }
                 if (run_left == 0) {
@@ -195,7 +274,7 @@ struct PoolThread {
                 }
                 --run_left;
                 const uint32_t nf = P.ring[wrap(ring0 + frame_at++)];
-                fill_frame(nf, a, in, n_args, f | label << 16 | depth << 22, wave + 1u);
+                fill_frame(nf, n_args, a, a1, a2, f | label << 16 | depth << 22, wave + 1u);
                 P.enter[wrap(enter0 + slot++)] = (uint16_t)nf;
                 if (in.last) return;
             } else {
@@ -206,7 +285,7 @@ struct PoolThread {
                     case PI_MUL: set(in.dst, a * b); break;
                     case PI_MAX: set(in.dst, a > b ? a : b); break;
                     case PI_REM: set(in.dst, b == 0 ? 0 : a % b); break;
-                    case PI_CMP: set(in.dst, in.cmp == PC_LT ? a < b : (a == b) == (in.cmp == PC_EQ)); break;
+                    case PI_CMP: set(in.dst, holds(in.cmp, a, b)); break;
                     case PI_MOV: set(in.dst, a); break;
                     case PI_CONST: set(in.dst, prog.consts[in.imm]); break;
                     case PI_ARG: set(in.dst, P.words[in.imm * z.cap + f]); break;
@@ -239,11 +318,11 @@ struct PoolThread {
     }
 };
 
-// Frames a round may enter: one per thread while the pool has frames to spare for what they may call (`div` each).  A reserve
+// Frames a round may enter: one per thread while the pool has frames to spare for what they may call (2^div_shift each).  A reserve
 // of (depth + 1) x (calls per body) frames stays untouched by rounds that enter two or more, so that a single frame at a
 // time -- plain depth-first recursion -- always gets through where the depth is bounded.
 __device__ __forceinline__ uint32_t pool_width(const PoolSizes& z, uint32_t avail) {
-    return max(1u, avail > z.reserve ? (avail - z.reserve) / z.div : 0u);
+    return max(1u, avail > z.reserve ? (avail - z.reserve) >> z.div_shift : 0u);
 }
 
 __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ PoolProgram program,
