@@ -68,6 +68,7 @@ struct alignas(128) HotCounter {
 struct Control {
     HotCounter qcount[3];         // tokens in the queue of wave w at [w % 3]
     HotCounter cell_count;        // ready cells queued so far, all waves (length of cell_items)
+    HotCounter unary_count[2];    // interleaved execution: unary operators queued so far (left, right half of W)
     HotCounter leaf_count;        // ready leaves queued so far (length of leaf_items)
     HotCounter frame_count;
     HotCounter bar;               // grid barrier arrivals of the scheduler kernel (monotone)
@@ -141,6 +142,7 @@ struct DevCtx {
     uint4*    cell_link;          // [work_cap] per grouped cell: where its operands come from and its state goes (rdf_group_link_kernel)
     uint32_t* group_ends;         // [wave_cap + 2]: cells per group, then (after the scatter) the end of each group
     LeafItem* leaf_items;         // every leaf in the order it was reached
+    uint2*    unary_items[2];     // interleaved execution: {result frame, operand frame} of the unary operators, by half of W
     uint32_t  work_cap;
     uint32_t* op_l;               // per frame: operand frames of the operator that made its state
     uint32_t* op_r;               //            (leaf: op_l = LEAF_MARK, op_r = token id)

@@ -293,26 +293,34 @@ __device__ void run_token(const DevCtx& c, const SharedProgram& sp, const LocalQ
                     set_status(c, RDF_ERR_BAD_ARG);
                     return;
                 }
+                // (four terms per load: the lanes read different rows, and every load is a request per lane)
                 const float* h = c.arena + (size_t)ref * c.S;
                 float acc = c.b_s[0];
-                for (int k = 0; k < c.H; ++k) acc = fmaf(__ldg(&c.W_s[k]), __ldcg(&h[k]), acc);
+#pragma unroll 4
+                for (int k = 0; k < c.H; k += 4) {
+                    const float4 x = ldcg4(h + k), w = __ldg(reinterpret_cast<const float4*>(c.W_s + k));
+                    acc = fmaf(w.w, x.w, fmaf(w.z, x.z, fmaf(w.y, x.y, fmaf(w.x, x.x, acc))));
+                }
                 r[in.dst] = acc > 0.f;
                 break;
             }
             case VM_VCHILD: {
-                // a unary vector operator: queued like a cell whose second operand is the marker of the operator
-                uint32_t i, slot = 0;
-                aggregated_inc2(&c.ctl->cell_count.v, &c.ctl->qcount[(wave + 1) % 3].v, i, slot);
+                // a unary vector operator: the list of its half of W
+                // (threads of both halves get here together: one place per thread on the counter of its half)
+                const int half = in.dst ? 1 : 0;
+                const unsigned here = __activemask(), mine = __match_any_sync(here, half);
+                const uint32_t lane = threadIdx.x % 32, leader = __ffs(mine) - 1;
+                uint32_t i = lane == leader ? atomicAdd(&c.ctl->unary_count[half].v, (uint32_t)__popc(mine)) : 0u;
+                const uint32_t slot = aggregated_inc(&c.ctl->qcount[(wave + 1) % 3].v);
+                i = __shfl_sync(here, i, leader) + __popc(mine & ((1u << lane) - 1u));
                 if (i >= c.work_cap || slot >= c.qcap) {
                     set_status(c, RDF_ERR_QUEUE_FULL);
                     return;
                 }
-                CellItem it;
-                it.out = (uint32_t)tag; it.l = (uint32_t)r[in.a]; it.r = in.dst ? CHILD_R_MARK : CHILD_L_MARK;
-                it.valid = 1u;
-                c.cell_items[i] = it;
-                c.op_l[tag] = it.l;
-                c.op_r[tag] = it.r;
+                const uint32_t x = (uint32_t)r[in.a];
+                c.unary_items[half][i] = make_uint2((uint32_t)tag, x);
+                c.op_l[tag] = x;
+                c.op_r[tag] = half ? CHILD_R_MARK : CHILD_L_MARK;
                 ++st.cells;
                 store_token(&c.q[(wave + 1) & 1][slot], tag, (int64_t)(uint32_t)tag, (uint32_t)in.imm);
                 break;
@@ -630,19 +638,70 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
 }
 
 
-static inline int interleaved_smem_bytes(int H) { return 2 * H * 33 * (int)sizeof(float); }
+// Vector operators of the interleaved execution.  A group of operators of one kind: rows xs[item][0 .. K) in shared memory,
+// outputs tanh(W[:, k0 : k0 + K] x + b).  A warp computes 16 items x 16 outputs, a thread 2 x 4 of them: its 8 lanes along the
+// items read 8 consecutive rows and its 4 lanes along the outputs 4 consecutive rows of W with 128-bit loads (row strides of
+// an odd number of 16-byte pieces: no bank conflicts, one pass each), 6 loads for 32 FMAs.  W stays in shared memory for the
+// whole kernel up to H = IL_SMEM_W_H; wider ones are read through L1.  The terms of a sum are added in index order (a Switch
+// decides on the sign of a sum over the state: another order could flip it).
+static const int IL_SMEM_W_H = 128;
+__host__ __device__ inline int il_stride(int K) { return K + (K % 8 == 0 ? 4 : 8); }
+__host__ __device__ inline int il_out_warps(int H) { return H < 128 ? (H + 15) / 16 : 8; }
+__host__ __device__ inline int il_group_max(int H) { return 32 / il_out_warps(H) * 16; }         // items that the 32 warps cover
+static inline int interleaved_smem_bytes(int H) {
+    return (il_group_max(H) * il_stride(2 * H) + (H <= IL_SMEM_W_H ? H * il_stride(2 * H) : 0)) * (int)sizeof(float);
+}
+
+template <bool SMEM_W>
+__device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int stride, const float* w_rows, int w_stride, int K, uint32_t out0,
+                                         uint32_t out1, int row0, int jw, int lane) {
+    const int H = c.H, og = lane >> 3;
+    const float* x0 = xs + (size_t)row0 * stride;
+    const float* x1 = x0 + 8 * stride;
+    for (int j0 = jw * 16 + og; j0 < H; j0 += 128) {
+        const float* wr[4];
+        float acc[2][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = min(j0 + 4 * q, H - 1);                  // (a row past the last output repeats the last one: not stored)
+            wr[q] = w_rows + (size_t)j * w_stride;
+            acc[0][q] = acc[1][q] = __ldg(&c.b[j]);
+        }
+#pragma unroll 2
+        for (int k = 0; k < K; k += 4) {
+            const float4 xa = *reinterpret_cast<const float4*>(x0 + k), xb = *reinterpret_cast<const float4*>(x1 + k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = SMEM_W ? *reinterpret_cast<const float4*>(wr[q] + k) : __ldg(reinterpret_cast<const float4*>(wr[q] + k));
+                acc[0][q] = fmaf(w.w, xa.w, fmaf(w.z, xa.z, fmaf(w.y, xa.y, fmaf(w.x, xa.x, acc[0][q]))));
+                acc[1][q] = fmaf(w.w, xb.w, fmaf(w.z, xb.z, fmaf(w.y, xb.y, fmaf(w.x, xb.x, acc[1][q]))));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = j0 + 4 * q;
+            if (j >= H) break;
+            if (out0 < c.frame_cap) c.arena[(size_t)out0 * c.S + j] = tanhf(acc[0][q]);
+            if (out1 < c.frame_cap) c.arena[(size_t)out1 * c.S + j] = tanhf(acc[1][q]);
+        }
+    }
+}
 
 // Token scheduling and vector operators interleaved wave by wave, for programs in which a Switch reads a vector
 // value (RDF_OP_GATE): the tokens of wave w may read any state whose operator was queued before wave w, so every
 // wave ends with the operators it queued -- leaves E[tok], unary operators tanh(W_half x + b), cells
-// tanh(W [x_l ; x_r] + b) -- in groups of 32 operators per block.
+// tanh(W [x_l ; x_r] + b) -- a list each, in groups of one kind per block (as many as the warps cover, fewer while that
+// leaves blocks without a group: a wave is as long as its longest block).
 // Two grid barriers per wave (tokens | operators).  fp32, H <= INTERLEAVED_MAX_H.
+// What bounds it: the FMA and load issue of the wide waves and the latency of the narrow ones.  8192 seeds, H = 128, 44
+// waves: groups of 32 with the kinds mixed (unary operators as cells with a zero half) and tokens on the first blocks only
+// 4.24 ms, this 1.86 ms (operators 2.9 -> 1.25, tokens 1.0 -> 0.33).
 __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
     extern __shared__ __align__(16) unsigned char il_smem[];
     load_program(c, sp);
     ThreadStats st;
-    uint32_t generation = 0, wave = 0, widest = 0, done_cells = 0, done_leaves = 0;
+    uint32_t generation = 0, wave = 0, widest = 0, done[3] = {0u, 0u, 0u}, done_leaves = 0;      // cells, left, right unary operators
     long long cyc_s = 0, cyc_o = 0, cyc_b = 0, t_mark = clock64();
     auto lap = [&](long long& acc) {
         const long long now = clock64();
@@ -650,8 +709,17 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         t_mark = now;
     };
     const int H = c.H, lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    float* xs = reinterpret_cast<float*>(il_smem);                  // [2H][33]: operand rows of a group of 32 operators, transposed
-    const uint32_t gwarp = blockIdx.x * (blockDim.x / 32) + warp, n_warps = gridDim.x * (blockDim.x / 32);
+    float* xs = reinterpret_cast<float*>(il_smem);
+    const bool smem_w = H <= IL_SMEM_W_H;
+    const int w_stride = smem_w ? il_stride(2 * H) : 2 * H;
+    float* ws = xs + il_group_max(H) * il_stride(2 * H);
+    if (smem_w)
+        for (int p = threadIdx.x; p < H * (H / 2); p += blockDim.x) {
+            const int j = p / (H / 2), k = (p % (H / 2)) * 4;
+            *reinterpret_cast<float4*>(ws + (size_t)j * w_stride + k) = __ldg(reinterpret_cast<const float4*>(c.W + (size_t)j * 2 * H + k));
+        }
+    const int out_warps = il_out_warps(H), iw = warp / out_warps, jw = warp % out_warps;
+    const uint32_t gwarp = warp * gridDim.x + blockIdx.x, n_warps = gridDim.x * (blockDim.x / 32);      // (consecutive warps on different SMs)
     for (;; ++wave) {
         const uint32_t n = ld_volatile_u32(&c.ctl->qcount[wave % 3].v);
         if (n == 0) break;
@@ -662,72 +730,63 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         widest = max(widest, n);
         if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl->qcount[(wave + 2) % 3].v = 0;
         const Token* q = c.q[wave & 1];
-        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-            run_token(c, sp, nullptr, wave, load_token(&q[i]), st);
+        for (uint32_t i = gwarp * 32u + lane; i < n; i += n_warps * 32u) run_token(c, sp, nullptr, wave, load_token(&q[i]), st);
         __syncthreads();
         lap(cyc_s);
         if (!grid_barrier(c, &c.ctl->bar.v, generation)) break;
         lap(cyc_b);
         // ---- the operators this wave queued
         const uint32_t n_leaf = min(ld_volatile_u32(&c.ctl->leaf_count.v), c.work_cap);
-        const uint32_t n_cell = min(ld_volatile_u32(&c.ctl->cell_count.v), c.work_cap);
+        uint32_t end[3];
+        end[0] = min(ld_volatile_u32(&c.ctl->cell_count.v), c.work_cap);
+        end[1] = min(ld_volatile_u32(&c.ctl->unary_count[0].v), c.work_cap);
+        end[2] = min(ld_volatile_u32(&c.ctl->unary_count[1].v), c.work_cap);
         for (uint32_t i = done_leaves + gwarp; i < n_leaf; i += n_warps) {
             const LeafItem it = c.leaf_items[i];
             const float* e = c.E + (size_t)it.tok * c.D;
             float* out = c.arena + (size_t)it.slot * c.S;
             for (int k = lane; k < H; k += 32) out[k] = __ldg(&e[k]);
         }
-        // Unary operators and cells, 32 at a time per block: a unary operator on x is the cell on [x ; 0] (left half of
-        // W) or [0 ; x] (right half), so one loop serves all three.  The operand rows of the group are staged
-        // transposed (xs[k][item], rows padded to 33 floats: conflict-free both ways); warp w then computes outputs
-        // 4w .. 4w+3 (+128, ...) of all 32 items, lane = item, the weight rows read as uniform vector loads.
-        for (uint32_t g0 = done_cells + blockIdx.x * 32u; g0 < n_cell; g0 += gridDim.x * 32u) {
-            const uint32_t cnt = min(32u, n_cell - g0);
+        const uint32_t total = end[0] - done[0] + end[1] - done[1] + end[2] - done[2];
+        const uint32_t G = min((uint32_t)il_group_max(H), ((total + gridDim.x - 1) / gridDim.x + 15u) & ~15u);
+        const uint32_t g0 = G ? (end[0] - done[0] + G - 1) / G : 0u, g1 = G ? (end[1] - done[1] + G - 1) / G : 0u, g2 = G ? (end[2] - done[2] + G - 1) / G : 0u;
+        for (uint32_t g = blockIdx.x; g < g0 + g1 + g2; g += gridDim.x) {
+            const int kind = g < g0 ? 0 : g < g0 + g1 ? 1 : 2;
+            const uint32_t first = done[kind] + (g - (kind == 0 ? 0u : kind == 1 ? g0 : g0 + g1)) * G, cnt = min(G, end[kind] - first);
+            const int K = kind == 0 ? 2 * H : H, stride = il_stride(K);
             __syncthreads();                                        // (the previous group's operands are no longer read)
-            CellItem it = CellItem{0u, 0u, 0u, 0u};
-            bool ok = false;
-            if ((uint32_t)warp < cnt) {
-                it = c.cell_items[g0 + warp];
-                const bool unary = it.r == CHILD_L_MARK || it.r == CHILD_R_MARK;
-                ok = it.l < c.frame_cap && (unary || it.r < c.frame_cap) && it.out < c.frame_cap;
+            for (uint32_t i = warp; i < cnt; i += 32u) {
+                uint32_t l, r = 0u;
+                if (kind == 0) {
+                    const CellItem it = c.cell_items[first + i];
+                    l = it.l; r = it.r;
+                } else l = c.unary_items[kind - 1][first + i].y;
+                const bool ok = l < c.frame_cap && r < c.frame_cap;
                 if (!ok && lane == 0) set_status(c, RDF_ERR_BAD_ARG);
-                for (int k = lane; k < H; k += 32) {
-                    float a = 0.f, b2 = 0.f;
-                    if (ok) {
-                        const float x = __ldcg(&c.arena[(size_t)it.l * c.S + k]);
-                        if (it.r == CHILD_R_MARK) b2 = x; else a = x;
-                        if (!unary) b2 = __ldcg(&c.arena[(size_t)it.r * c.S + k]);
-                    }
-                    xs[(size_t)k * 33 + warp] = a;
-                    xs[(size_t)(H + k) * 33 + warp] = b2;
+                for (int k = lane * 4; k < K; k += 128) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (ok) v = k < H ? ldcg4(c.arena + (size_t)l * c.S + k) : ldcg4(c.arena + (size_t)r * c.S + (k - H));
+                    *reinterpret_cast<float4*>(xs + (size_t)i * stride + k) = v;
                 }
             }
+            // this thread's two items: rows row0 and row0 + 8 of the group
+            const int row0 = iw * 16 + (lane & 7);
+            uint32_t out[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t at = (uint32_t)row0 + 8u * i;
+                out[i] = at >= cnt ? 0xFFFFFFFFu : kind == 0 ? c.cell_items[first + at].out : c.unary_items[kind - 1][first + at].x;
+            }
             __syncthreads();
-            // lane = item of the group; its output row
-            const uint32_t out_row = (uint32_t)lane < cnt ? c.cell_items[g0 + lane].out : 0xFFFFFFFFu;
-            for (int j0 = warp * 4; j0 < H; j0 += 128) {
-                float acc[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[q] = c.b[j0 + q];
-                const float4* w0 = reinterpret_cast<const float4*>(c.W + (size_t)j0 * 2 * H);
-                const int K4 = 2 * H / 4;
-                for (int k4 = 0; k4 < K4; ++k4) {
-                    float4 w[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) w[q] = __ldg(w0 + (size_t)q * K4 + k4);
-                    const float x0 = xs[(size_t)(4 * k4 + 0) * 33 + lane], x1 = xs[(size_t)(4 * k4 + 1) * 33 + lane];
-                    const float x2 = xs[(size_t)(4 * k4 + 2) * 33 + lane], x3 = xs[(size_t)(4 * k4 + 3) * 33 + lane];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        acc[q] = fmaf(w[q].w, x3, fmaf(w[q].z, x2, fmaf(w[q].y, x1, fmaf(w[q].x, x0, acc[q]))));
-                }
-                if (out_row < c.frame_cap)
-                    *reinterpret_cast<float4*>(c.arena + (size_t)out_row * c.S + j0) =
-                        make_float4(tanhf(acc[0]), tanhf(acc[1]), tanhf(acc[2]), tanhf(acc[3]));
+            const int k0 = kind == 2 ? H : 0;
+            if ((uint32_t)(iw * 16) < cnt) {
+                if (smem_w) il_group<true>(c, xs, stride, ws + k0, w_stride, K, out[0], out[1], row0, jw, lane);
+                else il_group<false>(c, xs, stride, c.W + k0, w_stride, K, out[0], out[1], row0, jw, lane);
             }
         }
         done_leaves = n_leaf;
-        done_cells = n_cell;
+#pragma unroll
+        for (int q2 = 0; q2 < 3; ++q2) done[q2] = end[q2];
         __syncthreads();
         lap(cyc_o);
         if (!grid_barrier(c, &c.ctl->bar.v, generation)) break;
@@ -1206,6 +1265,7 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.table = P.take<char>(L.table_bytes);
     L.cell_items = P.take<CellItem>(L.work_cap);
     L.leaf_items = P.take<LeafItem>(L.work_cap);
+    for (size_t& u : L.unary_items) u = P.take<uint2>(g->interleaved ? L.work_cap : 0);
     L.cell_sorted = P.take<CellItem>(L.clustered ? L.work_cap : 0);
     L.cell_link = P.take<uint4>(L.clustered ? L.work_cap : 0);
     const size_t vf = g->has_vector_ops ? L.frame_cap : 0;
@@ -1289,8 +1349,9 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
     CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_operator_kernel<false>, 256, 128 * THIN_RESIDENT_MAX_H));
     if (per_sm < 1) return RDF_ERR_CUDA;
-    CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, interleaved_smem_bytes(INTERLEAVED_MAX_H)));
-    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel, 1024, interleaved_smem_bytes(INTERLEAVED_MAX_H)));
+    const int il_smem = std::max(interleaved_smem_bytes(IL_SMEM_W_H), interleaved_smem_bytes(INTERLEAVED_MAX_H));      // the two largest configurations
+    CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem));
+    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel, 1024, il_smem));
     if (per_sm < 1) return RDF_ERR_CUDA;
     CUDA_OK(cudaFuncSetAttribute(rdf_scheduler_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * LQ_CAP * sizeof(Token))));
     CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_scheduler_kernel, 1024, 2 * LQ_CAP * sizeof(Token)));
@@ -1365,6 +1426,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
     c.cell_link = reinterpret_cast<uint4*>(ws + L.cell_link);
     c.group_ends = reinterpret_cast<uint32_t*>(ws + L.group_ends);
     c.leaf_items = reinterpret_cast<LeafItem*>(ws + L.leaf_items);
+    for (int k = 0; k < 2; ++k) c.unary_items[k] = reinterpret_cast<uint2*>(ws + L.unary_items[k]);
     c.work_cap = L.work_cap;
     c.op_l = reinterpret_cast<uint32_t*>(ws + L.op_l);
     c.op_r = reinterpret_cast<uint32_t*>(ws + L.op_r);

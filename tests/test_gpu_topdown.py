@@ -133,3 +133,10 @@ def test_topdown_full_size_as_benchmarked():
     # an instance that is not decisive may have grown another tree: the totals then differ by at most its size
     slack = sum(2 * (2 ** (D + 1)) for d in decisive if not d)
     assert abs(st["invocations"] - total) <= slack, (st["invocations"], total, slack)
+
+
+@pytest.mark.parametrize("H,D,B", [(4, 5, 40), (20, 6, 33), (124, 5, 30), (128, 5, 30), (132, 4, 30), (256, 4, 20)])
+def test_topdown_hidden_sizes(H, D, B):
+    """Hidden sizes on both sides of the warp tiles (16 outputs) and of the switch from weights in shared memory (H <= 128)
+    to weights read through the cache; groups of one and of several warps along the items."""
+    test_topdown_recursion_states_and_shapes(H, D, B)
