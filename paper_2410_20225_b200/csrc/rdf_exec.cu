@@ -833,10 +833,10 @@ __global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
 // RNN32: the fp32 TreeRNN alone (no TreeLSTM code in the kernel): few enough registers for two blocks per SM, which is what
 // the FFMA tiles need to hide their shared-memory and barrier latencies.
 template <bool TC, bool RNN32 = false>
-__global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_operator_kernel(const __grid_constant__ DevCtx c) {
-    __shared__ typename std::conditional<TC, TcShared, LstmSmem>::type smem;   // (the TreeRNN tiles and patches use the first part of LstmSmem)
-    const bool lstm = RNN32 ? false : c.lstm != 0;
-    extern __shared__ unsigned char dyn_smem[];                      // TC: resident weight slices + operand stages
+__global__ void __launch_bounds__(TC ? TC_THREADS : 256, TC ? 1 : 2) rdf_operator_kernel(const __grid_constant__ DevCtx c) {
+    __shared__ typename std::conditional<TC, TcShared, typename std::conditional<RNN32, LstmSmem, int>::type>::type smem;   // (tiles, or rows of thin patches)
+    const bool lstm = TC ? c.lstm != 0 : !RNN32;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];        // TC: resident weight slices + operand stages; TreeLSTM: tile stages
     if (c.ctl->forward_status != 0) return;                          // the scheduler failed: the lists are not to be trusted
     TcState tc;
     if constexpr (TC) {
@@ -846,8 +846,8 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
     }
     // fp32 TreeRNN, narrow waves: this block's 16 columns of W stay in shared memory for all waves
     const float4* wres = nullptr;
-    if constexpr (!TC) {
-        if (!lstm && c.H <= THIN_RESIDENT_MAX_H) {
+    if constexpr (RNN32) {
+        if (c.H <= THIN_RESIDENT_MAX_H) {
             float4* wr = reinterpret_cast<float4*>(dyn_smem);
             const int K2 = 2 * c.H, units_n = (c.H + 15) / 16, cg0 = blockIdx.x % units_n;
             for (int q = threadIdx.x; q < (K2 / 4) * 16; q += blockDim.x) {
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
                 asm volatile("fence.proxy.async;" ::: "memory");      // the operand rows it wrote are read by tile copies after the barrier
             }
         } else {
-            if constexpr (!RNN32) lstm_forward_tiles<3>(c, smem, 0, n_leaf);
+            if constexpr (!RNN32) lstm_forward_wave<3>(c, reinterpret_cast<float*>(dyn_smem), 0, n_leaf);
         }
         __syncthreads();
         lap(cyc_c);
@@ -918,16 +918,14 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_oper
             if (k > 0) wv = c.wave_marks[k - 1];                         // in flight during this wave
             if (cur.w <= cur.z) continue;
             const uint32_t first = min(cur.z, c.work_cap), nc = min(cur.w, c.work_cap) - first;
-            bool done = false;
             if constexpr (!RNN32) {
-                lstm_forward_tiles<5>(c, smem, first, nc);
-                done = true;
+                lstm_forward_wave<5>(c, reinterpret_cast<float*>(dyn_smem), first, nc);
+            } else {
+                // thin patches while they fit in two rounds over the grid, tiles for wide waves
+                if (c.H <= 384 && ((nc + 7) / 8) * ((c.H + 15) / 16) <= 2 * gridDim.x)
+                    rnn_cell_thin(c, reinterpret_cast<float*>(&smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
+                else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, nc);
             }
-            // thin patches while they fit in two rounds over the grid, tiles for wide waves
-            if (done) {
-            } else if (c.H <= 384 && ((nc + 7) / 8) * ((c.H + 15) / 16) <= 2 * gridDim.x)
-                rnn_cell_thin(c, reinterpret_cast<float*>(&smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
-            else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, nc);
             __syncthreads();
             lap(cyc_c);
             alive = grid_barrier(c, &c.ctl->bar_ops.v, generation);
@@ -1346,9 +1344,10 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn));
     CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_operator_kernel<true>, TC_THREADS, max_dyn));
     if (per_sm < 1) return RDF_ERR_CUDA;
-    CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
-    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_operator_kernel<false>, 256, 128 * THIN_RESIDENT_MAX_H));
+    CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lstm_tile_bytes()));
+    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_operator_kernel<false>, 256, lstm_tile_bytes()));
     if (per_sm < 1) return RDF_ERR_CUDA;
+    S->lstm32_per_sm = std::min(per_sm, 2);
     const int il_smem = std::max(interleaved_smem_bytes(IL_SMEM_W_H), interleaved_smem_bytes(INTERLEAVED_MAX_H));      // the two largest configurations
     CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem));
     CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel, 1024, il_smem));
@@ -1654,7 +1653,8 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
             co.cell_items = reinterpret_cast<CellItem*>(c.cell_ops);          // the operator kernels read the cells in depth order
             oargs[0] = (void*)&co;
             if (c.lstm)
-                RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false>, dim3(S->grid), dim3(256), oargs, 0, stream)));
+                RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false>, dim3(S->grid * S->lstm32_per_sm), dim3(256), oargs,
+                                                    lstm_tile_bytes(), stream)));
             else {
                 RDF_KERNEL(S, rdf_leaf_rows_kernel<<<8 * S->grid, 256, 0, stream>>>(c));
                 if (c.n_groups > 1) {

@@ -1,133 +1,145 @@
 // Binary TreeLSTM, forward tiles (fp32 FMA).
 //   cell: [i; f_l; f_r; o; u] = W [h_l; h_r] + b,  c = s(i) tanh(u) + s(f_l) c_l + s(f_r) c_r,  h = s(o) tanh(c)
 //   leaf: [i; o; u] = W_x E[tok] + b_x,            c = s(i) tanh(u),                           h = s(o) tanh(c)
-// One thread accumulates all NG gate pre-activations of its 4 x 4 (row, hidden unit) patch.
+// A tile is 16 RT rows x 16 hidden units; a thread accumulates all NG gates of one unit of RT rows, so the gate arithmetic
+// fuses into the epilogue.  Rows and weight rows lie in shared memory as they lie in memory (K contiguous, 32 at a time,
+// copied asynchronously two steps deep; row stride of an odd number of 16-byte pieces) and are read with 128-bit loads:
+// RT + NG loads for 4 RT NG FMAs.
+// Why so small: a wave of an ordinary batch has some 800 cells.  64 rows x 64 units made 39 tiles of 25 us each for 148 SMs;
+// 64 x 16 makes 130, a quarter as long; 32 x 16 (two blocks per SM) is taken while 64 rows leave blocks without a tile.
+// 601 trees, H = 148, 12 waves and the leaves: operators 0.767 -> 0.484 ms.
 #pragma once
-#include "rdf_exec.h"
+#include "rdf_tc.cuh"
 
 __device__ __forceinline__ float sigmoid_f(float x) { return 1.f / (1.f + expf(-x)); }
 
-template <int NG>
-__device__ void lstm_forward_tiles(const DevCtx& c, LstmSmem& sm, uint32_t first, uint32_t n_items) {
+static const int LT_UNITS = 16, LT_K = 32, LT_LD = LT_K + 4;
+static const int LT_STAGE = (64 + 5 * LT_UNITS) * LT_LD;                   // floats of a stage
+inline size_t lstm_tile_bytes() { return (size_t)2 * LT_STAGE * sizeof(float); }
+
+template <int NG, int RT>
+__device__ void lstm_forward_tiles(const DevCtx& c, float* smem, uint32_t first, uint32_t n_items) {
     constexpr bool CELL = NG == 5;
+    constexpr int ROWS = 16 * RT, PIECES = (ROWS + NG * LT_UNITS) * (LT_K / 4), PER = (PIECES + 255) / 256;
     const int H = c.H, S = c.S, G = c.G;
-    const int Kdim = CELL ? 2 * H : c.D;
-    const int split = CELL ? H : c.D;          // k < split comes from the first source row
+    const int Kdim = CELL ? 2 * H : c.D, split = CELL ? H : c.D;           // k < split comes from the first source row
     const float* Wm = CELL ? c.W : c.W_x;
     const float* bias = CELL ? c.b : c.b_x;
-    const int tiles_m = (n_items + TM - 1) / TM, tiles_n = (H + TN - 1) / TN;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int lrow = threadIdx.x / 4, lk = (threadIdx.x % 4) * 4;
-    for (int tile = blockIdx.x; tile < tiles_m * tiles_n; tile += gridDim.x) {
-        const int tm = tile / tiles_n, tn = tile % tiles_n;
-        const int row0 = tm * TM, col0 = tn * TN;
-        const int arow = row0 + lrow;
-        const float *xl = nullptr, *xr = nullptr;
-        if (arow < (int)n_items) {
-            if constexpr (CELL) {
-                const uint4 it = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + arow]));   // {out, l, r, -}
-                xl = c.arena + (size_t)it.y * S;
-                xr = c.arena + (size_t)it.z * S;
+    const int tiles_n = (H + LT_UNITS - 1) / LT_UNITS, tiles = (int)((n_items + ROWS - 1) / ROWS) * tiles_n;
+    const int tu = threadIdx.x % 16, tr = threadIdx.x / 16;                // unit; rows tr + 16 i
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int row0 = (tile / tiles_n) * ROWS, u0 = (tile % tiles_n) * LT_UNITS;
+        // the 16-byte pieces this thread copies per step: rows of the operands, then rows of the gates' weights
+        const float *src[PER], *src2[PER];
+        uint32_t valid = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            const int p = threadIdx.x + 256 * q, r = p / (LT_K / 4);
+            src[q] = src2[q] = c.W;
+            if (p >= PIECES) continue;
+            if (r < ROWS) {
+                if (row0 + r < (int)n_items) {
+                    valid |= 1u << q;
+                    if constexpr (CELL) {
+                        const uint4 it = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + row0 + r]));   // {out, l, r, -}
+                        src[q] = c.arena + (size_t)it.y * S;
+                        src2[q] = c.arena + (size_t)it.z * S - H;
+                    } else {
+                        src[q] = c.E + (size_t)__ldcg(&c.leaf_items[row0 + r].tok) * c.D;
+                    }
+                }
             } else {
-                const uint2 it = __ldcg(reinterpret_cast<const uint2*>(&c.leaf_items[arow]));  // {slot, tok}
-                xl = c.E + (size_t)it.y * c.D;
+                const int g = (r - ROWS) / LT_UNITS, u = u0 + (r - ROWS) % LT_UNITS;
+                if (u < H) {
+                    valid |= 1u << q;
+                    src[q] = Wm + (size_t)(g * H + u) * Kdim;
+                    src2[q] = src[q];
+                }
             }
         }
-        const int bcol = col0 + lrow;
-        float acc[NG][4][4];
+        auto fetch = [&](int k0, int stage) {
+            const uint32_t dst = smem_u32(smem + stage * LT_STAGE);
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int p = threadIdx.x + 256 * q, r = p / (LT_K / 4), kq = (p % (LT_K / 4)) * 4, k = k0 + kq;
+                if (p < PIECES)
+                    cp_async16(dst + 4 * (r * LT_LD + kq), (k < split ? src[q] : k < Kdim ? src2[q] : src[q] - k) + k, ((valid >> q) & 1u) && k < Kdim);
+            }
+            cp_async_commit();
+        };
+        float acc[NG][RT];
 #pragma unroll
         for (int g = 0; g < NG; ++g)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[g][i][j] = 0.f;
-        for (int k0 = 0; k0 < Kdim; k0 += TK) {
-            const int k = k0 + lk;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 b[NG];
-            if (xl && k < Kdim) a = k < split ? ldcg4(xl + k) : ldcg4(xr + (k - split));
-#pragma unroll
-            for (int g = 0; g < NG; ++g) {
-                b[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (bcol < H && k < Kdim)
-                    b[g] = __ldg(reinterpret_cast<const float4*>(Wm + (size_t)(g * H + bcol) * Kdim + k));
-            }
+            for (int i = 0; i < RT; ++i) acc[g][i] = 0.f;
+        __syncthreads();                                                   // (the previous tile's stages are no longer read)
+        fetch(0, 0);
+        const int steps = (Kdim + LT_K - 1) / LT_K;
+        for (int st = 0; st < steps; ++st) {
+            if (st + 1 < steps) fetch((st + 1) * LT_K, (st + 1) & 1);
+            else cp_async_commit();
+            cp_async_wait<1>();
             __syncthreads();
-            sm.As[lk + 0][lrow] = a.x; sm.As[lk + 1][lrow] = a.y; sm.As[lk + 2][lrow] = a.z; sm.As[lk + 3][lrow] = a.w;
+            const float* As = smem + (st & 1) * LT_STAGE + tr * LT_LD;
+            const float* Bs = smem + (st & 1) * LT_STAGE + (ROWS + tu) * LT_LD;
+#pragma unroll 4
+            for (int k = 0; k < LT_K; k += 4) {
+                float4 a[RT];
 #pragma unroll
-            for (int g = 0; g < NG; ++g) {
-                sm.Bs[g][lk + 0][lrow] = b[g].x; sm.Bs[g][lk + 1][lrow] = b[g].y;
-                sm.Bs[g][lk + 2][lrow] = b[g].z; sm.Bs[g][lk + 3][lrow] = b[g].w;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < TK; ++kk) {
-                const float4 av = *reinterpret_cast<const float4*>(&sm.As[kk][ty * 4]);
-                const float aa[4] = {av.x, av.y, av.z, av.w};
+                for (int i = 0; i < RT; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * LT_LD + k);
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
-                    const float4 bv = *reinterpret_cast<const float4*>(&sm.Bs[g][kk][tx * 4]);
-                    const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
+                    const float4 b = *reinterpret_cast<const float4*>(Bs + g * LT_UNITS * LT_LD + k);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[g][i][j] = fmaf(aa[i], bb[j], acc[g][i][j]);
+                    for (int i = 0; i < RT; ++i)
+                        acc[g][i] = fmaf(a[i].w, b.w, fmaf(a[i].z, b.z, fmaf(a[i].y, b.y, fmaf(a[i].x, b.x, acc[g][i]))));
                 }
             }
+            __syncthreads();
         }
-        const int col = col0 + tx * 4;
-        if (col < H) {
-            float bz[NG][4];
+        const int u = u0 + tu;
+        if (u >= H) continue;
+        float bz[NG];
 #pragma unroll
-            for (int g = 0; g < NG; ++g) {
-                const float4 t = __ldg(reinterpret_cast<const float4*>(bias + g * H + col));
-                bz[g][0] = t.x; bz[g][1] = t.y; bz[g][2] = t.z; bz[g][3] = t.w;
+        for (int g = 0; g < NG; ++g) bz[g] = __ldg(bias + g * H + u);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const int row = row0 + tr + 16 * i;
+            if (row >= (int)n_items) continue;
+            float v[NG], cc;
+            uint32_t out;
+            if constexpr (CELL) {
+                const uint4 it = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + row]));
+                out = it.x;
+                const float cl = __ldcg(c.arena + (size_t)it.y * S + H + u), cr = __ldcg(c.arena + (size_t)it.z * S + H + u);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) v[g] = sigmoid_f(acc[g][i] + bz[g]);
+                v[4] = tanhf(acc[4][i] + bz[4]);
+                cc = v[0] * v[4] + v[1] * cl + v[2] * cr;
+            } else {
+                out = __ldcg(&c.leaf_items[row].slot);
+                v[0] = sigmoid_f(acc[0][i] + bz[0]);
+                v[1] = sigmoid_f(acc[1][i] + bz[1]);
+                v[2] = tanhf(acc[2][i] + bz[2]);
+                cc = v[0] * v[2];
             }
+            float* st = c.arena + (size_t)out * S;
+            st[u] = v[CELL ? 3 : 1] * tanhf(cc);
+            st[H + u] = cc;
+            if (c.gates) {
+                float* gt = c.gates + (size_t)out * G;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int row = row0 + ty * 4 + i;
-                if (row >= (int)n_items) continue;
-                float hv[4], cv[4], gv[NG][4];
-                uint32_t out;
-                if constexpr (CELL) {
-                    const uint4 it = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + row]));
-                    out = it.x;
-                    const float4 cl4 = ldcg4(c.arena + (size_t)it.y * S + H + col);
-                    const float4 cr4 = ldcg4(c.arena + (size_t)it.z * S + H + col);
-                    const float cl[4] = {cl4.x, cl4.y, cl4.z, cl4.w}, cr[4] = {cr4.x, cr4.y, cr4.z, cr4.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float gi = sigmoid_f(acc[0][i][j] + bz[0][j]);
-                        const float fl = sigmoid_f(acc[1][i][j] + bz[1][j]);
-                        const float fr = sigmoid_f(acc[2][i][j] + bz[2][j]);
-                        const float go = sigmoid_f(acc[3][i][j] + bz[3][j]);
-                        const float gu = tanhf(acc[4][i][j] + bz[4][j]);
-                        cv[j] = gi * gu + fl * cl[j] + fr * cr[j];
-                        hv[j] = go * tanhf(cv[j]);
-                        gv[0][j] = gi; gv[1][j] = fl; gv[2][j] = fr; gv[3][j] = go; gv[4][j] = gu;
-                    }
-                } else {
-                    out = __ldcg(&c.leaf_items[row].slot);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float gi = sigmoid_f(acc[0][i][j] + bz[0][j]);
-                        const float go = sigmoid_f(acc[1][i][j] + bz[1][j]);
-                        const float gu = tanhf(acc[2][i][j] + bz[2][j]);
-                        cv[j] = gi * gu;
-                        hv[j] = go * tanhf(cv[j]);
-                        gv[0][j] = gi; gv[1][j] = go; gv[2][j] = gu;
-                    }
-                }
-                float* st = c.arena + (size_t)out * S;
-                *reinterpret_cast<float4*>(st + col) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-                *reinterpret_cast<float4*>(st + H + col) = make_float4(cv[0], cv[1], cv[2], cv[3]);
-                if (c.gates) {
-                    float* gt = c.gates + (size_t)out * G;
-#pragma unroll
-                    for (int g = 0; g < NG; ++g)
-                        *reinterpret_cast<float4*>(gt + g * H + col) = make_float4(gv[g][0], gv[g][1], gv[g][2], gv[g][3]);
-                }
+                for (int g = 0; g < NG; ++g) gt[g * H + u] = v[g];
             }
         }
     }
+    cp_async_wait<0>();
+}
+
+// 64 rows per tile when that gives every block a tile
+template <int NG>
+__device__ __forceinline__ void lstm_forward_wave(const DevCtx& c, float* smem, uint32_t first, uint32_t n_items) {
+    const uint32_t tiles_n = (c.H + LT_UNITS - 1) / LT_UNITS;
+    if ((n_items + 63u) / 64u * tiles_n >= gridDim.x) lstm_forward_tiles<NG, 4>(c, smem, first, n_items);
+    else lstm_forward_tiles<NG, 2>(c, smem, first, n_items);
 }
