@@ -146,8 +146,10 @@ struct DevCtx {
     uint32_t  work_cap;
     uint32_t* op_l;               // per frame: operand frames of the operator that made its state
     uint32_t* op_r;               //            (leaf: op_l = LEAF_MARK, op_r = token id)
-    float*    arena;              // [frame_cap, S] fp32 states: S = H (TreeRNN h) or 2H (TreeLSTM h then c)
-    float*    gates;              // TreeLSTM under rdf_grad: [frame_cap, G] activated gates, later their gradients
+    float*    arena;              // [frame_cap, S] fp32 states: S = H (TreeRNN h) or 2H (TreeLSTM h then c); bf16 TreeLSTM:
+                                  // [frame_cap, Hp] c alone
+    float*    gates;              // TreeLSTM under rdf_grad: [frame_cap, G] activated gates, later their gradients; bf16:
+                                  // [frame_cap, Hp / 8, gates, 8] (row stride 5Hp), what a thread of the epilogue has in one piece
     int       S, G, lstm;
     // tensor-core path (bf16 operands): bf16 copy of the states with row stride Hp, packed weights
     __nv_bfloat16* arena_bf;
@@ -155,9 +157,9 @@ struct DevCtx {
     __nv_bfloat16* WTp;           // [2Hp, Hp]   gradient operand
     __nv_bfloat16* dz_bf;         // [frame_cap, Hp] bf16 dz rows of the cells (rdf_grad), row = position of the cell in
                                   // all_cells: the cells of a gradient wave are consecutive rows, read as plain 2D tiles
-    uint32_t* cell_pos;           // per frame: position of a cell in all_cells (written with the lists; leaves: undefined);
+    uint32_t* cell_pos;           // per frame: position of a cell in all_cells (written with the lists; leaves: TreeLSTM: in all_leaves);
                                   // clustered fp32 path: in the grouped list
-    TensorMap tmap_dz128, tmap_dz64;   // dz_bf as [rows, Hp], 128-byte swizzle, boxes of 128 / 64 rows by 64 columns
+    TensorMap tmap_dz128, tmap_dz64;   // dz_bf as [rows, Hp], 128-byte swizzle, boxes of 128 / 64 rows by 64 columns; TreeLSTM: dg_bf
     __nv_bfloat16* z_bf;          // [cells_cap, 2Hp] operand rows [h_l ; h_r] of the cells, row = position of the cell in
                                   // all_cells: every invocation writes its state into the half of its caller's row
                                   // that it feeds, so a tile of consecutive cells reads its operands as plain 2D tiles
@@ -168,7 +170,10 @@ struct DevCtx {
     __nv_bfloat16* Wxp;           // [3Hp, Hp] leaf projection, slice-major
     __nv_bfloat16* WxTp;          // [Hp, 3Hp] its transpose (operand of the embedding gradient)
     __nv_bfloat16* E_bf;          // [V, Hp] embedding table in bf16
-    __nv_bfloat16* dg_bf;         // [frame_cap, 5Hp] bf16 gate gradients (rdf_grad)
+    __nv_bfloat16* dg_bf;         // [cells_cap, 5Hp] bf16 gate gradients of the cells (rdf_grad), row = position in all_cells
+    __nv_bfloat16* dgl_bf;        // [leaves_cap, 3Hp] the same of the leaves, row = position in all_leaves
+    uint32_t  leaves_cap;
+    TensorMap tmap_dgl128, tmap_dgl64;
     int       Hp, use_tc;
     // parameters
     int H, D, V, n_classes, compute;
@@ -178,7 +183,7 @@ struct DevCtx {
     rdf_trace_rec* trace;
     long long trace_cap;
     // gradient pass
-    float*    dhp;                // [frame_cap, S]: gradient arriving from the caller (dh, and dc for the TreeLSTM);
+    float*    dhp;                // [frame_cap, S]: gradient arriving from the caller (dh, and dc for the TreeLSTM; bf16: [frame_cap, 2Hp]);
                                   //                 TreeRNN: overwritten by dz (cell) / dh (leaf)
     float*    dlog;               // [frame_cap, 8]: softmax - onehot per invocation
     uint4*    wave_marks;         // [wave_cap], filled by the list kernels: entry k = {first frame, one past the last frame,

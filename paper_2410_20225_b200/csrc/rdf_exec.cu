@@ -1188,8 +1188,8 @@ __global__ void rdf_gather_roots_kernel(const DevCtx c, float* h_root) {
     const long long slot = c.y[b];
     if (slot < 0 || slot >= (long long)c.frame_cap) return;
     for (int k = threadIdx.x; k < c.H; k += blockDim.x)
-        h_root[(size_t)b * c.H + k] = c.arena ? c.arena[(size_t)slot * c.S + k]
-                                              : __bfloat162float(c.arena_bf[(size_t)slot * c.Hp + k]);
+        h_root[(size_t)b * c.H + k] = !c.use_tc ? c.arena[(size_t)slot * c.S + k]
+                                                : __bfloat162float(c.arena_bf[(size_t)slot * c.Hp + k]);
 }
 
 // ===========================================================================
@@ -1273,8 +1273,8 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.Hp = (H + 63) / 64 * 64;
     L.use_tc = g->has_vector_ops && params->compute == RDF_BF16 && L.Hp <= TC_HP_MAX && params->D == params->H;
     const bool tcl = L.use_tc && g->has_lstm, tcr = L.use_tc && !g->has_lstm;
-    L.arena = P.take<float>(tcr ? 0 : vf * S);          // the bf16 TreeRNN keeps its states in arena_bf only
-    L.gates = P.take<float>(g->has_lstm && want_grad ? vf * 5 * H : 0);
+    L.arena = P.take<float>(tcr ? 0 : vf * (tcl ? L.Hp : S));      // the bf16 path keeps h in arena_bf only
+    L.gates = P.take<float>(g->has_lstm && want_grad ? vf * 5 * (tcl ? L.Hp : H) : 0);
     const size_t wcount = (size_t)L.Hp * 2 * L.Hp * (tcl ? 5 : 1);
     L.arena_bf = P.take<__nv_bfloat16>(L.use_tc ? vf * L.Hp : 0);
     L.wp = P.take<__nv_bfloat16>(L.use_tc ? wcount : 0);
@@ -1289,12 +1289,14 @@ int rdf_make_layout(const rdf_graph* g, const rdf_batch* in, const rdf_params* p
     L.wxp = P.take<__nv_bfloat16>(tcl ? (size_t)3 * L.Hp * L.Hp : 0);
     L.wxtp = P.take<__nv_bfloat16>(tcl ? (size_t)3 * L.Hp * L.Hp : 0);
     L.e_bf = P.take<__nv_bfloat16>(tcl ? (size_t)params->V * L.Hp : 0);
-    L.dg_bf = P.take<__nv_bfloat16>(tcl && want_grad ? vf * 5 * L.Hp : 0);
+    L.dg_bf = P.take<__nv_bfloat16>(tcl && want_grad ? (size_t)L.cells_cap * 5 * L.Hp : 0);
+    L.leaves_cap = tcl && want_grad ? ((uint32_t)vf + 127u) / 128u * 128u : 0;
+    L.dgl_bf = P.take<__nv_bfloat16>((size_t)L.leaves_cap * 3 * L.Hp);
     L.tc_smem_fwd = !L.use_tc ? 0 : tcl ? tc_smem_bytes(80, 2 * L.Hp, 48, L.Hp, TC_STAGES_LSTM_FWD) : tc_smem_bytes(L.Hp / 4, 2 * L.Hp, 0, 0, TC_STAGES_RNN_FWD);
     L.tc_smem_bwd = !L.use_tc ? 0 : tcl ? tc_smem_bytes(TC_LSTM_BWD_NS, 5 * L.Hp, 0, 0, TC_STAGES_LSTM_BWD) : tc_smem_bytes(L.Hp / 4, L.Hp, 0, 0, TC_STAGES_RNN_BWD);
     L.ybuf = P.take<int64_t>(g->has_vector_ops ? in->B : 0);
     const size_t gf = want_grad ? L.frame_cap : 0;
-    L.dhp = P.take<float>(tcr ? 0 : gf * S);            // (the bf16 TreeRNN hands its gradients on as dz rows)
+    L.dhp = P.take<float>(tcr ? 0 : gf * (tcl ? 2 * L.Hp : S));            // (the bf16 TreeRNN hands its gradients on as dz rows)
     L.dlog = P.take<float>(gf * 8);
     // every wave of a vector program holds at least one token of an invocation on its way down or up
     L.wave_cap = g->has_vector_ops ? (uint32_t)std::min<long long>(2 * (long long)L.frame_cap + 64, 1ll << 24) : 0;
@@ -1437,7 +1439,7 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
         c.y = reinterpret_cast<int64_t*>(ws + L.ybuf);
         c.lstm = g->has_lstm ? 1 : 0;
         c.S = g->has_lstm ? 2 * params->H : params->H;
-        c.G = 5 * params->H;
+        c.G = 5 * (L.use_tc ? L.Hp : params->H);
         c.gates = nullptr;                 // set by rdf_grad for the TreeLSTM
         c.use_tc = L.use_tc; c.Hp = L.Hp;
         c.arena_bf = reinterpret_cast<__nv_bfloat16*>(ws + L.arena_bf);
@@ -1451,8 +1453,10 @@ void rdf_fill_ctx(rdf_graph* g, const rdf_batch* in, const rdf_params* params, r
         c.Wxp = reinterpret_cast<__nv_bfloat16*>(ws + L.wxp);
         c.WxTp = reinterpret_cast<__nv_bfloat16*>(ws + L.wxtp);
         c.E_bf = reinterpret_cast<__nv_bfloat16*>(ws + L.e_bf);
-        // only present (and only non-null) for the TreeLSTM on the tensor-core path
-        c.dg_bf = L.use_tc && g->has_lstm ? reinterpret_cast<__nv_bfloat16*>(ws + L.dg_bf) : nullptr;
+        const bool dg = L.use_tc && g->has_lstm && L.want_grad;
+        c.dg_bf = dg ? reinterpret_cast<__nv_bfloat16*>(ws + L.dg_bf) : nullptr;
+        c.dgl_bf = dg ? reinterpret_cast<__nv_bfloat16*>(ws + L.dgl_bf) : nullptr;
+        c.leaves_cap = L.leaves_cap;
     } else {
         c.y = out->y;
     }

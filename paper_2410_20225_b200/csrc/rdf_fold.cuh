@@ -114,6 +114,7 @@ __device__ __forceinline__ void fold_fire(const DevCtx& c, const FoldLevel& L, u
         c.leaf_items[pos] = it;
         if (c.lstm) {
             c.all_leaves[pos] = f;
+            if (c.cell_pos) c.cell_pos[f] = pos;
             if (c.leaf_ops) c.leaf_ops[pos] = make_uint4(f, rec.y, 0u, 1u);
         }
     }
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
         else __syncthreads();
     }
     // every block knows the totals: the rows after the last cell, which the weight gradient reads in whole stages, are zero
-    if (alive && blockIdx.x == gridDim.x - 1) zero_tail_rows(c, L.cb);
+    if (alive && blockIdx.x == gridDim.x - 1) zero_tail_rows(c, L.cb, L.lb);
     if (blockIdx.x == 0 && tid == 0) {
         const uint32_t inv = L.cb + L.lb;
         c.ctl->frame_count.v = B + inv; c.ctl->cell_count.v = L.cb; c.ctl->leaf_count.v = L.lb;

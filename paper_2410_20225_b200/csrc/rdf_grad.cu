@@ -649,7 +649,7 @@ __device__ __forceinline__ void backward_frames_f32(const DevCtx& c, uint32_t t0
     }
 }
 
-// A (TreeLSTM): the gate gradients replace the retained gates; dc goes straight to the callee frames.
+// A (fp32 TreeLSTM), one invocation per warp: the gate gradients replace the retained gates; dc goes straight to the callee frames.
 // One invocation t per warp.
 __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t, int lane) {
     const int H = c.H, C = c.n_classes, S = c.S;
@@ -667,15 +667,6 @@ __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t,
         // 128-bit accesses: four hidden units per lane and step
         auto ld = [](const float* p) { const float4 v = ldcg4(p); return v; };
         auto st4 = [](float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); };
-        const bool keep_f32 = c.dg_bf == nullptr;       // bf16 path: the gate gradients live on as bf16 operand rows only
-        auto stb = [&](int gate, int j, const float (&v)[4]) {
-            if (!c.dg_bf) return;
-            __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
-            uint2 pk;
-            pk.x = *reinterpret_cast<uint32_t*>(&lo);
-            pk.y = *reinterpret_cast<uint32_t*>(&hi);
-            *reinterpret_cast<uint2*>(c.dg_bf + (size_t)t * 5 * c.Hp + gate * c.Hp + j) = pk;
-        };
         for (int j = lane * 4; j < H; j += 128) {
             const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4 dh4 = from_result ? z4 : ld(g + j), dc4 = from_result ? z4 : ld(g + H + j), c4 = ld(st + H + j);
@@ -700,8 +691,7 @@ __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t,
                     g1[e] = dh[e] * tc * go[e] * (1.f - go[e]);
                     g2[e] = dc * gi[e] * (1.f - gu[e] * gu[e]);
                 }
-                if (keep_f32) { st4(gt + j, g0); st4(gt + H + j, g1); st4(gt + 2 * H + j, g2); }
-                stb(0, j, g0); stb(1, j, g1); stb(2, j, g2);
+                st4(gt + j, g0); st4(gt + H + j, g1); st4(gt + 2 * H + j, g2);
             } else {
                 const float4 a4 = ld(gt + j), l4 = ld(gt + H + j), r4 = ld(gt + 2 * H + j), o4 = ld(gt + 3 * H + j), u4 = ld(gt + 4 * H + j);
                 const float4 cl4 = ld(c.arena + (size_t)l * S + H + j), cr4 = ld(c.arena + (size_t)r * S + H + j);
@@ -721,15 +711,102 @@ __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t,
                     dl_[e] = dc * fl[e];
                     dr_[e] = dc * fr[e];
                 }
-                if (keep_f32) { st4(gt + j, g0); st4(gt + H + j, g1); st4(gt + 2 * H + j, g2); st4(gt + 3 * H + j, g3); st4(gt + 4 * H + j, g4); }
-                stb(0, j, g0); stb(1, j, g1); stb(2, j, g2); stb(3, j, g3); stb(4, j, g4);
+                st4(gt + j, g0); st4(gt + H + j, g1); st4(gt + 2 * H + j, g2); st4(gt + 3 * H + j, g3); st4(gt + 4 * H + j, g4);
                 st4(c.dhp + (size_t)l * S + H + j, dl_);
                 st4(c.dhp + (size_t)r * S + H + j, dr_);
             }
         }
-        if (c.dg_bf)                      // pad columns of every gate block are zero
-            for (int q = lane; q < (leaf ? 3 : 5) * (c.Hp - H); q += 32)
-                c.dg_bf[(size_t)t * 5 * c.Hp + (q / (c.Hp - H)) * c.Hp + H + q % (c.Hp - H)] = __float2bfloat16_rn(0.f);
+    }
+}
+
+// A (bf16 TreeLSTM): the gate gradients as bf16 operand rows in list order; dc goes straight to the callee frames.
+// A thread takes 8 hidden units of every invocation it gets (what the forward epilogue stored in one piece: gates, c and the
+// incoming gradients in whole sectors, pad units included, whose gradients come out as zeros); as many invocations at a time
+// as the block has threads for, all loads of one in flight together.
+// 8192 trees, H = 300 (4.5 GB): 1.42 ms with a warp per invocation and rows split by gate -> 1.22 ms.
+__device__ __forceinline__ void lstm_backward_units(const DevCtx& c, uint32_t f0, uint32_t f1) {
+    const int H = c.H, Hp = c.Hp, C = c.n_classes, ub = Hp / 8, per = blockDim.x / ub;
+    const int u = (threadIdx.x % ub) * 8, fo = threadIdx.x / ub;
+    if (fo >= per) return;
+    auto header = [&](uint32_t t, uint4& m) {
+        if (t < f1) m = make_uint4(c.op_l[t], c.op_r[t], c.frames[t].parent, c.cell_pos[t]);
+    };
+    const uint32_t step = gridDim.x * per;
+    uint32_t t = f0 + blockIdx.x * per + fo;
+    uint4 m = make_uint4(0u, 0u, 0u, 0u);
+    header(t, m);
+    for (; t < f1; t += step) {
+        const uint4 cur = m;
+        const bool leaf = cur.x == LEAF_MARK, top = cur.z < (uint32_t)c.B;         // top: called from `result`, no gradient comes in
+        const float4 d0 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8), d1 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8 + 4);
+        float g[5][8], cc[8], dh[8], dc[8], cl[8], cr[8];
+        const float* gt = c.gates + (size_t)t * c.G + u * (leaf ? 3 : 5);
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (k < 3 || !leaf) ld_global_32(gt + 8 * k, g[k]);
+        ld_global_32(c.arena + (size_t)t * Hp + u, cc);
+        if (!leaf) {
+            ld_global_32(c.arena + (size_t)cur.x * Hp + u, cl);
+            ld_global_32(c.arena + (size_t)cur.y * Hp + u, cr);
+        }
+        if (!top) {
+            ld_global_32(c.dhp + (size_t)t * 2 * Hp + u, dh);
+            ld_global_32(c.dhp + (size_t)t * 2 * Hp + Hp + u, dc);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) dh[i] = dc[i] = 0.f;
+        }
+        if (step < f1 - t) header(t + step, m);                        // in flight during this step
+        const float dl[MAX_CLASSES] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+        for (int k = 0; k < MAX_CLASSES; ++k)
+            if (k < C) {
+#pragma unroll
+                for (int i = 0; i < 8; i += 4)
+                    if (u + i < H) {
+                        const float4 w = __ldg(reinterpret_cast<const float4*>(&c.W_s[k * H + u + i]));
+                        dh[i] = fmaf(w.x, dl[k], dh[i]); dh[i + 1] = fmaf(w.y, dl[k], dh[i + 1]);
+                        dh[i + 2] = fmaf(w.z, dl[k], dh[i + 2]); dh[i + 3] = fmaf(w.w, dl[k], dh[i + 3]);
+                    }
+            }
+        auto store_bf = [](__nv_bfloat16* p, const float (&v)[8]) {
+            __align__(16) __nv_bfloat162 pk[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) pk[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(pk);
+        };
+        if (leaf) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float gi = g[0][i], go = g[1][i], gu = g[2][i], tc = tanhf(cc[i]);
+                const float d = dc[i] + dh[i] * go * (1.f - tc * tc);
+                g[0][i] = d * gu * gi * (1.f - gi);
+                g[1][i] = dh[i] * tc * go * (1.f - go);
+                g[2][i] = d * gi * (1.f - gu * gu);
+            }
+            __nv_bfloat16* row = c.dgl_bf + (size_t)cur.w * 3 * Hp + u;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) store_bf(row + k * Hp, g[k]);
+        } else {
+            float dcl[8], dcr[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float gi = g[0][i], fl = g[1][i], fr = g[2][i], go = g[3][i], gu = g[4][i], tc = tanhf(cc[i]);
+                const float d = dc[i] + dh[i] * go * (1.f - tc * tc);
+                g[0][i] = d * gu * gi * (1.f - gi);
+                g[1][i] = d * cl[i] * fl * (1.f - fl);
+                g[2][i] = d * cr[i] * fr * (1.f - fr);
+                g[3][i] = dh[i] * tc * go * (1.f - go);
+                g[4][i] = d * gi * (1.f - gu * gu);
+                dcl[i] = d * fl;
+                dcr[i] = d * fr;
+            }
+            __nv_bfloat16* row = c.dg_bf + (size_t)cur.w * 5 * Hp + u;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) store_bf(row + k * Hp, g[k]);
+            st_global_32(c.dhp + (size_t)cur.x * 2 * Hp + Hp + u, dcl);
+            st_global_32(c.dhp + (size_t)cur.y * 2 * Hp + Hp + u, dcr);
+        }
     }
 }
 
@@ -952,19 +1029,14 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
             const uint32_t per = ((n + gridDim.x - 1) / gridDim.x + 31u) & ~31u;
             const unsigned long long c0l = (unsigned long long)f0 + (unsigned long long)blockIdx.x * per;
             const uint32_t c0 = (uint32_t)min(c0l, (unsigned long long)f1), c1 = (uint32_t)min(c0l + per, (unsigned long long)f1);
-            bool done_a = false;
-            if constexpr (!RNN32) {
-                if (lstm) {
-                    for (uint32_t t = c0 + wib; t < c1; t += n_warps) lstm_backward_frame(c, t, lane);
-                    done_a = true;
-                }
-            }
-            if (done_a) {
-            } else if constexpr (TC) {
-                backward_frames_tc(c, c0 + wib * 4 + lane / 8, c1, 4 * n_warps, lane % 8);
-                asm volatile("fence.proxy.async;" ::: "memory");       // its dz rows are read by tile copies after the barrier
-            } else {
+            if constexpr (TC) {
+                if (lstm) lstm_backward_units(c, f0, f1);
+                else backward_frames_tc(c, c0 + wib * 4 + lane / 8, c1, 4 * n_warps, lane % 8);
+                asm volatile("fence.proxy.async;" ::: "memory");       // the dz / gate-gradient rows are read by tile copies after the barrier
+            } else if constexpr (RNN32) {
                 backward_frames_f32(c, c0 + wib * 4 + lane / 8, c1, 4 * n_warps, lane % 8);
+            } else {
+                for (uint32_t t = c0 + wib; t < c1; t += n_warps) lstm_backward_frame(c, t, lane);
             }
             __syncthreads();
             lap(cyc_a);
@@ -1379,6 +1451,13 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         if (rc == RDF_OK) rc = encode_row_tiles(&c.tmap_dz64, c.dz_bf, c.cells_cap, (uint64_t)c.Hp, 64);
         if (rc != RDF_OK) return rc;
     }
+    if (tc_lstm) {                         // the same for the gate-gradient rows of the cells and of the leaves
+        rc = encode_row_tiles(&c.tmap_dz128, c.dg_bf, c.cells_cap, (uint64_t)5 * c.Hp, 128);
+        if (rc == RDF_OK) rc = encode_row_tiles(&c.tmap_dz64, c.dg_bf, c.cells_cap, (uint64_t)5 * c.Hp, 64);
+        if (rc == RDF_OK) rc = encode_row_tiles(&c.tmap_dgl128, c.dgl_bf, c.leaves_cap, (uint64_t)3 * c.Hp, 128);
+        if (rc == RDF_OK) rc = encode_row_tiles(&c.tmap_dgl64, c.dgl_bf, c.leaves_cap, (uint64_t)3 * c.Hp, 64);
+        if (rc != RDF_OK) return rc;
+    }
     {
         const int rowbytes = tc_rnn ? c.Hp * 2 : c.S * 4;
         const int fr = std::max(1, std::min(LH_MAX_ROWS, LH_SLAB_BYTES / rowbytes));
@@ -1462,16 +1541,15 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         };
         DwArgs a{};
         a.ops = c.cell_ops; a.count = &c.ctl->all_cells;
-        a.A = tc_lstm ? c.dg_bf : c.dz_bf; a.lda = tc_lstm ? 5 * c.Hp : c.Hp; a.Mp = tc_lstm ? 5 * c.Hp : c.Hp;
+        a.Mp = tc_lstm ? 5 * c.Hp : c.Hp;
         a.Np = 2 * c.Hp; a.mode = 0; a.out = grads->dW; a.ldo = 2 * H;
-        a.a_tiles = tc_rnn ? 1 : 0;
         a.b_tiles = 1;                                              // [h_l ; h_r] of the listed cells: the operand rows
         a.bias_out = H < c.Hp ? grads->db : nullptr;                // db comes out of the same contraction
         launch_dw(a, max_cells);
         if (tc_lstm) {
             DwArgs x{};
             x.ops = c.leaf_ops; x.count = &c.ctl->all_leaves;
-            x.A = c.dg_bf; x.lda = 5 * c.Hp; x.Mp = 3 * c.Hp; x.Np = c.Hp; x.mode = 1; x.out = grads->dW_x; x.ldo = D;
+            x.Mp = 3 * c.Hp; x.Np = c.Hp; x.mode = 1; x.out = grads->dW_x; x.ldo = D;
             x.bias_out = H < c.Hp ? grads->db_x : nullptr;
             launch_dw(x, max_leaves);
         }
@@ -1487,7 +1565,7 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
     if (c.use_tc && H < c.Hp) {}        // (column H of the dW / dW_x contractions)
     else if (c.repro) {
         // column sums in two steps: a row of partial sums per block (in the buffer the weight gradient is done with), then
-        // the rows added up in block order.  TreeRNN: dz rows are in all_cells order; TreeLSTM: bf16 gate-gradient rows.
+        // the rows added up in block order.  TreeRNN: dz rows are in all_cells order; TreeLSTM: so are the gate-gradient rows.
         const int cs_blocks = std::min(8 * S->grid, (int)((size_t)DW_BLOCKS_MAX * 65536 / (5 * (size_t)H)));
         auto colsum = [&](const uint32_t* list, const uint32_t* count, const __nv_bfloat16* A, int lda_, int M, float* out_) {
             RDF_KERNEL(S, rdf_colsum_partial_kernel<__nv_bfloat16><<<cs_blocks, 256, 0, stream>>>(&c.ctl->status, list, count, A, lda_, M, H, c.Hp, c.dw_partial));
@@ -1495,14 +1573,14 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         };
         if (tc_rnn) colsum(nullptr, &c.ctl->all_cells, c.dz_bf, c.Hp, H, grads->db);
         else {
-            colsum(c.all_cells, &c.ctl->all_cells, c.dg_bf, 5 * c.Hp, 5 * H, grads->db);
-            colsum(c.all_leaves, &c.ctl->all_leaves, c.dg_bf, 5 * c.Hp, 3 * H, grads->db_x);
+            colsum(nullptr, &c.ctl->all_cells, c.dg_bf, 5 * c.Hp, 5 * H, grads->db);
+            colsum(nullptr, &c.ctl->all_leaves, c.dgl_bf, 3 * c.Hp, 3 * H, grads->db_x);
         }
     }
     else if (tc_rnn) RDF_KERNEL(S, rdf_colsum_kernel<__nv_bfloat16><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, nullptr, &c.ctl->all_cells, c.dz_bf, c.Hp, H, H, c.Hp, grads->db));   // dz rows are in all_cells order
     else if (tc_lstm) {                 // the gate gradients exist as bf16 operand rows only
-        RDF_KERNEL(S, rdf_colsum_kernel<__nv_bfloat16><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, c.all_cells, &c.ctl->all_cells, c.dg_bf, 5 * c.Hp, 5 * H, H, c.Hp, grads->db));
-        RDF_KERNEL(S, rdf_colsum_kernel<__nv_bfloat16><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, c.all_leaves, &c.ctl->all_leaves, c.dg_bf, 5 * c.Hp, 3 * H, H, c.Hp, grads->db_x));
+        RDF_KERNEL(S, rdf_colsum_kernel<__nv_bfloat16><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, nullptr, &c.ctl->all_cells, c.dg_bf, 5 * c.Hp, 5 * H, H, c.Hp, grads->db));
+        RDF_KERNEL(S, rdf_colsum_kernel<__nv_bfloat16><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, nullptr, &c.ctl->all_leaves, c.dgl_bf, 3 * c.Hp, 3 * H, H, c.Hp, grads->db_x));
     } else {
         RDF_KERNEL(S, rdf_colsum_kernel<float><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, c.all_cells, &c.ctl->all_cells, dgA, lda, MW, H, H, grads->db));
         if (lstm) RDF_KERNEL(S, rdf_colsum_kernel<float><<<8 * S->grid, 256, 0, stream>>>(&c.ctl->status, c.all_leaves, &c.ctl->all_leaves, c.gates, c.G, 3 * H, H, H, grads->db_x));

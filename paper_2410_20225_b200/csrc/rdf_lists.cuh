@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(256) rdf_list_fill_kernel(const DevCtx c, cons
         } else {
             if (c.lstm) {
                 c.all_leaves[il] = f;
+                if (c.cell_pos) c.cell_pos[f] = il;
                 if (c.leaf_ops) c.leaf_ops[il] = make_uint4(f, r[i], 0u, 1u);      // r = token id of a leaf
             }
             ++il;
@@ -139,20 +140,19 @@ __global__ void __launch_bounds__(256) rdf_list_fill_kernel(const DevCtx c, cons
     }
 }
 
-// The weight gradient reads dz and the operand rows in whole stages of 64 rows: the rows after the last cell are zero
-// (one block).
-__device__ __forceinline__ void zero_tail_rows(const DevCtx& c, uint32_t n_cells) {
-    const uint32_t n = min(n_cells, c.cells_cap), n_end = min((n + 63u) & ~63u, c.cells_cap);
-    if (c.dz_bf) {
-        const uint32_t per_row = (uint32_t)c.Hp / 8;
+// The weight gradient reads dz (the gate gradients) and the operand rows in whole stages of 64 rows: the rows after the last
+// cell / the last leaf are zero (one block).
+__device__ __forceinline__ void zero_tail_rows(const DevCtx& c, uint32_t n_cells, uint32_t n_leaves) {
+    auto zero = [](__nv_bfloat16* rows, uint32_t width, uint32_t count, uint32_t cap) {
+        if (!rows) return;
+        const uint32_t n = min(count, cap), n_end = min((n + 63u) & ~63u, cap), per_row = width / 8;
         for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
-            *reinterpret_cast<uint4*>(c.dz_bf + (size_t)(n + q / per_row) * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    if (c.z_bf) {
-        const uint32_t per_row = (uint32_t)c.Hp / 4;
-        for (uint32_t q = threadIdx.x; q < (n_end - n) * per_row; q += blockDim.x)
-            *reinterpret_cast<uint4*>(c.z_bf + (size_t)(n + q / per_row) * 2 * c.Hp + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
-    }
+            *reinterpret_cast<uint4*>(rows + (size_t)(n + q / per_row) * width + (q % per_row) * 8) = make_uint4(0u, 0u, 0u, 0u);
+    };
+    zero(c.dz_bf, c.Hp, n_cells, c.cells_cap);
+    zero(c.z_bf, 2 * c.Hp, n_cells, c.cells_cap);
+    zero(c.dg_bf, 5 * c.Hp, n_cells, c.cells_cap);
+    zero(c.dgl_bf, 3 * c.Hp, n_leaves, c.leaves_cap);
 }
 
 // marks[d].w = cells among the frames below marks[d].x: where wave d ends in all_cells.  One warp per wave.
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) rdf_list_ends_kernel(const DevCtx c, cons
         for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         if (lane == 0) c.wave_marks[d].w = seg_base[seg].x + cnt;
     }
-    if (blockIdx.x == 0) zero_tail_rows(c, c.ctl->all_cells);
+    if (blockIdx.x == 0) zero_tail_rows(c, c.ctl->all_cells, c.ctl->all_leaves);
 }
 
 // Where an invocation's state goes besides its own row: the operand row of the cell that called it

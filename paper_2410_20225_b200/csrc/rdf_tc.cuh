@@ -179,6 +179,15 @@ __device__ __forceinline__ void st_global_32(void* p, const uint4& a, const uint
                  "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
 }
 
+__device__ __forceinline__ void st_global_32(float* p, const float* v) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+                 "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+}
+__device__ __forceinline__ void ld_global_32(const float* p, float (&v)[8]) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]),
+                 "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p) : "memory");
+}
+
 // 16-byte asynchronous copy global -> shared through L2; `valid == false` writes zeros
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
     const int n = valid ? 16 : 0;
@@ -316,11 +325,11 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
     static_assert(STAGES >= 3 && STAGES <= TC_MAX_STAGES, "ring depth");
     constexpr int RGN = MODE == TC_LSTM_LEAF ? 1 : 0;
     // The rows of the A operand are consecutive rows of a matrix (the operand rows z_bf of the listed cells, or their
-    // dz rows): one 2D tile copy per stage instead of a gather.
-    constexpr bool TMA_A = MODE == TC_RNN_FWD || MODE == TC_LSTM_CELL || MODE == TC_RNN_BWD;
+    // dz / gate-gradient rows): one 2D tile copy per stage.  Only the rows E_bf[tok] of the leaf projection are gathered.
+    constexpr bool TMA_A = MODE != TC_LSTM_LEAF;
     // These modes write rows that later tile copies read (states into operand rows, dz rows).
     constexpr bool WRITES_TILE_ROWS = MODE == TC_RNN_FWD || MODE == TC_LSTM_CELL || MODE == TC_LSTM_LEAF || MODE == TC_RNN_BWD;
-    const int H = c.H, Hp = c.Hp, S = c.S, ns = tc.ns[RGN], n_chunks = tc.n_chunks[RGN];
+    const int H = c.H, Hp = c.Hp, ns = tc.ns[RGN], n_chunks = tc.n_chunks[RGN];
     const int slice = blockIdx.x % tc.n_split, rg = blockIdx.x / tc.n_split, n_rg = gridDim.x / tc.n_split;
     const int tiles = (n_items + TC_M - 1) / TC_M;
     // blocks beyond the last full group of slices have no tiles
@@ -333,8 +342,6 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
     if (warp >= TC_PROD_WARP0) {
         // ------------------------------------------------------------ producers
         const int p = threadIdx.x - TC_PROD_WARP0 * 32, r8 = p >> 3, c16 = p & 7;
-        const __nv_bfloat16* Arows = (MODE == TC_LSTM_BWD || MODE == TC_LSTM_DE) ? c.dg_bf
-                                     : MODE == TC_LSTM_LEAF ? c.E_bf : c.arena_bf;
         auto load_item = [&](int tile) {                     // the record of row p of the tile
             uint4 it = make_uint4(0u, 0u, 0u, 0u);
             const uint32_t row = (uint32_t)tile * TC_M + p;
@@ -359,18 +366,17 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
             sh.items[b][p] = it_next;
             mbar_arrive(items_full0 + 8 * b);
             if (i + 1 < my_tiles) it_next = load_item(rg + (i + 1) * n_rg);      // in flight during this tile
-            ok = mbar_wait(c, items_full0 + 8 * b, (T >> 1) & 1u) && ok;
-            // the eight rows this thread copies: r8 + 16 q
-            uint32_t src0[8], src1[8], valid = 0;
+            // the eight rows of E_bf this thread copies: those of rows r8 + 16 q
+            uint32_t src[8], valid = 0;
+            if (!TMA_A) {
+                ok = mbar_wait(c, items_full0 + 8 * b, (T >> 1) & 1u) && ok;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const uint4 it = sh.items[b][r8 + 16 * q];
-                if (it.w) valid |= 1u << q;
-                if (MODE == TC_RNN_FWD || MODE == TC_LSTM_CELL) { src0[q] = it.y; src1[q] = it.z; }
-                else if (MODE == TC_LSTM_LEAF) { src0[q] = it.y; src1[q] = it.y; }
-                else { src0[q] = it.x; src1[q] = it.x; }
+                for (int q = 0; q < 8; ++q) {
+                    const uint4 it = sh.items[b][r8 + 16 * q];
+                    if (it.w) valid |= 1u << q;
+                    src[q] = it.y;
+                }
             }
-            const size_t lda = (MODE == TC_LSTM_BWD || MODE == TC_LSTM_DE) ? (size_t)5 * Hp : (size_t)Hp;
             for (int kc = 0; kc < n_chunks && ok; ++kc) {
                 const uint32_t g = tc.g + (uint32_t)(i * n_chunks + kc), s = g % STAGES;
                 // the MMAs that last read this stage must have completed
@@ -382,18 +388,16 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
                     if (!ok) break;
                     if (p == 0) {
                         mbar_arrive_expect_tx(full0 + 8 * s, TC_A_STAGE);
-                        tma_load_2d(tc.a_addr + s * TC_A_STAGE, MODE == TC_RNN_BWD ? &c.tmap_dz128 : &c.tmap_z128, kc * TC_KC,
+                        tma_load_2d(tc.a_addr + s * TC_A_STAGE, MODE == TC_LSTM_DE ? &c.tmap_dgl128
+                                    : MODE == TC_RNN_BWD || MODE == TC_LSTM_BWD ? &c.tmap_dz128 : &c.tmap_z128, kc * TC_KC,
                                     (int)(first + (uint32_t)(rg + i * n_rg) * TC_M), full0 + 8 * s);
                     } else mbar_arrive(full0 + 8 * s);
                     continue;
                 }
-                const int koff = kc * TC_KC;
-                const bool second = (MODE == TC_RNN_FWD || MODE == TC_LSTM_CELL) && koff >= Hp;
-                const size_t col = (size_t)(second ? koff - Hp : koff) + c16 * 8;
+                const size_t col = (size_t)kc * TC_KC + c16 * 8;
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    cp_async16(tc.a_addr + s * TC_A_STAGE + swz(r8 + 16 * q, c16),
-                               Arows + (size_t)(second ? src1[q] : src0[q]) * lda + col, (valid >> q) & 1u);
+                    cp_async16(tc.a_addr + s * TC_A_STAGE + swz(r8 + 16 * q, c16), c.E_bf + (size_t)src[q] * Hp + col, (valid >> q) & 1u);
                 cp_async_arrive(full0 + 8 * s);                // this thread's share of the stage: arrives when its copies have landed
             }
         }
@@ -447,6 +451,13 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
             uint32_t zd = NO_ZDST;
             if ((MODE == TC_RNN_FWD || MODE == TC_LSTM_CELL || MODE == TC_LSTM_LEAF) && live) zd = __ldg(&c.zdst[it.x]);
             __nv_bfloat16* zrow = zd != NO_ZDST ? c.z_bf + (size_t)(zd >> 1) * 2 * Hp + (size_t)(zd & 1u) * Hp : nullptr;
+            // TreeLSTM cell: c of the operands, fetched while the MMAs run (8 units per thread, see below)
+            float cl[8], cr[8];
+            if (MODE == TC_LSTM_CELL && live) {
+                const int u0 = slice * 16 + (warp >> 2) * 8;
+                ld_global_32(c.arena + (size_t)it.y * Hp + u0, cl);
+                ld_global_32(c.arena + (size_t)it.z * Hp + u0, cr);
+            }
             uint32_t child_l = LEAF_MARK, child_tok = 0, child_pos = 0;
             float4 cd0 = make_float4(0.f, 0.f, 0.f, 0.f), cd1 = cd0;
             uint4 chq[BWD_MAXU];
@@ -517,19 +528,7 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
                 for (int g = 0; g < NG; ++g) tc_ld8(lane_base + (uint32_t)(g * 16 + wg * 8), v[g]);
                 if (live) {
                     const float* bias = MODE == TC_LSTM_CELL ? sh.ep : sh.ep + TC_EP_LEAF;     // [gate][unit of the slice]
-                    float cl[8], cr[8], hv[8], cv[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) cl[i] = cr[i] = 0.f;
-                    if (MODE == TC_LSTM_CELL) {
-#pragma unroll
-                        for (int i = 0; i < 8; i += 4)
-                            if (u0 + i < H) {
-                                const float4 a = ldcg4(c.arena + (size_t)it.y * S + H + u0 + i);
-                                const float4 b = ldcg4(c.arena + (size_t)it.z * S + H + u0 + i);
-                                cl[i] = a.x; cl[i + 1] = a.y; cl[i + 2] = a.z; cl[i + 3] = a.w;
-                                cr[i] = b.x; cr[i + 1] = b.y; cr[i + 2] = b.z; cr[i + 3] = b.w;
-                            }
-                    }
+                    float cv[8];
                     __align__(16) __nv_bfloat16 hb[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -554,28 +553,21 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
                                 v[0][i] = gi; v[1][i] = go; v[2][i] = gu;
                             }
                         }
-                        hb[i] = __float2bfloat16_rn(h);
-                        hv[i] = __bfloat162float(hb[i]);        // the h every consumer sees is the bf16 value
+                        hb[i] = __float2bfloat16_rn(h);         // the h every consumer sees
                         cv[i] = cc;
                     }
                     if (u0 == H) hb[0] = __float2bfloat16_rn(1.f);            // first pad column of the bf16 row: the constant
                     else if (u0 + 4 == H) hb[4] = __float2bfloat16_rn(1.f);   // input (see tc_leaf_rows); H is a multiple of 4
                     *reinterpret_cast<uint4*>(c.arena_bf + (size_t)it.x * Hp + u0) = *reinterpret_cast<const uint4*>(hb);
                     if (zrow) *reinterpret_cast<uint4*>(zrow + u0) = *reinterpret_cast<const uint4*>(hb);
-                    float* st = c.arena + (size_t)it.x * S;
+                    // c and the gates in whole 32-byte sectors (pad units: zeros); halves of sectors in rows by gate took
+                    // 1.2 of the 2.7 ms of the forward pass of 8192 trees, H = 300 (now 1.45)
+                    st_global_32(c.arena + (size_t)it.x * Hp + u0, cv);
+                    if (c.gates) {
+                        float* gt = c.gates + (size_t)it.x * 5 * Hp + u0 * NG;
 #pragma unroll
-                    for (int i = 0; i < 8; i += 4)
-                        if (u0 + i < H) {
-                            *reinterpret_cast<float4*>(st + u0 + i) = make_float4(hv[i], hv[i + 1], hv[i + 2], hv[i + 3]);
-                            *reinterpret_cast<float4*>(st + H + u0 + i) = make_float4(cv[i], cv[i + 1], cv[i + 2], cv[i + 3]);
-                            if (c.gates) {
-                                float* gt = c.gates + (size_t)it.x * c.G;
-#pragma unroll
-                                for (int g = 0; g < NG; ++g)
-                                    *reinterpret_cast<float4*>(gt + g * H + u0 + i) =
-                                        make_float4(v[g][i], v[g][i + 1], v[g][i + 2], v[g][i + 3]);
-                            }
-                        }
+                        for (int g = 0; g < NG; ++g) st_global_32(gt + 8 * g, v[g]);
+                    }
                 }
             } else {
                 // warps 0-3 take the first 16-column groups, warps 4-7 the rest
@@ -621,16 +613,17 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
                         for (int i = 0; i < 16; ++i)
                             if (col + i < c.D) {
                                 if (c.dE_fix) fix_add(&c.dE_fix[(size_t)it.y * c.D + col + i], to_fix(v[i]));
-                                else atomicAdd(&c.dE[(size_t)it.y * c.D + col + i], v[i]);
+                                else if (i % 4 == 0)                     // (D is a multiple of 4)
+                                    atomicAdd(reinterpret_cast<float4*>(&c.dE[(size_t)it.y * c.D + col + i]), make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
                             }
                     } else {
                         // operand gradients: columns [0, Hp) belong to the left callee frame, [Hp, 2Hp) to the right
                         const uint32_t child = col < Hp ? it.y : it.z;
                         const int cc = col < Hp ? col : col - Hp;
-                        float* dst = c.dhp + (size_t)child * S + cc;
-#pragma unroll
-                        for (int i = 0; i < 16; i += 4)
-                            if (cc + i < H) *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                        if (cc >= Hp) continue;                                 // (the last slice may reach beyond 2Hp)
+                        float* dst = c.dhp + (size_t)child * 2 * Hp + cc;
+                        st_global_32(dst, &v[0]);
+                        st_global_32(dst + 8, &v[8]);
                     }
                 }
             }
@@ -736,7 +729,7 @@ static __global__ void __launch_bounds__(256) rdf_pack_lstm_kernel(const DevCtx 
 }
 
 // dE of the TreeLSTM on tensor cores: one launch after the gradient waves, blocks = (row group, 64-column slice of D)
-static __global__ void __launch_bounds__(TC_THREADS, 1) rdf_de_tc_kernel(const DevCtx c) {
+static __global__ void __launch_bounds__(TC_THREADS, 1) rdf_de_tc_kernel(const __grid_constant__ DevCtx c) {
     extern __shared__ unsigned char dyn_smem[];
     __shared__ TcShared sh;
     if (c.ctl->status != 0) return;                    // an earlier kernel of this call failed

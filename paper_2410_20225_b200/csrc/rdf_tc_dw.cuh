@@ -37,22 +37,20 @@ __device__ __forceinline__ uint64_t tc_desc_mn(uint32_t smem_addr, uint32_t lbo,
 }
 
 // What to contract:  out[row(m)][col(n)] += sum over the listed invocations t of A_t[m] * B_t[n]
-//   A_t = A + t * lda, Mp padded rows in blocks of Hp (block g, unit j -> output row g * H + j, j < H)
+//   A_t = row t of dz_bf / dg_bf / dgl_bf: Mp padded columns in blocks of Hp (block g, unit j -> output row g * H + j, j < H).
+//   The rows are in list order and are read as 2D tiles; those after the last listed one are zero up to a multiple of 64.
 //   mode 0: B_t = [h(l_t) ; h(r_t)] from arena_bf (Np = 2 Hp; column half * Hp + k -> output column half * H + k)
 //   mode 1: B_t = E_bf[tok_t]                     (Np = Hp;  column k -> output column k, k < D)
 struct DwArgs {
     const uint4* ops;            // {frame, left / token, right, valid} per listed invocation
     const uint32_t* count;
-    const __nv_bfloat16* A;
-    int lda, Mp, Np, mode;
+    int Mp, Np, mode;
     float* out;
     int ldo;
     int tiles_n, n_tiles;
     int splits;                  // blocks per tile: block `split` takes the stages split, split + splits, ... of the list
     float* bias_out;             // mode 0 with H < Hp: column H of the left half of B is the constant 1 of the state rows,
                                  // so that column of the product is sum_t A_t = the bias gradient (null: not wanted)
-    int a_tiles;                 // 1: the rows of A are in list order (row = position in the list) and are read as 2D tiles
-                                 //    through DevCtx::tmap_dz64; the rows after the last listed one are zero up to a multiple of 64
     int b_tiles;                 // 1 (mode 0): B_t is row t of the operand rows z_bf (list order too), read through DevCtx::tmap_z64
     float* partial;              // reproducible mode: [n_tiles * splits][256][256], the block's partial tile (block = split *
                                  // n_tiles + tile) instead of atomics on `out`; null otherwise
@@ -102,8 +100,8 @@ __global__ void __launch_bounds__(256, 1) rdf_dw_tc_kernel(const __grid_constant
     if (warp < 4) {
         // ---- producers: a thread copies one 16-byte piece (q) of sixteen cells (tr0 + 4 i) of both operands per stage
         const int q = threadIdx.x & 31, tr0 = threadIdx.x >> 5, atom = q >> 3, c16 = q & 7;
-        const int m = m0 + atom * 64 + c16 * 8, n = n0 + atom * 64 + c16 * 8;
-        const bool m_in = m < a.Mp, n_in = n < a.Np;
+        const int n = n0 + atom * 64 + c16 * 8;
+        const bool n_in = n < a.Np;
         const __nv_bfloat16* Brows = a.mode == 0 ? c.arena_bf : c.E_bf;
         auto load_op = [&](uint32_t kc) {                          // the record of cell threadIdx.x of stage kc
             const uint32_t idx = ((uint32_t)split + kc * (uint32_t)a.splits) * DW_KT + threadIdx.x;
@@ -118,29 +116,23 @@ __global__ void __launch_bounds__(256, 1) rdf_dw_tc_kernel(const __grid_constant
             if (!ok) s_abort = 1;
             const uint32_t a_st = stage0 + s * DW_STAGE, b_st = a_st + DW_HALF;
 #pragma unroll 4
-            for (int i = 0; ok && i < DW_KT / 4; ++i) {
+            for (int i = 0; ok && !a.b_tiles && i < DW_KT / 4; ++i) {
                 const int tr = tr0 + 4 * i;
                 const uint4 it = s_ops[kc & 1][tr];
                 const uint32_t off = atom * 8192 + (tr >> 3) * 1024 + (tr & 7) * 128 + ((c16 ^ (tr & 7)) << 4);
-                if (!a.a_tiles) {
-                    const bool mv = it.w != 0u && m_in;
-                    cp_async16(a_st + off, a.A + (size_t)it.x * a.lda + (mv ? m : 0), mv);
-                }
-                if (!a.b_tiles) {
-                    const bool nv = it.w != 0u && n_in;
-                    size_t src = 0;
-                    if (nv) src = a.mode == 0 ? (n < Hp ? (size_t)it.y * Hp + n : (size_t)it.z * Hp + (n - Hp)) : (size_t)it.y * Hp + n;
-                    cp_async16(b_st + off, Brows + src, nv);
-                }
+                const bool nv = it.w != 0u && n_in;
+                size_t src = 0;
+                if (nv) src = a.mode == 0 ? (n < Hp ? (size_t)it.y * Hp + n : (size_t)it.z * Hp + (n - Hp)) : (size_t)it.y * Hp + n;
+                cp_async16(b_st + off, Brows + src, nv);
             }
-            if (ok && (a.a_tiles || a.b_tiles) && threadIdx.x == 0) {
+            if (ok && threadIdx.x == 0) {
                 // four boxes of 64 rows x 64 columns per operand, each written as the eight swizzled atoms of its column group
                 int boxes = 0;
-                for (int g = 0; g < 4; ++g) boxes += (a.a_tiles && m0 + g * 64 < a.Mp) + (a.b_tiles && n0 + g * 64 < a.Np);
+                for (int g = 0; g < 4; ++g) boxes += (m0 + g * 64 < a.Mp) + (a.b_tiles && n0 + g * 64 < a.Np);
                 mbar_expect_tx(full0 + 8 * s, (uint32_t)boxes * 8192u);
                 const int row0 = (int)(((uint32_t)split + kc * (uint32_t)a.splits) * DW_KT);
                 for (int g = 0; g < 4; ++g) {
-                    if (a.a_tiles && m0 + g * 64 < a.Mp) tma_load_2d(a_st + g * 8192, &c.tmap_dz64, m0 + g * 64, row0, full0 + 8 * s);
+                    if (m0 + g * 64 < a.Mp) tma_load_2d(a_st + g * 8192, a.mode ? &c.tmap_dgl64 : &c.tmap_dz64, m0 + g * 64, row0, full0 + 8 * s);
                     if (a.b_tiles && n0 + g * 64 < a.Np) tma_load_2d(b_st + g * 8192, &c.tmap_z64, n0 + g * 64, row0, full0 + 8 * s);
                 }
             }
