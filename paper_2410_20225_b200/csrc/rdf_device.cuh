@@ -69,6 +69,7 @@ struct Control {
     HotCounter qcount[3];         // tokens in the queue of wave w at [w % 3]
     HotCounter cell_count;        // ready cells queued so far, all waves (length of cell_items)
     HotCounter unary_count[2];    // interleaved execution: unary operators queued so far (left, right half of W)
+    HotCounter tile_next[2][3];   // fp32 wide waves, forward / gradient: tiles handed out (a wave in three uses the same word, see WideTiles)
     HotCounter leaf_count;        // ready leaves queued so far (length of leaf_items)
     HotCounter frame_count;
     HotCounter bar;               // grid barrier arrivals of the scheduler kernel (monotone)

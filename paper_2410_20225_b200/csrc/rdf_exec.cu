@@ -394,6 +394,86 @@ __device__ void rnn_cell_tiles(const DevCtx& c, GemmSmem& sm, uint32_t first, ui
     }
 }
 
+// The same for wide waves: 128 x 128 tiles (see WT).  1.05 M cells, H = 256, in 16 waves: 8.8 -> 7.3 ms.
+__device__ void rnn_cell_tiles_wide(const DevCtx& c, float* sm, const WideTiles& wt, uint32_t first, uint32_t n_items) {
+    const int H = c.H, K2 = 2 * c.H;
+    const int tiles_n = (H + WT - 1) / WT, tiles = (int)((n_items + WT - 1) / WT) * tiles_n, steps = (K2 + WT_K - 1) / WT_K;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int ty = (warp / 2) * 4 + lane / 8, tx = (warp % 2) * 8 + lane % 8;          // rows ty + 16 i, columns tx + 16 j
+    const int cr = threadIdx.x / 4, ck = (threadIdx.x % 4) * 4;                        // copies: rows cr, cr + 64, k ck ..
+    int* s_next = reinterpret_cast<int*>(sm + WT_STAGES * WT_STAGE) - 1;              // (a stage does not fill its last row)
+    wt.start();
+    for (int tile = blockIdx.x; tile < tiles;) {
+        const int row0 = (tile / tiles_n) * WT, col0 = (tile % tiles_n) * WT;
+        uint32_t l[2], r[2];
+        bool va[2], vb[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int row = row0 + cr + 64 * q;
+            va[q] = row < (int)n_items; vb[q] = col0 + cr + 64 * q < H;
+            l[q] = r[q] = 0u;
+            if (va[q]) {
+                const uint4 it = __ldcg(reinterpret_cast<const uint4*>(&c.cell_items[first + row]));   // {out, l, r, -}
+                l[q] = it.y; r[q] = it.z;
+            }
+        }
+        auto fetch = [&](int st) {
+            const int k = st * WT_K + ck;
+            const uint32_t dst = smem_u32(sm + (st % WT_STAGES) * WT_STAGE + cr * WT_LD + ck);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const bool v = va[q] && k < K2, w = vb[q] && k < K2;
+                cp_async16(dst + 4 * 64 * q * WT_LD, v ? c.arena + (size_t)(k < H ? l[q] : r[q]) * H + (k < H ? k : k - H) : c.arena, v);
+                cp_async16(dst + 4 * (WT + 64 * q) * WT_LD, w ? c.W + (size_t)(col0 + cr + 64 * q) * K2 + k : c.W, w);
+            }
+            cp_async_commit();
+        };
+        float acc[8][8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        __syncthreads();                                                   // (the stages of the tile before are no longer read)
+        if (threadIdx.x == 0) *s_next = wt.take();
+        fetch(0);
+        fetch(1);                                                          // (beyond the last step: zeros)
+        for (int st = 0; st < steps; ++st) {
+            cp_async_wait<1>();
+            __syncthreads();
+            fetch(st + 2);
+            const float* As = sm + (st % WT_STAGES) * WT_STAGE + ty * WT_LD;
+            const float* Bs = sm + (st % WT_STAGES) * WT_STAGE + (WT + tx) * WT_LD;
+#pragma unroll
+            for (int k = 0; k < WT_K; k += 4) {
+                float4 a[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * WT_LD + k);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4 b = *reinterpret_cast<const float4*>(Bs + 16 * j * WT_LD + k);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        acc[i][j] = fmaf(a[i].w, b.w, fmaf(a[i].z, b.z, fmaf(a[i].y, b.y, fmaf(a[i].x, b.x, acc[i][j]))));
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + ty + 16 * i;
+            if (row >= (int)n_items) continue;
+            float* out = c.arena + (size_t)__ldcg(&c.cell_items[first + row].out) * H;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int col = col0 + tx + 16 * j;
+                if (col < H) out[col] = tanhf(acc[i][j] + __ldg(&c.b[col]));
+            }
+        }
+        __syncthreads();
+        tile = *s_next;
+    }
+    cp_async_wait<0>();
+}
+
 // Narrow waves (a few dozen ready cells, e.g. the tail of a deep chain): the 64 x 64 tiles would keep
 // a handful of blocks busy with a long dependent k-loop.  Here one block step computes an 8 cell x 16
 // column patch with the whole contraction spread over its threads: thread = (cell, column, half of k),
@@ -834,9 +914,9 @@ __global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
 // the FFMA tiles need to hide their shared-memory and barrier latencies.
 template <bool TC, bool RNN32 = false>
 __global__ void __launch_bounds__(TC ? TC_THREADS : 256, TC ? 1 : 2) rdf_operator_kernel(const __grid_constant__ DevCtx c) {
-    __shared__ typename std::conditional<TC, TcShared, typename std::conditional<RNN32, LstmSmem, int>::type>::type smem;   // (tiles, or rows of thin patches)
+    __shared__ typename std::conditional<TC, TcShared, int>::type smem;
     const bool lstm = TC ? c.lstm != 0 : !RNN32;
-    extern __shared__ __align__(16) unsigned char dyn_smem[];        // TC: resident weight slices + operand stages; TreeLSTM: tile stages
+    extern __shared__ __align__(16) unsigned char dyn_smem[];        // TC: resident weight slices + operand stages; fp32: tile stages, resident columns
     if (c.ctl->forward_status != 0) return;                          // the scheduler failed: the lists are not to be trusted
     TcState tc;
     if constexpr (TC) {
@@ -848,7 +928,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, TC ? 1 : 2) rdf_operato
     const float4* wres = nullptr;
     if constexpr (RNN32) {
         if (c.H <= THIN_RESIDENT_MAX_H) {
-            float4* wr = reinterpret_cast<float4*>(dyn_smem);
+            float4* wr = reinterpret_cast<float4*>(dyn_smem + FP32_TILE_BYTES);
             const int K2 = 2 * c.H, units_n = (c.H + 15) / 16, cg0 = blockIdx.x % units_n;
             for (int q = threadIdx.x; q < (K2 / 4) * 16; q += blockDim.x) {
                 const int k4 = q / 16, col = cg0 * 16 + q % 16;
@@ -901,6 +981,8 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, TC ? 1 : 2) rdf_operato
             lap(cyc_b);
         }
     } else {
+        WideTiles wide;
+        wide.next = c.ctl->tile_next[0];
         // fp32 path: the same order.  With the clustered path this kernel fires the wide depths (scheduler waves below
         // d_split) and the clusters have fired the deeper ones before it.
         uint32_t nw = min(c.ctl->n_depth_waves, c.wave_cap);
@@ -923,8 +1005,12 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, TC ? 1 : 2) rdf_operato
             } else {
                 // thin patches while they fit in two rounds over the grid, tiles for wide waves
                 if (c.H <= 384 && ((nc + 7) / 8) * ((c.H + 15) / 16) <= 2 * gridDim.x)
-                    rnn_cell_thin(c, reinterpret_cast<float*>(&smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
-                else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, nc);
+                    rnn_cell_thin(c, reinterpret_cast<float*>(dyn_smem), wres, first, nc);      // 8 x 2H + 128 floats <= 26 KB
+                else if (wide_tiles_pay(nc, c.H)) {
+                    rnn_cell_tiles_wide(c, reinterpret_cast<float*>(dyn_smem), wide, first, nc);
+                    ++wide.wave;
+                }
+                else rnn_cell_tiles(c, *reinterpret_cast<GemmSmem*>(dyn_smem), first, nc);
             }
             __syncthreads();
             lap(cyc_c);
@@ -1360,8 +1446,8 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     S->grid = sms;                 // one persistent block per SM
     {   // the fp32 TreeRNN kernels: two blocks per SM where they fit
         int a = 0;
-        CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
-        CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, rdf_operator_kernel<false, true>, 256, 128 * THIN_RESIDENT_MAX_H));
+        CUDA_OK(cudaFuncSetAttribute(rdf_operator_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fp32_smem_bytes(0, THIN_RESIDENT_MAX_H)));
+        CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, rdf_operator_kernel<false, true>, 256, fp32_smem_bytes(0, THIN_RESIDENT_MAX_H)));
         S->rnn32_per_sm = std::max(1, std::min(2, a));
     }
     S->device = dev;
@@ -1686,7 +1772,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                 }
                 // ... the wide ones with the whole grid
                 RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_operator_kernel<false, true>, dim3(S->grid * S->rnn32_per_sm),
-                                                    dim3(256), oargs, thin_resident_bytes(0, c.H), stream)));
+                                                    dim3(256), oargs, fp32_smem_bytes(0, c.H), stream)));
             }
         }
         rdf_mark(S, 4, stream);

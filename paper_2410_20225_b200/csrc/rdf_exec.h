@@ -13,12 +13,24 @@ struct __align__(16) GemmSmem {
     float Bs[TK][TN + 4];     // [k][column of the tile]
 };
 
-// TreeLSTM tiles: the same 64 x 64 tile for up to five gate blocks at once, so that all gates of a
-// hidden unit end up in one thread and the gate arithmetic fuses into the epilogue
-struct __align__(16) LstmSmem {
-    float As[TK][TM + 4];
-    float Bs[5][TK][TN + 4];
+// Wide waves: tiles of 128 x 128, 8 x 8 outputs per thread, a ring of three stages of 16 k filled by asynchronous copies.  Rows
+// of A (and of W where it is read along k) lie in the stage as in memory, 16 k each, 20 words apart.
+static const int WT = 128, WT_K = 16, WT_LD = WT_K + 4, WT_STAGES = 3, WT_STAGE = 2 * WT * WT_LD;      // (floats of a stage)
+static const size_t FP32_TILE_BYTES = (size_t)WT_STAGES * WT_STAGE * sizeof(float);       // (also holds GemmSmem and the patches)
+// The tiles of a wide wave are handed out one by one: of two blocks on an SM the older one gets its instructions issued first
+// and would otherwise be done long before the other (a third of the time of the wide gradient waves).
+struct WideTiles {
+    HotCounter* next;          // three words: the one of wave w is cleared during wave w - 1, when wave w - 3 + 1 is long done
+    uint32_t wave = 0;
+    __device__ void start() const { if (blockIdx.x == 0 && threadIdx.x == 0) next[(wave + 1) % 3].v = 0u; }
+    __device__ int take() const { return (int)(gridDim.x + atomicAdd(&next[wave % 3].v, 1u)); }
 };
+// Which tile for a wave: rounds over the grid, a 64 x 64 tile taking WT_SMALL of the time of a large one (a quarter of the work
+// at about half its rate: 26 and 47 TFLOP/s)
+__device__ __forceinline__ bool wide_tiles_pay(uint32_t n_items, int n_cols) {
+    const uint32_t large = (n_items + WT - 1) / WT * ((n_cols + WT - 1) / WT), small = (n_items + TM - 1) / TM * ((n_cols + TN - 1) / TN);
+    return (large + gridDim.x - 1) / gridDim.x * 9u <= (small + gridDim.x - 1) / gridDim.x * 4u;
+}
 
 __device__ __forceinline__ float4 ldcg4(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
 
@@ -39,6 +51,8 @@ __device__ __forceinline__ void gemm_tile_step(const GemmSmem& sm, int tx, int t
 // 128 * H bytes, while that fits beside the tiles
 static const int THIN_RESIDENT_MAX_H = 384;
 inline size_t thin_resident_bytes(int lstm, int H) { return !lstm && H <= THIN_RESIDENT_MAX_H ? (size_t)128 * H : 0; }
+// dynamic shared memory of the fp32 kernels: tile stages (or the rows of a patch), then the resident columns
+inline size_t fp32_smem_bytes(int lstm, int H) { return FP32_TILE_BYTES + thin_resident_bytes(lstm, H); }
 
 static const int DW_BLOCKS_MAX = 256;        // blocks of the tensor-core weight-gradient pass (reproducible mode: one partial tile each)
 static const int LIST_SEG = 2048;            // frames per segment of the list kernels (256 threads x 8)

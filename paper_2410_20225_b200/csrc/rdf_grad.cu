@@ -864,6 +864,91 @@ __device__ void backward_operand_tiles(const DevCtx& c, GemmSmem& sm, uint32_t f
     }
 }
 
+// The same for wide waves: 128 x 128 tiles (see WT); W is read along its columns, as it lies: pairs of them per multiply-add.
+// 1.05 M cells, H = 256, in 16 waves: 7.5 -> 5.8 ms (47 TFLOP/s of 64).
+__device__ void backward_operand_tiles_wide(const DevCtx& c, float* sm, const WideTiles& wt, uint32_t first, uint32_t n_items, const float* A, int lda, int Kdim) {
+    const int H = c.H, K2 = 2 * c.H, S = c.S;
+    const int tiles_n = (K2 + WT - 1) / WT, tiles = (int)((n_items + WT - 1) / WT) * tiles_n, steps = (Kdim + WT_K - 1) / WT_K;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int ty = (warp / 2) * 4 + lane / 8, tx = (warp % 2) * 8 + lane % 8;          // rows ty + 16 i, columns 4 tx .., 64 + 4 tx ..
+    const int cr = threadIdx.x / 4, ck = (threadIdx.x % 4) * 4;                        // copies of A: rows cr, cr + 64, k ck ..
+    const int bk = threadIdx.x / 16, bn = (threadIdx.x % 16) * 4;                      // copies of W: k bk, columns bn, bn + 64
+    int* s_next = reinterpret_cast<int*>(sm + WT_STAGES * WT_STAGE) - 1;              // (a stage does not fill its last row)
+    wt.start();
+    for (int tile = blockIdx.x; tile < tiles;) {
+        const int row0 = (tile / tiles_n) * WT, col0 = (tile % tiles_n) * WT;
+        const float* src[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int row = row0 + cr + 64 * q;
+            src[q] = row < (int)n_items ? A + (size_t)__ldcg(&c.all_cells[first + row]) * lda : nullptr;
+        }
+        auto fetch = [&](int st) {
+            const int k = st * WT_K + ck, kb = st * WT_K + bk;
+            float* stage = sm + (st % WT_STAGES) * WT_STAGE;
+            const uint32_t da = smem_u32(stage + cr * WT_LD + ck), db = smem_u32(stage + WT * WT_LD + bk * WT + bn);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const bool v = src[q] && k < Kdim, w = kb < Kdim && col0 + bn + 64 * q < K2;
+                cp_async16(da + 4 * 64 * q * WT_LD, v ? src[q] + k : c.W, v);
+                cp_async16(db + 4 * 64 * q, w ? c.W + (size_t)kb * K2 + col0 + bn + 64 * q : c.W, w);
+            }
+            cp_async_commit();
+        };
+        f32x2 acc[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+        __syncthreads();                                                   // (the stages of the tile before are no longer read)
+        if (threadIdx.x == 0) *s_next = wt.take();
+        fetch(0);
+        fetch(1);                                                          // (beyond the last step: zeros)
+        for (int st = 0; st < steps; ++st) {
+            cp_async_wait<1>();
+            __syncthreads();
+            fetch(st + 2);
+            const float* As = sm + (st % WT_STAGES) * WT_STAGE + ty * WT_LD;
+            const float* Bs = sm + (st % WT_STAGES) * WT_STAGE + WT * WT_LD + tx * 4;
+#pragma unroll
+            for (int k = 0; k < WT_K; k += 4) {
+                float4 a[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(As + 16 * i * WT_LD + k);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(Bs + (k + e) * WT), b1 = *reinterpret_cast<const ulonglong2*>(Bs + (k + e) * WT + 64);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float x = e == 0 ? a[i].x : e == 1 ? a[i].y : e == 2 ? a[i].z : a[i].w;
+                        const f32x2 xx = pack2(x, x);
+                        acc[i][0] = fma2(xx, b0.x, acc[i][0]); acc[i][1] = fma2(xx, b0.y, acc[i][1]);
+                        acc[i][2] = fma2(xx, b1.x, acc[i][2]); acc[i][3] = fma2(xx, b1.y, acc[i][3]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = row0 + ty + 16 * i;
+            if (row >= (int)n_items) continue;
+            const uint32_t t = __ldcg(&c.all_cells[first + row]), l = __ldcg(&c.op_l[t]), r = __ldcg(&c.op_r[t]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int col = col0 + tx * 4 + 64 * j;
+                if (col >= K2) continue;
+                float4 v;
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(acc[i][2 * j]));
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(v.z), "=f"(v.w) : "l"(acc[i][2 * j + 1]));
+                *reinterpret_cast<float4*>(c.dhp + (size_t)(col < H ? l : r) * S + (col < H ? col : col - H)) = v;
+            }
+        }
+        __syncthreads();
+        tile = *s_next;
+    }
+    cp_async_wait<0>();
+}
+
 // Narrow waves: an 8 cell x 32 column patch of [dh_l ; dh_r] = W^T dz per block step;
 // thread = (cell, 4 columns, quarter of the contraction over j).  The thread that ends up with the four
 // sums finishes the callee they belong to right away (what the per-invocation pass would do one wave
@@ -963,8 +1048,8 @@ __device__ void backward_operand_thin(const DevCtx& c, float* zs, const float4* 
 template <bool TC, bool RNN32 = false>         // RNN32: the fp32 TreeRNN alone, two blocks per SM (see rdf_operator_kernel)
 __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_backward_kernel(const __grid_constant__ DevCtx c) {
     const bool lstm = RNN32 ? false : c.lstm != 0;
-    __shared__ typename std::conditional<TC, TcShared, LstmSmem>::type smem;   // fp32: tiles use the first part; thin patches stage rows in it
-    extern __shared__ unsigned char dyn_smem[];                      // tensor-core path: resident W^T slice + A stages
+    __shared__ typename std::conditional<TC, TcShared, int>::type smem;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];        // TC: resident W^T slice + A stages; fp32: tile stages, resident columns
     if (c.ctl->forward_status != 0) return;                          // the forward pass failed: nothing to differentiate
     TcState tc;
     if constexpr (TC) {
@@ -976,7 +1061,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
     const float4* wres = nullptr;
     if constexpr (!TC) {
         if (!lstm && c.H <= THIN_RESIDENT_MAX_H) {
-            float4* wr = reinterpret_cast<float4*>(dyn_smem);
+            float4* wr = reinterpret_cast<float4*>(dyn_smem + FP32_TILE_BYTES);
             const int K2 = 2 * c.H, units_n = (K2 + 31) / 32, cg0 = blockIdx.x % units_n;
             for (int q = threadIdx.x; q < c.H * 8; q += blockDim.x) {
                 const int j = q / 8, col = cg0 * 32 + (q % 8) * 4;
@@ -1003,6 +1088,8 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
     // clustered gradient pass (fp32 TreeRNN, deep recursions): this kernel runs the wide call depths only, up to d_split
     const bool clustered = !TC && !lstm && depth_groups(c) > 1u;
     const uint32_t d_split = clustered ? c.ctl->d_split : 0u;
+    WideTiles wide;
+    wide.next = c.ctl->tile_next[1];
     for (uint32_t k = 0; k < nw; ++k) {
         const uint4 cur = wv;
         if (k + 1 < nw) wv = c.wave_marks[k + 1];                    // in flight during this wave
@@ -1051,11 +1138,15 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
                 if (lstm) tc_pipe<TC_LSTM_BWD, TC_STAGES_LSTM_BWD>(c, tc, smem, first, end - first);
                 else tc_pipe<TC_RNN_BWD, TC_STAGES_RNN_BWD>(c, tc, smem, first, end - first);
             } else {
-                if (lstm) backward_operand_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, end - first, c.gates, c.G, 5 * c.H);
-                else if (c.H <= 512 && ((end - first + 7) / 8) * ((2 * c.H + 31) / 32) <= 2 * gridDim.x) {
-                    backward_operand_thin(c, reinterpret_cast<float*>(&smem), wres, first, end - first);   // 8 x H + 800 floats <= 26 KB
+                const float* A = lstm ? c.gates : c.dhp;
+                const int lda = lstm ? c.G : c.H, Kdim = lstm ? 5 * c.H : c.H;
+                if (!lstm && c.H <= 512 && ((end - first + 7) / 8) * ((2 * c.H + 31) / 32) <= 2 * gridDim.x) {
+                    backward_operand_thin(c, reinterpret_cast<float*>(dyn_smem), wres, first, end - first);   // 8 x H + 800 floats <= 26 KB
                     thin = true;
-                } else backward_operand_tiles(c, *reinterpret_cast<GemmSmem*>(&smem), first, end - first, c.dhp, c.H, c.H);
+                } else if (wide_tiles_pay(end - first, 2 * c.H)) {
+                    backward_operand_tiles_wide(c, reinterpret_cast<float*>(dyn_smem), wide, first, end - first, A, lda, Kdim);
+                    ++wide.wave;
+                } else backward_operand_tiles(c, *reinterpret_cast<GemmSmem*>(dyn_smem), first, end - first, A, lda, Kdim);
             }
             __syncthreads();
             lap(cyc_c);
@@ -1232,7 +1323,7 @@ inline size_t bwd_cluster_smem_bytes(int H) {
 //   mode 1: B_t = E[tok_t]           (N = D)    -> dW_x (TreeLSTM leaves)
 // A block owns a tile of 16 RM x 16 RN outputs (a thread RM x RN of them) and every splits-th stage of 16 invocations; the
 // rows of three stages are on their way (cp.async) while one is multiplied.  What bounds it is shared memory: RM + RN words
-// for RM RN multiply-adds of a thread, hence 8 x 8 per thread (two blocks per SM; 8 x 16 leaves room for one: 7.75 ms).
+// for RM RN multiply-adds of a thread, hence 8 x 8 per thread (two blocks per SM; 8 x 16 leaves room for one: 7.75 ms; one block of two groups in step: 7.9 ms).
 // 1.31 M cells, H = 256 (344 GFLOP): 12.7 (64 x 64 tiles, 4 x 4 per thread, one stage at a time) -> 7.3 ms, 47 TFLOP/s of 64.
 struct OuterArgs {
     const uint32_t* list;
@@ -1545,17 +1636,17 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
         // narrow ones after them (both leave at once when there is nothing for them to do)
         const bool clusters = c.n_groups > 1 && !c.lstm && H <= 512;
         if (c.lstm) {
-            CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
+            CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fp32_smem_bytes(0, THIN_RESIDENT_MAX_H)));
             RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_backward_kernel<false>, dim3(S->grid), dim3(256), args,
-                                                thin_resident_bytes(c.lstm, c.H), stream)));
+                                                fp32_smem_bytes(c.lstm, c.H), stream)));
         } else {
             // fp32 TreeRNN: as many blocks per SM as both of its persistent kernels take
             int per_sm = 0;
-            CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * THIN_RESIDENT_MAX_H));
-            CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_backward_kernel<false, true>, 256, 128 * THIN_RESIDENT_MAX_H));
+            CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fp32_smem_bytes(0, THIN_RESIDENT_MAX_H)));
+            CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_backward_kernel<false, true>, 256, fp32_smem_bytes(0, THIN_RESIDENT_MAX_H)));
             per_sm = std::max(1, std::min(per_sm, S->rnn32_per_sm));
             RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_backward_kernel<false, true>, dim3(S->grid * per_sm), dim3(256), args,
-                                                thin_resident_bytes(0, c.H), stream)));
+                                                fp32_smem_bytes(0, c.H), stream)));
         }
         if (clusters) {
             cudaLaunchConfig_t cfg = {};
