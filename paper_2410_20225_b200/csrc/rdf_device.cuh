@@ -150,7 +150,7 @@ struct DevCtx {
     float*    arena;              // [frame_cap, S] fp32 states: S = H (TreeRNN h) or 2H (TreeLSTM h then c); bf16 TreeLSTM:
                                   // [frame_cap, Hp] c alone
     float*    gates;              // TreeLSTM under rdf_grad: [frame_cap, G] activated gates, later their gradients; bf16:
-                                  // [frame_cap, Hp / 8, gates, 8] (row stride 5Hp), what a thread of the epilogue has in one piece
+                                  // [frame_cap, 5, Hp] (leaves: the first 3), written by whole sectors of 8 units
     int       S, G, lstm;
     // tensor-core path (bf16 operands): bf16 copy of the states with row stride Hp, packed weights
     __nv_bfloat16* arena_bf;

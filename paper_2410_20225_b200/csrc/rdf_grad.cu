@@ -719,93 +719,93 @@ __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t,
     }
 }
 
+// tanh to a few units in the last place without a branch, so that independent ones overlap: x from -0.55 to 0.55 by Lambert's
+// continued fraction x / (1 + x^2 / (3 + x^2 / (5 + x^2 / (7 + x^2 / 9)))) as a quotient of polynomials, else 1 - 2 / (e^2|x| + 1).
+__device__ __forceinline__ float tanh_select(float x) {
+    const float y = x * x, a = fabsf(x);
+    const float small = x * __fdividef(fmaf(y, y + 105.f, 945.f), fmaf(y, fmaf(y, 15.f, 420.f), 945.f));
+    const float large = 1.f - __fdividef(2.f, expf(fminf(2.f * a, 40.f)) + 1.f);
+    return a < 0.55f ? small : copysignf(large, x);
+}
+
 // A (bf16 TreeLSTM): the gate gradients as bf16 operand rows in list order; dc goes straight to the callee frames.
-// A thread takes 8 hidden units of every invocation it gets (what the forward epilogue stored in one piece: gates, c and the
-// incoming gradients in whole sectors, pad units included, whose gradients come out as zeros); as many invocations at a time
-// as the block has threads for, all loads of one in flight together.
-// 8192 trees, H = 300 (4.5 GB): 1.42 ms with a warp per invocation and rows split by gate -> 1.22 ms.
+// A thread takes 4 hidden units of every invocation it gets, pad units included (their gradients come out as zeros); as many
+// invocations at a time as the block has threads for, all loads of one in flight together, and one code for leaves and cells,
+// which meet in a warp.  Memory-bound; the lanes of a load cover whole lines (gates in blocks of 8 units, 160 bytes from lane to
+// lane, spent as long on cache tags as on bytes).
+// 8192 trees, H = 300 (4.5 GB): 1.42 ms (a warp per invocation) -> 1.22 (8 units per thread, 13 warps) -> 0.93; 416 / 1024 threads
+// 1.00 / 1.11.
 __device__ __forceinline__ void lstm_backward_units(const DevCtx& c, uint32_t f0, uint32_t f1) {
-    const int H = c.H, Hp = c.Hp, C = c.n_classes, ub = Hp / 8, per = blockDim.x / ub;
-    const int u = (threadIdx.x % ub) * 8, fo = threadIdx.x / ub;
+    const int H = c.H, Hp = c.Hp, C = c.n_classes, ub = Hp / 4, per = blockDim.x / ub;
+    const int u = (threadIdx.x % ub) * 4, fo = threadIdx.x / ub;
     if (fo >= per) return;
-    auto header = [&](uint32_t t, uint4& m) {
-        if (t < f1) m = make_uint4(c.op_l[t], c.op_r[t], c.frames[t].parent, c.cell_pos[t]);
+    auto header = [&](uint32_t t) { return make_uint4(c.op_l[t], c.op_r[t], c.frames[t].parent, c.cell_pos[t]); };
+    auto ld = [](const float* q, float (&v)[4]) {
+        const float4 x = ldcg4(q);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    };
+    auto store_bf = [](__nv_bfloat16* q, const float (&v)[4]) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+        *reinterpret_cast<uint2*>(q) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
     };
     const uint32_t step = gridDim.x * per;
     uint32_t t = f0 + blockIdx.x * per + fo;
     uint4 m = make_uint4(0u, 0u, 0u, 0u);
-    header(t, m);
+    if (t < f1) m = header(t);
     for (; t < f1; t += step) {
         const uint4 cur = m;
         const bool leaf = cur.x == LEAF_MARK, top = cur.z < (uint32_t)c.B;         // top: called from `result`, no gradient comes in
-        const float4 d0 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8), d1 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8 + 4);
-        float g[5][8], cc[8], dh[8], dc[8], cl[8], cr[8];
-        const float* gt = c.gates + (size_t)t * c.G + u * (leaf ? 3 : 5);
+        float g[5][4], cc[4], dh[4], dc[4], cl[4], cr[4];
+        const float* gt = c.gates + (size_t)t * c.G + u;
 #pragma unroll
-        for (int k = 0; k < 5; ++k)
-            if (k < 3 || !leaf) ld_global_32(gt + 8 * k, g[k]);
-        ld_global_32(c.arena + (size_t)t * Hp + u, cc);
+        for (int k = 0; k < 3; ++k) ld(gt + k * Hp, g[k]);
         if (!leaf) {
-            ld_global_32(c.arena + (size_t)cur.x * Hp + u, cl);
-            ld_global_32(c.arena + (size_t)cur.y * Hp + u, cr);
+            ld(gt + 3 * Hp, g[3]);
+            ld(gt + 4 * Hp, g[4]);
+            ld(c.arena + (size_t)cur.x * Hp + u, cl);
+            ld(c.arena + (size_t)cur.y * Hp + u, cr);
         }
+        ld(c.arena + (size_t)t * Hp + u, cc);
         if (!top) {
-            ld_global_32(c.dhp + (size_t)t * 2 * Hp + u, dh);
-            ld_global_32(c.dhp + (size_t)t * 2 * Hp + Hp + u, dc);
+            ld(c.dhp + (size_t)t * 2 * Hp + u, dh);
+            ld(c.dhp + (size_t)t * 2 * Hp + Hp + u, dc);
         } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) dh[i] = dc[i] = 0.f;
+            for (int i = 0; i < 4; ++i) dh[i] = dc[i] = 0.f;
         }
-        if (step < f1 - t) header(t + step, m);                        // in flight during this step
+        const float4 d0 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8), d1 = *reinterpret_cast<const float4*>(c.dlog + (size_t)t * 8 + 4);
+        if (step < f1 - t) m = header(t + step);                       // in flight during this step
         const float dl[MAX_CLASSES] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+        if (u < H) {
 #pragma unroll
-        for (int k = 0; k < MAX_CLASSES; ++k)
-            if (k < C) {
+            for (int k = 0; k < MAX_CLASSES; ++k)
+                if (k < C) {
+                    const float4 w = __ldg(reinterpret_cast<const float4*>(&c.W_s[k * H + u]));
+                    dh[0] = fmaf(w.x, dl[k], dh[0]); dh[1] = fmaf(w.y, dl[k], dh[1]);
+                    dh[2] = fmaf(w.z, dl[k], dh[2]); dh[3] = fmaf(w.w, dl[k], dh[3]);
+                }
+        }
 #pragma unroll
-                for (int i = 0; i < 8; i += 4)
-                    if (u + i < H) {
-                        const float4 w = __ldg(reinterpret_cast<const float4*>(&c.W_s[k * H + u + i]));
-                        dh[i] = fmaf(w.x, dl[k], dh[i]); dh[i + 1] = fmaf(w.y, dl[k], dh[i + 1]);
-                        dh[i + 2] = fmaf(w.z, dl[k], dh[i + 2]); dh[i + 3] = fmaf(w.w, dl[k], dh[i + 3]);
-                    }
-            }
-        auto store_bf = [](__nv_bfloat16* p, const float (&v)[8]) {
-            __align__(16) __nv_bfloat162 pk[4];
+        for (int i = 0; i < 4; ++i) {
+            const float gi = g[0][i], fl = g[1][i], fr = g[2][i], go = leaf ? fl : g[3][i], gu = leaf ? fr : g[4][i];
+            const float tc = tanh_select(cc[i]);
+            const float d = dc[i] + dh[i] * go * (1.f - tc * tc);
+            g[0][i] = d * gu * gi * (1.f - gi);
+            g[3][i] = dh[i] * tc * go * (1.f - go);
+            g[4][i] = d * gi * (1.f - gu * gu);
+            g[1][i] = leaf ? g[3][i] : d * cl[i] * fl * (1.f - fl);
+            g[2][i] = leaf ? g[4][i] : d * cr[i] * fr * (1.f - fr);
+            cl[i] = d * fl;
+            cr[i] = d * fr;
+        }
+        __nv_bfloat16* row = leaf ? c.dgl_bf + (size_t)cur.w * 3 * Hp + u : c.dg_bf + (size_t)cur.w * 5 * Hp + u;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) pk[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-            *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(pk);
-        };
-        if (leaf) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float gi = g[0][i], go = g[1][i], gu = g[2][i], tc = tanhf(cc[i]);
-                const float d = dc[i] + dh[i] * go * (1.f - tc * tc);
-                g[0][i] = d * gu * gi * (1.f - gi);
-                g[1][i] = dh[i] * tc * go * (1.f - go);
-                g[2][i] = d * gi * (1.f - gu * gu);
-            }
-            __nv_bfloat16* row = c.dgl_bf + (size_t)cur.w * 3 * Hp + u;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) store_bf(row + k * Hp, g[k]);
-        } else {
-            float dcl[8], dcr[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float gi = g[0][i], fl = g[1][i], fr = g[2][i], go = g[3][i], gu = g[4][i], tc = tanhf(cc[i]);
-                const float d = dc[i] + dh[i] * go * (1.f - tc * tc);
-                g[0][i] = d * gu * gi * (1.f - gi);
-                g[1][i] = d * cl[i] * fl * (1.f - fl);
-                g[2][i] = d * cr[i] * fr * (1.f - fr);
-                g[3][i] = dh[i] * tc * go * (1.f - go);
-                g[4][i] = d * gi * (1.f - gu * gu);
-                dcl[i] = d * fl;
-                dcr[i] = d * fr;
-            }
-            __nv_bfloat16* row = c.dg_bf + (size_t)cur.w * 5 * Hp + u;
-#pragma unroll
-            for (int k = 0; k < 5; ++k) store_bf(row + k * Hp, g[k]);
-            st_global_32(c.dhp + (size_t)cur.x * 2 * Hp + Hp + u, dcl);
-            st_global_32(c.dhp + (size_t)cur.y * 2 * Hp + Hp + u, dcr);
+        for (int k = 0; k < 3; ++k) store_bf(row + k * Hp, g[k]);
+        if (!leaf) {
+            store_bf(row + 3 * Hp, g[3]);
+            store_bf(row + 4 * Hp, g[4]);
+            *reinterpret_cast<float4*>(c.dhp + (size_t)cur.x * 2 * Hp + Hp + u) = make_float4(cl[0], cl[1], cl[2], cl[3]);
+            *reinterpret_cast<float4*>(c.dhp + (size_t)cur.y * 2 * Hp + Hp + u) = make_float4(cr[0], cr[1], cr[2], cr[3]);
         }
     }
 }
@@ -1045,9 +1045,11 @@ __device__ void backward_operand_thin(const DevCtx& c, float* zs, const float4* 
     }
 }
 
-template <bool TC, bool RNN32 = false>         // RNN32: the fp32 TreeRNN alone, two blocks per SM (see rdf_operator_kernel)
-__global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_backward_kernel(const __grid_constant__ DevCtx c) {
-    const bool lstm = RNN32 ? false : c.lstm != 0;
+// RNN32: the fp32 TreeRNN alone, two blocks per SM (see rdf_operator_kernel); TCL: the bf16 TreeLSTM (TC alone: the bf16 TreeRNN)
+static const int LSTM_BWD_THREADS = 640;      // (see lstm_backward_units)
+template <bool TC, bool RNN32 = false, bool TCL = false>
+__global__ void __launch_bounds__(TCL ? LSTM_BWD_THREADS : TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_backward_kernel(const __grid_constant__ DevCtx c) {
+    constexpr bool lstm = TC ? TCL : !RNN32;
     __shared__ typename std::conditional<TC, TcShared, int>::type smem;
     extern __shared__ __align__(16) unsigned char dyn_smem[];        // TC: resident W^T slice + A stages; fp32: tile stages, resident columns
     if (c.ctl->forward_status != 0) return;                          // the forward pass failed: nothing to differentiate
@@ -1117,7 +1119,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
             const unsigned long long c0l = (unsigned long long)f0 + (unsigned long long)blockIdx.x * per;
             const uint32_t c0 = (uint32_t)min(c0l, (unsigned long long)f1), c1 = (uint32_t)min(c0l + per, (unsigned long long)f1);
             if constexpr (TC) {
-                if (lstm) lstm_backward_units(c, f0, f1);
+                if constexpr (lstm) lstm_backward_units(c, f0, f1);
                 else backward_frames_tc(c, c0 + wib * 4 + lane / 8, c1, 4 * n_warps, lane % 8);
                 asm volatile("fence.proxy.async;" ::: "memory");       // the dz / gate-gradient rows are read by tile copies after the barrier
             } else if constexpr (RNN32) {
@@ -1135,7 +1137,7 @@ __global__ void __launch_bounds__(TC ? TC_THREADS : 256, RNN32 ? 2 : 1) rdf_back
         bool thin = false;
         if (end > first) {
             if constexpr (TC) {
-                if (lstm) tc_pipe<TC_LSTM_BWD, TC_STAGES_LSTM_BWD>(c, tc, smem, first, end - first);
+                if constexpr (lstm) tc_pipe<TC_LSTM_BWD, TC_STAGES_LSTM_BWD>(c, tc, smem, first, end - first);
                 else tc_pipe<TC_RNN_BWD, TC_STAGES_RNN_BWD>(c, tc, smem, first, end - first);
             } else {
                 const float* A = lstm ? c.gates : c.dhp;
@@ -1628,8 +1630,9 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
     CUDA_OK(cudaGetLastError());
     void* args[] = {(void*)&c};
     if (c.use_tc) {
-        CUDA_OK(cudaFuncSetAttribute(rdf_backward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, L.tc_smem_bwd));
-        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_backward_kernel<true>, dim3(S->grid), dim3(TC_THREADS), args,
+        void (*kernel)(DevCtx) = lstm ? rdf_backward_kernel<true, false, true> : rdf_backward_kernel<true>;
+        CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L.tc_smem_bwd));
+        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)kernel, dim3(S->grid), dim3(lstm ? LSTM_BWD_THREADS : TC_THREADS), args,
                                             (size_t)L.tc_smem_bwd, stream)));
     } else {
         // deep recursions (cells grouped by the forward pass): the grid-wide kernel runs the wide depths, the clusters the

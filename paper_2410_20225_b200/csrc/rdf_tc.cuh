@@ -319,7 +319,7 @@ __device__ __forceinline__ float tc_sigmoid(float x) { return fmaf(0.5f, tc_tanh
 
 // The tile loop over n_items ready operators (see TcMode), 128 rows per tile.  Rows come from
 // cell_items / leaf_items (forward modes) or from cell_ops / leaf_ops at [first ..] (gradient modes).
-// Called by all TC_THREADS threads of the block; returns when every tile has been written out.
+// Called by all threads of the block (those beyond TC_THREADS have no part in it); returns when every tile has been written out.
 template <int MODE, int STAGES>
 __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t first, uint32_t n_items) {
     static_assert(STAGES >= 3 && STAGES <= TC_MAX_STAGES, "ring depth");
@@ -339,7 +339,8 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
     const uint32_t acc_full0 = smem_u32(&sh.acc_full[0]), acc_empty0 = smem_u32(&sh.acc_empty[0]);
     const uint32_t items_full0 = smem_u32(&sh.items_full[0]);
     bool ok = true;
-    if (warp >= TC_PROD_WARP0) {
+    if (warp >= TC_THREADS / 32) {
+    } else if (warp >= TC_PROD_WARP0) {
         // ------------------------------------------------------------ producers
         const int p = threadIdx.x - TC_PROD_WARP0 * 32, r8 = p >> 3, c16 = p & 7;
         auto load_item = [&](int tile) {                     // the record of row p of the tile
@@ -564,9 +565,9 @@ __device__ void tc_pipe(const DevCtx& c, TcState& tc, TcShared& sh, uint32_t fir
                     // 1.2 of the 2.7 ms of the forward pass of 8192 trees, H = 300 (now 1.45)
                     st_global_32(c.arena + (size_t)it.x * Hp + u0, cv);
                     if (c.gates) {
-                        float* gt = c.gates + (size_t)it.x * 5 * Hp + u0 * NG;
+                        float* gt = c.gates + (size_t)it.x * 5 * Hp + u0;
 #pragma unroll
-                        for (int g = 0; g < NG; ++g) st_global_32(gt + 8 * g, v[g]);
+                        for (int g = 0; g < NG; ++g) st_global_32(gt + g * Hp, v[g]);
                     }
                 }
             } else {
