@@ -725,6 +725,11 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
 // whole kernel up to H = IL_SMEM_W_H; wider ones are read through L1.  The terms of a sum are added in index order (a Switch
 // decides on the sign of a sum over the state: another order could flip it).
 static const int IL_SMEM_W_H = 128;
+// One cluster of 8 blocks runs a call while instances x (H + 16) stay below this.  Besides its faster barrier, the acquire of a
+// grid barrier drops the block's local memory (spilled registers, label arrays) from L1 twice per wave.  Grid -> cluster, depth 10:
+// 8 instances, H = 16: 0.450 -> 0.289 ms; 64, H = 128: 0.852 -> 0.759; 400, H = 16: 0.603 -> 0.497; 100, H = 128: 0.856 -> 0.809;
+// 200, H = 64: 0.699 -> 0.795.
+static const long long IL_CLUSTER_WORK = 15500;
 __host__ __device__ inline int il_stride(int K) { return K + (K % 8 == 0 ? 4 : 8); }
 __host__ __device__ inline int il_out_warps(int H) { return H < 128 ? (H + 15) / 16 : 8; }
 __host__ __device__ inline int il_group_max(int H) { return 32 / il_out_warps(H) * 16; }         // items that the 32 warps cover
@@ -776,6 +781,8 @@ __device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int s
 // What bounds it: the FMA and load issue of the wide waves and the latency of the narrow ones.  8192 seeds, H = 128, 44
 // waves: groups of 32 with the kinds mixed (unary operators as cells with a zero half) and tokens on the first blocks only
 // 4.24 ms, this 1.86 ms (operators 2.9 -> 1.25, tokens 1.0 -> 0.33).
+// CLUSTER: the whole grid is one cluster, whose barrier takes a fifth of the time of the grid barrier (see IL_CLUSTER_WORK).
+template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
     extern __shared__ __align__(16) unsigned char il_smem[];
@@ -800,6 +807,11 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         }
     const int out_warps = il_out_warps(H), iw = warp / out_warps, jw = warp % out_warps;
     const uint32_t gwarp = warp * gridDim.x + blockIdx.x, n_warps = gridDim.x * (blockDim.x / 32);      // (consecutive warps on different SMs)
+    auto barrier = [&]() {
+        if (!CLUSTER) return grid_barrier(c, &c.ctl->bar.v, generation);
+        cluster_sync_all();                                         // (blocks that have left count as arrived)
+        return ld_volatile_i32(&c.ctl->status) == 0;
+    };
     for (;; ++wave) {
         const uint32_t n = ld_volatile_u32(&c.ctl->qcount[wave % 3].v);
         if (n == 0) break;
@@ -813,7 +825,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         for (uint32_t i = gwarp * 32u + lane; i < n; i += n_warps * 32u) run_token(c, sp, nullptr, wave, load_token(&q[i]), st);
         __syncthreads();
         lap(cyc_s);
-        if (!grid_barrier(c, &c.ctl->bar.v, generation)) break;
+        if (!barrier()) break;
         lap(cyc_b);
         // ---- the operators this wave queued
         const uint32_t n_leaf = min(ld_volatile_u32(&c.ctl->leaf_count.v), c.work_cap);
@@ -832,7 +844,10 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         const uint32_t g0 = G ? (end[0] - done[0] + G - 1) / G : 0u, g1 = G ? (end[1] - done[1] + G - 1) / G : 0u, g2 = G ? (end[2] - done[2] + G - 1) / G : 0u;
         for (uint32_t g = blockIdx.x; g < g0 + g1 + g2; g += gridDim.x) {
             const int kind = g < g0 ? 0 : g < g0 + g1 ? 1 : 2;
-            const uint32_t first = done[kind] + (g - (kind == 0 ? 0u : kind == 1 ? g0 : g0 + g1)) * G, cnt = min(G, end[kind] - first);
+            // (no arrays by index: they would live in local memory, which the barrier's acquire has just dropped from L1)
+            const uint32_t first = (kind == 0 ? done[0] : kind == 1 ? done[1] : done[2]) + (g - (kind == 0 ? 0u : kind == 1 ? g0 : g0 + g1)) * G;
+            const uint32_t cnt = min(G, (kind == 0 ? end[0] : kind == 1 ? end[1] : end[2]) - first);
+            const uint2* unary = kind == 2 ? c.unary_items[1] : c.unary_items[0];
             const int K = kind == 0 ? 2 * H : H, stride = il_stride(K);
             __syncthreads();                                        // (the previous group's operands are no longer read)
             for (uint32_t i = warp; i < cnt; i += 32u) {
@@ -840,7 +855,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
                 if (kind == 0) {
                     const CellItem it = c.cell_items[first + i];
                     l = it.l; r = it.r;
-                } else l = c.unary_items[kind - 1][first + i].y;
+                } else l = unary[first + i].y;
                 const bool ok = l < c.frame_cap && r < c.frame_cap;
                 if (!ok && lane == 0) set_status(c, RDF_ERR_BAD_ARG);
                 for (int k = lane * 4; k < K; k += 128) {
@@ -855,7 +870,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const uint32_t at = (uint32_t)row0 + 8u * i;
-                out[i] = at >= cnt ? 0xFFFFFFFFu : kind == 0 ? c.cell_items[first + at].out : c.unary_items[kind - 1][first + at].x;
+                out[i] = at >= cnt ? 0xFFFFFFFFu : kind == 0 ? c.cell_items[first + at].out : unary[first + at].x;
             }
             __syncthreads();
             const int k0 = kind == 2 ? H : 0;
@@ -869,7 +884,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         for (int q2 = 0; q2 < 3; ++q2) done[q2] = end[q2];
         __syncthreads();
         lap(cyc_o);
-        if (!grid_barrier(c, &c.ctl->bar.v, generation)) break;
+        if (!barrier()) break;
         lap(cyc_b);
     }
     flush_stats(c, st);
@@ -1415,6 +1430,16 @@ ExecState* rdf_state_of(rdf_graph* g) {
     return static_cast<ExecState*>(g->dev);
 }
 
+// The interleaved kernel as one cluster of CLUSTER_CTAS blocks
+static cudaLaunchConfig_t il_cluster_config(cudaLaunchAttribute* at, size_t smem, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(CLUSTER_CTAS); cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 1;
+    return cfg;
+}
+
 int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     (void)g;
     int dev = 0;
@@ -1437,9 +1462,17 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     if (per_sm < 1) return RDF_ERR_CUDA;
     S->lstm32_per_sm = std::min(per_sm, 2);
     const int il_smem = std::max(interleaved_smem_bytes(IL_SMEM_W_H), interleaved_smem_bytes(INTERLEAVED_MAX_H));      // the two largest configurations
-    CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem));
-    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel, 1024, il_smem));
+    CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem));
+    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel<false>, 1024, il_smem));
     if (per_sm < 1) return RDF_ERR_CUDA;
+    {
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = il_cluster_config(at, il_smem, nullptr);
+        int n = 0;
+        S->il_cluster = cudaFuncSetAttribute(rdf_interleaved_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&n, rdf_interleaved_kernel<true>, &cfg) == cudaSuccess && n > 0;
+        cudaGetLastError();
+    }
     CUDA_OK(cudaFuncSetAttribute(rdf_scheduler_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * LQ_CAP * sizeof(Token))));
     CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_scheduler_kernel, 1024, 2 * LQ_CAP * sizeof(Token)));
     if (per_sm < 1) return RDF_ERR_CUDA;
@@ -1707,9 +1740,15 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         const int blocks = L.frame_cap <= FS_ONE_BLOCK ? 1 : S->grid;
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_fold_kernel, dim3(blocks), dim3(FS_CHUNK), args, 0, stream)));
     } else if (g->interleaved)
-        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel, dim3(S->grid), dim3(1024), args,
-                                            (size_t)interleaved_smem_bytes(c.H), stream)));
-    else
+    {
+        if (S->il_cluster && in->B * (c.H + 16ll) < IL_CLUSTER_WORK) {
+            cudaLaunchAttribute at[1];
+            const cudaLaunchConfig_t cfg = il_cluster_config(at, (size_t)interleaved_smem_bytes(c.H), stream);
+            RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_interleaved_kernel<true>, c)));
+        } else
+            RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel<false>, dim3(S->grid), dim3(1024), args,
+                                                (size_t)interleaved_smem_bytes(c.H), stream)));
+    } else
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_scheduler_kernel, dim3(S->grid), dim3(1024), args,
                                             2 * LQ_CAP * sizeof(Token), stream)));
     rdf_mark(S, 2, stream);

@@ -135,8 +135,10 @@ def test_topdown_full_size_as_benchmarked():
     assert abs(st["invocations"] - total) <= slack, (st["invocations"], total, slack)
 
 
-@pytest.mark.parametrize("H,D,B", [(4, 5, 40), (20, 6, 33), (124, 5, 30), (128, 5, 30), (132, 4, 30), (256, 4, 20)])
+@pytest.mark.parametrize("H,D,B", [(4, 5, 40), (20, 6, 33), (124, 5, 30), (128, 5, 30), (132, 4, 30), (256, 4, 20),
+                                   (20, 4, 440), (124, 4, 110), (124, 4, 112), (132, 4, 120)])
 def test_topdown_hidden_sizes(H, D, B):
     """Hidden sizes on both sides of the warp tiles (16 outputs) and of the switch from weights in shared memory (H <= 128)
-    to weights read through the cache; groups of one and of several warps along the items."""
+    to weights read through the cache; groups of one and of several warps along the items; one
+    cluster (B (H + 16) < 15500) and the whole grid."""
     test_topdown_recursion_states_and_shapes(H, D, B)
