@@ -212,6 +212,125 @@ __global__ void __launch_bounds__(256) rdf_loss_heads_kernel(const DevCtx c, int
     }
 }
 
+// ---- the same pass for fp32 rows of up to 128 NQ units and up to NC classes, a warp on its own: four rows at a time stay in
+// registers from the logits to dW_s (a lane has units 4 lane + 128 q), one transposing reduction leaves logit (row, class) on lane
+// 8 row + class, where softmax, loss and dlog of all four rows are computed at once.  16 warps per SM with 4 KB each
+// in flight, nothing waits for a block; the slab form above spends 22 k cycles per 48 rows on latencies.
+// 2.62 M rows, H = 256 (2.8 GB): 2.20 -> 0.65 ms (4.3 TB/s).
+template <int NQ, int NC>
+__global__ void __launch_bounds__(256, NQ < 3 ? 2 : 1) rdf_loss_rows_kernel(const DevCtx c) {
+    if (c.ctl->status != 0) return;                    // an earlier kernel of this call failed: its lists and rows are not to be trusted
+    __shared__ __align__(16) float s_w[NC][128 * NQ];  // W_s, then the block's share of dW_s
+    __shared__ float warp_loss[8], s_db[8];
+    const uint32_t B = (uint32_t)c.B, F = max(c.ctl->frame_count.v, B);
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, r = lane / 8, k = lane % 8, H = c.H;
+    for (int q = threadIdx.x; q < NC * 128 * NQ; q += 256) {
+        const int kk = q / (128 * NQ), j = q % (128 * NQ);
+        s_w[kk][j] = kk < c.n_classes && j < H ? c.W_s[kk * H + j] : 0.f;
+    }
+    if (threadIdx.x < 8) s_db[threadIdx.x] = 0.f;
+    __syncthreads();
+    const float bias = k < c.n_classes ? c.b_s[k] : -INFINITY;
+    float acc[NQ][4][NC], loss = 0.f, db = 0.f;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int kk = 0; kk < NC; ++kk) acc[q][e][kk] = 0.f;
+    const uint32_t step = gridDim.x * 32u;             // rows of a round: 4 per warp
+    auto label_of = [&](uint32_t f) { return f < F ? __ldg(&c.label[(int)c.frames[f].arg]) : 0; };
+    uint32_t f0 = B + (blockIdx.x * 8u + warp) * 4u;
+    int lab = label_of(f0 + r);
+    for (; f0 < F; f0 += step) {
+        float4 x[4][NQ];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int j = lane * 4 + 128 * q;
+                x[i][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (j < H && f0 + i < F) x[i][q] = *reinterpret_cast<const float4*>(c.arena + (size_t)(f0 + i) * c.S + j);
+            }
+        const int lab_ahead = step < F - f0 ? label_of(f0 + step + r) : 0;     // two dependent loads, in flight during this round
+        float z[32];
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            if (kk < NC) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const float4 w = *reinterpret_cast<const float4*>(&s_w[kk < NC ? kk : 0][lane * 4 + 128 * q]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        s[i] = fmaf(w.w, x[i][q].w, fmaf(w.z, x[i][q].z, fmaf(w.y, x[i][q].y, fmaf(w.x, x[i][q].x, s[i]))));
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[8 * i + kk] = s[i];
+        }
+#pragma unroll
+        for (int n = 16; n > 0; n >>= 1)               // (half of the values go to the other half of the lanes)
+#pragma unroll
+            for (int i = 0; i < n; ++i) {
+                const bool up = lane & n;
+                const float mine = up ? z[i + n] : z[i], other = up ? z[i] : z[i + n];
+                z[i] = mine + __shfl_xor_sync(0xffffffffu, other, n);
+            }
+        const float zz = z[0] + bias;                  // logit of (row r, class k)
+        float m = zz;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        const float ex = expf(zz - m);                 // (a class that does not exist: 0)
+        float sum = ex;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const bool live = f0 + r < F;
+        const float d = live && k < c.n_classes ? ex / sum - (k == lab ? 1.f : 0.f) : 0.f;
+        if (live) c.dlog[(size_t)(f0 + r) * 8 + k] = d;
+        const float zl = __shfl_sync(0xffffffffu, zz, 8 * r + (lab & 7));
+        if (live && k == 0) loss += logf(sum) + m - (lab >= 0 && lab < c.n_classes ? zl : 0.f);
+        db += d;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int kk = 0; kk < NC; ++kk) {
+                const float dk = __shfl_sync(0xffffffffu, d, 8 * i + kk);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    acc[q][0][kk] = fmaf(dk, x[i][q].x, acc[q][0][kk]); acc[q][1][kk] = fmaf(dk, x[i][q].y, acc[q][1][kk]);
+                    acc[q][2][kk] = fmaf(dk, x[i][q].z, acc[q][2][kk]); acc[q][3][kk] = fmaf(dk, x[i][q].w, acc[q][3][kk]);
+                }
+            }
+        lab = lab_ahead;
+    }
+    // the warps' shares added up in shared memory, one warp after the other
+    for (int o = 16; o >= 8; o >>= 1) db += __shfl_xor_sync(0xffffffffu, db, o);
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    for (int w = 0; w < 8; ++w) {
+        __syncthreads();
+        if (warp != w) continue;
+        if (lane < 8) s_db[lane] += db;
+        if (lane == 0) warp_loss[w] = loss;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int kk = 0; kk < NC; ++kk) {
+                float4* t = reinterpret_cast<float4*>(&s_w[kk][lane * 4 + 128 * q]);
+                const float4 old = w ? *t : make_float4(0.f, 0.f, 0.f, 0.f);
+                *t = make_float4(old.x + acc[q][0][kk], old.y + acc[q][1][kk], old.z + acc[q][2][kk], old.w + acc[q][3][kk]);
+            }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < c.n_classes * H; q += 256) atomicAdd(&c.dW_s[q], s_w[q / H][q % H]);
+    if (threadIdx.x < c.n_classes) atomicAdd(&c.db_s[threadIdx.x], s_db[threadIdx.x]);
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += warp_loss[w];
+        c.loss_partial[blockIdx.x] = t;
+    }
+}
+
 // ---- the same pass for the bf16 workloads (rows = the bf16 h of arena_bf), with the two small contractions on the tensor cores
 // (warp-level mma.sync m16n8k16: the shapes are [64 rows x Hp] x [Hp x 8 classes] and [Hp x 64 rows] x [64 x 8],
 // far too small for a tcgen05 tile).  States are bf16 already; W_s and dlog enter as a bf16 pair hi + lo
@@ -1618,6 +1737,10 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
             const int smem_mma = 2 * LM_ROWS * (c.Hp * 2 + 16);
             CUDA_OK(cudaFuncSetAttribute(rdf_loss_heads_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_mma));
             RDF_KERNEL(S, rdf_loss_heads_mma_kernel<<<loss_blocks, 256, smem_mma, stream>>>(c));
+        } else if (params->n_classes <= 5 && H <= 384) {       // (wider rows, more classes: too many registers for rows and sums)
+            if (H <= 128) RDF_KERNEL(S, rdf_loss_rows_kernel<1, 5><<<loss_blocks, 256, 0, stream>>>(c));
+            else if (H <= 256) RDF_KERNEL(S, rdf_loss_rows_kernel<2, 5><<<loss_blocks, 256, 0, stream>>>(c));
+            else RDF_KERNEL(S, rdf_loss_rows_kernel<3, 5><<<loss_blocks, 256, 0, stream>>>(c));
         } else {
             CUDA_OK(cudaFuncSetAttribute(rdf_loss_heads_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             RDF_KERNEL(S, rdf_loss_heads_kernel<false><<<loss_blocks, 256, smem, stream>>>(c, fr, rowbytes));

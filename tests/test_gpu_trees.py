@@ -491,3 +491,23 @@ def test_clustered_depths(H, chains, depth):
     cfg["params"]["b"] = (0.1 * np.random.default_rng(H).standard_normal(H)).astype(np.float32)
     st, _ = check_grad(cfg, workers=WORKERS)
     assert st["clusters"] > 1 and st["waves_backward"] >= depth
+
+
+@pytest.mark.parametrize("H", [4, 60, 128, 132, 256, 260, 384, 388])
+def test_fp32_gradient_tile_edges(H):
+    """Hidden sizes on both sides of the loss head's unit groups (128 units; beyond 384 rows move through shared memory) and of
+    the weight gradient's tiles (64 x 128 and 128 x 128), a few dozen trees with single leaves among them: the tail of every
+    tile and of every round of rows.  Tolerance: the file's fp32 bound."""
+    rng = np.random.default_rng(H)
+    p = workloads.treernn_params(3, 70, H, H)
+    tb = workloads.tree_batch_from_shapes([workloads.random_split_shape(rng, L) for L in [1, 2, 1] + [int(x) for x in rng.integers(1, 30, 37)]], 7, vocab=70)
+    check_grad({"trees": tb, "params": p})
+
+
+def test_fp32_wide_wave_tiles():
+    """Waves wide enough for the 128 x 128 tiles in both directions (32 768 cells, H = 132: two tile columns forward, three in the
+    gradient pass, none of them full), and odd trees that leave a ragged last tile row."""
+    rng = np.random.default_rng(8)
+    p = workloads.treernn_params(3, 70, 132, 132)
+    shapes = [workloads.perfect_tree_shape(15)] * 2 + [workloads.random_split_shape(rng, int(L)) for L in rng.integers(1, 40, 21)]
+    check_grad({"trees": workloads.tree_batch_from_shapes(shapes, 7, vocab=70), "params": p}, workers=WORKERS)
