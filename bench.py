@@ -508,7 +508,7 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     lstm = case.cell == "lstm"
     mm = "tensor" if case.use_tc else "alu"
     if not case.use_tc and not lstm:
-        add("rdf_group_count/scan/scatter_kernel", "group", "hbm", 48.0 * C, "16 B cell record read twice and written once")
+        add("rdf_group_kernel", "group", "hbm", 48.0 * C, "16 B cell record read twice and written once")
     add("rdf_operator_kernel", "operators", mm, case.flops_fwd(),
         "cell contraction 2*2H*H per cell" + (" (x5 gates) + leaf projection 2*D*3H per leaf" if lstm else ""))
     add("rdf_gather_roots_kernel", "roots", "hbm", tb.B * H * (4.0 + (2 if case.use_tc and not lstm else 4)), "root rows read and written")

@@ -152,7 +152,7 @@ struct ClDepth {
 struct ClRings {
     ClDepth  depth[CL_RING];
     uint4    rec[CL_RING][CL_SLOTS];           // {cell, left, right, -}
-    uint4    link[CL_RING][CL_SLOTS];          // see rdf_group_link_kernel
+    uint4    link[CL_RING][CL_SLOTS];          // see rdf_group_kernel
     uint32_t end[CL_RING];                     // list end between steps t - 1 and t
     uint64_t rows_full[3];                     // rows of step t complete: mbarrier t % 3
     uint64_t rows_read[4];                     // rows of step t read by every block: mbarrier t % 4

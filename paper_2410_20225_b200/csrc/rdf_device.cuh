@@ -75,6 +75,7 @@ struct Control {
     HotCounter bar;               // grid barrier arrivals of the scheduler kernel (monotone)
     HotCounter bar2;              // barrier counter of the backward kernel
     HotCounter bar_ops;           // barrier counter of the operator kernel
+    HotCounter bar_group;         // barrier counter of the grouping kernel
     int32_t  status;
     uint32_t waves, waves_backward, max_wave_tokens, max_probe, max_depth;
     uint32_t all_cells;           // backward: cells seen so far (length of the all-cells list)
@@ -140,7 +141,7 @@ struct DevCtx {
     // batched operators
     CellItem* cell_items;         // every cell in the order it became ready (general scheduler)
     CellItem* cell_sorted;        // clustered fp32 path: the cells grouped by (cluster of their instance, call depth)
-    uint4*    cell_link;          // [work_cap] per grouped cell: where its operands come from and its state goes (rdf_group_link_kernel)
+    uint4*    cell_link;          // [work_cap] per grouped cell: where its operands come from and its state goes (rdf_group_kernel)
     uint32_t* group_ends;         // [wave_cap + 2]: cells per group, then (after the scatter) the end of each group
     LeafItem* leaf_items;         // every leaf in the order it was reached
     uint2*    unary_items[2];     // interleaved execution: {result frame, operand frame} of the unary operators, by half of W

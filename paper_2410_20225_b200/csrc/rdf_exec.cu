@@ -1154,11 +1154,8 @@ __device__ __forceinline__ uint32_t cell_bucket(const DevCtx& c, const uint4& it
     return (__ldcg(&c.finst[it.x]) % groups) * stride + d;
 }
 
-__global__ void __launch_bounds__(256) rdf_group_count_kernel(const DevCtx c) {
-    if (c.ctl->status != 0) return;
+__device__ __forceinline__ void group_count(const DevCtx& c, uint32_t groups, uint32_t stride) {
     const uint32_t n = min(c.ctl->all_cells, c.work_cap), lane = threadIdx.x % 32;
-    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
-    if (groups <= 1u) return;
     for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * blockDim.x) {
         const uint32_t i = i0 + lane;
         const uint32_t k = i < n ? cell_bucket(c, c.cell_ops[i], groups, stride) : 0u;
@@ -1168,16 +1165,14 @@ __global__ void __launch_bounds__(256) rdf_group_count_kernel(const DevCtx c) {
 }
 
 // counts -> first position of each bucket (one block; buckets 1 .. groups * stride - 1)
-__global__ void __launch_bounds__(1024) rdf_group_scan_kernel(const DevCtx c) {
+__device__ __forceinline__ void group_scan(const DevCtx& c, uint32_t top) {
     __shared__ uint32_t warp_sum[32];
     __shared__ uint32_t carry;
-    if (c.ctl->status != 0) return;
-    if (depth_groups(c) <= 1u) return;
-    const uint32_t top = depth_groups(c) * depth_stride(c) - 1u;
+    const uint32_t n_warps = blockDim.x / 32;
     const uint32_t lane = threadIdx.x % 32, warp = threadIdx.x / 32;
     if (threadIdx.x == 0) carry = 0;
     __syncthreads();
-    for (uint32_t h0 = 1; h0 <= top; h0 += 1024) {
+    for (uint32_t h0 = 1; h0 <= top; h0 += blockDim.x) {
         const uint32_t h = h0 + threadIdx.x;
         const uint32_t v = h <= top ? c.group_ends[h] : 0u;
         uint32_t x = v;
@@ -1188,7 +1183,7 @@ __global__ void __launch_bounds__(1024) rdf_group_scan_kernel(const DevCtx c) {
         if (lane == 31) warp_sum[warp] = x;
         __syncthreads();
         if (warp == 0) {
-            uint32_t w = warp_sum[lane];
+            uint32_t w = lane < n_warps ? warp_sum[lane] : 0u;
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
                 if ((int)lane >= o) w += y;
@@ -1199,18 +1194,15 @@ __global__ void __launch_bounds__(1024) rdf_group_scan_kernel(const DevCtx c) {
         const uint32_t before = carry + (warp ? warp_sum[warp - 1] : 0u) + x - v;
         if (h <= top) c.group_ends[h] = before;
         __syncthreads();
-        if (threadIdx.x == 1023) carry = before + v;
+        if (threadIdx.x == blockDim.x - 1) carry = before + v;
         __syncthreads();
     }
 }
 
 // every cell to its bucket; afterwards group_ends[k] is where bucket k ends (it starts where bucket k - 1 ends;
 // bucket group * stride + 0 is empty, so it ends where the previous group ends)
-__global__ void __launch_bounds__(256) rdf_group_scatter_kernel(const DevCtx c) {
-    if (c.ctl->status != 0) return;
+__device__ __forceinline__ void group_scatter(const DevCtx& c, uint32_t groups, uint32_t stride) {
     const uint32_t n = min(c.ctl->all_cells, c.work_cap), lane = threadIdx.x % 32;
-    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
-    if (groups <= 1u) return;
     for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * blockDim.x) {
         const uint32_t i = i0 + lane;
         const uint4 it = i < n ? c.cell_ops[i] : make_uint4(0u, 0u, 0u, 0u);
@@ -1230,10 +1222,7 @@ __global__ void __launch_bounds__(256) rdf_group_scatter_kernel(const DevCtx c) 
 
 // Which depths are wide enough for the whole grid (clustered path): up to the last one that has more than `threshold` cells
 // over all groups; the deeper ones are left to the clusters.
-__global__ void __launch_bounds__(256) rdf_group_split_kernel(const DevCtx c, uint32_t threshold) {
-    if (c.ctl->status != 0) return;
-    const uint32_t groups = depth_groups(c), stride = depth_stride(c);
-    if (groups <= 1u) return;
+__device__ __forceinline__ void group_split(const DevCtx& c, uint32_t groups, uint32_t stride, uint32_t threshold) {
     for (uint32_t h = 1 + blockIdx.x * blockDim.x + threadIdx.x; h < stride; h += gridDim.x * blockDim.x) {
         uint32_t total = 0;
         for (uint32_t gq = 0; gq < groups; ++gq) total += c.group_ends[(size_t)gq * stride + h] - c.group_ends[(size_t)gq * stride + h - 1];
@@ -1245,11 +1234,8 @@ __global__ void __launch_bounds__(256) rdf_group_split_kernel(const DevCtx c, ui
 // leaf, else the place of that cell among the cells of its (group, depth), at most CL_NO_SLOT; z = the place of the calling
 // cell, | the operand port << 6.  The clusters hand states on from one depth to the next: a program whose operands lie
 // further apart than one call depth (calls that waited for other calls) is left to the grid-wide kernels.
-__global__ void __launch_bounds__(256) rdf_group_link_kernel(const DevCtx c) {
-    if (c.ctl->status != 0) return;
-    const uint32_t groups = depth_groups(c), stride = depth_stride(c), split = c.ctl->d_split;
-    if (groups <= 1u) return;
-    const uint32_t n = min(c.ctl->all_cells, c.work_cap), B = (uint32_t)c.B;
+__device__ __forceinline__ void group_link(const DevCtx& c, uint32_t groups, uint32_t stride) {
+    const uint32_t split = ld_volatile_u32(&c.ctl->d_split), n = min(c.ctl->all_cells, c.work_cap), B = (uint32_t)c.B;
     auto depth_of = [&](uint32_t f) { return (c.frames[f].label >> FRAME_WAVE_SHIFT) + 1u; };
     auto place = [&](uint32_t f) {
         const uint32_t k = cell_bucket(c, make_uint4(f, 0u, 0u, 1u), groups, stride);
@@ -1281,6 +1267,28 @@ __global__ void __launch_bounds__(256) rdf_group_link_kernel(const DevCtx c) {
         c.cell_link[p] = link;
     }
     if (!regular) atomicMax(&c.ctl->d_split, stride - 1u);
+}
+
+// The five steps, one kernel with grid barriers between them: a shallow recursion (which has nothing to group, as the device
+// alone knows) pays for one launch.  512 trees, H = 64:
+// 0.018 -> 0.007 ms, the call 156 -> 153 us; 64 chains of 4096 and 16 trees of height 16: 0.14 -> 0.23 ms of 43.
+__global__ void __launch_bounds__(256) rdf_group_kernel(const __grid_constant__ DevCtx c, uint32_t threshold) {
+    if (c.ctl->status != 0) return;
+    const uint32_t groups = depth_groups(c), stride = depth_stride(c), top = groups * stride - 1u;
+    if (groups <= 1u) return;
+    uint32_t generation = 0;
+    auto barrier = [&]() { return grid_barrier(c, &c.ctl->bar_group.v, generation); };
+    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k <= top + 1u && k < c.wave_cap + 2u; k += gridDim.x * blockDim.x) c.group_ends[k] = 0u;
+    if (!barrier()) return;
+    group_count(c, groups, stride);
+    if (!barrier()) return;
+    if (blockIdx.x == 0) group_scan(c, top);
+    if (!barrier()) return;
+    group_scatter(c, groups, stride);
+    if (!barrier()) return;
+    group_split(c, groups, stride, threshold);
+    if (!barrier()) return;
+    group_link(c, groups, stride);
 }
 
 // root states: h_root[b] = state(frame y[b])
@@ -1861,13 +1869,9 @@ int rdf_launch_lists(const rdf_batch* in, char* ws, const Layout& L, ExecState* 
 // The cells grouped by (cluster of their instance, call depth) for the clustered fp32 kernels, forward and gradient.
 int rdf_launch_depth_groups(char* ws, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream) {
     if (c.n_groups <= 1) return RDF_OK;
-    CUDA_OK(cudaMemsetAsync(ws + L.group_ends, 0, ((size_t)L.wave_cap + 2) * sizeof(uint32_t), stream));
-    RDF_KERNEL(S, rdf_group_count_kernel<<<2 * S->grid, 256, 0, stream>>>(c));
-    RDF_KERNEL(S, rdf_group_scan_kernel<<<1, 1024, 0, stream>>>(c));
-    RDF_KERNEL(S, rdf_group_scatter_kernel<<<2 * S->grid, 256, 0, stream>>>(c));
-    RDF_KERNEL(S, rdf_group_split_kernel<<<S->grid, 256, 0, stream>>>(c, 40u * (uint32_t)c.n_groups));
-    RDF_KERNEL(S, rdf_group_link_kernel<<<4 * S->grid, 256, 0, stream>>>(c));
-    CUDA_OK(cudaGetLastError());
+    uint32_t threshold = 40u * (uint32_t)c.n_groups;
+    void* args[] = {(void*)&c, (void*)&threshold};
+    RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_group_kernel, dim3(2 * S->grid), dim3(256), args, 0, stream)));
     return RDF_OK;
 }
 
