@@ -511,3 +511,10 @@ def test_fp32_wide_wave_tiles():
     p = workloads.treernn_params(3, 70, 132, 132)
     shapes = [workloads.perfect_tree_shape(15)] * 2 + [workloads.random_split_shape(rng, int(L)) for L in rng.integers(1, 40, 21)]
     check_grad({"trees": workloads.tree_batch_from_shapes(shapes, 7, vocab=70), "params": p}, workers=WORKERS)
+
+
+@pytest.mark.parametrize("H,B", [(4, 3), (20, 40), (148, 12), (148, 170)])
+def test_fp32_treelstm_tile_rows(H, B):
+    """Waves of every tile height (64, 32 and 16 rows), hidden sizes and contraction lengths that fill no tile and no step.
+    Tolerance: the file's fp32 bound."""
+    check_forward(_lstm_cfg(B, 300, H), cell="lstm")
