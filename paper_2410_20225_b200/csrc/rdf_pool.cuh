@@ -70,13 +70,16 @@ struct Pool {
     uint16_t* ring;          // [cap] free frames, oldest first
 };
 
-// k consecutive places on a shared counter for every thread that gets here together: one atomic per group
-__device__ __forceinline__ uint32_t pool_take(uint32_t* counter, uint32_t k) {
+// a place on a shared counter for every thread that gets here together: one atomic per group
+__device__ __forceinline__ uint32_t pool_take(uint32_t* counter) {
     const uint32_t group = __activemask(), lane = threadIdx.x & 31u, leader = __ffs(group) - 1;
     uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(counter, k * __popc(group));
-    return __shfl_sync(group, base, leader) + k * __popc(group & ((1u << lane) - 1u));
+    if (lane == leader) base = atomicAdd(counter, (uint32_t)__popc(group));
+    return __shfl_sync(group, base, leader) + __popc(group & ((1u << lane) - 1u));
 }
+
+static const int POOL_RUN_BITS = 6;                     // calls that follow one another: at most POOL_MAX_CODE
+static_assert(POOL_MAX_CODE < (1 << POOL_RUN_BITS), "a run of calls fits the bits of reserve");
 
 struct PoolThread {
     static const int T = POOL_THREADS;
@@ -95,11 +98,27 @@ struct PoolThread {
         set_status(c, code);
         sh.stop = 1;
     }
-    __device__ __forceinline__ void give_back(uint32_t f) { P.ring[wrap(ring_tail + pool_take(&sh.freed[par], 1u))] = (uint16_t)f; }
-    // k frames for calls that follow one another, and their places on the stack (first of each); false: the pool is exhausted
+    __device__ __forceinline__ void give_back(uint32_t f) { P.ring[wrap(ring_tail + pool_take(&sh.freed[par]))] = (uint16_t)f; }
+    // k frames for calls that follow one another, and their places on the stack (first of each); false: the pool is exhausted.
+    // The threads that get here together may make different numbers of calls (branches of a body, different functions): a
+    // prefix sum over the lanes, one ballot per bit of k (k < 2^BITS).
+    template <int BITS>
     __device__ __forceinline__ bool reserve(uint32_t k, uint32_t& frame_at, uint32_t& slot) {
-        frame_at = pool_take(&sh.taken[par], k);
-        slot = pool_take(&sh.entered[par], k);
+        const uint32_t group = __activemask(), lane = threadIdx.x & 31u, leader = __ffs(group) - 1, lower = (1u << lane) - 1u;
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int b = 0; b < BITS; ++b) {
+            const uint32_t m = __ballot_sync(group, (k >> b) & 1u);
+            before += (uint32_t)__popc(m & lower) << b;
+            total += (uint32_t)__popc(m) << b;
+        }
+        uint32_t f0 = 0, s0 = 0;
+        if (lane == leader) {
+            f0 = atomicAdd(&sh.taken[par], total);
+            s0 = atomicAdd(&sh.entered[par], total);
+        }
+        frame_at = __shfl_sync(group, f0, leader) + before;
+        slot = __shfl_sync(group, s0, leader) + before;
         if (frame_at + k <= avail) return true;
         sh.stop = 2;
         return false;
@@ -116,7 +135,7 @@ struct PoolThread {
             return;
         }
         ++matches;
-        const uint32_t at = match0 + pool_take(&sh.matched[par], 1u);
+        const uint32_t at = match0 + pool_take(&sh.matched[par]);
         if (at < z.cap) P.match[at] = (uint16_t)(f | node << 13);
         else sh.stop = 2;                                   // (only bodies with several match nodes can have more matches than frames)
     }
@@ -148,7 +167,7 @@ struct PoolThread {
     }
     __device__ __forceinline__ void tail_call(uint32_t f, uint32_t h, uint32_t label, int64_t a0, int64_t a1, int64_t a2, uint32_t depth, uint32_t wave) {
         fill_frame(f, P.prog->labels[label].n_args, a0, a1, a2, (h & ~(63u << 22)) | depth << 22, wave);
-        P.enter[wrap(enter0 + pool_take(&sh.entered[par], 1u))] = (uint16_t)f;      // (one token per frame: the deque holds all frames)
+        P.enter[wrap(enter0 + pool_take(&sh.entered[par]))] = (uint16_t)f;      // (one token per frame: the deque holds all frames)
     }
     __device__ __forceinline__ static int64_t pick(const PoolOperand& o, int64_t a0, int64_t a1, int64_t a2) {
         return (o.reg == 0 ? a0 : o.reg == 1 ? a1 : o.reg == 2 ? a2 : 0ll) + (int64_t)o.imm;
@@ -166,7 +185,7 @@ struct PoolThread {
         const uint32_t k = act.n_calls;
         uint32_t depth, frame_at, slot;
         invocations += k;
-        if (!push_tag(h, depth) || !reserve(k, frame_at, slot)) return -1;
+        if (!push_tag(h, depth) || !reserve<2>(k, frame_at, slot)) return -1;      // (1 to 3 calls)
 #pragma unroll
         for (uint32_t q = 0; q < 3; ++q)
             if (q < k) {
@@ -270,7 +289,7 @@ struct PoolThread {
                 }
                 if (run_left == 0) {
                     run_left = in.n_run;
-                    if (!reserve(run_left, frame_at, slot)) return;
+                    if (!reserve<POOL_RUN_BITS>(run_left, frame_at, slot)) return;
                 }
                 --run_left;
                 const uint32_t nf = P.ring[wrap(ring0 + frame_at++)];
@@ -381,7 +400,10 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         }
         if (ne + nm == 0) {
             if (!more) break;
-            continue;
+            if (avail > z.cap / 2) continue;
+            if (tid == 0) sh.stop = 2;                       // (no token holds the missing frames: not a state this kernel gets into)
+            __syncthreads();
+            break;
         }
         // ---- this round's tokens: completed matches for the first warps, frames to enter for the others
         const uint32_t width = pool_width(z, avail);

@@ -639,3 +639,52 @@ def test_recursion_deeper_than_a_pool():
     y, _ = g.eval_int(torch.tensor(xs, dtype=torch.int64, device="cuda"), max_invocations=sum(xs) + len(xs))
     assert y.tolist() == [v * (v + 1) // 2 for v in xs]
     assert g.stats()["invocations"] == sum(xs) + len(xs) and g.stats()["waves"] >= 20000
+
+
+def _mixed_counts(kind):
+    """Bodies whose branches make different numbers of calls: threads of one warp then reserve different numbers of frames."""
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f = rdf.Function("f", 1)
+    n = f.param()
+    call = lambda fn, g, d: fn.call(g, fn.sub(fn.param(), fn.const(d)))  # noqa: E731
+    small = f.lt(n, f.const(2))
+    if kind == "0-1-2":
+        one, two = f.add(call(f, 1, 1), f.const(1)), f.add(call(f, 1, 1), call(f, 1, 2))
+        f.ret(f.if_(small, f.const(1), f.if_(f.lt(n, f.const(6)), one, two)))
+        return [r, f]
+    if kind == "0-1-2-3":                         # more conditions than the fixed shapes take: the interpreter's runs of calls
+        c1, c2, c3 = f.const(1), f.const(2), f.const(3)
+        rest = f.rem(n, c3)
+        c = [f.call(1, f.sub(n, k)) for k in (c1, c2, c3)]
+        three = f.if_(f.lt(rest, c2), f.sub(c[0], c[1]), f.add(f.max(c[0], c[1]), c[2]))
+        f.ret(f.if_(f.lt(n, c2), n, f.if_(f.lt(rest, c1), f.add(c[0], f.const(1)), three)))
+        return [r, f]
+    if kind == "1-3":
+        three = f.add(f.max(call(f, 1, 2), call(f, 1, 3)), call(f, 1, 4))
+        f.ret(f.if_(small, n, f.if_(f.eq(f.rem(n, f.const(2)), f.const(0)), three, f.add(call(f, 1, 1), f.const(3)))))
+        return [r, f]
+    g = rdf.Function("g", 1)                      # mutual: f makes two calls, g three or one, h one
+    m = g.param()
+    h = rdf.Function("h", 1)
+    h.ret(h.add(call(h, 1, 1), h.const(7)))
+    f.ret(f.if_(small, n, f.add(call(f, 2, 1), call(f, 3, 2))))
+    g.ret(g.if_(g.lt(m, g.const(3)), g.const(2),
+                g.if_(g.lt(m, g.const(6)), call(g, 1, 1), g.sub(g.add(call(g, 1, 1), call(g, 2, 2)), call(g, 3, 3)))))
+    return [r, f, g, h]
+
+
+@pytest.mark.parametrize("mode", [rdf.TAGS_PATH, rdf.TAGS_FRAME])
+@pytest.mark.parametrize("kind", ["0-1-2", "0-1-2-3", "1-3", "mutual"])
+def test_pool_executor_branches_with_different_numbers_of_calls(kind, mode):
+    """Values and numbers of calls of programs whose branches (or functions) make one, two or three calls, at one block's
+    batch and at many chunks per block."""
+    fs = _mixed_counts(kind)
+    want = [_evaluate(fs, v) for v in range(12)]
+    g = rdf.Graph(fs, 0, mode)
+    for B in (1, 37, 1000, 30000):
+        x_host = np.random.default_rng(B).integers(0, 12, size=B)
+        calls = int(sum(want[v][1] for v in x_host))
+        y, _ = g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=calls)
+        assert y.tolist() == [want[v][0] for v in x_host], (kind, B)
+        assert g.stats()["invocations"] == calls, (kind, B)
