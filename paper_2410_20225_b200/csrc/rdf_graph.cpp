@@ -671,6 +671,7 @@ struct Lower {
             kseg = cont_segment(K);
         }
         g->labels.push_back(L);
+        g->label_caller.push_back(cur_func);
         label_entry_seg.push_back(entry_seg[callee]);
         label_kseg.push_back(kseg);
         return (int)g->labels.size() - 1;
@@ -1397,11 +1398,15 @@ struct PoolBuilder {
             const int w = word0 + M.port_base;
             out.match[k] = PoolMatch{(int16_t)new_pc[M.cont_pc], (uint8_t)M.n_ports, (uint8_t)w, ((1u << M.n_ports) - 1u) << w};
         }
-        // most frames one segment takes (over its branches: an upper bound)
+        // most frames one segment takes (over its branches: an upper bound; a tail call to the caller's own function keeps
+        // its frame, one to another function takes a new one)
         for (size_t k = 0; k + 1 < seg.size(); ++k) {
             const int end = seg[k + 1] < n ? new_pc[seg[k + 1]] : out.n_code;
             int calls = 0;
-            for (int i = new_pc[seg[k]]; i < end; ++i) calls += out.code[i].op == PI_CALL && !out.code[i].tail;
+            for (int i = new_pc[seg[k]]; i < end; ++i) {
+                const PoolInstr& in = out.code[i];
+                if (in.op == PI_CALL) calls += !in.tail || g->labels[in.imm].callee != g->label_caller[in.imm];
+            }
             int& most = entries.count(seg[k]) ? out.calls_entry : out.calls_cont;
             most = std::max(most, calls);
         }

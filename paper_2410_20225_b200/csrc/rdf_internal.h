@@ -153,6 +153,7 @@ struct rdf_graph {
     std::vector<LabelInfo> labels;
     std::vector<int64_t> consts;
     std::vector<int32_t> label_callee, label_local;   // the same two fields of `labels`, as plain arrays for rdf_graph_describe
+    std::vector<int32_t> label_caller;                // per label: the function whose body makes the call
     int32_t result_entry_pc = 0;
     int32_t n_ports_total = 0;
     int32_t max_calls_per_body = 1;

@@ -688,3 +688,32 @@ def test_pool_executor_branches_with_different_numbers_of_calls(kind, mode):
         y, _ = g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=calls)
         assert y.tolist() == [want[v][0] for v in x_host], (kind, B)
         assert g.stats()["invocations"] == calls, (kind, B)
+
+
+def _tail_to_another():
+    """f(n) = n < 1 ? 1 : g(f(n-1) + f(n-1)), g(m) = m + 1: a completed match calls another function, which takes a frame."""
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f = rdf.Function("f", 1)
+    n = f.param()
+    m = f.sub(n, f.const(1))
+    f.ret(f.if_(f.lt(n, f.const(1)), f.const(1), f.call(2, f.add(f.call(1, m), f.call(1, m)))))
+    g = rdf.Function("g", 1)
+    g.ret(g.add(g.param(), g.const(1)))
+    return [r, f, g]
+
+
+@pytest.mark.parametrize("mode", [rdf.TAGS_PATH, rdf.TAGS_FRAME])
+@pytest.mark.parametrize("B,n_hi", [(60000, 12), (3000, 12), (1, 12)])
+def test_pool_executor_tail_calls_of_another_function(B, n_hi, mode):
+    """Full binary recursions fill the pools to their last frames while matches complete that need frames themselves: every
+    result is written (a pool with path tags has no other executor behind it)."""
+    fs = _tail_to_another()
+    want = [_evaluate(fs, v) for v in range(n_hi + 1)]
+    g = rdf.Graph(fs, 0, mode)
+    x_host = np.random.default_rng(2).integers(0 if B > 1 else n_hi, n_hi + 1, size=B)
+    calls = int(sum(want[v][1] for v in x_host))
+    y = torch.full((B,), -1, dtype=torch.int64, device="cuda")
+    g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=calls, y=y)
+    assert y.tolist() == [want[v][0] for v in x_host]
+    assert g.stats()["invocations"] == calls
