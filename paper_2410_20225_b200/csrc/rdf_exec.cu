@@ -1639,7 +1639,7 @@ static uint32_t pool_frames(const PoolProgram& P, const ExecState* S) {
     return smem <= fixed ? 0u : (uint32_t)std::min<size_t>((smem - fixed) / pool_frame_bytes(P), POOL_MAX_FRAMES) & ~7u;
 }
 // The pool executor: how many frames a block has, and how the instances are dealt out.
-static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, cudaStream_t stream) {
+static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, bool fallback, cudaStream_t stream) {
     const PoolProgram& P = g->pool_prog;
     const size_t smem = pool_smem_bytes(S);
     PoolSizes z{};
@@ -1656,6 +1656,7 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     z.refill = POOL_THREADS / 3;
     z.max_calls = (unsigned long long)in->max_invocations;
     z.max_parked = (unsigned long long)L.table_cap * std::max<size_t>(1, g->match.size());
+    z.fallback = fallback;
     rdf_mark(S, 1, stream);
     CUDA_OK(cudaFuncSetAttribute(rdf_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RDF_KERNEL(S, rdf_pool_kernel<<<grid, POOL_THREADS, smem, stream>>>(c, P, z));
@@ -1684,9 +1685,11 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                       (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B) &&
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);
     if (pool) {
-        const int rc = rdf_launch_pool(g, in, L, S, c, stream);
+        // bounded depth, one match per frame: a pool always suffices (should it not, the call ends with a status)
+        const bool fallback = !(g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1);
+        const int rc = rdf_launch_pool(g, in, L, S, c, fallback, stream);
         if (rc != RDF_OK) return rc;
-        if (g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1) {      // bounded depth, one match per frame: a pool always suffices
+        if (!fallback) {
             for (int k = 2; k <= 5; ++k) rdf_mark(S, k, stream);
             S->last_ctl = c.ctl;
             S->last_stream = stream;

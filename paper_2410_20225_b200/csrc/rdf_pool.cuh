@@ -43,6 +43,7 @@ struct PoolSizes {
     uint32_t max_depth;      // path tags: labels that fit the packed tag; frame tags: no limit (0xFFFFFFFF)
     unsigned long long max_calls;   // frame tags: Call firings the caller allows
     unsigned long long max_parked;  // path tags: operands the token store of the call holds
+    int      fallback;       // the general scheduler is launched behind this kernel for a pool that is exhausted
 };
 
 struct PoolShared {
@@ -453,7 +454,9 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         __threadfence();
         volatile Control* k = c.ctl;
         k->tokens = k->invocations + (unsigned long long)c.B;
-        if (!k->pool_exhausted) {
+        if (k->pool_exhausted) {
+            if (!z.fallback) set_status(c, RDF_ERR_QUEUE_FULL);
+        } else {
             if (c.tag_mode == RDF_TAGS_FRAME && k->invocations > z.max_calls) set_status(c, RDF_ERR_FRAMES_FULL);
             if (c.tag_mode == RDF_TAGS_PATH && k->store_inserts > z.max_parked) set_status(c, RDF_ERR_STORE_FULL);
         }
