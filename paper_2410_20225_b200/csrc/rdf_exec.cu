@@ -433,6 +433,7 @@ __device__ void rnn_cell_tiles_wide(const DevCtx& c, float* sm, const WideTiles&
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        cp_async_wait<0>();                                                // (nor written: its zeros beyond the last step have landed)
         __syncthreads();                                                   // (the stages of the tile before are no longer read)
         if (threadIdx.x == 0) *s_next = wt.take();
         fetch(0);

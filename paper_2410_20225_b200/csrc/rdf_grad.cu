@@ -1019,6 +1019,7 @@ __device__ void backward_operand_tiles_wide(const DevCtx& c, float* sm, const Wi
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+        cp_async_wait<0>();                                                // (nor written: its zeros beyond the last step have landed)
         __syncthreads();                                                   // (the stages of the tile before are no longer read)
         if (threadIdx.x == 0) *s_next = wt.take();
         fetch(0);

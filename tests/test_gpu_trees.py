@@ -518,3 +518,12 @@ def test_fp32_treelstm_tile_rows(H, B):
     """Waves of every tile height (64, 32 and 16 rows), hidden sizes and contraction lengths that fill no tile and no step.
     Tolerance: the file's fp32 bound."""
     check_forward(_lstm_cfg(B, 300, H), cell="lstm")
+
+
+@pytest.mark.parametrize("H", [68, 256])
+def test_fp32_wide_tiles_one_after_another(H):
+    """More wide tiles in a wave than thread blocks, so that a block starts tile after tile in the same stages, with contraction
+    lengths that end in the middle of a step (H = 68) and of the ring (H = 256: 32 steps forward, 16 back, three stages)."""
+    p = workloads.treernn_params(3, 70, H, H)
+    shapes = [workloads.perfect_tree_shape(16)] * 2
+    check_grad({"trees": workloads.tree_batch_from_shapes(shapes, 7, vocab=70), "params": p}, workers=WORKERS)
