@@ -811,7 +811,12 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
     auto barrier = [&]() {
         if (!CLUSTER) return grid_barrier(c, &c.ctl->bar.v, generation);
         cluster_sync_all();                                         // (blocks that have left count as arrived)
-        return ld_volatile_i32(&c.ctl->status) == 0;
+        // one read per block: a faster block may be in the next phase already and set an error there, and a block goes on or
+        // leaves as a whole
+        __shared__ int good;
+        if (threadIdx.x == 0) good = ld_volatile_i32(&c.ctl->status) == 0;
+        __syncthreads();
+        return good != 0;
     };
     for (;; ++wave) {
         const uint32_t n = ld_volatile_u32(&c.ctl->qcount[wave % 3].v);

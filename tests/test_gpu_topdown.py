@@ -142,3 +142,31 @@ def test_topdown_hidden_sizes(H, D, B):
     to weights read through the cache; groups of one and of several warps along the items; one
     cluster (B (H + 16) < 15500) and the whole grid."""
     test_topdown_recursion_states_and_shapes(H, D, B)
+
+
+def test_topdown_errors_in_one_cluster():
+    """Calls that one thread-block cluster runs (small batches) and that end with a status in any of their waves -- the frame
+    table full after each of many different numbers of invocations, a token that is no row of the table: every block leaves, and
+    the next call has the states of an undisturbed one."""
+    V, H, D, B = 50, 32, 7, 24
+    P = workloads.topdown_params(7, V, H)
+    P["b_s"][0] = -100.0                          # full trees
+    tb = workloads.topdown_batch(7, B, V)
+    total = B * (1 + (2 ** (D + 1) - 1) + (2 ** (D + 1) - 2))
+    g = rdf.Graph(*rdf.topdown_program(D), rdf.TAGS_FRAME)
+    dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(P)
+    want = g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0]
+    bad = dict(dt, tok=dt["tok"].clone())
+    bad["tok"][B // 2] = V
+
+    def code(trees, max_invocations):
+        try:
+            g.eval_trees(trees, dp, rdf.F32, max_invocations=max_invocations)
+        except rdf.RdfError as e:
+            return e.code
+        return 0
+
+    for m in [B, B + 1, 3 * B] + list(range(5 * B, total, 311)) + [total - 1]:
+        assert code(dt, m) == -6, m
+    assert code(bad, total) == -2
+    assert torch.equal(g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0], want)
