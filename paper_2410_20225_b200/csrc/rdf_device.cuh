@@ -91,6 +91,7 @@ struct Control {
     float    loss;
     int32_t  forward_status;      // status word at the end of the forward pass and the loss head
     uint32_t next_chunk, blocks_done, pool_exhausted;   // rdf_pool.cuh
+    uint4    il_state[2];         // interleaved execution: where the grid carries on after a cluster ({wave, cells, left, right done}, {leaves done, widest})
     uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
 };
 static_assert(sizeof(Control) <= 4096, "the control block is 4 KB");

@@ -726,11 +726,18 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
 // whole kernel up to H = IL_SMEM_W_H; wider ones are read through L1.  The terms of a sum are added in index order (a Switch
 // decides on the sign of a sum over the state: another order could flip it).
 static const int IL_SMEM_W_H = 128;
-// One cluster of 8 blocks runs a call while instances x (H + 16) stay below this.  Besides its faster barrier, the acquire of a
-// grid barrier drops the block's local memory (spilled registers, label arrays) from L1 twice per wave.  Grid -> cluster, depth 10:
-// 8 instances, H = 16: 0.450 -> 0.289 ms; 64, H = 128: 0.852 -> 0.759; 400, H = 16: 0.603 -> 0.497; 100, H = 128: 0.856 -> 0.809;
-// 200, H = 64: 0.699 -> 0.795.
-static const long long IL_CLUSTER_WORK = 15500;
+// One cluster of 8 blocks runs the waves of a call while they are narrow: up to IL_CLUSTER_TOKENS tokens, and tokens x H x H
+// up to IL_CLUSTER_FMA.  How wide the waves get is up to the values (the gate) and the depth limit, so the kernel looks at each
+// wave and leaves the rest of the call to the grid at the first one that is wider.  Besides its faster barrier, the acquire of a
+// grid barrier drops the block's local memory (spilled registers, label arrays) from L1 twice per wave.
+// Grid alone / this / cluster alone, us: 8 seeds, H = 16, depth 10: 523 / 335 / 327; 100, H = 128: 862 / 846 / 915; 20, H = 256,
+// depth 8: 1806 / 1580 / 1586; 64 full trees, H = 128, depth 10: 1031 / 1016 / 7660; 64, H = 128, depth 18: 1636 / 1620 / 2990.
+// The limit on tokens x H x H at 2^23 instead: 100, H = 128: 826, but 20, H = 256: 1687; at 2^25: 927 and 1588.
+static const uint32_t IL_CLUSTER_TOKENS = 8192;
+static const unsigned long long IL_CLUSTER_FMA = 16ull << 20;
+__host__ __device__ inline bool il_narrow(unsigned long long tokens, int H) {
+    return tokens <= IL_CLUSTER_TOKENS && tokens * (unsigned long long)(H * H) <= IL_CLUSTER_FMA;
+}
 __host__ __device__ inline int il_stride(int K) { return K + (K % 8 == 0 ? 4 : 8); }
 __host__ __device__ inline int il_out_warps(int H) { return H < 128 ? (H + 15) / 16 : 8; }
 __host__ __device__ inline int il_group_max(int H) { return 32 / il_out_warps(H) * 16; }         // items that the 32 warps cover
@@ -782,14 +789,17 @@ __device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int s
 // What bounds it: the FMA and load issue of the wide waves and the latency of the narrow ones.  8192 seeds, H = 128, 44
 // waves: groups of 32 with the kinds mixed (unary operators as cells with a zero half) and tokens on the first blocks only
 // 4.24 ms, this 1.86 ms (operators 2.9 -> 1.25, tokens 1.0 -> 0.33).
-// CLUSTER: the whole grid is one cluster, whose barrier takes a fifth of the time of the grid barrier (see IL_CLUSTER_WORK).
+// CLUSTER: the whole grid is one cluster, whose barrier takes a fifth of the time of the grid barrier; it leaves at the first wave
+// that is not il_narrow, and the form for the whole grid, launched behind it, carries on from the queues.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
     extern __shared__ __align__(16) unsigned char il_smem[];
+    const uint4 from = c.ctl->il_state[0], from2 = c.ctl->il_state[1];         // (zeros unless a cluster has run waves of this call)
+    if (!CLUSTER && (c.ctl->status != 0 || c.ctl->qcount[from.x % 3u].v == 0u)) return;
     load_program(c, sp);
     ThreadStats st;
-    uint32_t generation = 0, wave = 0, widest = 0, done[3] = {0u, 0u, 0u}, done_leaves = 0;      // cells, left, right unary operators
+    uint32_t generation = 0, wave = from.x, widest = from2.y, done[3] = {from.y, from.z, from.w}, done_leaves = from2.x;   // cells, left, right unary operators
     long long cyc_s = 0, cyc_o = 0, cyc_b = 0, t_mark = clock64();
     auto lap = [&](long long& acc) {
         const long long now = clock64();
@@ -808,15 +818,17 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         }
     const int out_warps = il_out_warps(H), iw = warp / out_warps, jw = warp % out_warps;
     const uint32_t gwarp = warp * gridDim.x + blockIdx.x, n_warps = gridDim.x * (blockDim.x / 32);      // (consecutive warps on different SMs)
-    auto barrier = [&]() {
+    auto barrier = [&](bool look) {
         if (!CLUSTER) return grid_barrier(c, &c.ctl->bar.v, generation);
         cluster_sync_all();                                         // (blocks that have left count as arrived)
         // one read per block: a faster block may be in the next phase already and set an error there, and a block goes on or
         // leaves as a whole
         __shared__ int good;
-        if (threadIdx.x == 0) good = ld_volatile_i32(&c.ctl->status) == 0;
-        __syncthreads();
-        return good != 0;
+        if (look) {
+            if (threadIdx.x == 0) good = ld_volatile_i32(&c.ctl->status) == 0;
+            __syncthreads();
+        }
+        return !look || good != 0;
     };
     for (;; ++wave) {
         const uint32_t n = ld_volatile_u32(&c.ctl->qcount[wave % 3].v);
@@ -825,13 +837,14 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
             set_status(c, RDF_ERR_WAVE_LIMIT);
             break;
         }
+        if (CLUSTER && !il_narrow(n, H)) break;
         widest = max(widest, n);
         if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl->qcount[(wave + 2) % 3].v = 0;
         const Token* q = c.q[wave & 1];
         for (uint32_t i = gwarp * 32u + lane; i < n; i += n_warps * 32u) run_token(c, sp, nullptr, wave, load_token(&q[i]), st);
         __syncthreads();
         lap(cyc_s);
-        if (!barrier()) break;
+        if (!barrier(true)) break;
         lap(cyc_b);
         // ---- the operators this wave queued
         const uint32_t n_leaf = min(ld_volatile_u32(&c.ctl->leaf_count.v), c.work_cap);
@@ -890,14 +903,18 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         for (int q2 = 0; q2 < 3; ++q2) done[q2] = end[q2];
         __syncthreads();
         lap(cyc_o);
-        if (!barrier()) break;
+        if (!barrier(false)) break;        // (an operator's error is seen after the next tokens: its row is merely wrong)
         lap(cyc_b);
     }
     flush_stats(c, st);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         c.ctl->waves = wave;
         c.ctl->max_wave_tokens = widest;
-        c.ctl->cyc[0] = cyc_s; c.ctl->cyc[1] = cyc_o; c.ctl->cyc[2] = cyc_b;
+        c.ctl->cyc[0] += cyc_s; c.ctl->cyc[1] += cyc_o; c.ctl->cyc[2] += cyc_b;
+        if (CLUSTER) {
+            c.ctl->il_state[0] = make_uint4(wave, done[0], done[1], done[2]);
+            c.ctl->il_state[1] = make_uint4(done_leaves, widest, 0u, 0u);
+        }
         c.ctl->forward_status = c.ctl->status;
     }
 }
@@ -1758,13 +1775,13 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_fold_kernel, dim3(blocks), dim3(FS_CHUNK), args, 0, stream)));
     } else if (g->interleaved)
     {
-        if (S->il_cluster && in->B * (c.H + 16ll) < IL_CLUSTER_WORK) {
+        if (S->il_cluster && il_narrow((unsigned long long)in->B, c.H)) {
             cudaLaunchAttribute at[1];
             const cudaLaunchConfig_t cfg = il_cluster_config(at, (size_t)interleaved_smem_bytes(c.H), stream);
             RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_interleaved_kernel<true>, c)));
-        } else
-            RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel<false>, dim3(S->grid), dim3(1024), args,
-                                                (size_t)interleaved_smem_bytes(c.H), stream)));
+        }
+        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel<false>, dim3(S->grid), dim3(1024), args,
+                                            (size_t)interleaved_smem_bytes(c.H), stream)));
     } else
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_scheduler_kernel, dim3(S->grid), dim3(1024), args,
                                             2 * LQ_CAP * sizeof(Token), stream)));

@@ -170,3 +170,45 @@ def test_topdown_errors_in_one_cluster():
         assert code(dt, m) == -6, m
     assert code(bad, total) == -2
     assert torch.equal(g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0], want)
+
+
+def _full_trees(B, D, H, V=50):
+    P = workloads.topdown_params(7, V, H)
+    P["b_s"][0] = -100.0                          # the gate never stops: 2^d expansions per seed at depth d
+    g = rdf.Graph(*rdf.topdown_program(D), rdf.TAGS_FRAME)
+    tb = workloads.topdown_batch(7, B, V)
+    total = B * (1 + (2 ** (D + 1) - 1) + (2 ** (D + 1) - 2))
+    return g, P, tb, total
+
+
+@pytest.mark.parametrize("B,D,H", [(1, 9, 128), (3, 12, 16), (8, 9, 100), (40, 6, 256), (1, 1, 4)])
+def test_topdown_waves_that_outgrow_a_cluster(B, D, H):
+    """A call that starts in one thread-block cluster and is handed to the whole grid at its first wide wave (tokens x H x H
+    beyond 2^24, or more than 8192 tokens), and one that never gets there: states, invocations and waves."""
+    g, P, tb, total = _full_trees(B, D, H)
+    want = np.array([direct.topdown(P, int(t), D, {}) for t in tb.tok[:B]])
+    dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(P)
+    for _ in range(2):
+        h = g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0].cpu().numpy()
+        st = g.stats()
+        assert st["invocations"] == total and st["waves"] == 4 * (D + 1)
+        assert np.abs(h - want).max() / np.abs(want).max() <= TOL
+
+
+def test_topdown_wide_waves_of_few_seeds_use_the_device():
+    """64 seeds that grow full trees (waves of 65 536 tokens) take no longer than 512 of them."""
+    ms = []
+    for B in (64, 512):
+        g, P, tb, total = _full_trees(B, 10, 128)
+        dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(P)
+        for _ in range(3):
+            g.eval_trees(dt, dp, rdf.F32, check=False, max_invocations=total)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        e[0].record()
+        for _ in range(5):
+            g.eval_trees(dt, dp, rdf.F32, check=False, max_invocations=total)
+        e[1].record()
+        torch.cuda.synchronize()
+        g.stats()
+        ms.append(e[0].elapsed_time(e[1]) / 5)
+    assert ms[0] < ms[1], ms
