@@ -249,19 +249,22 @@ typedef struct {
     int32_t  status;             /* RDF_OK or the first RDF_ERR_* the device recorded */
     uint32_t waves;              /* scheduler waves run (forward) */
     uint32_t waves_backward;
-    uint32_t max_wave_tokens;    /* widest wave */
+    uint32_t max_wave_tokens;    /* widest wave (integer programs that run out of shared memory: an upper bound when the call has
+                                    more than 65 792 waves) */
     uint64_t invocations;        /* Call firings */
     uint64_t tokens;             /* tokens taken from the wave queues */
     uint64_t store_inserts;      /* operands parked in the token store */
     uint64_t store_matches;      /* firings completed by a match */
-    uint64_t store_probes;       /* hash slots inspected (PATH mode) */
-    uint32_t max_probe;          /* longest probe sequence */
+    uint64_t store_probes;       /* hash slots inspected (PATH mode; 0 for a call that ran out of shared memory, where an
+                                    operand has its place in the frame of its invocation) */
+    uint32_t max_probe;          /* longest probe sequence (likewise) */
     uint32_t max_depth;          /* deepest tag (PATH mode) */
     uint64_t cells;              /* batched cell firings */
     uint64_t leaves;             /* batched leaf firings */
     /* SM clock cycles spent by thread block 0.  Forward: token scheduling (scheduler kernel), batched
        operators (operator kernel), waiting at grid barriers (both).  Gradient kernel: per-invocation
-       work, batched operand gradients, waiting at grid barriers. */
+       work, batched operand gradients, waiting at grid barriers.  (Integer programs that run out of shared memory have no
+       grid barriers: all of block 0's time is cycles_schedule.) */
     uint64_t cycles_schedule, cycles_batch, cycles_barrier;
     uint64_t cycles_bwd_frames, cycles_bwd_batch, cycles_bwd_barrier;
     uint32_t kernel_launches;    /* kernels of the library that the last call launched (host count; memsets and copies excluded) */

@@ -64,6 +64,7 @@ struct alignas(128) HotCounter {
     uint32_t v;
 };
 
+static const int POOL_BINS = 256;             // pool executor: waves whose tokens are counted in shared memory
 // Counters and control words, one 4 KB block at the start of the workspace.
 struct Control {
     HotCounter qcount[3];         // tokens in the queue of wave w at [w % 3]
@@ -91,6 +92,7 @@ struct Control {
     float    loss;
     int32_t  forward_status;      // status word at the end of the forward pass and the loss head
     uint32_t next_chunk, blocks_done, pool_exhausted;   // rdf_pool.cuh
+    uint32_t wave_tokens[POOL_BINS];                    // tokens per wave of the call
     uint4    il_state[2];         // interleaved execution: where the grid carries on after a cluster ({wave, cells, left, right done}, {leaves done, widest})
     uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
 };

@@ -1656,7 +1656,7 @@ int rdf_check_common(rdf_graph* g, const rdf_batch* in, const rdf_params* params
     return RDF_OK;
 }
 
-static size_t pool_smem_bytes(const ExecState* S) { return std::min<size_t>(S->smem_per_sm / POOL_PER_SM - 2048, S->smem_per_block - 1024); }
+static size_t pool_smem_bytes(const ExecState* S) { return std::min<size_t>(S->smem_per_sm / POOL_PER_SM - 1024, S->smem_per_block) - sizeof(PoolShared) - 256; }
 static uint32_t pool_frames(const PoolProgram& P, const ExecState* S) {
     const size_t fixed = pool_fixed_bytes(P), smem = pool_smem_bytes(S);
     return smem <= fixed ? 0u : (uint32_t)std::min<size_t>((smem - fixed) / pool_frame_bytes(P), POOL_MAX_FRAMES) & ~7u;
@@ -1680,6 +1680,13 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     z.max_calls = (unsigned long long)in->max_invocations;
     z.max_parked = (unsigned long long)L.table_cap * std::max<size_t>(1, g->match.size());
     z.fallback = fallback;
+    z.n_match = (uint32_t)std::max(1, P.n_match);
+    z.match_step = pool_tokens_share(P) ? -1 : 1;
+    // Tokens per wave from POOL_BINS on are counted in the queue that this executor does not use; with path tags and no call
+    // that waits for another one a wave is a call depth, and there are not that many.
+    const bool few_waves = in->max_invocations < POOL_BINS || (g->tag_mode == RDF_TAGS_PATH && !P.late_calls);
+    z.late_waves = few_waves ? 0u : (uint32_t)std::min<long long>(std::min<long long>(in->max_invocations, 65536), (long long)L.qcap * (long long)(sizeof(Token) / 4));
+    if (z.late_waves) CUDA_OK(cudaMemsetAsync(c.q[0], 0, (size_t)z.late_waves * sizeof(uint32_t), stream));
     rdf_mark(S, 1, stream);
     CUDA_OK(cudaFuncSetAttribute(rdf_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RDF_KERNEL(S, rdf_pool_kernel<<<grid, POOL_THREADS, smem, stream>>>(c, P, z));
@@ -1691,6 +1698,7 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
 // of fib(18) (8361 calls) takes 0.10 ms in a pool and 0.22 in waves, fib(22) (57 313) 0.36 and 0.30, fib(24) (150 049) 0.87
 // and 0.34, eight of fib(22) 0.36 and 0.34; but 32 of fib(24) 0.90 and 1.58.
 static const long long POOL_CALLS = 40000, POOL_MANY = 32;
+static const uint32_t POOL_MIN_FRAMES = 15 * POOL_THREADS / 4;   // (bodies of up to three operators with two operands each)
 
 // zero what must start at zero, upload the program, seed, run all waves
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,
@@ -1703,7 +1711,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     const bool fold = g->fold && !out->trace;
     // Integer programs run out of shared memory.  The general scheduler has what that executor does not: trace records, a
     // bound on the width of a wave, the waits and waves that rdf_set_limits limits, and the cooperative probes.
-    const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= 4u * POOL_THREADS && S->wait_cycles == 0 &&
+    const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= POOL_MIN_FRAMES && S->wait_cycles == 0 &&
                       S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
                       (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B) &&
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);

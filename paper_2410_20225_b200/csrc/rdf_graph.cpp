@@ -1396,7 +1396,7 @@ struct PoolBuilder {
         for (int k = 0; k < out.n_match; ++k) {
             const MatchNode& M = g->match[k];
             const int w = word0 + M.port_base;
-            out.match[k] = PoolMatch{(int16_t)new_pc[M.cont_pc], (uint8_t)M.n_ports, (uint8_t)w, ((1u << M.n_ports) - 1u) << w};
+            out.match[k] = PoolMatch{(int16_t)new_pc[M.cont_pc], (uint8_t)M.n_ports, (uint8_t)w, (1u << M.n_ports) - 1u};
         }
         // most frames one segment takes (over its branches: an upper bound; a tail call to the caller's own function keeps
         // its frame, one to another function takes a new one)
@@ -1405,6 +1405,7 @@ struct PoolBuilder {
             int calls = 0;
             for (int i = new_pc[seg[k]]; i < end; ++i) {
                 const PoolInstr& in = out.code[i];
+                if (in.op == PI_CALL && !entries.count(seg[k])) out.late_calls = 1;
                 if (in.op == PI_CALL) calls += !in.tail || g->labels[in.imm].callee != g->label_caller[in.imm];
             }
             int& most = entries.count(seg[k]) ? out.calls_entry : out.calls_cont;

@@ -107,7 +107,7 @@ struct alignas(16) PoolLabel {
 struct PoolMatch {
     int16_t  cont;
     uint8_t  n_ports, word0;         // its ports are words word0 .. of the frame
-    uint32_t all;                    // bits of its ports
+    uint32_t all;                    // a bit per port
 };
 // Common shapes of a segment, run without the interpreter, everything in registers (operand registers 0 .. 2: the arguments
 // or the operands of the match; 3: zero).
@@ -135,6 +135,7 @@ struct alignas(16) PoolProgram {
     int32_t   n_code, n_labels, n_match, result_entry;
     int32_t   words, n_regs;         // 64-bit words per frame, registers per thread
     int32_t   calls_entry, calls_cont;   // most frames taken by a segment that enters a function / that carries on after a match
+    int32_t   late_calls, pad[3];        // some call waits for another one
     PoolInstr code[POOL_MAX_CODE];
     PoolLabel labels[POOL_MAX_LABELS];
     PoolMatch match[POOL_MAX_MATCH];

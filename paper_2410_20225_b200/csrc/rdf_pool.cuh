@@ -43,6 +43,9 @@ struct PoolSizes {
     uint32_t max_depth;      // path tags: labels that fit the packed tag; frame tags: no limit (0xFFFFFFFF)
     unsigned long long max_calls;   // frame tags: Call firings the caller allows
     unsigned long long max_parked;  // path tags: operands the token store of the call holds
+    uint32_t n_match;        // match nodes, at least 1
+    int      match_step;     // -1, 1: direction in which Pool::match grows
+    uint32_t late_waves;     // PoolThread::n_late
     int      fallback;       // the general scheduler is launched behind this kernel for a pool that is exhausted
 };
 
@@ -52,11 +55,15 @@ struct PoolShared {
     uint32_t taken[2];       // frames taken in the round
     uint32_t freed[2];       // frames given back in the round
     uint32_t next_chunk;
+    uint32_t waves[POOL_BINS];   // tokens per wave (of the block), the first POOL_BINS waves
     int      stop;           // 1: an error, 2: the pool is exhausted
 };
 
 inline size_t pool_fixed_bytes(const PoolProgram& P) { return sizeof(PoolProgram) + (size_t)(P.n_regs + 1) * POOL_THREADS * 8; }
-inline size_t pool_frame_bytes(const PoolProgram& P) { return 8 * (size_t)P.words + 4 + 4 + 2 + 2 + 2; }
+inline bool pool_tokens_share(const PoolProgram& P) { return P.n_match <= 1; }       // one token per frame at most: Pool::match
+inline size_t pool_frame_bytes(const PoolProgram& P) {
+    return 8 * (size_t)P.words + 4 + 4 * (size_t)std::max(1, P.n_match) + 2 + 2 + (pool_tokens_share(P) ? 0 : 2);
+}
 static const uint32_t POOL_MAX_FRAMES = 1u << 13;       // a completed match: frame | node << 13
 
 // The pool's arrays in dynamic shared memory
@@ -65,9 +72,11 @@ struct Pool {
     int64_t*  regs;          // [n_regs + 1][T]; the last one is zero
     int64_t*  words;         // [words][cap]: arguments while the frame waits to be entered, then the operands of its match nodes
     uint32_t* head;          // [cap] frame word
-    uint32_t* state;         // [cap] waiting to be entered: calls above it; then the operands that have arrived
+    uint32_t* state;         // [n_match][cap] waiting to be entered (the first row): its wave; then per match node the operands that
+                             // have arrived [7:0] and the latest wave one of them arrived in [31:8]
     uint16_t* enter;         // [cap] frames to enter, oldest first (a deque)
-    uint16_t* match;         // [cap] stack of completed matches
+    uint16_t* match;         // stack of completed matches; one match node (a frame has one token then): it grows down from the end of
+                             // `enter`, more of them: an array of its own
     uint16_t* ring;          // [cap] free frames, oldest first
 };
 
@@ -90,7 +99,9 @@ struct PoolThread {
     PoolShared& sh;
     uint32_t tid;
     uint32_t ring0, avail, ring_tail, enter0, match0, par;  // this round: first free frame, free frames, where frames go back, tops of the stacks
-    uint32_t invocations = 0, inserts = 0, matches = 0, max_depth = 0, max_wave = 0;
+    uint32_t invocations = 0, inserts = 0, matches = 0, max_depth = 0, max_wave = 0;     // (max_wave: from POOL_BINS on)
+    uint32_t* late_waves;    // tokens per wave from POOL_BINS on (global memory, n_late of them; later ones count in the last)
+    uint32_t n_late;
 
     __device__ __forceinline__ int64_t val(uint32_t reg, int32_t imm) const { return P.regs[reg * T + tid] + (int64_t)imm; }
     __device__ __forceinline__ void set(uint32_t reg, int64_t v) { P.regs[reg * T + tid] = v; }
@@ -125,19 +136,58 @@ struct PoolThread {
         return false;
     }
 
+    // Waves.  The pool does not run in waves, but a token has one all the same -- that of the token that made its call, plus
+    // one; a match fires in the latest wave one of its operands arrived in -- and what the general scheduler reports of its
+    // waves (their number, the widest one) and refuses because of them is the same here.
+    // A token of wave `wave` is taken.  (There are at most 2^24 waves: 24 bits wherever a wave is kept.)
+    __device__ __forceinline__ bool count_wave(uint32_t wave) {
+        if (wave < (uint32_t)POOL_BINS) {
+            atomicAdd(&sh.waves[wave], 1u);
+            return true;
+        }
+        if (wave >= c.wave_limit) {
+            error(RDF_ERR_WAVE_LIMIT);
+            return false;
+        }
+        max_wave = max(max_wave, wave);
+        if (n_late) atomicAdd(&late_waves[min(wave - (uint32_t)POOL_BINS, n_late - 1u)], 1u);
+        return true;
+    }
+
     // The operand `v` arrives at port `port` of match node `node` in frame f; the last one makes the match a token.
-    __device__ __forceinline__ void deliver(uint32_t f, uint32_t node, uint32_t port, int64_t v) {
+    __device__ __forceinline__ void deliver(uint32_t f, uint32_t node, uint32_t port, int64_t v, uint32_t wave) {
         const PoolMatch M = P.prog->match[node];
         P.words[(M.word0 + port) * z.cap + f] = v;
         __threadfence_block();
-        const uint32_t bit = 1u << (M.word0 + port), before = atomicOr(&P.state[f], bit);
-        if (((before | bit) & M.all) != M.all) {
-            ++inserts;
-            return;
+        uint32_t* state = &P.state[node * z.cap + f];
+        if (M.n_ports == 2) {                               // one exchange: the second operand gets the first one's word, and nobody follows
+            const uint32_t there = atomicExch(state, wave << 8 | 1u);
+            if (there == 0u) {
+                ++inserts;
+                return;
+            }
+            *state = max(there, wave << 8 | 1u);
+        } else {
+            const uint32_t bit = 1u << port;
+            uint32_t there = atomicCAS(state, 0u, wave << 8 | bit);
+            while (there != 0u) {
+                const uint32_t both = max(there & ~0xFFu, wave << 8) | (there & 0xFFu) | bit;
+                if ((both & 0xFFu) == M.all) {              // (nobody follows the last one)
+                    *state = both;
+                    break;
+                }
+                const uint32_t seen = there;
+                there = atomicCAS(state, seen, both);
+                if (there == seen) there = 0u;
+            }
+            if (there == 0u) {
+                ++inserts;
+                return;
+            }
         }
         ++matches;
         const uint32_t at = match0 + pool_take(&sh.matched[par]);
-        if (at < z.cap) P.match[at] = (uint16_t)(f | node << 13);
+        if (at < z.cap) P.match[z.match_step * (int)at] = (uint16_t)(f | node << 13);
         else sh.stop = 2;                                   // (only bodies with several match nodes can have more matches than frames)
     }
 
@@ -182,7 +232,7 @@ struct PoolThread {
         if (e.n_cond > 1 && holds(e.cmp[1], pick(e.a[1], a0, a1, a2), pick(e.b[1], a0, a1, a2))) which = 1;
         if (e.n_cond > 0 && holds(e.cmp[0], pick(e.a[0], a0, a1, a2), pick(e.b[0], a0, a1, a2))) which = 0;
         const PoolAction& act = e.act[which];
-        if (act.n_calls == 0) return give_value(f, h, pick(act.ops[0], a0, a1, a2));
+        if (act.n_calls == 0) return give_value(f, h, pick(act.ops[0], a0, a1, a2), wave);
         const uint32_t k = act.n_calls;
         uint32_t depth, frame_at, slot;
         invocations += k;
@@ -202,13 +252,13 @@ struct PoolThread {
     }
 
     // Return_i: frame f (its word h) has the value v.  Returns the code to go on with (in frame f, r0 = v), or -1.
-    __device__ __forceinline__ int give_value(uint32_t& f, uint32_t& h, int64_t v) {
+    __device__ __forceinline__ int give_value(uint32_t& f, uint32_t& h, int64_t v, uint32_t wave) {
         for (;;) {
             const PoolLabel L = P.prog->labels[(h >> 16) & 63u];
             give_back(f);
             f = h & 0xFFFFu;
             if (L.k_kind == K_PORT) {
-                deliver(f, L.k_node, L.k_port, v);
+                deliver(f, L.k_node, L.k_port, v, wave);
                 return -1;
             }
             h = P.head[f];
@@ -226,6 +276,7 @@ struct PoolThread {
         int pc;
         if (node >= 0) {
             const PoolMatch M = prog.match[node];
+            wave = P.state[node * z.cap + f] >> 8;
             const int64_t* w = P.words + M.word0 * z.cap + f;
             const int64_t p0 = w[0], p1 = w[z.cap], p2 = M.n_ports > 2 ? w[2 * z.cap] : 0ll;
             const PoolCont& q = prog.cont_of[min(node, POOL_MAX_CONT - 1)];
@@ -233,13 +284,13 @@ struct PoolThread {
                 uint32_t depth;
                 ++invocations;
                 if (push_tag(h, depth))
-                    tail_call(f, h, q.label, pick(q.ops[0], p0, p1, p2), pick(q.ops[1], p0, p1, p2), pick(q.ops[2], p0, p1, p2), depth, 1u);
+                    tail_call(f, h, q.label, pick(q.ops[0], p0, p1, p2), pick(q.ops[1], p0, p1, p2), pick(q.ops[2], p0, p1, p2), depth, wave + 1u);
                 return;
             }
             if (node < POOL_MAX_CONT && q.op >= PI_ADD && q.op <= PI_MAX) {
                 const int64_t a = pick(q.a, p0, p1, p2), b = pick(q.b, p0, p1, p2);
                 const int64_t r = q.op == PI_ADD ? a + b : q.op == PI_SUB ? a - b : q.op == PI_MUL ? a * b : a > b ? a : b;
-                pc = give_value(f, h, r + (int64_t)q.imm);
+                pc = give_value(f, h, r + (int64_t)q.imm, wave);
                 if (pc < 0) return;
             } else {
                 set(0, p0); set(1, p1);
@@ -258,7 +309,8 @@ struct PoolThread {
             }
             wave = P.state[f];
             P.state[f] = 0u;
-            max_wave = max(max_wave, wave);
+            for (uint32_t k = 1; k < z.n_match; ++k) P.state[k * z.cap + f] = 0u;
+            if (!count_wave(wave)) return;
             if (fast >= 0) {
                 pc = enter_fast(f, h, prog.entry_of[fast], wave);
                 if (pc < 0) return;
@@ -276,7 +328,7 @@ struct PoolThread {
                 const int64_t b = val(in.rb, in.ib);
                 if (!holds(in.cmp, a, b)) pc = in.imm;
             } else if (in.op == PI_RET) {
-                pc = give_value(f, h, a);
+                pc = give_value(f, h, a, wave);
                 if (pc < 0) return;
             } else if (in.op == PI_CALL) {
                 const uint32_t label = (uint32_t)in.imm, n_args = prog.labels[label].n_args;
@@ -311,7 +363,7 @@ struct PoolThread {
                     case PI_ARG: set(in.dst, P.words[in.imm * z.cap + f]); break;
                     case PI_JMP: pc = in.imm; break;
                     case PI_PORT:
-                        deliver(f, in.imm, in.cmp, a);
+                        deliver(f, in.imm, in.cmp, a, wave);
                         if (in.last) return;
                         break;
                     case PI_TREE: {
@@ -362,19 +414,27 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         P.regs = reinterpret_cast<int64_t*>(p); p += (size_t)(program.n_regs + 1) * T * 8;
         P.words = reinterpret_cast<int64_t*>(p); p += (size_t)program.words * z.cap * 8;
         P.head = reinterpret_cast<uint32_t*>(p); p += (size_t)z.cap * 4;
-        P.state = reinterpret_cast<uint32_t*>(p); p += (size_t)z.cap * 4;
+        P.state = reinterpret_cast<uint32_t*>(p); p += (size_t)z.n_match * z.cap * 4;
         P.enter = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2;
-        P.match = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2;
+        if (z.match_step < 0) P.match = P.enter + z.cap - 1;
+        else { P.match = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2; }
         P.ring = reinterpret_cast<uint16_t*>(p);
     }
     for (uint32_t i = tid; i < z.cap; i += T) P.ring[i] = (uint16_t)i;
     P.regs[program.n_regs * T + tid] = 0ll;
-    if (tid == 0) sh = PoolShared{};
+    if (tid == 0) {
+        sh.entered[0] = sh.entered[1] = sh.matched[0] = sh.matched[1] = sh.taken[0] = sh.taken[1] = sh.freed[0] = sh.freed[1] = 0u;
+        sh.stop = 0;
+    }
+    for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += T) sh.waves[i] = 0u;
+    const long long t_start = clock64();
     const uint32_t B = (uint32_t)c.B, chunks = (B + z.chunk - 1) / z.chunk;
     uint32_t ib = min(B, blockIdx.x * z.chunk), ie = min(B, ib + z.chunk);       // instances this block has taken and not yet started
     bool more = blockIdx.x < chunks;
     PoolThread t{c, z, P, sh, tid};
-    uint32_t ebase = 0, ne = 0, nm = 0, ring0 = 0, avail = z.cap, par = 0, widest = 0;      // frames to enter, completed matches
+    t.late_waves = reinterpret_cast<uint32_t*>(c.q[0]);
+    t.n_late = z.late_waves;
+    uint32_t ebase = 0, ne = 0, nm = 0, ring0 = 0, avail = z.cap, par = 0;      // frames to enter, completed matches
     unsigned long long tokens = 0;
     __syncthreads();
     for (uint32_t round = 0;; ++round) {
@@ -413,11 +473,10 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         uint32_t f = 0xFFFFFFFFu;
         int node = -1;
         if (tid < mm) {
-            const uint32_t v = P.match[nm - 1u - tid];
+            const uint32_t v = P.match[z.match_step * (int)(nm - 1u - tid)];
             f = v & (POOL_MAX_FRAMES - 1u);
             node = (int)(v >> 13);
         } else if (tid >= w0 && tid - w0 < me) f = P.enter[t.wrap(ebase + ne - 1u - (tid - w0))];
-        widest = max(widest, ne + nm);
         tokens += mm + me;
         t.ring0 = ring0; t.avail = avail; t.ring_tail = t.wrap(ring0 + avail);
         t.enter0 = t.wrap(ebase + ne - me); t.match0 = nm - mm; t.par = par;
@@ -445,13 +504,39 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
     st.invocations = t.invocations; st.max_depth = t.max_depth;
     st.sc.inserts = t.inserts; st.sc.matches = t.matches;
     flush_stats(c, st);
-    const uint32_t w = __reduce_max_sync(0xffffffffu, t.max_wave);
-    if ((tid & 31u) == 0) atomicMax(&c.ctl->waves, w + 1u);
-    if (tid == 0) atomicMax(&c.ctl->max_wave_tokens, widest);
+    uint32_t w = t.max_wave;
+    for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += T)
+        if (sh.waves[i]) {
+            atomicAdd(&c.ctl->wave_tokens[i], sh.waves[i]);
+            w = max(w, i);
+        }
+    w = __reduce_max_sync(0xffffffffu, w);
+    if ((tid & 31u) == 0 && (w || tid == 0)) atomicMax(&c.ctl->waves, w + 1u);
+    if (blockIdx.x == 0 && tid == 0) c.ctl->cyc[0] = clock64() - t_start;
     __threadfence();
     __syncthreads();
-    if (tid == 0 && atomicAdd(&c.ctl->blocks_done, 1u) == gridDim.x - 1u) {
-        __threadfence();
+    if (tid == 0) sh.next_chunk = atomicAdd(&c.ctl->blocks_done, 1u);
+    __syncthreads();
+    if (sh.next_chunk != gridDim.x - 1u) return;
+    __threadfence();
+    // the widest wave of the call
+    uint32_t wide = 0, late = 0;
+    const uint32_t n_waves = ld_volatile_u32(&c.ctl->waves);
+    for (uint32_t i = tid; i < min(n_waves, (uint32_t)POOL_BINS); i += T) wide = max(wide, __ldcg(&c.ctl->wave_tokens[i]));
+    if (n_waves > (uint32_t)POOL_BINS)
+        for (uint32_t i = tid; i < min(n_waves - (uint32_t)POOL_BINS, t.n_late); i += T) {
+            const uint32_t v = __ldcg(&t.late_waves[i]);
+            (i + 1u < t.n_late ? wide : late) = max(v, i + 1u < t.n_late ? wide : late);
+        }
+    wide = __reduce_max_sync(0xffffffffu, wide);
+    late = __reduce_max_sync(0xffffffffu, late);
+    if ((tid & 31u) == 0) {
+        atomicMax(&c.ctl->max_wave_tokens, max(wide, late));
+        // (the last bin is a sum over waves, and an upper bound only)
+        if (c.tag_mode == RDF_TAGS_PATH && wide > c.qcap && !c.ctl->pool_exhausted) set_status(c, RDF_ERR_QUEUE_FULL);
+    }
+    __syncthreads();
+    if (tid == 0) {
         volatile Control* k = c.ctl;
         k->tokens = k->invocations + (unsigned long long)c.B;
         if (k->pool_exhausted) {

@@ -717,3 +717,83 @@ def test_pool_executor_tail_calls_of_another_function(B, n_hi, mode):
     g.eval_int(torch.from_numpy(x_host).cuda(), max_invocations=calls, y=y)
     assert y.tolist() == [want[v][0] for v in x_host]
     assert g.stats()["invocations"] == calls
+
+
+# what rdf_last_status reports of a run, whichever executor ran it
+REPORTED = ("invocations", "tokens", "waves", "max_wave_tokens", "store_inserts", "store_matches", "max_depth")
+
+
+def _same_report(functions, result, mode, x, calls):
+    """The call once out of the pools and once, traced, through the general scheduler."""
+    g = rdf.Graph(functions, result, mode)
+    y, _ = g.eval_int(x, max_invocations=calls)
+    mine = g.stats()
+    y2, _ = g.eval_int(x, max_invocations=calls, trace_capacity=2 * calls + 64)
+    general = g.stats()
+    assert torch.equal(y, y2)
+    assert {k: mine[k] for k in REPORTED} == {k: general[k] for k in REPORTED}
+
+
+@pytest.mark.parametrize("name,mode,hi,B", [("fib", rdf.TAGS_PATH, 15, 700), ("fib", rdf.TAGS_FRAME, 15, 700), ("tak", rdf.TAGS_FRAME, 15, 60),
+                                            ("ack", rdf.TAGS_FRAME, 9, 50), ("primes", rdf.TAGS_FRAME, 400, 40), ("find", rdf.TAGS_FRAME, 8, 300),
+                                            ("0-1-2", rdf.TAGS_PATH, 14, 900), ("0-1-2-3", rdf.TAGS_FRAME, 14, 900), ("mutual", rdf.TAGS_FRAME, 12, 900),
+                                            ("tail", rdf.TAGS_PATH, 9, 900)])
+def test_pool_executor_reports_the_waves_of_the_graph(name, mode, hi, B):
+    """Number of waves and the widest one are those of the graph executed in waves (which is what rdf_batch.max_wave_tokens and
+    rdf_set_limits are about), also beyond 256 waves, behind matches and with several matches per body."""
+    programs_ = {"fib": rdf.fib_program, "tak": lambda: rdf.tak_program(10, 5), "ack": rdf.ack_program, "primes": rdf.primes_program,
+                 "find": lambda: rdf.find_program(200), "tail": lambda: (_tail_to_another(), 0)}
+    fs, r = programs_[name]() if name in programs_ else (_mixed_counts(name), 0)
+    xs = np.random.default_rng(3).integers(0, hi + 1, size=B)
+    xs[0] = hi
+    g = rdf.Graph(fs, r, mode)
+    x = torch.from_numpy(xs).cuda()
+    g.eval_int(x, max_invocations=3_000_000)
+    _same_report(fs, r, mode, x, g.stats()["invocations"])
+
+
+def test_pool_executor_reports_the_waves_of_random_programs():
+    x = torch.arange(9, dtype=torch.int64, device="cuda").repeat(20)
+    for seed in range(60):
+        fs = _random_program(seed)
+        try:
+            g = rdf.Graph(fs, 0, rdf.TAGS_FRAME)
+        except rdf.RdfError:
+            continue
+        g.eval_int(x, max_invocations=1_000_000)
+        _same_report(fs, 0, rdf.TAGS_FRAME, x, g.stats()["invocations"])
+
+
+@pytest.mark.parametrize("max_invocations", [300, 1000, 3000, 20000, 60000, 102000])
+def test_pool_executor_refuses_what_the_queues_would(max_invocations):
+    """Path tags: a bound on the invocations that is too small for a wave or for the store is the status of the general scheduler."""
+    g = rdf.Graph(*rdf.fib_program(), rdf.TAGS_PATH)
+    x = torch.full((64,), 15, dtype=torch.int64, device="cuda")          # 64 x 1973 calls
+
+    def code(**kw):
+        try:
+            g.eval_int(x, max_invocations=max_invocations, **kw)
+        except rdf.RdfError as e:
+            return e.code
+        return 0
+    assert code() == code(trace_capacity=300000)
+
+
+def test_pool_executor_wave_limit():
+    """A chain of more calls than there may be waves (2^24) ends with the status of the general scheduler, whatever the bound on
+    the invocations."""
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f = rdf.Function("down", 1)
+    n = f.param()
+    f.ret(f.if_(f.lt(n, f.const(1)), f.const(0), f.call(1, f.sub(n, f.const(1)))))
+    g = rdf.Graph([r, f], 0, rdf.TAGS_FRAME)
+    x = torch.full((32,), (1 << 24) // 16, dtype=torch.int64, device="cuda")
+    assert not g.eval_int(x, max_invocations=40 << 20)[0].any() and g.stats()["waves"] == (1 << 24) // 16 + 2
+    x[7] = (1 << 24) + 5
+    code = 0
+    try:
+        g.eval_int(x, max_invocations=40 << 20)
+    except rdf.RdfError as e:
+        code = e.code
+    assert code == -8
