@@ -1706,14 +1706,16 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     rdf_mark(S, 0, stream);
     S->launches = 0;
     CUDA_OK(cudaMemsetAsync(ws + L.ctl, 0, 4096, stream));
+    // a bound of the caller's on the width of a wave, which only the general scheduler runs into
+    const bool any_width = in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B;
     // Structural recursion over the input trees has its own scheduler; a traced call records every firing of the graph and
     // goes through the general one.
-    const bool fold = g->fold && !out->trace;
+    const bool fold = g->fold && !out->trace && any_width;
     // Integer programs run out of shared memory.  The general scheduler has what that executor does not: trace records, a
     // bound on the width of a wave, the waits and waves that rdf_set_limits limits, and the cooperative probes.
     const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= POOL_MIN_FRAMES && S->wait_cycles == 0 &&
                       S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
-                      (in->max_wave_tokens <= 0 || in->max_wave_tokens >= in->max_invocations + in->B) &&
+                      any_width &&
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);
     if (pool) {
         // bounded depth, one match per frame: a pool always suffices (should it not, the call ends with a status)

@@ -152,7 +152,7 @@ __device__ __forceinline__ void fold_children(const DevCtx& c, const uint4& rec,
 __device__ __forceinline__ bool fold_room(const DevCtx& c, const FoldLevel& L, uint32_t cells) {
     const uint64_t end = (uint64_t)L.fb + L.n + 2ull * cells;
     if (end > c.frame_cap) { set_status(c, RDF_ERR_FRAMES_FULL); return false; }
-    if (2ull * cells > c.qcap) { set_status(c, RDF_ERR_QUEUE_FULL); return false; }
+    if (2ull * cells > c.qcap) { set_status(c, RDF_ERR_QUEUE_FULL); return false; }      // (the records of the level would not fit)
     // (in token waves a level costs one on the way down and one on the way up)
     if (cells && 2ull * (L.d + 1u) + 3u > c.wave_limit) { set_status(c, RDF_ERR_WAVE_LIMIT); return false; }
     return true;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
     const uint32_t tid = threadIdx.x, lane = tid % 32, warp = tid / 32, B = (uint32_t)c.B;
     uint4* const tq[2] = {reinterpret_cast<uint4*>(c.q[0]), reinterpret_cast<uint4*>(c.q[1])};
     FoldLevel L{B, B, 0u, 0u, 0u};
-    uint32_t generation = 0, g = 0, stretch = 0, widest = B;
+    uint32_t generation = 0, g = 0, stretch = 0;
     const long long t_start = clock64();
     bool in_shared = false, alive = true;
     if (3ull > c.wave_limit) { set_status(c, RDF_ERR_WAVE_LIMIT); alive = false; }
@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
                         fold_fire(c, L, tid, valid, rec, arg, kid, rank, stay ? sh.q[(L.d + 1) & 1] : tq[(L.d + 1) & 1],
                                   stay ? nullptr : c.level_counts + (g % 3u) * c.level_cap);
                     fold_next(c, L, total);
-                    widest = max(widest, L.n);
                     in_shared = stay;
                     __syncthreads();
                 } while (L.n && L.n <= FS_CHUNK && ++k < FS_STRETCH);
@@ -233,14 +232,14 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
                 if (tid == 0) {
                     uint4* s = &c.ctl->fold_state[2 * (stretch & 1u)];
                     s[0] = make_uint4(L.n, L.fb, L.cb, L.lb);
-                    s[1] = make_uint4(L.d, widest, 0u, 0u);
+                    s[1] = make_uint4(L.d, 0u, 0u, 0u);
                 }
             }
             if (gridDim.x > 1 && !grid_barrier(c, &c.ctl->bar.v, generation)) { alive = false; break; }
             const uint4* s = &c.ctl->fold_state[2 * (stretch & 1u)];     // (two slots in turn: block 0 may be a stretch ahead)
             if (blockIdx.x != 0) {
                 const uint4 a = __ldcg(s), b = __ldcg(s + 1);
-                L.n = a.x; L.fb = a.y; L.cb = a.z; L.lb = a.w; L.d = b.x; widest = b.y;
+                L.n = a.x; L.fb = a.y; L.cb = a.z; L.lb = a.w; L.d = b.x;
             }
             in_shared = false;
             ++stretch;
@@ -297,7 +296,6 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
         }
         if (!room) { alive = false; break; }
         fold_next(c, L, total);
-        widest = max(widest, L.n);
         ++g;
         if (gridDim.x > 1) alive = grid_barrier(c, &c.ctl->bar.v, generation);
         else __syncthreads();
@@ -312,7 +310,9 @@ __global__ void __launch_bounds__(FS_CHUNK, 1) rdf_fold_kernel(const __grid_cons
         c.ctl->call_waves = L.d;
         // in terms of the token waves of the graph: a call per invocation, a return per invocation, one more for `result`
         c.ctl->waves = 2u * L.d + 1u;
-        c.ctl->max_wave_tokens = widest;
+        // (the widest wave: its calls and returns belong to invocations none of which is below another one, and no such set
+        // is larger than that of the leaves)
+        c.ctl->max_wave_tokens = max(B, L.lb);
         c.ctl->invocations = inv; c.ctl->tokens = (unsigned long long)B + 2ull * inv;
         c.ctl->store_inserts = c.ctl->store_matches = c.ctl->cells = L.cb;
         c.ctl->leaves = L.lb;

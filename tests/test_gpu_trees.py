@@ -527,3 +527,41 @@ def test_fp32_wide_tiles_one_after_another(H):
     p = workloads.treernn_params(3, 70, H, H)
     shapes = [workloads.perfect_tree_shape(16)] * 2
     check_grad({"trees": workloads.tree_batch_from_shapes(shapes, 7, vocab=70), "params": p}, workers=WORKERS)
+
+
+@pytest.mark.parametrize("cell", ["rnn", "lstm"])
+def test_queue_bound_of_structural_recursion(cell, monkeypatch):
+    """The widest wave that a call reports is enough as the queue bound of any later call (a traced one runs the token waves, in
+    which returning values take places beside the calls), and a bound that the token waves do not fit is refused as by them."""
+    rng = np.random.default_rng(4)
+    p = (workloads.treernn_params if cell == "rnn" else workloads.treelstm_params)(7, 50, 8, 8)
+    g = rdf.Graph(*rdf.tree_net_program(cell), rdf.TAGS_FRAME)
+    make = rdf.Graph._batch
+
+    def code(dt, dp, bound, **kw):
+        def bounded(d):
+            b = make(d)
+            b.max_wave_tokens = bound
+            return b
+        monkeypatch.setattr(rdf.Graph, "_batch", staticmethod(bounded))
+        try:
+            g.eval_trees(dt, dp, **kw)
+        except rdf.RdfError as e:
+            return e.code
+        finally:
+            monkeypatch.setattr(rdf.Graph, "_batch", staticmethod(make))
+        return 0
+    for B, leaves in ((1, 1), (1, 40), (60, 25), (700, 9)):
+        tb = workloads.tree_batch_from_shapes([workloads.random_split_shape(rng, int(rng.integers(max(1, leaves // 2), leaves + 1))) for _ in range(B)], 7, vocab=50)
+        dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(p)
+        h, _ = g.eval_trees(dt, dp)
+        reported = g.stats()["max_wave_tokens"]
+        g.eval_trees(dt, dp, trace_capacity=2 * tb.N + 64)
+        width = g.stats()["max_wave_tokens"]
+        assert width <= reported <= (tb.N + B) // 2
+        assert code(dt, dp, reported, trace_capacity=2 * tb.N + 64) == 0
+        # (waves of up to 1024 tokens stay in one block and need no queue)
+        for bound in (width, max(B, width - 1)):
+            assert code(dt, dp, bound) == code(dt, dp, bound, trace_capacity=2 * tb.N + 64) == (0 if bound >= width or width <= 1024 else -7)
+        assert B < 700 or width > 1024
+        assert torch.equal(g.eval_trees(dt, dp)[0], h)
