@@ -671,7 +671,9 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
                 } while (m != 0 && m <= blockDim.x && k < NARROW_STRETCH && wave < c.wave_limit &&
                          ld_volatile_i32(&c.ctl->status) == 0);
                 // hand the next wave back to the global queue (tokens beyond the local capacity are there already)
-                for (uint32_t i = threadIdx.x; i < min(m, LQ_CAP); i += blockDim.x) {
+                // (a queue bound below the width of the block: the stretch needed no queue, the wave it ends with does)
+                if (m > c.qcap) set_status(c, RDF_ERR_QUEUE_FULL);
+                for (uint32_t i = threadIdx.x; i < min(min(m, LQ_CAP), c.qcap); i += blockDim.x) {
                     const Token t = load_local_token(&lq.buf[wave & 1][i]);
                     store_token(&c.q[wave & 1][i], t.tag, t.datum, t.pc);
                 }

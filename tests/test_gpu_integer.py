@@ -797,3 +797,27 @@ def test_pool_executor_wave_limit():
     except rdf.RdfError as e:
         code = e.code
     assert code == -8
+
+
+def test_queue_bound_at_the_end_of_a_narrow_stretch():
+    """Waves of up to 1024 tokens stay in one block; the wave with which it hands back to the grid must fit the queue: too many
+    tokens for the bound, or 4096 narrow waves of more tokens than the bound."""
+    fs, r = rdf.fib_program()
+    g = rdf.Graph(fs, r, rdf.TAGS_FRAME)
+    x = torch.full((2,), 18, dtype=torch.int64, device="cuda")
+    d = rdf.Function("down", 1)
+    n = d.param()
+    d.ret(d.if_(d.lt(n, d.const(1)), d.const(0), d.add(n, d.call(1, d.sub(n, d.const(1))))))
+    res = rdf.Function("result", 1)
+    res.ret(res.add(res.call(1, res.param()), res.call(1, res.param())))
+    chain = rdf.Graph([res, d], 0, rdf.TAGS_FRAME)
+    long = torch.full((3,), 5000, dtype=torch.int64, device="cuda")
+
+    def code(graph, xs, calls, bound):
+        try:
+            graph.eval_int(xs, max_invocations=calls, max_wave_tokens=bound)
+        except rdf.RdfError as e:
+            return e.code
+        return 0
+    assert code(g, x, 2 * 8361, 100) == -7 and code(g, x, 2 * 8361, 8361) == 0
+    assert code(chain, long, 6 * 5001, 5) == -7 and code(chain, long, 6 * 5001, 6) == 0
