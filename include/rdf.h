@@ -247,10 +247,12 @@ typedef struct {                 /* all device, fp32, shapes of the parameters; 
 
 typedef struct {
     int32_t  status;             /* RDF_OK or the first RDF_ERR_* the device recorded */
-    uint32_t waves;              /* scheduler waves run (forward) */
+    uint32_t waves;              /* scheduler waves run (forward); an upper bound for an integer program of which a long instance
+                                    was left to the whole device */
     uint32_t waves_backward;
     uint32_t max_wave_tokens;    /* widest wave; an upper bound for structural recursion over the input trees (the number of
-                                    leaves) and for integer programs that run out of shared memory in more than 65 792 waves */
+                                    leaves) and for integer programs that run out of shared memory in more than 65 792 waves or
+                                    of which a long instance was left to the whole device */
     uint64_t invocations;        /* Call firings */
     uint64_t tokens;             /* tokens taken from the wave queues */
     uint64_t store_inserts;      /* operands parked in the token store */

@@ -77,6 +77,7 @@ struct Control {
     HotCounter bar2;              // barrier counter of the backward kernel
     HotCounter bar_ops;           // barrier counter of the operator kernel
     HotCounter bar_group;         // barrier counter of the grouping kernel
+    HotCounter blocks_done;       // pool kernel: blocks that have run all their instances
     int32_t  status;
     uint32_t waves, waves_backward, max_wave_tokens, max_probe, max_depth;
     uint32_t all_cells;           // backward: cells seen so far (length of the all-cells list)
@@ -91,7 +92,9 @@ struct Control {
     unsigned long long cyc[6];    // block 0: forward schedule / batch / barrier, backward frames / batch / barrier
     float    loss;
     int32_t  forward_status;      // status word at the end of the forward pass and the loss head
-    uint32_t next_chunk, blocks_done, pool_exhausted;   // rdf_pool.cuh
+    uint32_t next_chunk, pool_exhausted;   // rdf_pool.cuh
+    uint32_t hand_claims, hand_mask, hand_frames, scheduler_done;   // blocks that have a place to leave their calls in, that have left
+                                                        // them, and the frames these had
     uint32_t wave_tokens[POOL_BINS];                    // tokens per wave of the call
     uint4    il_state[2];         // interleaved execution: where the grid carries on after a cluster ({wave, cells, left, right done}, {leaves done, widest})
     uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
@@ -100,6 +103,14 @@ static_assert(sizeof(Control) <= 4096, "the control block is 4 KB");
 
 // A tensor map as the driver encodes it (128 opaque bytes; the host fills it with cuTensorMapEncodeTiled).
 struct alignas(64) TensorMap { unsigned long long opaque[16]; };
+
+// What the general scheduler needs to know of the pool kernel before it (rdf_pool.cuh)
+struct PoolCarry {
+    uint32_t cap, words, word0, n_match;        // PoolSizes, PoolProgram
+    size_t   slot_bytes;                        // a block's frames in the second wave queue
+    size_t   pair_n, arrived_n, table_n;        // elements of the token store to clear
+    unsigned long long max_parked;
+};
 
 struct DevCtx {
     // lowered program (copied into the workspace at every call)
@@ -118,7 +129,8 @@ struct DevCtx {
     uint32_t qcap;
     // structural recursion (rdf_fold.cuh)
     int       fold_label[3], fold_right[2];
-    int       after_pool;         // general scheduler behind the pool kernel: it runs only if a pool was exhausted
+    int       after_pool;         // general scheduler behind the pool kernel: it runs only what a pool could not, or left to it
+    PoolCarry pool;
     uint32_t* level_counts;       // [3][level_cap]: cells per chunk of a level, three levels in turn
     uint32_t  level_cap;
     // frames (frame-form tags)

@@ -571,6 +571,7 @@ __device__ __forceinline__ void flush_stats(const DevCtx& c, const ThreadStats& 
     }
 }
 
+__device__ bool pool_take_over(const DevCtx& c, uint32_t& generation);       // rdf_pool.cuh
 static const uint32_t NARROW_STRETCH = 4096;   // waves block 0 runs alone before it meets the grid again
 
 // The scheduler: all waves of token processing, for integer and for vector programs.  Only tokens are
@@ -579,16 +580,16 @@ static const uint32_t NARROW_STRETCH = 4096;   // waves block 0 runs alone befor
 __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
     __shared__ uint32_t lq_count[3], lq_ctr[3];
-    if (c.after_pool && !c.ctl->pool_exhausted) return;              // (the pool kernel has run the call)
     extern __shared__ __align__(16) unsigned char lq_smem[];         // local queue of narrow stretches: 2 x LQ_CAP tokens
     LocalQ lq;
     lq.buf[0] = reinterpret_cast<Token*>(lq_smem);
     lq.buf[1] = lq.buf[0] + LQ_CAP;
     lq.count = lq_count;
     lq.ctr = lq_ctr;
-    load_program(c, sp);
     ThreadStats st;
     uint32_t generation = 0, wave = 0, widest = 0;
+    if (c.after_pool && !pool_take_over(c, generation)) return;      // (the pool kernel has run the call)
+    load_program(c, sp);
     long long cyc_s = 0, cyc_b = 0, t_mark = clock64();
     auto lap = [&](long long& acc) {
         const long long now = clock64();
@@ -712,11 +713,20 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
         lap(cyc_b);
     }
     flush_stats(c, st);
+    const bool rest = c.after_pool && c.ctl->pool_exhausted == 0;    // the rest of a call that began in the pool kernel
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        c.ctl->waves = wave;
-        c.ctl->max_wave_tokens = widest;
-        c.ctl->cyc[0] = cyc_s; c.ctl->cyc[2] = cyc_b;
+        c.ctl->waves = rest ? c.ctl->waves + wave : wave;
+        c.ctl->max_wave_tokens = rest ? c.qcap : widest;
+        c.ctl->cyc[0] = rest ? c.ctl->cyc[0] + cyc_s : cyc_s; c.ctl->cyc[2] = cyc_b;
         c.ctl->forward_status = c.ctl->status;      // what the operator kernel checks before it starts
+    }
+    if (!rest) return;
+    // (path tags: the operands of the whole call against the token store it has)
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&c.ctl->scheduler_done, 1u) == gridDim.x - 1u && c.tag_mode == RDF_TAGS_PATH) {
+        __threadfence();
+        if (*reinterpret_cast<volatile unsigned long long*>(&c.ctl->store_inserts) > c.pool.max_parked) set_status(c, RDF_ERR_STORE_FULL);
     }
 }
 
@@ -1658,13 +1668,22 @@ int rdf_check_common(rdf_graph* g, const rdf_batch* in, const rdf_params* params
     return RDF_OK;
 }
 
+// One block runs an instance to its end, so a few large instances are better spread over the device wave by wave: one call
+// of fib(18) (8361 calls) takes 0.10 ms in a pool and 0.22 in waves, fib(22) (57 313) 0.36 and 0.30, fib(24) (150 049) 0.87
+// and 0.34, eight of fib(22) 0.36 and 0.34; but 32 of fib(24) 0.90 and 1.58.  What the mean does not show -- a long instance among
+// short ones -- the blocks find out (rdf_pool.cuh: POOL_ACTIVE): 64 calls, one of them fib(24) / fib(27) / fib(30) and the rest fib(5),
+// take 0.45 / 0.53 / 0.97 ms, in waves 0.35 / 0.42 / 0.86, in pools alone 0.83 / 5.0 / 22.9.  The launch behind the pool kernel
+// that this needs, mostly with nothing to do, costs 1024 calls of fib 169 -> 178 us.
+static const long long POOL_CALLS = 40000, POOL_MANY = 32;
+static const uint32_t POOL_MIN_FRAMES = 15 * POOL_THREADS / 4;   // (bodies of up to three operators with two operands each)
+
 static size_t pool_smem_bytes(const ExecState* S) { return std::min<size_t>(S->smem_per_sm / POOL_PER_SM - 1024, S->smem_per_block) - sizeof(PoolShared) - 256; }
 static uint32_t pool_frames(const PoolProgram& P, const ExecState* S) {
     const size_t fixed = pool_fixed_bytes(P), smem = pool_smem_bytes(S);
     return smem <= fixed ? 0u : (uint32_t)std::min<size_t>((smem - fixed) / pool_frame_bytes(P), POOL_MAX_FRAMES) & ~7u;
 }
 // The pool executor: how many frames a block has, and how the instances are dealt out.
-static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, bool fallback, cudaStream_t stream) {
+static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, bool& fallback, cudaStream_t stream) {
     const PoolProgram& P = g->pool_prog;
     const size_t smem = pool_smem_bytes(S);
     PoolSizes z{};
@@ -1681,8 +1700,19 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     z.refill = POOL_THREADS / 3;
     z.max_calls = (unsigned long long)in->max_invocations;
     z.max_parked = (unsigned long long)L.table_cap * std::max<size_t>(1, g->match.size());
-    z.fallback = fallback;
     z.n_match = (uint32_t)std::max(1, P.n_match);
+    c.pool.cap = z.cap; c.pool.words = (uint32_t)P.words; c.pool.word0 = (uint32_t)P.word0; c.pool.n_match = z.n_match;
+    c.pool.slot_bytes = pool_dump_bytes(P, z.cap); c.pool.max_parked = z.max_parked;
+    c.pool.pair_n = L.pair_bytes / sizeof(Slot); c.pool.arrived_n = L.arrived_bytes / sizeof(uint32_t); c.pool.table_n = L.table_bytes / sizeof(Slot);
+    // A long instance may be left to the general scheduler, where the call may have one; path tags do not keep the labels of
+    // calls that took over their caller's frame, and a store of the caller's own size is held against the whole call at once.
+    if (in->max_invocations > POOL_CALLS && S->hash_slots == 0 && !(g->tag_mode == RDF_TAGS_PATH && P.tails)) {
+        z.hand_slots = (uint32_t)std::min<size_t>(POOL_ACTIVE, (size_t)L.qcap * sizeof(Token) / c.pool.slot_bytes);
+        const double us = 20.0 + (double)(L.pair_bytes + L.arrived_bytes + L.table_bytes) / 6e6;         // (cleared at 6 TB/s)
+        z.hand_after = (long long)(us * 1e-3 * S->clock_khz);
+        fallback = fallback || z.hand_slots > 0;
+    }
+    z.fallback = fallback;
     z.match_step = pool_tokens_share(P) ? -1 : 1;
     // Tokens per wave from POOL_BINS on are counted in the queue that this executor does not use; with path tags and no call
     // that waits for another one a wave is a call depth, and there are not that many.
@@ -1695,12 +1725,6 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     CUDA_OK(cudaGetLastError());
     return RDF_OK;
 }
-
-// One block runs an instance to its end, so a few large instances are better spread over the device wave by wave: one call
-// of fib(18) (8361 calls) takes 0.10 ms in a pool and 0.22 in waves, fib(22) (57 313) 0.36 and 0.30, fib(24) (150 049) 0.87
-// and 0.34, eight of fib(22) 0.36 and 0.34; but 32 of fib(24) 0.90 and 1.58.
-static const long long POOL_CALLS = 40000, POOL_MANY = 32;
-static const uint32_t POOL_MIN_FRAMES = 15 * POOL_THREADS / 4;   // (bodies of up to three operators with two operands each)
 
 // zero what must start at zero, upload the program, seed, run all waves
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,
@@ -1721,7 +1745,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);
     if (pool) {
         // bounded depth, one match per frame: a pool always suffices (should it not, the call ends with a status)
-        const bool fallback = !(g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1);
+        bool fallback = !(g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1);
         const int rc = rdf_launch_pool(g, in, L, S, c, fallback, stream);
         if (rc != RDF_OK) return rc;
         if (!fallback) {
@@ -1732,8 +1756,6 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
             return RDF_OK;
         }
         c.after_pool = 1;
-        RDF_KERNEL(S, rdf_pool_fallback_kernel<<<2 * S->grid, 256, 0, stream>>>(c, L.pair_bytes / sizeof(Slot), L.arrived_bytes / sizeof(uint32_t),
-                                                                               L.table_bytes / sizeof(Slot)));
     } else if (fold) {
         CUDA_OK(cudaMemsetAsync(ws + L.level_counts, 0, (size_t)3 * L.level_cap * sizeof(uint32_t), stream));
     } else if (g->tag_mode == RDF_TAGS_FRAME) {
@@ -1751,7 +1773,9 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
             // page-locked, so that the copy below is asynchronous to the host (made once per graph)
             if (S->tables) { if (S->tables_pinned) cudaFreeHost(S->tables); else free(S->tables); }
             S->tables = nullptr; S->tables_bytes = 0;
-            if (S->may_allocate) {
+            cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+            CUDA_OK(cudaStreamIsCapturing(stream, &capturing));
+            if (S->may_allocate && capturing == cudaStreamCaptureStatusNone) {
                 CUDA_OK(cudaHostAlloc(reinterpret_cast<void**>(&S->tables), bytes, cudaHostAllocDefault));
                 S->tables_pinned = true;
             } else {

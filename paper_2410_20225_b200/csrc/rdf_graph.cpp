@@ -1385,7 +1385,7 @@ struct PoolBuilder {
         // frames: the arguments share their words with the operands of the match nodes, unless they are read late
         out.n_labels = (int)g->labels.size(); out.n_match = (int)g->match.size();
         out.result_entry = new_pc[g->result_entry_pc];
-        const int word0 = late_args ? max_args : 0;
+        const int word0 = out.word0 = late_args ? max_args : 0;
         out.words = std::max(max_args, word0 + g->n_ports_total);
         if (out.words > POOL_MAX_WORDS) return false;
         for (int k = 0; k < out.n_labels; ++k) {
@@ -1406,7 +1406,9 @@ struct PoolBuilder {
             for (int i = new_pc[seg[k]]; i < end; ++i) {
                 const PoolInstr& in = out.code[i];
                 if (in.op == PI_CALL && !entries.count(seg[k])) out.late_calls = 1;
-                if (in.op == PI_CALL) calls += !in.tail || g->labels[in.imm].callee != g->label_caller[in.imm];
+                if (in.op != PI_CALL) continue;
+                if (in.tail && g->labels[in.imm].callee == g->label_caller[in.imm]) out.tails = 1;
+                else ++calls;
             }
             int& most = entries.count(seg[k]) ? out.calls_entry : out.calls_cont;
             most = std::max(most, calls);

@@ -135,7 +135,7 @@ struct alignas(16) PoolProgram {
     int32_t   n_code, n_labels, n_match, result_entry;
     int32_t   words, n_regs;         // 64-bit words per frame, registers per thread
     int32_t   calls_entry, calls_cont;   // most frames taken by a segment that enters a function / that carries on after a match
-    int32_t   late_calls, pad[3];        // some call waits for another one
+    int32_t   late_calls, tails, word0, pad;   // some call waits for another one; some call takes over its caller's frame; word of port 0
     PoolInstr code[POOL_MAX_CODE];
     PoolLabel labels[POOL_MAX_LABELS];
     PoolMatch match[POOL_MAX_MATCH];

@@ -31,6 +31,12 @@
 
 static const int POOL_THREADS = 768, POOL_PER_SM = 1;   // threads of a block, blocks per SM (131 072 calls of fib: 512 threads 6.7 ms, 768 5.5,
                                                         // 1024 6.2, two blocks of 256 6.7: more threads leave each fewer frames)
+// A block runs its instances to their end, and an instance far larger than the others would keep one block busy long after the
+// device has run out of work (one of fib(30), 2.7 M calls, 22.9 ms).  When at most POOL_ACTIVE blocks are left, one with more tokens
+// pending than threads all the while leaves them to the general scheduler, which spreads a wave over the device: its frames, parked operands and the calls to be entered go there as they
+// are.  Before that it runs as long as the other way costs: some 20 us to get going, and the clearing of the token store
+// (PoolSizes::hand_after).
+static const uint32_t POOL_ACTIVE = 8;
 static const uint32_t POOL_ROOT = 0x80000000u;          // frame word of an instance's `result` context: | instance
 // Frame word of an invocation: parent frame [15:0], label [21:16], depth of the tag [27:22] (path tags)
 
@@ -45,10 +51,13 @@ struct PoolSizes {
     unsigned long long max_parked;  // path tags: operands the token store of the call holds
     uint32_t n_match;        // match nodes, at least 1
     int      match_step;     // -1, 1: direction in which Pool::match grows
+    uint32_t hand_slots;     // places for the frames of a block that leaves its calls to the general scheduler
+    long long hand_after;    // clock cycles it runs on its own before it does
     uint32_t late_waves;     // PoolThread::n_late
     int      fallback;       // the general scheduler is launched behind this kernel for a pool that is exhausted
 };
 
+static const int POOL_LEAVE = 3;
 struct PoolShared {
     uint32_t entered[2];     // frames to enter pushed in the round (by parity)
     uint32_t matched[2];     // completed matches pushed in the round
@@ -56,11 +65,14 @@ struct PoolShared {
     uint32_t freed[2];       // frames given back in the round
     uint32_t next_chunk;
     uint32_t waves[POOL_BINS];   // tokens per wave (of the block), the first POOL_BINS waves
-    int      stop;           // 1: an error, 2: the pool is exhausted
+    uint32_t hand;           // 1 + the place the block leaves its frames in
+    uint32_t left[3];        // of a block that leaves them: first free frame, free frames, frames to enter
+    long long alone;         // since when few others are left (clock cycles; 0: they are not)
+    int      stop;           // 1: an error, 2: the pool is exhausted, POOL_LEAVE: the block leaves its calls
 };
 
 inline size_t pool_fixed_bytes(const PoolProgram& P) { return sizeof(PoolProgram) + (size_t)(P.n_regs + 1) * POOL_THREADS * 8; }
-inline bool pool_tokens_share(const PoolProgram& P) { return P.n_match <= 1; }       // one token per frame at most: Pool::match
+__host__ __device__ inline bool pool_tokens_share(const PoolProgram& P) { return P.n_match <= 1; }       // one token per frame at most: Pool::match
 inline size_t pool_frame_bytes(const PoolProgram& P) {
     return 8 * (size_t)P.words + 4 + 4 * (size_t)std::max(1, P.n_match) + 2 + 2 + (pool_tokens_share(P) ? 0 : 2);
 }
@@ -90,6 +102,20 @@ __device__ __forceinline__ uint32_t pool_take(uint32_t* counter) {
 
 static const int POOL_RUN_BITS = 6;                     // calls that follow one another: at most POOL_MAX_CODE
 static_assert(POOL_MAX_CODE < (1 << POOL_RUN_BITS), "a run of calls fits the bits of reserve");
+
+// A block's frames on their way to the general scheduler, in the second wave queue
+struct PoolDump {
+    int64_t  *words;
+    uint32_t *head, *state, *id;                // id: frame id, ~0: no frame; state ~0: to be entered
+    __device__ PoolDump(const DevCtx& c, uint32_t slot) {
+        char* p = reinterpret_cast<char*>(c.q[1]) + slot * c.pool.slot_bytes;
+        words = reinterpret_cast<int64_t*>(p);
+        head = reinterpret_cast<uint32_t*>(words + (size_t)c.pool.words * c.pool.cap);
+        state = head + c.pool.cap;
+        id = state + (size_t)c.pool.n_match * c.pool.cap;
+    }
+};
+inline size_t pool_dump_bytes(const PoolProgram& P, uint32_t cap) { return (size_t)cap * (8 * (size_t)P.words + 8 + 4 * (size_t)std::max(1, P.n_match)); }
 
 struct PoolThread {
     static const int T = POOL_THREADS;
@@ -161,12 +187,12 @@ struct PoolThread {
         __threadfence_block();
         uint32_t* state = &P.state[node * z.cap + f];
         if (M.n_ports == 2) {                               // one exchange: the second operand gets the first one's word, and nobody follows
-            const uint32_t there = atomicExch(state, wave << 8 | 1u);
+            const uint32_t mine = wave << 8 | 1u << port, there = atomicExch(state, mine);
             if (there == 0u) {
                 ++inserts;
                 return;
             }
-            *state = max(there, wave << 8 | 1u);
+            *state = max(there, mine) | M.all;
         } else {
             const uint32_t bit = 1u << port;
             uint32_t there = atomicCAS(state, 0u, wave << 8 | bit);
@@ -397,34 +423,87 @@ __device__ __forceinline__ uint32_t pool_width(const PoolSizes& z, uint32_t avai
     return max(1u, avail > z.reserve ? (avail - z.reserve) >> z.div_shift : 0u);
 }
 
+__device__ __forceinline__ Pool pool_arrays(unsigned char* p, uint32_t cap, int n_regs, int words, uint32_t n_match, int match_step) {
+    Pool P;
+    P.prog = reinterpret_cast<const PoolProgram*>(p);
+    p += sizeof(PoolProgram);
+    P.regs = reinterpret_cast<int64_t*>(p); p += (size_t)(n_regs + 1) * POOL_THREADS * 8;
+    P.words = reinterpret_cast<int64_t*>(p); p += (size_t)words * cap * 8;
+    P.head = reinterpret_cast<uint32_t*>(p); p += (size_t)cap * 4;
+    P.state = reinterpret_cast<uint32_t*>(p); p += (size_t)n_match * cap * 4;
+    P.enter = reinterpret_cast<uint16_t*>(p); p += (size_t)cap * 2;
+    if (match_step < 0) P.match = P.enter + cap - 1;
+    else { P.match = reinterpret_cast<uint16_t*>(p); p += (size_t)cap * 2; }
+    P.ring = reinterpret_cast<uint16_t*>(p);
+    return P;
+}
+
+// The frames of a block that leaves its calls, as they lie.  (On its own: it takes everything from shared memory, so that the
+// rounds keep nothing in registers for it.)
+__device__ __noinline__ void pool_leave(const DevCtx& c, unsigned char* smem, const PoolShared& sh) {
+    const PoolProgram& prog = *reinterpret_cast<const PoolProgram*>(smem);
+    const uint32_t cap = c.pool.cap, slot = sh.hand - 1u, ring0 = sh.left[0], avail = sh.left[1], enter0 = 0u, ne = sh.left[2];
+    const Pool P = pool_arrays(smem, cap, prog.n_regs, prog.words, c.pool.n_match, pool_tokens_share(prog) ? -1 : 1);
+    constexpr uint32_t T = POOL_THREADS;
+    uint8_t* kind = reinterpret_cast<uint8_t*>(P.regs);      // 0 free, 1 entered, 2 to be entered (18 KB and more, for 8192 frames at most)
+    const uint32_t tid = threadIdx.x, n_match = c.pool.n_match;
+    auto wrap = [&](uint32_t at) { return at >= cap ? at - cap : at; };
+    for (uint32_t i = tid; i < cap; i += T) kind[i] = 1u;
+    __syncthreads();
+    for (uint32_t i = tid; i < avail; i += T) kind[P.ring[wrap(ring0 + i)]] = 0u;
+    for (uint32_t i = tid; i < ne; i += T) kind[P.enter[wrap(enter0 + i)]] = 2u;
+    __syncthreads();
+    const PoolDump d(c, slot);
+    for (uint32_t i = tid; i < cap; i += T) {
+        const uint32_t head = P.head[i];
+        uint32_t id = 0xFFFFFFFFu;
+        if (kind[i]) id = head & POOL_ROOT ? head & ~POOL_ROOT : (uint32_t)c.B + aggregated_inc(&c.ctl->hand_frames);
+        d.id[i] = id;
+        d.head[i] = head;
+        for (uint32_t k = 0; k < c.pool.words; ++k) d.words[(size_t)k * cap + i] = P.words[k * cap + i];
+        for (uint32_t k = 0; k < n_match; ++k) d.state[(size_t)k * cap + i] = kind[i] == 2u ? 0xFFFFFFFFu : P.state[k * cap + i];
+    }
+    if (tid == 0) atomicOr(&c.ctl->hand_mask, 1u << slot);
+}
+
+// Every 32 rounds, one thread: has another block failed; does this one leave its calls?  pending: it has no more instances to start
+// and more tokens than threads.  (On its own and seldom: the read of the other blocks' count takes a third of a round.)
+__device__ __noinline__ void pool_look(const DevCtx& c, const PoolSizes& z, PoolShared& sh, bool pending) {
+    if (ld_volatile_i32(&c.ctl->status) != 0) sh.stop = 1;
+    if (!pending || z.hand_slots == 0u || sh.stop != 0) return;
+    if (gridDim.x - ld_volatile_u32(&c.ctl->blocks_done.v) > POOL_ACTIVE) {
+        sh.alone = 0ll;
+        return;
+    }
+    const long long now = clock64();
+    if (sh.alone == 0ll) sh.alone = now;
+    else if (now - sh.alone >= z.hand_after) {
+        const uint32_t slot = atomicAdd(&c.ctl->hand_claims, 1u);
+        if (slot < z.hand_slots) {
+            sh.hand = slot + 1u;
+            atomicCAS(&sh.stop, 0, POOL_LEAVE);              // (unless the pool is exhausted in this very round)
+        }
+        sh.alone = now;
+    }
+}
+
 __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ PoolProgram program,
                                                                              const __grid_constant__ PoolSizes z) {
     constexpr uint32_t T = POOL_THREADS;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PoolShared sh;
     const uint32_t tid = threadIdx.x;
-    Pool P;
     {
-        unsigned char* p = smem;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(p);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(smem);
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&program);
         for (uint32_t i = tid; i < sizeof(PoolProgram) / 4; i += T) dst[i] = src[i];
-        P.prog = reinterpret_cast<const PoolProgram*>(p);
-        p += sizeof(PoolProgram);
-        P.regs = reinterpret_cast<int64_t*>(p); p += (size_t)(program.n_regs + 1) * T * 8;
-        P.words = reinterpret_cast<int64_t*>(p); p += (size_t)program.words * z.cap * 8;
-        P.head = reinterpret_cast<uint32_t*>(p); p += (size_t)z.cap * 4;
-        P.state = reinterpret_cast<uint32_t*>(p); p += (size_t)z.n_match * z.cap * 4;
-        P.enter = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2;
-        if (z.match_step < 0) P.match = P.enter + z.cap - 1;
-        else { P.match = reinterpret_cast<uint16_t*>(p); p += (size_t)z.cap * 2; }
-        P.ring = reinterpret_cast<uint16_t*>(p);
     }
+    const Pool P = pool_arrays(smem, z.cap, program.n_regs, program.words, z.n_match, z.match_step);
     for (uint32_t i = tid; i < z.cap; i += T) P.ring[i] = (uint16_t)i;
     P.regs[program.n_regs * T + tid] = 0ll;
     if (tid == 0) {
         sh.entered[0] = sh.entered[1] = sh.matched[0] = sh.matched[1] = sh.taken[0] = sh.taken[1] = sh.freed[0] = sh.freed[1] = 0u;
-        sh.stop = 0;
+        sh.stop = 0; sh.hand = 0u; sh.alone = 0ll;
     }
     for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += T) sh.waves[i] = 0u;
     const long long t_start = clock64();
@@ -434,8 +513,9 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
     PoolThread t{c, z, P, sh, tid};
     t.late_waves = reinterpret_cast<uint32_t*>(c.q[0]);
     t.n_late = z.late_waves;
-    uint32_t ebase = 0, ne = 0, nm = 0, ring0 = 0, avail = z.cap, par = 0;      // frames to enter, completed matches
+    uint32_t ne = 0, nm = 0, ring0 = 0, avail = z.cap, par = 0;      // frames to enter, completed matches
     unsigned long long tokens = 0;
+    bool leaving = false;
     __syncthreads();
     for (uint32_t round = 0;; ++round) {
         // ---- more instances, while few tokens are pending and at most half of the frames are in use
@@ -446,7 +526,7 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
                 P.head[f] = POOL_ROOT | inst;
                 P.words[f] = c.x ? c.x[inst] : (int64_t)c.tree_root[inst];
                 P.state[f] = 0u;
-                P.enter[t.wrap(ebase + ne + tid)] = (uint16_t)f;
+                P.enter[t.wrap(ne + tid)] = (uint16_t)f;
             }
             ib += k; ne += k; avail -= k;
             ring0 = t.wrap(ring0 + k);
@@ -469,22 +549,22 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         // ---- this round's tokens: completed matches for the first warps, frames to enter for the others
         const uint32_t width = pool_width(z, avail);
         const uint32_t mm = min(min(nm, T), z.cont_calls ? width : T), w0 = (mm + 31u) & ~31u;
-        const uint32_t me = min(min(ne, T - w0), z.cont_calls && mm ? (width > mm ? width - mm : 0u) : width);
+        const uint32_t me = leaving ? 0u : min(min(ne, T - w0), z.cont_calls && mm ? (width > mm ? width - mm : 0u) : width);
         uint32_t f = 0xFFFFFFFFu;
         int node = -1;
         if (tid < mm) {
             const uint32_t v = P.match[z.match_step * (int)(nm - 1u - tid)];
             f = v & (POOL_MAX_FRAMES - 1u);
             node = (int)(v >> 13);
-        } else if (tid >= w0 && tid - w0 < me) f = P.enter[t.wrap(ebase + ne - 1u - (tid - w0))];
+        } else if (tid >= w0 && tid - w0 < me) f = P.enter[t.wrap(ne - 1u - (tid - w0))];
         tokens += mm + me;
         t.ring0 = ring0; t.avail = avail; t.ring_tail = t.wrap(ring0 + avail);
-        t.enter0 = t.wrap(ebase + ne - me); t.match0 = nm - mm; t.par = par;
+        t.enter0 = ne - me; t.match0 = nm - mm; t.par = par;
         __syncthreads();
         if (f != 0xFFFFFFFFu) t.run(f, node);
         if (tid == 0) {
             sh.entered[par ^ 1u] = 0u; sh.matched[par ^ 1u] = 0u; sh.freed[par ^ 1u] = 0u; sh.taken[par ^ 1u] = 0u;
-            if ((round & 255u) == 255u && ld_volatile_i32(&c.ctl->status) != 0) sh.stop = 1;       // another block failed
+            if ((round & 31u) == 31u) pool_look(c, z, sh, !more && ib >= ie && ne + nm >= T);
             if (c.tag_mode == RDF_TAGS_FRAME && tokens > 2ull * (z.max_calls + B) + T) {             // more calls than the caller allows
                 set_status(c, RDF_ERR_FRAMES_FULL);
                 sh.stop = 1;
@@ -495,8 +575,17 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         nm = nm - mm + sh.matched[par];
         ring0 = t.wrap(ring0 + sh.taken[par]);
         avail = avail - sh.taken[par] + sh.freed[par];
-        if (sh.stop) break;
+        const int stop = sh.stop;
+        if (stop) {
+            if (stop != POOL_LEAVE || nm == 0) break;        // (completed matches first: what is left are frames to enter and parked operands)
+            leaving = true;
+        }
         par ^= 1u;
+    }
+    if (sh.stop == POOL_LEAVE && ne) {
+        if (tid == 0) { sh.left[0] = ring0; sh.left[1] = avail; sh.left[2] = ne; }
+        __syncthreads();
+        pool_leave(c, smem, sh);
     }
     // ---- counters, and (the block that ends last) the verdict on the capacities of the call
     if (sh.stop == 2 && tid == 0) c.ctl->pool_exhausted = 1;
@@ -515,7 +604,7 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
     if (blockIdx.x == 0 && tid == 0) c.ctl->cyc[0] = clock64() - t_start;
     __threadfence();
     __syncthreads();
-    if (tid == 0) sh.next_chunk = atomicAdd(&c.ctl->blocks_done, 1u);
+    if (tid == 0) sh.next_chunk = atomicAdd(&c.ctl->blocks_done.v, 1u);
     __syncthreads();
     if (sh.next_chunk != gridDim.x - 1u) return;
     __threadfence();
@@ -549,18 +638,78 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
     }
 }
 
-// The call again for the general scheduler, when a block of the pool kernel ran out of frames (recursion deeper than a pool):
-// what that scheduler expects cleared and seeded.
-__global__ void __launch_bounds__(256) rdf_pool_fallback_kernel(const DevCtx c, size_t pair_n, size_t arrived_n, size_t table_n) {
-    if (!c.ctl->pool_exhausted) return;
+// In front of the general scheduler: what the pool kernel could not run (a block ran out of frames: recursion deeper than a
+// pool) is seeded again from the start, what blocks have left is put where that scheduler expects it.  False: nothing to do.
+__device__ __noinline__ bool pool_take_over(const DevCtx& c, uint32_t& generation) {
+    const bool again = c.ctl->pool_exhausted != 0;
+    const uint32_t left = c.ctl->hand_mask;
+    if (!again && (left == 0u || c.ctl->status != 0)) return false;
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i = i0; i < pair_n; i += stride) reinterpret_cast<uint4*>(c.pair_slots)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (size_t i = i0; i < arrived_n; i += stride) c.arrived[i] = 0u;
-    for (size_t i = i0; i < table_n; i += stride) reinterpret_cast<uint4*>(c.table)[i] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-    for (long long b = (long long)i0; b < c.B; b += (long long)stride) seed_instance(c, b);
-    if (i0 == 0) {
-        Control* k = c.ctl;
-        k->invocations = k->tokens = k->store_inserts = k->store_matches = 0ull;
-        k->status = 0; k->waves = k->max_wave_tokens = k->max_depth = 0u;
+    for (size_t i = i0; i < c.pool.pair_n; i += stride) reinterpret_cast<uint4*>(c.pair_slots)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = i0; i < c.pool.arrived_n; i += stride) c.arrived[i] = 0u;
+    for (size_t i = i0; i < c.pool.table_n; i += stride) reinterpret_cast<uint4*>(c.table)[i] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    if (again) {
+        for (long long b = (long long)i0; b < c.B; b += (long long)stride) seed_instance(c, b);
+        if (i0 == 0) {
+            Control* k = c.ctl;
+            k->invocations = k->tokens = k->store_inserts = k->store_matches = 0ull;
+            k->status = 0; k->waves = k->max_wave_tokens = k->max_depth = 0u;
+        }
+        return grid_barrier(c, &c.ctl->bar.v, generation);
     }
+    // frame ids: every call that the pools have made counts as one (those that have come over have the first ones), so that the
+    // table is full after as many calls as ever
+    if (i0 == 0) c.ctl->frame_count.v = (uint32_t)c.B + (uint32_t)c.ctl->invocations;
+    if (!grid_barrier(c, &c.ctl->bar.v, generation)) return false;
+    const uint32_t cap = c.pool.cap;
+    for (size_t i = i0; i < (size_t)32 * cap; i += stride) {
+        const uint32_t slot = (uint32_t)(i / cap), f = (uint32_t)(i % cap);
+        if (!((left >> slot) & 1u)) continue;
+        const PoolDump d(c, slot);
+        const uint32_t id = d.id[f], head = d.head[f];
+        if (id == 0xFFFFFFFFu) continue;
+        const bool root = head & POOL_ROOT;
+        const uint32_t label = root ? 0u : (head >> 16) & 63u;
+        uint64_t tag;
+        if (c.tag_mode == RDF_TAGS_FRAME) {
+            tag = id;
+            Frame fr;
+            fr.parent = root ? LEAF_MARK : d.id[head & 0xFFFFu]; fr.label = label; fr.arg = d.words[f];
+            c.frames[tag] = fr;
+            const int n_args = root ? 1 : c.labels[label].n_args;
+            for (int k = 1; k < n_args; ++k) c.frame_args[(size_t)tag * 2 + k - 1] = d.words[(size_t)k * cap + f];
+        } else {
+            uint64_t path = 0;
+            uint32_t depth = 0, q = f;
+            while (!(d.head[q] & POOL_ROOT) && depth < 64u) {
+                path |= (uint64_t)((d.head[q] >> 16) & 63u) << (c.label_bits * depth++);
+                q = d.head[q] & 0xFFFFu;
+            }
+            tag = path_root((long long)(d.head[q] & ~POOL_ROOT)) | (uint64_t)depth << RDF_DEPTH_SHIFT | path;
+        }
+        if (d.state[f] == 0xFFFFFFFFu) {
+            const uint32_t at = atomicAdd(&c.ctl->qcount[0].v, 1u);
+            if (at >= c.qcap) {
+                set_status(c, RDF_ERR_QUEUE_FULL);
+                continue;
+            }
+            store_token(&c.q[0][at], tag, d.words[f], (uint32_t)(root ? c.result_entry_pc : c.labels[label].entry_pc));
+            atomicAdd(&c.ctl->tokens, ~0ull);                // (counted when the call was made, and once more when it is run)
+            continue;
+        }
+        for (int n = 0; n < c.n_match; ++n) {
+            const MatchNode M = c.match[n];
+            const uint32_t there = d.state[(size_t)n * cap + f] & 0xFFu;
+            if (there == (1u << M.n_ports) - 1u) continue;   // (has fired)
+            for (int p = 0; p < M.n_ports; ++p) {
+                if (!((there >> p) & 1u)) continue;
+                const int64_t v = d.words[(size_t)(c.pool.word0 + M.port_base + p) * cap + f];
+                StoreCounters sc;                            // (they have been counted)
+                int64_t regs[3];
+                if (c.tag_mode == RDF_TAGS_FRAME) dense_deliver(c, M, n, tag, p, v, regs, sc);
+                else if (hash_insert_or_consume(c, n, tag, v, regs[0], sc) < 0) set_status(c, RDF_ERR_STORE_FULL);
+            }
+        }
+    }
+    return grid_barrier(c, &c.ctl->bar.v, generation);
 }

@@ -558,19 +558,19 @@ def _evaluate(functions, x):
     """The program by direct recursion over its expressions: (value, calls)."""
     calls = [0]
 
-    def call(k, a):
+    def call(k, *args):
         fn, memo = functions[k], {}
 
         def ev(i):
             if i not in memo:
                 op, p, q, s, imm = fn.exprs[i]
                 if op == bd.OP_PARAM:
-                    memo[i] = a
+                    memo[i] = args[imm]
                 elif op == bd.OP_CONST:
                     memo[i] = imm
                 elif op == bd.OP_CALL:
                     calls[0] += 1
-                    memo[i] = call(imm, ev(p))
+                    memo[i] = call(imm, *[ev(e) for e in (p, q, s)[:functions[imm].n_params]])
                 elif op == bd.OP_IF:
                     memo[i] = ev(q) if ev(p) else ev(s)
                 else:
@@ -821,3 +821,115 @@ def test_queue_bound_at_the_end_of_a_narrow_stretch():
         return 0
     assert code(g, x, 2 * 8361, 100) == -7 and code(g, x, 2 * 8361, 8361) == 0
     assert code(chain, long, 6 * 5001, 5) == -7 and code(chain, long, 6 * 5001, 6) == 0
+
+
+# ------------------------------------------- a long instance among short ones
+def _wide_program(kind):
+    """Recursions that fill a pool: binary under path and frame tags, three operands per match, a parameter read behind a
+    condition that waited for a call, several matches per body, calls of other functions behind a match."""
+    if kind == "tail":
+        return _tail_to_another()
+    r = rdf.Function("result", 1)
+    r.ret(r.add(r.call(1, r.param()), r.const(2)))
+    f = rdf.Function("f", 1)
+    n = f.param()
+    m = f.sub(n, f.const(1))
+    small = f.lt(n, f.const(1))
+    if kind == "binary":
+        f.ret(f.if_(small, f.const(1), f.sub(f.mul(f.call(1, m), f.const(3)), f.call(1, m))))
+        return [r, f]
+    if kind == "ternary":
+        g = rdf.Function("g", 3)
+        g.ret(g.add(g.sub(g.param(0), g.param(1)), g.mul(g.param(2), g.const(2))))
+        f.ret(f.if_(small, n, f.call(2, f.call(1, m), n, f.add(f.call(1, m), f.const(1)))))
+        return [r, f, g]
+    if kind == "late":
+        g = rdf.Function("g", 1)
+        g.ret(g.rem(g.param(), g.const(3)))
+        two = f.add(f.call(1, f.sub(n, f.const(1))), f.call(1, f.sub(n, f.const(1))))
+        f.ret(f.if_(small, f.const(1), f.if_(f.lt(f.call(2, n), f.const(5)), two, n)))
+        return [r, f, g]
+    a, b, c = f.call(1, m), f.call(1, m), f.call(1, f.sub(n, f.const(3)))
+    f.ret(f.if_(small, n, f.add(f.max(a, f.mul(b, f.const(2))), c)))          # "matches"
+    return [r, f]
+
+
+@pytest.mark.parametrize("kind,mode,big", [("binary", rdf.TAGS_PATH, 16), ("binary", rdf.TAGS_FRAME, 17), ("tail", rdf.TAGS_PATH, 15), ("tail", rdf.TAGS_FRAME, 16),
+                                           ("ternary", rdf.TAGS_FRAME, 16), ("late", rdf.TAGS_FRAME, 16), ("matches", rdf.TAGS_FRAME, 15)])
+@pytest.mark.parametrize("n_big", [1, 5, 12])
+def test_long_instances_are_left_to_the_device(kind, mode, big, n_big):
+    """A few instances with most of the calls of a batch: their blocks leave them to the general scheduler when (nearly) all other
+    blocks are done -- frames, parked operands and calls to be entered.  Values and counts are those of the program."""
+    fs = _wide_program(kind)
+    memo = {v: _evaluate(fs, v) for v in (0, 1, 2, 3, 4)}
+    memo[big] = _evaluate(fs, big)
+    xs = np.random.default_rng(big).integers(0, 5, size=70)
+    xs[np.random.default_rng(n_big).permutation(70)[:n_big]] = big
+    calls = int(sum(memo[v][1] for v in xs))
+    g = rdf.Graph(fs, 0, mode)
+    x = torch.from_numpy(xs).cuda()
+    for bound in (calls, 3 * calls):
+        y, _ = g.eval_int(x, max_invocations=bound)
+        st = g.stats()
+        assert y.tolist() == [memo[v][0] for v in xs]
+        assert st["invocations"] == calls and st["tokens"] == calls + 70
+        left = st["max_wave_tokens"] == bound + 70           # (the bound it reports for a call that two executors share)
+        assert left or n_big > 1 or kind == "matches", st
+    general = rdf.Graph(fs, 0, mode)
+    general.set_limits(wave_limit=1 << 20)
+    general.eval_int(x, max_invocations=calls)
+    gs = general.stats()
+    assert {k: st[k] for k in ("store_inserts", "store_matches", "max_depth")} == {k: gs[k] for k in ("store_inserts", "store_matches", "max_depth")}
+    assert gs["waves"] <= st["waves"] and gs["max_wave_tokens"] <= st["max_wave_tokens"]
+    if mode == rdf.TAGS_FRAME:                    # one call too many is a status code
+        code = 0
+        try:
+            g.eval_int(x, max_invocations=calls - 1)
+        except rdf.RdfError as e:
+            code = e.code
+        assert code == -6
+
+
+def _ms(g, x, calls, n=5):
+    for _ in range(3):
+        g.eval_int(x, max_invocations=calls, check=False)
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    e[0].record()
+    for _ in range(n):
+        g.eval_int(x, max_invocations=calls, check=False)
+    e[1].record()
+    torch.cuda.synchronize()
+    g.stats()
+    return e[0].elapsed_time(e[1]) / n
+
+
+@pytest.mark.parametrize("big", [24, 27, 30])
+def test_one_long_instance_takes_no_longer_than_in_waves(big):
+    """64 calls of fib(5), one of them fib(30) (2.7 M calls): against the general scheduler alone (a wave limit selects it)."""
+    x = torch.full((64,), 5, dtype=torch.int64, device="cuda")
+    x[40] = big
+    calls = 63 * 15 + 2 * _fib_iter(big + 1) - 1
+    pool, waves = rdf.Graph(*rdf.fib_program(), rdf.TAGS_FRAME), rdf.Graph(*rdf.fib_program(), rdf.TAGS_FRAME)
+    waves.set_limits(wave_limit=1 << 20)
+    ms = _ms(pool, x, calls), _ms(waves, x, calls)
+    print("fib", big, "ms", ms)
+    assert ms[0] <= 1.5 * ms[1], ms               # (the time it runs on its own, and one wave per depth of what is left)
+
+
+@pytest.mark.parametrize("mode", [rdf.TAGS_PATH, rdf.TAGS_FRAME])
+def test_first_call_of_a_graph_under_capture(mode):
+    """Nothing in a call's launch needs an earlier call outside the capture."""
+    rdf.Graph(*rdf.tak_program(), rdf.TAGS_FRAME).eval_int(torch.zeros(1, dtype=torch.int64, device="cuda"), max_invocations=100)   # (library start-up)
+    x = torch.arange(64, dtype=torch.int64, device="cuda") % 16
+    y = torch.zeros_like(x)
+    g = rdf.Graph(*rdf.fib_program(), mode)
+    cg = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(cg):
+        g.eval_int(x, max_invocations=100000, check=False, y=y)
+    for shift in (0, 3):
+        x.copy_((torch.arange(64, device="cuda") + shift) % 16)
+        y.zero_()
+        cg.replay()
+        torch.cuda.synchronize()
+        assert y.tolist() == [_fib_iter(int(v)) for v in x]
