@@ -13,6 +13,7 @@
 
 #include "rdf_cluster.cuh"
 #include "rdf_exec.h"
+#include "rdf_math.cuh"
 #include "rdf_tc.cuh"
 #include "rdf_tc_dw.cuh"
 
@@ -836,15 +837,6 @@ __device__ __forceinline__ void lstm_backward_frame(const DevCtx& c, uint32_t t,
             }
         }
     }
-}
-
-// tanh to a few units in the last place without a branch, so that independent ones overlap: x from -0.55 to 0.55 by Lambert's
-// continued fraction x / (1 + x^2 / (3 + x^2 / (5 + x^2 / (7 + x^2 / 9)))) as a quotient of polynomials, else 1 - 2 / (e^2|x| + 1).
-__device__ __forceinline__ float tanh_select(float x) {
-    const float y = x * x, a = fabsf(x);
-    const float small = x * __fdividef(fmaf(y, y + 105.f, 945.f), fmaf(y, fmaf(y, 15.f, 420.f), 945.f));
-    const float large = 1.f - __fdividef(2.f, expf(fminf(2.f * a, 40.f)) + 1.f);
-    return a < 0.55f ? small : copysignf(large, x);
 }
 
 // A (bf16 TreeLSTM): the gate gradients as bf16 operand rows in list order; dc goes straight to the callee frames.
