@@ -1730,7 +1730,9 @@ extern "C" int rdf_grad(rdf_graph* g, const rdf_batch* in, const rdf_params* par
             const int smem_mma = 2 * LM_ROWS * (c.Hp * 2 + 16);
             CUDA_OK(cudaFuncSetAttribute(rdf_loss_heads_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_mma));
             RDF_KERNEL(S, rdf_loss_heads_mma_kernel<<<loss_blocks, 256, smem_mma, stream>>>(c));
-        } else if (params->n_classes <= 5 && H <= 384) {       // (wider rows, more classes: too many registers for rows and sums)
+        } else if (params->n_classes <= 5 && H <= 384) {
+            // (built for up to 5 classes; the slab form takes the others, up to 8, and rows beyond 384 units, whose four rows and
+            // sums do not fit the registers: 175 of 255 at 384)
             if (H <= 128) RDF_KERNEL(S, rdf_loss_rows_kernel<1, 5><<<loss_blocks, 256, 0, stream>>>(c));
             else if (H <= 256) RDF_KERNEL(S, rdf_loss_rows_kernel<2, 5><<<loss_blocks, 256, 0, stream>>>(c));
             else RDF_KERNEL(S, rdf_loss_rows_kernel<3, 5><<<loss_blocks, 256, 0, stream>>>(c));

@@ -565,3 +565,16 @@ def test_queue_bound_of_structural_recursion(cell, monkeypatch):
             assert code(dt, dp, bound) == code(dt, dp, bound, trace_capacity=2 * tb.N + 64) == (0 if bound >= width or width <= 1024 else -7)
         assert B < 700 or width > 1024
         assert torch.equal(g.eval_trees(dt, dp)[0], h)
+
+
+@pytest.mark.parametrize("cell,compute,H,C", [("rnn", rdf.F32, 60, 2), ("rnn", rdf.F32, 132, 3), ("rnn", rdf.F32, 260, 4), ("rnn", rdf.F32, 60, 6), ("rnn", rdf.F32, 256, 8),
+                                              ("rnn", rdf.F32, 388, 3), ("lstm", rdf.F32, 100, 3), ("lstm", rdf.F32, 100, 7), ("rnn", rdf.BF16, 100, 2),
+                                              ("rnn", rdf.BF16, 100, 8), ("lstm", rdf.BF16, 64, 3), ("lstm", rdf.BF16, 64, 8)])
+def test_loss_head_class_counts(cell, compute, H, C):
+    """Every form of the loss head with fewer classes than it is built for (padded) and with as many as the library takes."""
+    rng = np.random.default_rng(H + C)
+    bf16 = compute == rdf.BF16
+    p = (workloads.treernn_params if cell == "rnn" else workloads.treelstm_params)(3, 70, H, H, n_classes=C, bf16=bf16)
+    p["b_s"] = np.asarray(0.25 * np.arange(C) - 0.5, dtype=np.float32)
+    tb = workloads.tree_batch_from_shapes([workloads.random_split_shape(rng, int(L)) for L in rng.integers(1, 30, 40)], 7, vocab=70, n_classes=C)
+    check_grad({"trees": tb, "params": p}, compute, cell=cell)
