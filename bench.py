@@ -35,7 +35,7 @@ import workloads  # noqa: E402
 METRIC = "recursive_invocations_per_sec"
 UNIT = "invocations/s"
 WORKLOAD_NAMES = {
-    1: "config1: fib(n), 1024 calls, n~U[0,18], int64, packed path tags, forward",
+    1: "config1: fib(n), 1024 calls, n~U[0,18], int64, path tags, forward",
     2: "config2: TreeRNN forward, 512 random binary trees, H=64, fp32",
     3: "config3: TreeRNN forward+backward, 8192 trees (lognormal leaves, median 18), H=300, vocab 21000, 5-class loss at every node",
     4: "config4: binary TreeLSTM forward+backward, 8192 trees (same size mix), H=300, vocab 21000, 5-class loss at every node",
@@ -492,10 +492,13 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
                      "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak if peak else None, "peak_source": src,
                      "traffic": traffic.get((kernel, workload))})
 
-    fib = "rdf_pool_kernel" if getattr(case, "store", "thread") == "thread" else "rdf_scheduler_kernel"
-    add({"fib": fib, "topdown": "rdf_scheduler_kernel"}.get(case.cfg["kind"], "rdf_fold_kernel"), "schedule", "hbm", 128.0 * N,
-        "128 B per invocation: call token write+read, return token / store slot write+read, frame record")
     if case.cfg["kind"] == "fib":
+        if case.store == "thread":              # (the hash store belongs to the general scheduler)
+            add("rdf_pool_kernel", "schedule", "hbm", 16.0 * len(case.cfg["x"]),
+                "16 B per instance: argument read, result written (frames, tokens and operands stay in shared memory)")
+        else:
+            add("rdf_scheduler_kernel", "schedule", "hbm", 128.0 * N,
+                "128 B per invocation: call token write+read, return token / store slot write+read, frame record")
         return rows
     if case.cfg["kind"] == "topdown":
         rows.clear()
@@ -507,6 +510,8 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     Hp = 64 * ((H + 63) // 64)
     lstm = case.cell == "lstm"
     mm = "tensor" if case.use_tc else "alu"
+    add("rdf_fold_kernel", "schedule", "hbm", N * 36.0 + C * 20.0 + Lf * 8.0,
+        "per invocation: node words read, frame record and operand words written; list entry of a cell / leaf written")
     if not case.use_tc and not lstm:
         add("rdf_group_kernel", "group", "hbm", 48.0 * C, "16 B cell record read twice and written once")
     add("rdf_operator_kernel", "operators", mm, case.flops_fwd(),
@@ -514,7 +519,8 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     add("rdf_gather_roots_kernel", "roots", "hbm", tb.B * H * (4.0 + (2 if case.use_tc and not lstm else 4)), "root rows read and written")
     if case.grad:
         rowbytes = Hp * 2 if case.use_tc else H * 4 * (2 if lstm else 1)
-        add("rdf_loss_heads_kernel", "loss", "hbm", float(N) * (rowbytes + 32), "one state row read + 32 B of dlog written per invocation")
+        head = "rdf_loss_heads_mma_kernel" if case.use_tc else "rdf_loss_rows_kernel" if H <= 384 else "rdf_loss_heads_kernel"
+        add(head, "loss", "hbm", float(N) * (rowbytes + 32), "one state row read + 32 B of dlog written per invocation")
         bwd = C * 2.0 * H * (2 * H) * (5 if lstm else 1)
         add("rdf_backward_kernel", "backward", mm, bwd, "operand-gradient contraction W^T dz: 2*H*2H per cell" + (" (x5 gates)" if lstm else ""))
         dw = bwd + (Lf * 2.0 * H * 3 * H if lstm else 0.0)
@@ -647,7 +653,8 @@ def run(args):
         "dtype": case.dtype, "data": "synthetic",
         "config": {"workload": WORKLOAD_NAMES[args.workload] + (f" [scaled: {args.fib_batch} calls]" if args.fib_batch and args.workload == 1 else "")
                    + (f" [reduced: {args.override}]" if args.override else "")
-                   + (f" [store: {args.store} probes" + (f", load {args.hash_load}" if args.hash_load else "") + "]" if args.workload == 1 else ""),
+                   + (f" [store: {args.store} probes" + (f", load {args.hash_load}" if args.hash_load else "") + "]"
+                      if args.workload == 1 and args.store != "thread" else ""),
                    "invocations_per_step": case.N, "instances": cfg.get("B") or cfg["trees"].B,
                    "pass": "forward+backward" if cfg.get("grad") else "forward",
                    "timing": "CUDA events per step; 256 MB L2 flush between steps; inputs and parameters resident"},
