@@ -203,11 +203,14 @@ typedef struct {
     int32_t      H, D, V, n_classes;
     int32_t      reproducible;   /* rdf_grad with RDF_BF16 on the tensor-core path: 1 = the parameter gradients and the loss
                                     come out bit for bit the same on every call with the same inputs (the cells are put in
-                                    an order that depends on the input alone -- by call depth, then by the argument of the
-                                    invocation -- every floating-point sum has a fixed order, and the sums that many thread
-                                    blocks contribute to are exact integer sums in fixed point).  Slower; 0 = sums by
-                                    atomics in arrival order (equal up to rounding).  Invocations of one depth that share
-                                    an argument (a node reached twice) keep their arrival order.  UNSUPPORTED elsewhere. */
+                                    an order that depends on the input alone, every floating-point sum has a fixed order,
+                                    and the sums that many thread blocks contribute to are exact integer sums in fixed
+                                    point).  The order is by call depth; within a depth, structural recursion over the
+                                    input trees has the instances in the order of tree_root and each one's invocations
+                                    from left to right (another order of the same trees may change the last bits), other
+                                    programs the order of the invocations' arguments, where invocations that share an
+                                    argument (a node reached twice) keep their arrival order.  Slower; 0 = sums by atomics
+                                    in arrival order (equal up to rounding).  UNSUPPORTED elsewhere. */
     const float* E;              /* [V, D]                                          */
     const float* W;              /* TreeRNN [H, 2H]; TreeLSTM [5H, 2H] (i, f_l, f_r, o, u) */
     const float* b;              /* [H] or [5H]                                     */
@@ -359,10 +362,12 @@ int rdf_set_limits(rdf_graph* g, long long wait_cycles, long long wave_limit);
  * those events and writes up to `capacity` durations in milliseconds to the
  * host array `ms`, in this order:
  *   0 set-up (clears, program upload, seed tokens, weight packing)
- *   1 scheduler waves (tokens: tag push / pop, matching, lists of ready operators)
- *   2 grouping of the ready cells by height     3 operator waves (batched leaves and cells)
+ *   1 scheduling (tokens: tag push / pop, matching, lists of ready operators; input trees: level by level; integer
+ *     programs: the whole run)
+ *   2 lists and grouping of the cells (by call depth; deep fp32 recursions: by cluster of instances and call depth)
+ *   3 operator waves (batched leaves and cells)
  *   4 root states to the caller's buffer        5 loss head with dW_s, db_s
- *   6 lists of the gradient pass                7 gradient waves
+ *   6 empty (the gradient pass has the lists of the forward pass)   7 gradient waves
  *   8 dW (and dW_x)   9 db   10 dE (TreeLSTM; the TreeRNN's dE is formed during the waves)
  * (rdf_eval fills 0..4).  *n receives the number written. */
 enum { RDF_PHASE_SETUP = 0, RDF_PHASE_SCHEDULE, RDF_PHASE_GROUP, RDF_PHASE_OPERATORS, RDF_PHASE_ROOTS, RDF_PHASE_LOSS,

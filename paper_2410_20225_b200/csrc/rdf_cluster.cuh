@@ -16,8 +16,8 @@
 //   * a block tells the others when it has read the rows of a depth (an mbarrier in each of them), which is waited for
 //     before a push two depths later: nobody runs further ahead.
 // Cells of a depth beyond the first CL_SLOTS go through global memory (a cluster barrier orders those depths).
-// Measured per depth, 64 chains, H = 256 (weights in shared memory and states through L2 -> this): forward 4.9 -> 2.1 us,
-// gradient 5.0 -> 3.1 us.
+// Measured per depth, 64 chains, H = 256 (weights in shared memory and states through L2 -> this): forward 4.7 -> 1.86 us,
+// gradient 5.0 -> 1.96 us.
 #pragma once
 #include "rdf_tc.cuh"
 

@@ -20,9 +20,11 @@
 // call) run without the interpreter, from registers.
 //
 // What bounds it: the latency of a round -- some 400 dependent instructions per warp between two block barriers -- and the
-// frames that fit the shared memory, which limit the tokens of a round.
-// Measured, general scheduler -> this: 131 072 calls of fib(0..18) 36.3 -> 5.5 ms, 1024 calls 0.721 -> 0.17 ms, 8 calls of
-// fib(0..10) 0.137 -> 0.036 ms, 200 calls of tak 1.76 -> 0.75 ms (limited by the depth of the largest instance).
+// frames that fit the shared memory, which limit the tokens of a round.  (16 384 calls of fib(0..18): an instruction issued in
+// 55 % of the cycles, 19.3 warp instructions per call; warps stalled per issue: 2.6 on the fixed latency of the instruction
+// before, 2.2 at the barrier, 1.9 on shared memory.)
+// Measured, general scheduler -> this: 131 072 calls of fib(0..18) 36.3 -> 5.3 ms, 1024 calls 0.72 -> 0.18 ms, 8 calls of
+// fib(0..10) 0.137 -> 0.037 ms, 200 calls of tak 1.75 -> 0.80 ms (limited by the depth of the largest instance).
 // Handing calls of a busy block to idle ones through global memory was built and dropped: 200 calls of tak 0.90 -> 0.83 ms,
 // but 1024 calls of fib 0.23 -> 0.31 ms.
 // (Included by rdf_exec.cu only: it defines kernels.)
@@ -32,10 +34,10 @@
 static const int POOL_THREADS = 768, POOL_PER_SM = 1;   // threads of a block, blocks per SM (131 072 calls of fib: 512 threads 6.7 ms, 768 5.5,
                                                         // 1024 6.2, two blocks of 256 6.7: more threads leave each fewer frames)
 // A block runs its instances to their end, and an instance far larger than the others would keep one block busy long after the
-// device has run out of work (one of fib(30), 2.7 M calls, 22.9 ms).  When at most POOL_ACTIVE blocks are left, one with more tokens
-// pending than threads all the while leaves them to the general scheduler, which spreads a wave over the device: its frames, parked operands and the calls to be entered go there as they
-// are.  Before that it runs as long as the other way costs: some 20 us to get going, and the clearing of the token store
-// (PoolSizes::hand_after).
+// device has run out of work (one of fib(30), 2.7 M calls, 22.9 ms).  When at most POOL_ACTIVE blocks are left, one with more
+// tokens pending than threads all the while leaves them to the general scheduler, which spreads a wave over the device: its
+// frames, parked operands and the calls to be entered go there as they are.  Before that it runs as long as the other way
+// costs: some 20 us to get going, and the clearing of the token store (PoolSizes::hand_after).
 static const uint32_t POOL_ACTIVE = 8;
 static const uint32_t POOL_ROOT = 0x80000000u;          // frame word of an instance's `result` context: | instance
 // Frame word of an invocation: parent frame [15:0], label [21:16], depth of the tag [27:22] (path tags)
