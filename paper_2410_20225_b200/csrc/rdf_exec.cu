@@ -742,11 +742,13 @@ static const int IL_SMEM_W_H = 128;
 // up to IL_CLUSTER_FMA.  How wide the waves get is up to the values (the gate) and the depth limit, so the kernel looks at each
 // wave and leaves the rest of the call to the grid at the first one that is wider.  Besides its faster barrier, the acquire of a
 // grid barrier drops the block's local memory (spilled registers, label arrays) from L1 twice per wave.
-// Grid alone / this / cluster alone, us: 8 seeds, H = 16, depth 10: 523 / 335 / 327; 100, H = 128: 862 / 846 / 915; 20, H = 256,
-// depth 8: 1806 / 1580 / 1586; 64 full trees, H = 128, depth 10: 1031 / 1016 / 7660; 64, H = 128, depth 18: 1636 / 1620 / 2990.
-// The limit on tokens x H x H at 2^23 instead: 100, H = 128: 826, but 20, H = 256: 1687; at 2^25: 927 and 1588.
-static const uint32_t IL_CLUSTER_TOKENS = 8192;
-static const unsigned long long IL_CLUSTER_FMA = 16ull << 20;
+// Grid alone / this / cluster alone, us: 8 seeds, H = 16, depth 10: 523 / 335 / 327; 100, H = 128: 862 / 830 / 915; 20, H = 256,
+// depth 8: 1806 / 1580 / 1586; 64 full trees, H = 128, depth 10: 1031 / 1010 / 7660; 64, H = 128, depth 18: 1636 / 1600 / 2990.
+// Where the lines lie: with tokens x H x H up to 2^24, 500 seeds, H = 100, depth 6 take 584 us (grid 488), with 2^23 20 seeds,
+// H = 256 1687; with up to 8192 tokens 3000 seeds, H = 40, depth 4 take 379 (grid 310, this 318), with 2048 600 seeds, H = 16 533
+// (grid 586, this 484).
+static const uint32_t IL_CLUSTER_TOKENS = 4096;
+static const unsigned long long IL_CLUSTER_FMA = 10ull << 20;
 __host__ __device__ inline bool il_narrow(unsigned long long tokens, int H) {
     return tokens <= IL_CLUSTER_TOKENS && tokens * (unsigned long long)(H * H) <= IL_CLUSTER_FMA;
 }

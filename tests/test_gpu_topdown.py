@@ -139,8 +139,7 @@ def test_topdown_full_size_as_benchmarked():
                                    (20, 4, 440), (124, 4, 110), (124, 4, 112), (132, 4, 120)])
 def test_topdown_hidden_sizes(H, D, B):
     """Hidden sizes on both sides of the warp tiles (16 outputs) and of the switch from weights in shared memory (H <= 128)
-    to weights read through the cache; groups of one and of several warps along the items; one
-    cluster (B (H + 16) < 15500) and the whole grid."""
+    to weights read through the cache; groups of one and of several warps along the items."""
     test_topdown_recursion_states_and_shapes(H, D, B)
 
 
@@ -184,7 +183,7 @@ def _full_trees(B, D, H, V=50):
 @pytest.mark.parametrize("B,D,H", [(1, 9, 128), (3, 12, 16), (8, 9, 100), (40, 6, 256), (1, 1, 4)])
 def test_topdown_waves_that_outgrow_a_cluster(B, D, H):
     """A call that starts in one thread-block cluster and is handed to the whole grid at its first wide wave (tokens x H x H
-    beyond 2^24, or more than 8192 tokens), and one that never gets there: states, invocations and waves."""
+    beyond 10 x 2^20, or more than 4096 tokens), and one that never gets there: states, invocations and waves."""
     g, P, tb, total = _full_trees(B, D, H)
     want = np.array([direct.topdown(P, int(t), D, {}) for t in tb.tok[:B]])
     dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(P)
