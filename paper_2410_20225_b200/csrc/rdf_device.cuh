@@ -96,7 +96,7 @@ struct Control {
     uint32_t hand_claims, hand_mask, hand_frames, scheduler_done;   // blocks that have a place to leave their calls in, that have left
                                                         // them, and the frames these had
     uint32_t wave_tokens[POOL_BINS];                    // tokens per wave of the call
-    uint4    il_state[2];         // interleaved execution: where the grid carries on after a cluster ({wave, cells, left, right done}, {leaves done, widest})
+    uint4    il_state[2];         // interleaved execution: where the grid carries on after a cluster ({wave, cells, left, right done}, {leaves done, widest, 1: nothing is left})
     uint4    fold_state[4];       // rdf_fold.cuh: the level at which the grid carries on after a narrow stretch (two slots)
 };
 static_assert(sizeof(Control) <= 4096, "the control block is 4 KB");

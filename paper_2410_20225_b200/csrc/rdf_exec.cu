@@ -810,10 +810,13 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
     __shared__ SharedProgram sp;
     extern __shared__ __align__(16) unsigned char il_smem[];
     const uint4 from = c.ctl->il_state[0], from2 = c.ctl->il_state[1];         // (zeros unless a cluster has run waves of this call)
-    if (!CLUSTER && (c.ctl->status != 0 || c.ctl->qcount[from.x % 3u].v == 0u)) return;
+    // The cluster's own word that it has ended the call.  (Not the status word: a faster block may be in the first wave already and
+    // set an error there, and a block goes on or leaves as a whole.)
+    if (!CLUSTER && from2.z != 0u) return;
     load_program(c, sp);
     ThreadStats st;
     uint32_t generation = 0, wave = from.x, widest = from2.y, done[3] = {from.y, from.z, from.w}, done_leaves = from2.x;   // cells, left, right unary operators
+    bool wide = false;
     long long cyc_s = 0, cyc_o = 0, cyc_b = 0, t_mark = clock64();
     auto lap = [&](long long& acc) {
         const long long now = clock64();
@@ -851,7 +854,8 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
             set_status(c, RDF_ERR_WAVE_LIMIT);
             break;
         }
-        if (CLUSTER && !il_narrow(n, H)) break;
+        wide = CLUSTER && !il_narrow(n, H);
+        if (wide) break;
         widest = max(widest, n);
         if (blockIdx.x == 0 && threadIdx.x == 0) c.ctl->qcount[(wave + 2) % 3].v = 0;
         const Token* q = c.q[wave & 1];
@@ -927,7 +931,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
         c.ctl->cyc[0] += cyc_s; c.ctl->cyc[1] += cyc_o; c.ctl->cyc[2] += cyc_b;
         if (CLUSTER) {
             c.ctl->il_state[0] = make_uint4(wave, done[0], done[1], done[2]);
-            c.ctl->il_state[1] = make_uint4(done_leaves, widest, 0u, 0u);
+            c.ctl->il_state[1] = make_uint4(done_leaves, widest, wide ? 0u : 1u, 0u);
         }
         c.ctl->forward_status = c.ctl->status;
     }

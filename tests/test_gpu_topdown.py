@@ -194,6 +194,19 @@ def test_topdown_waves_that_outgrow_a_cluster(B, D, H):
         assert np.abs(h - want).max() / np.abs(want).max() <= TOL
 
 
+def test_topdown_errors_behind_a_cluster():
+    """Calls that a cluster hands to the whole grid and that end with a status there, some in the first wave the grid runs: every
+    block leaves, and the next call has the states of an undisturbed one."""
+    g, P, tb, total = _full_trees(8, 9, 100)
+    dt, dp = rdf.Graph.device_trees(tb), rdf.Graph.device_params(P)
+    want = g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0]
+    for m in list(range(8 * 31, total, 173)) + [total - 1]:
+        with pytest.raises(rdf.RdfError) as e:
+            g.eval_trees(dt, dp, rdf.F32, max_invocations=m)
+        assert e.value.code == -6, m
+    assert torch.equal(g.eval_trees(dt, dp, rdf.F32, max_invocations=total)[0], want)
+
+
 def test_topdown_wide_waves_of_few_seeds_use_the_device():
     """64 seeds that grow full trees (waves of 65 536 tokens) take no longer than 512 of them."""
     ms = []
