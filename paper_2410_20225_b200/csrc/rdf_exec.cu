@@ -961,6 +961,7 @@ __global__ void __launch_bounds__(256) rdf_seed_kernel(const DevCtx c) {
     if (b < c.B) seed_instance(c, b);
 }
 
+#include "rdf_lanes.cuh"
 #include "rdf_pool.cuh"
 
 // The operator kernel: the leaves first (they wait for nothing), then the cells in waves whose operands are complete;
@@ -1683,6 +1684,17 @@ int rdf_check_common(rdf_graph* g, const rdf_batch* in, const rdf_params* params
 static const long long POOL_CALLS = 40000, POOL_MANY = 32;
 static const uint32_t POOL_MIN_FRAMES = 15 * POOL_THREADS / 4;   // (bodies of up to three operators with two operands each)
 
+// The lane executor (rdf_lanes.cuh) for the programs it takes, unless a few instances may hold most of a large number of calls: a
+// block has 300 000 calls a millisecond, and one that leaves its calls has them less spread out than a pool (64 calls, one of them
+// fib(27) and the rest fib(5): 0.70 ms, with the pool executor in front 0.53).  Operators that are calls make so many waves that the
+// general scheduler is no help (one call of tak(18, 12, 6), 63 609 calls in 150 waves: 1.20 ms in waves, 0.36).
+static const long long LANE_CALLS = 100000, LANE_TAIL_CALLS = 400000;
+static bool lane_takes(const rdf_graph* g, const rdf_batch* in, const ExecState* S) {
+    if (!g->lanes || in->B >= (1ll << 30)) return false;
+    if (in->max_invocations <= LANE_CALLS || in->B >= S->grid) return true;
+    return g->lane_prog.cont == PI_CALL && in->max_invocations <= LANE_TAIL_CALLS * in->B;
+}
+
 static size_t pool_smem_bytes(const ExecState* S) { return std::min<size_t>(S->smem_per_sm / POOL_PER_SM - 1024, S->smem_per_block) - sizeof(PoolShared) - 256; }
 static uint32_t pool_frames(const PoolProgram& P, const ExecState* S) {
     const size_t fixed = pool_fixed_bytes(P), smem = pool_smem_bytes(S);
@@ -1732,6 +1744,47 @@ static int rdf_launch_pool(rdf_graph* g, const rdf_batch* in, const Layout& L, E
     return RDF_OK;
 }
 
+typedef void (*LaneKernel)(const DevCtx, const LaneProgram, const LaneSizes);
+static LaneKernel lane_kernel(const LaneProgram& P) {
+    static const LaneKernel k[2][3] = {{rdf_lanes_kernel<1, 2>, rdf_lanes_kernel<2, 2>, rdf_lanes_kernel<3, 2>},
+                                       {rdf_lanes_kernel<1, 3>, rdf_lanes_kernel<2, 3>, rdf_lanes_kernel<3, 3>}};
+    return k[P.n_ports - 2][P.n_args - 1];
+}
+static int rdf_launch_lanes(rdf_graph* g, const rdf_batch* in, const Layout& L, ExecState* S, DevCtx& c, bool& fallback, cudaStream_t stream) {
+    const LaneProgram& P = g->lane_prog;
+    const bool path = g->tag_mode == RDF_TAGS_PATH;
+    const size_t room = std::min<size_t>(S->smem_per_sm - 1024, S->smem_per_block) - sizeof(LaneShared) - 256 - lane_fixed_bytes();
+    LaneSizes z{};
+    z.cap = (uint32_t)std::min<size_t>(room / lane_frame_bytes(P.n_args, P.n_ports), POOL_MAX_FRAMES) & ~7u;
+    z.max_depth = path ? (uint32_t)(RDF_PATH_BITS / g->label_bits) : LN_NONE;
+    z.reserve = (path ? z.max_depth : 64u) + 2u;
+    z.max_calls = (unsigned long long)in->max_invocations;
+    z.max_parked = (unsigned long long)L.table_cap;
+    const bool few_waves = in->max_invocations < POOL_BINS || (path && P.cont != PI_CALL);
+    z.late_waves = few_waves ? 0u : (uint32_t)std::min<long long>(in->max_invocations, 65536);
+    if (z.late_waves) CUDA_OK(cudaMemsetAsync(c.q[0], 0, (size_t)z.late_waves * sizeof(uint32_t), stream));
+    const int grid = (int)std::min<long long>(S->grid, in->B);
+    z.first_wait = in->B < 2ll * grid * LN_WARPS ? LN_FIRST_WAIT : 0u;
+    // what a block may leave: its frames, the calls they have not made, its tokens and stocks, and the `result` contexts of these
+    c.pool.cap = z.cap * (uint32_t)P.n_ports + 4u * LN_THREADS;
+    c.pool.words = (uint32_t)g->pool_prog.words; c.pool.word0 = (uint32_t)g->pool_prog.word0; c.pool.n_match = 1;
+    c.pool.slot_bytes = pool_dump_bytes(g->pool_prog, c.pool.cap); c.pool.max_parked = z.max_parked;
+    c.pool.pair_n = L.pair_bytes / sizeof(Slot); c.pool.arrived_n = L.arrived_bytes / sizeof(uint32_t); c.pool.table_n = L.table_bytes / sizeof(Slot);
+    if (in->max_invocations > LANE_CALLS && S->hash_slots == 0) {
+        z.hand_slots = (uint32_t)std::min<size_t>(POOL_ACTIVE, (size_t)L.qcap * sizeof(Token) / c.pool.slot_bytes);
+        z.hand_after = (long long)((double)(L.pair_bytes + L.arrived_bytes + L.table_bytes) / 6e9 * S->clock_khz);      // (at 6 TB/s)
+        fallback = fallback || z.hand_slots > 0;
+    }
+    z.fallback = fallback;
+    rdf_mark(S, 1, stream);
+    const LaneKernel kernel = lane_kernel(P);
+    const size_t smem = lane_fixed_bytes() + z.cap * lane_frame_bytes(P.n_args, P.n_ports);
+    CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RDF_KERNEL(S, kernel<<<grid, LN_THREADS, smem, stream>>>(c, P, z));
+    CUDA_OK(cudaGetLastError());
+    return RDF_OK;
+}
+
 // zero what must start at zero, upload the program, seed, run all waves
 int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char* ws, const Layout& L, ExecState* S,
                        DevCtx& c, cudaStream_t stream) {
@@ -1745,14 +1798,15 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
     const bool fold = g->fold && !out->trace && any_width;
     // Integer programs run out of shared memory.  The general scheduler has what that executor does not: trace records, a
     // bound on the width of a wave, the waits and waves that rdf_set_limits limits, and the cooperative probes.
+    const bool lanes = lane_takes(g, in, S);
     const bool pool = g->pool && !out->trace && pool_frames(g->pool_prog, S) >= POOL_MIN_FRAMES && S->wait_cycles == 0 &&
                       S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
                       any_width &&
-                      (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B);
+                      (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B || lanes);
     if (pool) {
         // bounded depth, one match per frame: a pool always suffices (should it not, the call ends with a status)
         bool fallback = !(g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1);
-        const int rc = rdf_launch_pool(g, in, L, S, c, fallback, stream);
+        const int rc = lanes ? rdf_launch_lanes(g, in, L, S, c, fallback, stream) : rdf_launch_pool(g, in, L, S, c, fallback, stream);
         if (rc != RDF_OK) return rc;
         if (!fallback) {
             for (int k = 2; k <= 5; ++k) rdf_mark(S, k, stream);

@@ -1323,6 +1323,72 @@ struct PoolBuilder {
         }
     }
 
+    // One function, entered from `result` and from its own calls; one operator with two or three operands, each of them a call.
+    bool lane_shape(LaneProgram& q) const {
+        try {
+            if (out.n_match != 1 || out.match[0].n_ports > 3) return false;
+            const PoolInstr& top = out.code[out.result_entry];
+            need(top.op == PI_CALL && top.n_run == 1 && top.last);
+            const PoolLabel& first = out.labels[top.imm];
+            need(first.fast >= 0 && first.k_kind == K_SEG);
+            const PoolInstr& end = out.code[first.k_pc];
+            need(end.op == PI_OUT && end.ra == 0);
+            const PoolEntry& e = out.entry_of[first.fast];
+            const PoolCont& k = out.cont_of[0];
+            need(k.op != PI_HALT && e.n_cond > 0);
+            auto op = [](const PoolOperand& o) {
+                LaneOperand r{};
+                if (o.reg < 3) r.mask[o.reg] = ~0ull;
+                r.imm = o.imm;
+                return r;
+            };
+            q = LaneProgram{};
+            q.n_args = e.n_args; q.n_ports = out.match[0].n_ports;
+            q.n_cond = e.n_cond; q.call_at = q.ret_at = -1;
+            q.out_imm = end.ia;
+            q.label[3] = top.imm;
+            q.root[0] = op(plain(top.ra, top.ia, 1));
+            if (e.n_args > 1) q.root[1] = op(plain(top.rb, top.ib, 1));
+            if (e.n_args > 2) q.root[2] = op(plain(top.rc, top.ic, 1));
+            for (int c = 0; c < e.n_cond; ++c) { q.cmp[c] = e.cmp[c]; q.a[c] = op(e.a[c]); q.b[c] = op(e.b[c]); }
+            int calls = 1, returns = 0, order[3] = {-1, -1, -1};            // order[port]: which call feeds it
+            for (int c = 0; c <= e.n_cond; ++c) {
+                const PoolAction& act = e.act[c];
+                if (act.n_calls == 0) {
+                    if (returns) q.ret_at = c;
+                    q.ret[returns++] = op(act.ops[0]);
+                    continue;
+                }
+                need(q.call_at < 0 && act.n_calls == q.n_ports);
+                q.call_at = c;
+                for (int i = 0; i < act.n_calls; ++i) {
+                    const PoolLabel& L = out.labels[act.labels[i] & 0xFF];
+                    need(L.entry == first.entry && L.k_kind == K_PORT && L.k_node == 0 && L.k_port < q.n_ports && order[L.k_port] < 0);
+                    order[L.k_port] = i;
+                    q.port[i] = L.k_port;
+                    q.label[i] = act.labels[i] & 0xFF;
+                    for (int j = 0; j < 3; ++j) q.call[3 * i + j] = op(act.ops[3 * i + j]);
+                    ++calls;
+                }
+            }
+            need(q.call_at >= 0);
+            auto by_call = [&](PoolOperand o) { return op(PoolOperand{o.reg < q.n_ports ? order[o.reg] : 3, o.imm}); };
+            q.cont = k.op; q.cont_imm = k.imm;
+            if (k.op == PI_CALL) {
+                // (a call's depth is its wave otherwise, which rdf_lanes.cuh relies on where the depth is limited)
+                need(g->tag_mode == RDF_TAGS_FRAME && out.labels[k.label].entry == first.entry && out.labels[k.label].k_kind == K_RET);
+                for (int j = 0; j < 3; ++j) q.tail[j] = by_call(k.ops[j]);
+                ++calls;
+            } else {
+                q.ca = by_call(k.a);
+                q.cb = by_call(k.b);
+            }
+            return calls == out.n_labels;
+        } catch (const Fail&) {
+            return false;
+        }
+    }
+
     // false: not a program for the pool executor
     bool build() {
         if (g->has_vector_ops || g->has_loops || g->interleaved) return false;
@@ -1436,6 +1502,7 @@ extern "C" int rdf_graph_build(const rdf_program* prog, rdf_graph** out_graph) {
         detect_fold(P, g);
         PoolBuilder pool{g, g->pool_prog};
         g->pool = pool.build();
+        g->lanes = g->pool && pool.lane_shape(g->lane_prog);
     } catch (const Err& e) {
         delete g;
         return e.code;

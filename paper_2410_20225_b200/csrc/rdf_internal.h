@@ -144,6 +144,22 @@ struct alignas(16) PoolProgram {
     PoolCont  cont_of[POOL_MAX_CONT];    // by match node
 };
 
+// A program of one recursive function whose body returns a value or makes n_ports calls that meet in one operator (rdf_lanes.cuh).
+// Operands of conditions, returned values and calls: over the parameters; of the operator: over its operands in the order the calls
+// are made; of `root`: over the program's argument.
+struct LaneOperand { uint64_t mask[3]; int64_t imm; };      // the value whose mask is set, plus a constant
+struct LaneProgram {
+    int32_t n_args, n_ports;
+    int32_t n_cond, call_at, cmp[2];             // the first condition that holds: its action, else the last one; call_at: the one that makes the calls
+    int32_t cont, ret_at;                        // PI_ADD .. PI_MAX: ca op cb + cont_imm is returned; PI_CALL: `tail` are the parameters of the same function
+    int64_t cont_imm, out_imm;
+    LaneOperand a[2], b[2];
+    LaneOperand ret[2];                          // returned by the other actions, the second one by action ret_at
+    LaneOperand call[9], root[3];                // parameters of the calls, 3 each; of the call `result` makes
+    LaneOperand ca, cb, tail[3];
+    int32_t label[4], port[3];                   // labels of the calls, and (3) of the one `result` makes; the operator's ports they feed
+};
+
 struct rdf_graph {
     // literal graph (Section 3 transformation), for inspection
     std::vector<rdf_node> nodes;
@@ -171,6 +187,8 @@ struct rdf_graph {
     int32_t fold_right[2] = {0, 1};       // the child that operand 0 / 1 descends into: 0 left, 1 right
     bool pool = false;            // an integer program that fits the pool executor
     PoolProgram pool_prog{};
+    bool lanes = false;           // a call per thread
+    LaneProgram lane_prog{};
     bool interleaved = false;     // some Switch reads a vector value: operators run between the token waves
     std::vector<std::string> func_names;
     // per-run state owned by the executor (rdf_exec.cu)

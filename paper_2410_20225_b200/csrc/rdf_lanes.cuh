@@ -1,0 +1,857 @@
+// Integer programs of one recursive function, a call per thread.
+//
+// The pool executor (rdf_pool.cuh) runs a block's tokens in rounds, with barriers between them, and every call goes through its
+// stacks.  Programs of one common form -- one function whose body returns a value or makes two or three calls that meet in one
+// operator (fib, tak) -- run here instead: every lane of a warp holds one token in registers, a call that makes calls or a value
+// on its way to the operator that waits for it.  A lane with a call works out the parameters of the calls it makes and finds
+// those that return at once (their values go to the operator directly); it goes on with the first of the others and leaves the
+// rest, as {frame, which call}, on the warp's stack, where idle lanes take them.  A value that completes its operator is carried
+// on by the lane that brought it.  So no call goes through a queue, a frame exists only while an operator waits, and the warps of
+// a block meet only where one of them has nothing to do.
+//
+//   frame         in shared memory: parameters, operands that have arrived, {caller's frame, port}, wave of the invocation
+//   free frames   a list per warp (LN_FREE), the rest in a list of the block
+//   calls to make a stack per warp (LN_STACK); what it cannot hold, and the oldest of it when other warps have nothing to do,
+//                 in a stack of the block
+//
+// A block runs its instances to their end.  One that is left over with a long instance when few others are busy leaves it to the
+// general scheduler, as in the pool executor: tokens, operands that have arrived and calls to make go there (PoolDump).
+//
+// Frames may run out.  The last `reserve` of them are for one lane at a time (the favoured one): it runs the call it holds depth
+// first to its end, which takes a frame per level, while the other lanes that need a frame wait.  Path tags bound the levels; with
+// frame tags a recursion deeper than that ends in pool_exhausted, and the general scheduler behind this kernel runs the call.
+//
+// What bounds it: instructions and their latency, some 370 per iteration of a warp, which is 36 calls of fib (the pool executor: 19.3
+// per call); an instruction issued in 45 % of the cycles, warps stalled per issue 2.7 on the fixed latency of the one before, 1.4 on
+// branches, 1.1 on shared memory.  Few calls at a time take the latency of their longest chain, two iterations of 1.5 to 2 us per
+// level.  Measured, pool executor -> this: 131 072 calls of fib(0..18) 5.36 -> 2.9 ms, 8000 0.57 -> 0.33, 1024 0.175 -> 0.148, 8 of
+// fib(0..10) 39 -> 31 us; 200 calls of tak 0.90 -> 0.43 ms, 600 1.52 -> 0.58; 1000 full binary recursions of depth 17, whose frames no
+// pool holds, 94 -> 4.3 ms.  Tried: the returns of leaves as tokens of their own (34 instructions per call, 8.2 ms), the lists of the block
+// for every call (a lock: 1024 calls 258 us against 123), calls given to other blocks through global memory (no faster).
+//
+// The wave of a token is that of the pool executor: the caller's plus one, and the latest of an operator's operands.  Tokens per
+// wave follow from the invocations that made calls: NP in the next wave for each (and one more where the operator is a call).
+// (Included by rdf_exec.cu only: it defines kernels.)
+#pragma once
+#include "rdf_pool.cuh"
+
+// Warps of a block.  More of them hide more latency, but every lane holds the frames of a path down its call tree: 131 072 calls of
+// fib took 3.5 / 2.9 / 2.8 / 2.5 ms with 12 / 16 / 20 / 24, 1000 full binary recursions of depth 17 4.3 ms with 16, and with 24 they ran
+// out of frames and went on lane by lane.
+static const int LN_WARPS = 16, LN_THREADS = 32 * LN_WARPS;
+static const uint32_t LN_STACK = 128;                   // calls a warp keeps for itself
+static const uint32_t LN_FREE = 160, LN_FREE0 = 64, LN_STEP = 32;      // free frames it keeps: at most, at first; more at a time
+static const uint32_t LN_DEEP = 8;                      // free frames a lane should find when it begins a call
+static const uint32_t LN_SHARE = 8;                     // calls it needs to have to give some away
+// A block leaves its calls when it has run, on its own, as long as the clearing of the token store takes and LN_WIDE calls per wave so
+// far: a wave of the general scheduler takes some 10 us whatever its width.  (200 calls of tak: 424 calls per wave, better off here.)
+static const uint32_t LN_WIDE = 512;
+static const uint32_t LN_ROOT = 0x80000000u;            // link: the program's output of instance [30:0]
+static const uint32_t LN_FRAME = POOL_MAX_FRAMES - 1u;  // link: frame [12:0], port [14:13]
+static const uint32_t LN_NONE = 0xFFFFFFFFu, LN_ALL = 0xFFFFFFFFu;
+static const uint32_t LN_FIRST_WAIT = 1000;             // (so that the blocks' first warps have theirs before any block's second one)
+
+struct LaneSizes {
+    uint32_t cap;            // frames of a block
+    uint32_t reserve;        // frames of the block's list for the favoured lane
+    uint32_t max_depth;      // path tags: labels that fit the packed tag (no call is an operator then, and a call's depth is its wave); frame tags: LN_NONE
+    unsigned long long max_calls;   // frame tags: Call firings the caller allows
+    unsigned long long max_parked;  // path tags: operands the token store of the call holds
+    uint32_t late_waves;     // as PoolSizes
+    uint32_t hand_slots;     // as PoolSizes
+    long long hand_after;    // clock cycles: the clearing of the token store
+    uint32_t first_wait;     // clock cycles before warp k takes its first instances, times k
+    int      fallback;
+};
+
+// What a warp keeps besides its tokens
+struct LaneCold {
+    uint32_t fav, fav_base;      // the favoured lane, and the calls that lay on the stack before it
+    uint32_t first;              // it has not looked for work yet
+    uint32_t seen;               // instances known to be taken
+    uint32_t stock;              // the first instance of its stock (arguments: my_stock)
+};
+struct LaneShared {
+    uint32_t calling[POOL_BINS]; // invocations of the wave that made calls
+    uint32_t tails[POOL_BINS];   // calls of the wave made by an operator
+    uint32_t waves[POOL_BINS];   // tokens of the wave
+    uint32_t n_free, n_calls;    // in the block's lists
+    uint32_t lock;
+    uint32_t begun;              // instances the block has taken
+    uint32_t live;               // instances the block has begun and not ended
+    uint32_t hungry, gone;       // the warps that wait for work, that have left; a bit each
+    uint32_t inbox[LN_WARPS];    // calls another warp has put on the stack of one that waits
+    uint32_t scarce;             // a warp has found the block's list of free frames empty
+    uint32_t favoured;           // 1 + warp
+    uint32_t more, stop, done;   // more: there may be instances to take; stop: 1 an error, 2 frames have run out, POOL_LEAVE: the block leaves its calls
+    uint32_t scratch;
+    uint32_t hand, dumped;       // 1 + the place the block leaves its calls in; calls and `result` contexts left there
+    long long alone;             // since when few others are busy (clock cycles; 0: they are not) ...
+    uint32_t alone_calls;        // ... and the invocations that had made calls by then
+    LaneCold cold[LN_WARPS];
+};
+
+// The block's arrays in dynamic shared memory
+template <int NA, int NP>
+struct LaneArrays {
+    static const int NO = NP == 2 ? 1 : 3;       // operand words of a frame: of two operands the second one takes the place of parameter 0
+    int64_t  *args, *ops, *my_stock;
+    uint32_t *link_of, *wave_of, *state, *wmax;
+    uint16_t *free_list, *call_list, *my_free, *stacks, *my_calls;
+    __device__ __forceinline__ LaneArrays(unsigned char* top, const LaneSizes& z, uint32_t warp) {
+        auto array = [&](size_t bytes) { unsigned char* r = top; top += bytes; return r; };
+        args = reinterpret_cast<int64_t*>(array(8 * NA * z.cap));
+        ops = reinterpret_cast<int64_t*>(array(8 * NO * z.cap));
+        my_stock = reinterpret_cast<int64_t*>(array(8 * LN_WARPS * 32)) + warp * 32u;
+        link_of = reinterpret_cast<uint32_t*>(array(4 * z.cap));
+        wave_of = reinterpret_cast<uint32_t*>(array(4 * z.cap));
+        state = reinterpret_cast<uint32_t*>(array(4 * z.cap));
+        wmax = reinterpret_cast<uint32_t*>(array(NP == 2 ? 0 : 4 * z.cap));
+        stacks = reinterpret_cast<uint16_t*>(array(2 * LN_WARPS * LN_STACK));
+        my_calls = stacks + warp * LN_STACK;
+        free_list = reinterpret_cast<uint16_t*>(array(2 * z.cap));
+        call_list = reinterpret_cast<uint16_t*>(array(2 * (NP - 1) * z.cap));
+        my_free = reinterpret_cast<uint16_t*>(top) + warp * LN_FREE;
+    }
+};
+inline size_t lane_frame_bytes(int n_args, int n_ports) { return 8 * (size_t)(n_args + (n_ports == 2 ? 1 : 3)) + 12 + (n_ports == 2 ? 0 : 4) + 2 + 2 * (size_t)(n_ports - 1); }
+inline size_t lane_fixed_bytes() { return (size_t)LN_WARPS * (2 * (size_t)(LN_FREE + LN_STACK) + 8 * 32); }
+
+__device__ __forceinline__ uint32_t lane_vol(const uint32_t& w) { return *const_cast<const volatile uint32_t*>(&w); }
+__device__ __forceinline__ void lane_set(uint32_t& w, uint32_t v) { *const_cast<volatile uint32_t*>(&w) = v; }
+// what other warps change, read once for the whole warp: its lanes branch on it together
+__device__ __forceinline__ uint32_t lane_see(const uint32_t& w) { return __shfl_sync(LN_ALL, lane_vol(w), 0); }
+__device__ __forceinline__ uint32_t lane_exch(uint32_t* p, uint32_t v) {
+    uint32_t r;
+    asm volatile("atom.acq_rel.cta.shared::cta.exch.b32 %0, [%1], %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+    return r;
+}
+__device__ __forceinline__ uint32_t lane_or(uint32_t* p, uint32_t v) {
+    uint32_t r;
+    asm volatile("atom.acq_rel.cta.shared::cta.or.b32 %0, [%1], %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
+    return r;
+}
+
+// ---- the block's lists.  (Functions of their own, with everything in registers: they are not part of the loop over tokens.)
+__device__ __noinline__ void lane_error(Control* ctl, LaneShared& sh, int code) {
+    atomicCAS(&ctl->status, 0, code);
+    lane_set(sh.stop, 1u);
+}
+__device__ __forceinline__ bool lane_lock(Control* ctl, LaneShared& sh) {
+    uint32_t ok = 0;
+    if ((threadIdx.x & 31u) == 0u) {
+        for (uint32_t i = 0; i < (1u << 22) && !ok; ++i) {
+            ok = atomicCAS(&sh.lock, 0u, 1u) == 0u;
+            if (!ok && (i & 3u) == 3u) __nanosleep(32);
+        }
+        if (!ok) lane_error(ctl, sh, RDF_ERR_TIMEOUT);
+        __threadfence_block();
+    }
+    ok = __shfl_sync(LN_ALL, ok, 0);
+    __syncwarp();
+    return ok != 0u;
+}
+__device__ __forceinline__ void lane_unlock(LaneShared& sh) {
+    __syncwarp();
+    if ((threadIdx.x & 31u) == 0u) {
+        __threadfence_block();
+        atomicExch(&sh.lock, 0u);
+    }
+    __syncwarp();
+}
+// the k oldest calls of a warp to the block's stack: how many have gone
+__device__ __noinline__ uint32_t lane_spill_calls(Control* ctl, LaneShared& sh, uint16_t* list, const uint16_t* mine, uint32_t base, uint32_t k) {
+    if (!lane_lock(ctl, sh)) return 0u;
+    const uint32_t at = lane_see(sh.n_calls), lane = threadIdx.x & 31u;
+    for (uint32_t i = lane; i < k; i += 32u) list[at + i] = mine[(base + i) % LN_STACK];
+    __syncwarp();
+    if (lane == 0) lane_set(sh.n_calls, at + k);
+    lane_unlock(sh);
+    return k;
+}
+// calls from the block's stack, behind `top`: how many
+__device__ __noinline__ uint32_t lane_take_calls(Control* ctl, LaneShared& sh, const uint16_t* list, uint16_t* mine, uint32_t top) {
+    if (!lane_lock(ctl, sh)) return 0u;
+    const uint32_t lane = threadIdx.x & 31u, n = lane_see(sh.n_calls), k = min(n, 32u);
+    if (lane < k) mine[(top + lane) % LN_STACK] = list[n - k + lane];
+    __syncwarp();
+    if (lane == 0) lane_set(sh.n_calls, n - k);
+    lane_unlock(sh);
+    return k;
+}
+// The k oldest calls of a warp to one that waits, which has an empty stack and takes them from its beginning: how many have gone
+__device__ __noinline__ uint32_t lane_hand_calls(LaneShared& sh, uint16_t* stacks, const uint16_t* mine, uint32_t base, uint32_t k) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t to = LN_NONE;
+    if (lane == 0) {
+        const uint32_t waiting = lane_vol(sh.hungry);
+        if (waiting) {
+            to = __ffs(waiting) - 1u;
+            if (!((atomicAnd(&sh.hungry, ~(1u << to)) >> to) & 1u)) to = LN_NONE;      // (somebody else was first)
+        }
+    }
+    to = __shfl_sync(LN_ALL, to, 0);
+    if (to == LN_NONE) return 0u;
+    for (uint32_t i = lane; i < k; i += 32u) stacks[to * LN_STACK + i] = mine[(base + i) % LN_STACK];
+    __syncwarp();
+    if (lane == 0) {
+        __threadfence_block();
+        lane_set(sh.inbox[to], k);
+    }
+    __syncwarp();
+    return k;
+}
+// the last k of a warp's n free frames to the block's list: how many it has then
+__device__ __noinline__ uint32_t lane_spill_free(Control* ctl, LaneShared& sh, uint16_t* list, const uint16_t* mine, uint32_t n, uint32_t k) {
+    if (!lane_lock(ctl, sh)) return n;
+    const uint32_t at = lane_see(sh.n_free), lane = threadIdx.x & 31u;
+    for (uint32_t i = lane; i < k; i += 32u) list[at + i] = mine[n - k + i];
+    __syncwarp();
+    if (lane == 0) {
+        lane_set(sh.n_free, at + k);
+        lane_set(sh.scarce, 0u);
+    }
+    lane_unlock(sh);
+    return n - k;
+}
+// up to `want` more free frames for a warp that has n, all but `reserve` of the block's: how many it has then
+__device__ __noinline__ uint32_t lane_take_free(Control* ctl, LaneShared& sh, const uint16_t* list, uint16_t* mine, uint32_t n, uint32_t want, uint32_t reserve) {
+    if (!lane_lock(ctl, sh)) return n;
+    const uint32_t at = lane_see(sh.n_free), spare = at > reserve ? at - reserve : 0u, k = min(want, spare), lane = threadIdx.x & 31u;
+    for (uint32_t i = lane; i < k; i += 32u) mine[n + i] = list[at - k + i];
+    __syncwarp();
+    if (lane == 0) {
+        lane_set(sh.n_free, at - k);
+        if (k < want) lane_set(sh.scarce, 1u);               // (warps that wait give theirs back)
+    }
+    lane_unlock(sh);
+    return n + k;
+}
+// No lane of the warp that needs a frame gets one.  One warp of the block is favoured, one of its lanes, and that one has the
+// reserve.  Returns the frames the warp has.
+__device__ __noinline__ uint32_t lane_starved(Control* ctl, LaneShared& sh, const uint16_t* list, uint16_t* mine, uint32_t need, uint32_t cnt) {
+    const uint32_t lane = threadIdx.x & 31u;
+    LaneCold& k = sh.cold[threadIdx.x >> 5];
+    if (lane_see(k.fav) == LN_NONE) {
+        uint32_t got = 0;
+        if (lane == 0) got = atomicCAS(&sh.favoured, 0u, 1u) == 0u;
+        if (!__shfl_sync(LN_ALL, got, 0)) {
+            __nanosleep(200);
+            return 0u;
+        }
+        if (lane == 0) {
+            k.fav = __ffs(need) - 1u;
+            k.fav_base = cnt;
+        }
+        __syncwarp();
+    }
+    if (!((need >> lane_see(k.fav)) & 1u)) return 0u;
+    const uint32_t n = lane_take_free(ctl, sh, list, mine, 0u, 1u, 0u);
+    if (n == 0u && lane == 0) {                              // a recursion deeper than the reserve, and nothing left
+        ctl->pool_exhausted = 1;
+        lane_set(sh.stop, 2u);
+    }
+    return n;
+}
+// the favoured lane has ended its call; the warp has no free frames then
+__device__ __noinline__ void lane_favoured_done(Control* ctl, LaneShared& sh, uint16_t* list, const uint16_t* mine, uint32_t n_free) {
+    if (n_free) lane_spill_free(ctl, sh, list, mine, n_free, n_free);
+    if ((threadIdx.x & 31u) == 0u) {
+        sh.cold[threadIdx.x >> 5].fav = LN_NONE;
+        __threadfence_block();
+        atomicExch(&sh.favoured, 0u);
+    }
+    __syncwarp();
+}
+// n calls of wave w, beyond the waves that are counted in shared memory
+__device__ __noinline__ void lane_count_late(const DevCtx& c, const LaneSizes& z, LaneShared& sh, uint32_t w, uint32_t n) {
+    if (w >= c.wave_limit) lane_error(c.ctl, sh, RDF_ERR_WAVE_LIMIT);
+    atomicMax(&c.ctl->waves, w + 1u);
+    if (z.late_waves) atomicAdd(reinterpret_cast<uint32_t*>(c.q[0]) + min(w - (uint32_t)POOL_BINS, z.late_waves - 1u), n);
+}
+// an operand: one of up to three values (or none) plus a constant
+template <int N>
+__device__ __forceinline__ int64_t lane_pick(const LaneOperand& o, const int64_t* x) {
+    uint64_t r = (uint64_t)x[0] & o.mask[0];
+    if (N > 1) r |= (uint64_t)x[1] & o.mask[1];
+    if (N > 2) r |= (uint64_t)x[2] & o.mask[2];
+    return (int64_t)r + o.imm;
+}
+// Does a call with these parameters return at once?  Then v is its value.
+template <int NA>
+__device__ __forceinline__ bool lane_returns(const LaneProgram& p, const int64_t* x, int64_t& v) {
+    const int64_t a0 = lane_pick<NA>(p.a[0], x), b0 = lane_pick<NA>(p.b[0], x);
+    const bool first = p.cmp[0] == PC_LT ? a0 < b0 : (a0 == b0) == (p.cmp[0] == PC_EQ);
+    v = lane_pick<NA>(p.ret[0], x);
+    if (p.n_cond == 1) return first == (p.call_at != 0);
+    const int64_t a1 = lane_pick<NA>(p.a[1], x), b1 = lane_pick<NA>(p.b[1], x);
+    const bool second = p.cmp[1] == PC_LT ? a1 < b1 : (a1 == b1) == (p.cmp[1] == PC_EQ);
+    const int which = first ? 0 : second ? 1 : 2;
+    if (which == p.ret_at) v = lane_pick<NA>(p.ret[1], x);
+    return which != p.call_at;
+}
+// call q > 0 of frame f
+template <int NA, int NP>
+__device__ __forceinline__ void lane_load_call(const LaneProgram& p, const int64_t* args, const uint32_t* wave_of, uint32_t cap, uint32_t e, int64_t* a,
+                                               uint32_t& link, uint32_t& wave) {
+    const uint32_t f = e & LN_FRAME;
+    int64_t x[NA];
+#pragma unroll
+    for (int k = 0; k < NA; ++k) x[k] = args[k * cap + f];
+    wave = wave_of[f] + 1u;
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+        a[k] = lane_pick<NA>(p.call[1 * 3 + k], x);
+        if (NP > 2 && (e >> 13) == 2u) a[k] = lane_pick<NA>(p.call[2 * 3 + k], x);
+    }
+    link = e;
+}
+
+// A token: nothing, a call that makes calls (its parameters), a value (in a[0])
+enum { LN_IDLE = 0, LN_CALL = 1, LN_VALUE = 2 };
+// A warp's state where it is not in the loop over tokens
+template <int NA>
+struct LaneState {
+    int      mode;
+    int64_t  a[NA];
+    uint32_t link, wave;
+    uint32_t n_free, base, cnt, stock;
+    bool     got;
+};
+
+// ---- what a warp does that has nothing to do, and between blocks
+template <int NA, int NP>
+struct LaneSlow {
+    const DevCtx& c;
+    const LaneProgram& p;
+    const LaneSizes& z;
+    LaneShared& sh;
+    const LaneArrays<NA, NP> A;
+    const uint32_t lane, warp;
+    LaneState<NA> t;
+    __device__ __forceinline__ LaneSlow(const DevCtx& c_, const LaneProgram& p_, const LaneSizes& z_, LaneShared& sh_, unsigned char* smem, const LaneState<NA>& t_)
+        : c(c_), p(p_), z(z_), sh(sh_), A(smem, z_, threadIdx.x >> 5), lane(threadIdx.x & 31u), warp(threadIdx.x >> 5), t(t_) {}
+    __device__ __forceinline__ LaneCold& cold() const { return sh.cold[warp]; }
+
+    // A stock of instances, smaller the fewer are left
+    __device__ __forceinline__ bool take_instances() {
+        const uint32_t B = (uint32_t)c.B, seen = lane_see(cold().seen), left = B > seen ? B - seen : 0u;
+        const uint32_t k = min(32u, max(1u, left / (gridDim.x * LN_WARPS * 2u)));
+        uint32_t at = 0;
+        if (lane == 0) {
+            atomicAdd(&sh.live, k);                          // (before they are taken: no warp may think that the block has nothing)
+            at = atomicAdd(&c.ctl->next_chunk, k);
+        }
+        at = __shfl_sync(LN_ALL, at, 0);
+        const uint32_t n = at < B ? min(k, B - at) : 0u;
+        if (lane < n) A.my_stock[lane] = c.x[at + lane];
+        if (lane == 0) {
+            cold().seen = at + k; cold().stock = at;
+            if (n < k) {
+                atomicSub(&sh.live, k - n);
+                lane_set(sh.more, 0u);
+            }
+            if (n) atomicAdd(&sh.begun, n);
+        }
+        __syncwarp();
+        t.stock = n;
+        return n != 0u;
+    }
+    // The last warp, now and then: has another block failed; does this one leave its calls?
+    __device__ __forceinline__ void look_around() const {
+        uint32_t top = 0, calls = 0;                         // waves so far, and invocations that have made calls (of the first POOL_BINS waves)
+        for (uint32_t w = lane; w < (uint32_t)POOL_BINS; w += 32u) {
+            const uint32_t n = lane_vol(sh.calling[w]);
+            if (n) top = w;
+            calls += n;
+        }
+        top = __reduce_max_sync(LN_ALL, top);
+        calls = __reduce_add_sync(LN_ALL, calls);
+        if (lane == 0) {
+            if (ld_volatile_i32(&c.ctl->status) | (int)ld_volatile_u32(&c.ctl->pool_exhausted)) lane_set(sh.stop, 1u);
+            else if (z.hand_slots && !lane_vol(sh.more)) {
+                const long long now = clock64();
+                if (gridDim.x - ld_volatile_u32(&c.ctl->blocks_done.v) > POOL_ACTIVE) sh.alone = 0ll;
+                else if (sh.alone == 0ll) {
+                    sh.alone = now;
+                    sh.alone_calls = calls;
+                } else if (now - sh.alone >= z.hand_after && __popc(lane_vol(sh.hungry)) <= LN_WARPS / 2 && (calls - sh.alone_calls) * NP >= LN_WIDE * top) {
+                    sh.alone = 0ll;
+                    const uint32_t slot = atomicAdd(&c.ctl->hand_claims, 1u);
+                    if (slot < z.hand_slots) {
+                        sh.hand = slot + 1u;
+                        atomicCAS(&sh.stop, 0u, (uint32_t)POOL_LEAVE);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
+    // the warp has calls from elsewhere or leaves: it does not wait any more.  False: somebody is handing it calls
+    __device__ __forceinline__ bool retract() {
+        uint32_t was = 0;
+        if (lane == 0) was = (atomicAnd(&sh.hungry, ~(1u << warp)) >> warp) & 1u;
+        return __shfl_sync(LN_ALL, was, 0) != 0u;
+    }
+    __device__ __forceinline__ void take_inbox() {
+        for (uint32_t i = 0; i < (1u << 16) && lane_see(sh.inbox[warp]) == 0u; ++i) {}       // (whoever has claimed it writes at once)
+        t.cnt = lane_see(sh.inbox[warp]);
+        __threadfence_block();
+    }
+    // Nothing to do in the whole warp (no token, no call to make).  t.got: there is now; else nothing will come any more.
+    __device__ __forceinline__ void find_work() {
+        const long long t0 = clock64();
+        t.got = true;
+        if (lane_see(cold().fav) != LN_NONE) {
+            lane_favoured_done(c.ctl, sh, A.free_list, A.my_free, t.n_free);
+            t.n_free = 0u;
+        }
+        const long long wait = lane_see(cold().first) ? (long long)warp * z.first_wait : 0ll;
+        __syncwarp();
+        if (lane == 0) cold().first = 0u;
+        __syncwarp();
+        if (wait == 0ll && lane_see(sh.more) && take_instances()) return;
+        t.base = t.cnt = 0u;
+        bool waits = false;
+        for (uint32_t poll = 0;; ++poll) {
+            if (!waits) {
+                if (lane == 0) {
+                    lane_set(sh.inbox[warp], 0u);
+                    __threadfence_block();
+                    atomicOr(&sh.hungry, 1u << warp);        // from here on another warp may fill the stack
+                }
+                __syncwarp();
+                waits = true;
+            }
+            // one look, by one lane
+            enum { NOTHING = 0, LEAVE, INBOX, STACK, INSTANCES, EXPIRED, ALL_WAIT };
+            uint32_t what = NOTHING;
+            if (lane == 0) {
+                const long long spent = clock64() - t0;
+                if (lane_vol(sh.inbox[warp])) what = INBOX;
+                else if (lane_vol(sh.stop) | lane_vol(sh.done)) what = LEAVE;
+                else if (lane_vol(sh.n_calls)) what = STACK;
+                else if (lane_vol(sh.more)) what = spent >= wait ? INSTANCES : NOTHING;
+                else if (spent > (warp == 0 ? 32ll : 1ll) * c.spin_limit) what = EXPIRED;
+                else if (warp == 0 && lane_vol(sh.live) == 0u && (lane_vol(sh.hungry) | lane_vol(sh.gone)) == (uint32_t)((1ull << LN_WARPS) - 1ull)) what = ALL_WAIT;
+            }
+            what = __shfl_sync(LN_ALL, what, 0);
+            if (what == LEAVE) {
+                if (retract()) break;
+                what = INBOX;
+            }
+            if (what == INBOX) {
+                take_inbox();
+                return;
+            }
+            if (what == STACK || what == INSTANCES || what == EXPIRED) {
+                if (!retract()) {
+                    take_inbox();
+                    return;
+                }
+                waits = false;
+                if (what == EXPIRED) {
+                    // (it holds nothing that anybody waits for; warp 0: longer than 2^24 waves of one call after the other take)
+                    if (lane == 0) atomicOr(&sh.gone, 1u << warp);
+                    if (warp == 0 && lane == 0) lane_error(c.ctl, sh, RDF_ERR_TIMEOUT);
+                    break;
+                }
+                if (what == INSTANCES && take_instances()) return;
+                if (what == STACK) {
+                    t.cnt = lane_take_calls(c.ctl, sh, A.call_list, A.my_calls, 0u);
+                    if (t.cnt) return;
+                }
+                continue;
+            }
+            if (t.n_free && lane_see(sh.scarce)) t.n_free = lane_spill_free(c.ctl, sh, A.free_list, A.my_free, t.n_free, t.n_free);
+            if (what == ALL_WAIT) {
+                if (lane == 0) lane_set(sh.done, 1u);
+                break;
+            }
+            if (warp == LN_WARPS - 1 && (poll & 15u) == 15u) look_around();
+            __nanosleep(100);
+            __syncwarp();
+        }
+        t.got = false;
+    }
+};
+template <int NA, int NP>
+__device__ __noinline__ LaneState<NA> lane_slow(const DevCtx& c, const LaneProgram& p, const LaneSizes& z, LaneShared& sh, unsigned char* smem, const LaneState<NA> t, bool work) {
+    LaneSlow<NA, NP> s(c, p, z, sh, smem, t);
+    if (work) s.find_work();
+    else s.look_around();
+    return s.t;
+}
+
+// The calls of a block that leaves them, in the form of the pool executor's frames: a frame of this block is the entry of its
+// number, calls to make and the `result` contexts that wait for a value have entries behind them.
+template <int NA, int NP>
+__device__ __noinline__ void lane_leave(const DevCtx& c, const LaneProgram& p, const LaneSizes& z, LaneShared& sh, unsigned char* smem, const LaneState<NA> t) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n_entries = c.pool.cap;
+    const LaneArrays<NA, NP> A(smem, z, warp);
+    const PoolDump d(c, sh.hand - 1u);
+    // free frames: no wave
+    for (uint32_t i = lane; i < t.n_free; i += 32u) A.wave_of[A.my_free[i]] = LN_NONE;
+    for (uint32_t i = threadIdx.x; i < sh.n_free; i += LN_THREADS) A.wave_of[A.free_list[i]] = LN_NONE;
+    for (uint32_t i = threadIdx.x; i < n_entries; i += LN_THREADS) d.id[i] = LN_NONE;
+    __syncthreads();
+    // the word of an invocation: its caller's entry, the call's label, its depth.  A `result` context that waits gets its entry here
+    auto head = [&](uint32_t link, uint32_t wave) {
+        const uint32_t depth = z.max_depth == LN_NONE ? 0u : wave;
+        if (!(link & LN_ROOT)) return (link & LN_FRAME) | (uint32_t)p.label[link >> 13] << 16 | depth << 22;
+        const uint32_t at = z.cap + atomicAdd(&sh.dumped, 1u), inst = link & ~LN_ROOT;
+        if (at < n_entries) {
+            d.id[at] = inst; d.head[at] = POOL_ROOT | inst; d.state[at] = 0u;
+            d.words[at] = c.x[inst];
+        }
+        return at | (uint32_t)p.label[3] << 16 | depth << 22;
+    };
+    auto call = [&](const int64_t* a, uint32_t link, uint32_t wave) {
+        const uint32_t h = head(link, wave), at = z.cap + atomicAdd(&sh.dumped, 1u);
+        if (at >= n_entries) return;
+        d.id[at] = (uint32_t)c.B + atomicAdd(&c.ctl->hand_frames, 1u);
+        d.head[at] = h;
+        d.state[at] = 0xFFFFFFFFu;
+        for (int k = 0; k < NA; ++k) d.words[(size_t)k * n_entries + at] = a[k];
+    };
+    for (uint32_t f = threadIdx.x; f < z.cap; f += LN_THREADS) {
+        const uint32_t wave = A.wave_of[f];
+        if (wave == LN_NONE) continue;
+        d.id[f] = (uint32_t)c.B + atomicAdd(&c.ctl->hand_frames, 1u);
+        d.head[f] = head(A.link_of[f], wave);
+        uint32_t there = 0;
+        for (uint32_t q = 0; q < (uint32_t)NP; ++q) {
+            if (!((A.state[f] >> q) & 1u)) continue;
+            there |= 1u << p.port[q];
+            d.words[(size_t)(c.pool.word0 + p.port[q]) * n_entries + f] = NP == 2 ? (q == 0u ? A.ops : A.args)[f] : A.ops[q * z.cap + f];
+        }
+        d.state[f] = there;
+        // (its calls have been made and these operands parked: the counters of an operator come with its firing otherwise)
+        atomicAdd(&c.ctl->invocations, (unsigned long long)NP);
+        if (there) atomicAdd(&c.ctl->store_inserts, (unsigned long long)__popc(there));
+    }
+    auto waiting = [&](uint32_t e) {
+        int64_t a[NA];
+        uint32_t link, wave;
+        lane_load_call<NA, NP>(p, A.args, A.wave_of, z.cap, e, a, link, wave);
+        call(a, link, wave);
+    };
+    for (uint32_t i = lane; i < t.cnt; i += 32u) waiting(A.my_calls[(t.base + i) % LN_STACK]);
+    for (uint32_t i = threadIdx.x; i < sh.n_calls; i += LN_THREADS) waiting(A.call_list[i]);
+    if (lane < t.stock) {                                    // instances that have not begun: their `result` context is to be entered
+        const uint32_t at = z.cap + atomicAdd(&sh.dumped, 1u), inst = sh.cold[warp].stock + lane;
+        if (at < n_entries) {
+            d.id[at] = inst; d.head[at] = POOL_ROOT | inst; d.state[at] = 0xFFFFFFFFu;
+            d.words[at] = A.my_stock[lane];
+        }
+        atomicSub(&sh.begun, 1u);
+    }
+    if (t.mode == LN_CALL) call(t.a, t.link, t.wave);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (z.cap + sh.dumped > n_entries) lane_error(c.ctl, sh, RDF_ERR_QUEUE_FULL);
+        atomicOr(&c.ctl->hand_mask, 1u << (sh.hand - 1u));
+    }
+}
+
+template <int NA, int NP>
+__global__ void __launch_bounds__(LN_THREADS, 1) rdf_lanes_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ LaneProgram p,
+                                                                  const __grid_constant__ LaneSizes z) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ LaneShared sh;
+    const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u, lower = (1u << lane) - 1u, cap = z.cap;
+    const long long t_start = clock64();
+    const LaneArrays<NA, NP> A(smem, z, warp);
+    // free frames: every warp its share, the rest in the block's list
+    const uint32_t rest = cap - LN_WARPS * LN_FREE0;
+    for (uint32_t i = tid; i < rest; i += LN_THREADS) A.free_list[i] = (uint16_t)i;
+    for (uint32_t i = lane; i < LN_FREE0; i += 32u) A.my_free[i] = (uint16_t)(rest + warp * LN_FREE0 + i);
+    for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += LN_THREADS) sh.calling[i] = sh.tails[i] = 0u;
+    if (lane == 0) {
+        LaneCold& k = sh.cold[warp];
+        k.fav = LN_NONE;
+        k.fav_base = k.seen = k.stock = 0u;
+        k.first = 1u;
+    }
+    if (tid == 0) {
+        sh.n_free = rest;
+        sh.n_calls = sh.lock = sh.begun = sh.live = sh.hungry = sh.gone = sh.scarce = sh.favoured = 0u;
+        sh.more = 1u; sh.stop = sh.done = sh.hand = sh.dumped = 0u;
+        sh.alone = 0ll;
+    }
+    __syncthreads();
+
+    uint32_t n_free = LN_FREE0, base = 0, cnt = 0;      // of the warp: free frames; calls to make: my_calls[(base .. base + cnt) % LN_STACK], oldest first
+    uint32_t allowed = LN_ALL;                   // lanes that may take calls and frames (the favoured one, if there is one)
+    uint32_t room = (cap - LN_WARPS * LN_FREE0) / LN_WARPS;      // its share of the block's free frames, as last seen
+    uint32_t stock = 0;                          // instances taken and not begun
+    uint32_t stalls = 0;                         // iterations without a frame, one after the other
+    uint32_t fired = 0;                    // operators the lane has fired
+    int      mode = LN_IDLE;
+    int64_t  a[NA];
+    uint32_t link = 0, wave = 0;
+#pragma unroll
+    for (int k = 0; k < NA; ++k) a[k] = 0ll;
+    auto slow = [&](bool work) {
+        LaneState<NA> t{mode, {}, link, wave, n_free, base, cnt, stock, true};
+#pragma unroll
+        for (int k = 0; k < NA; ++k) t.a[k] = a[k];
+        t = lane_slow<NA, NP>(c, p, z, sh, smem, t, work);
+        mode = t.mode; link = t.link; wave = t.wave; n_free = t.n_free; base = t.base; cnt = t.cnt; stock = t.stock;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) a[k] = t.a[k];
+        return t.got;
+    };
+    // The operator has its operands x, the last of which arrived in `wave`: its value, or the call it is.
+    auto fire = [&](const int64_t* x) {
+        if (p.cont != PI_CALL) {
+            const int64_t s = lane_pick<NP>(p.ca, x), t = lane_pick<NP>(p.cb, x);
+            int64_t v = s + t;
+            if (p.cont != PI_ADD) {
+                if (p.cont == PI_SUB) v = s - t;
+                else if (p.cont == PI_MUL) v = s * t;
+                else v = s > t ? s : t;
+            }
+            a[0] = v + p.cont_imm;
+            mode = LN_VALUE;
+        } else {
+            int64_t v;
+#pragma unroll
+            for (int k = 0; k < NA; ++k) a[k] = lane_pick<NP>(p.tail[k], x);
+            wave += 1u;
+            if (wave < (uint32_t)POOL_BINS) atomicAdd(&sh.tails[wave], 1u);
+            else lane_count_late(c, z, sh, wave, 1u);
+            mode = LN_CALL;
+            if (lane_returns<NA>(p, a, v)) {
+                mode = LN_VALUE;
+                a[0] = v;
+            }
+        }
+    };
+    for (uint32_t it = 1;; ++it) {
+        __syncwarp();
+        if ((it & 7u) == 0u) {
+            if (warp == LN_WARPS - 1u && ((it & 31u) == 0u || (z.hand_slots && lane_see(sh.more) == 0u))) slow(false);
+            const uint32_t stop = lane_see(sh.stop);
+            if (stop && stop != (uint32_t)POOL_LEAVE) break;
+            if (stop) allowed = 0u;                  // (values are brought to where they wait; what is left are calls)
+            room = lane_see(sh.n_free) / LN_WARPS;
+            if (n_free > 2u * LN_STEP && allowed == LN_ALL && lane_see(sh.scarce)) n_free = lane_spill_free(c.ctl, sh, A.free_list, A.my_free, n_free, n_free - LN_STEP);
+            if (z.max_depth == LN_NONE && __any_sync(LN_ALL, (unsigned long long)fired * NP > z.max_calls)) {
+                if (lane == 0) lane_error(c.ctl, sh, RDF_ERR_FRAMES_FULL);
+                break;
+            }
+        }
+        // ---- idle lanes take calls to make
+        uint32_t idle = __ballot_sync(LN_ALL, mode == LN_IDLE);
+        if (allowed == 0u && !__any_sync(LN_ALL, mode == LN_VALUE)) break;
+        if (allowed != LN_ALL && (idle & allowed) && cnt <= lane_see(sh.cold[warp].fav_base)) {
+            lane_favoured_done(c.ctl, sh, A.free_list, A.my_free, n_free);
+            n_free = 0u;
+            allowed = LN_ALL;
+        }
+        if (cnt == 0u && idle == LN_ALL && stock == 0u && allowed != 0u) {
+            allowed = LN_ALL;
+            if (!slow(true)) break;
+            idle = __ballot_sync(LN_ALL, mode == LN_IDLE);
+        }
+        if (cnt == 0u && idle && allowed == LN_ALL && lane_see(sh.n_calls)) cnt = lane_take_calls(c.ctl, sh, A.call_list, A.my_calls, base);
+        // (few free frames: what runs is brought to its end before more is begun)
+        const uint32_t begin = idle == LN_ALL ? max(1u, (n_free + room) / LN_DEEP) : (n_free + room) / LN_DEEP;
+        idle &= allowed;
+        {
+            const uint32_t rank = __popc(idle & lower);
+            if (((idle >> lane) & 1u) && rank < min(cnt, begin)) {
+                lane_load_call<NA, NP>(p, A.args, A.wave_of, cap, A.my_calls[(base + cnt - 1u - rank) % LN_STACK], a, link, wave);
+                mode = LN_CALL;
+            }
+            if (cnt == 0u && stock && idle) {
+                // nothing to make: a few instances (each of them soon makes calls for all lanes)
+                const uint32_t k = min(min(stock, begin), 1u + (uint32_t)__popc(idle) / 8u);
+                if (((idle >> lane) & 1u) && rank < k) {
+                    const int64_t arg = A.my_stock[stock - 1u - rank];
+                    int64_t v;
+#pragma unroll
+                    for (int j = 0; j < NA; ++j) a[j] = lane_pick<1>(p.root[j], &arg);
+                    link = LN_ROOT | (sh.cold[warp].stock + stock - 1u - rank);
+                    wave = 1u;
+                    mode = LN_CALL;
+                    if (lane_returns<NA>(p, a, v)) {
+                        mode = LN_VALUE;
+                        a[0] = v;
+                    }
+                }
+                stock -= k;
+            }
+            cnt -= min((uint32_t)__popc(idle), min(cnt, begin));
+        }
+        // ---- calls make their calls
+        uint32_t inner = 0;                          // those that do not return at once
+        int64_t  r[NP][NA], x[3] = {0, 0, 0};
+        const bool calls = mode == LN_CALL;
+        if (calls) {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+#pragma unroll
+                for (int k = 0; k < NA; ++k) r[q][k] = lane_pick<NA>(p.call[3 * q + k], a);
+                if (!lane_returns<NA>(p, r[q], x[q])) inner |= 1u << q;
+            }
+        }
+        uint32_t need = __ballot_sync(LN_ALL, inner != 0u) & allowed;
+        const uint32_t n = __popc(need);
+        if (n_free < n) {
+            if (allowed == LN_ALL) n_free = lane_take_free(c.ctl, sh, A.free_list, A.my_free, n_free, n - n_free + LN_STEP, z.reserve);
+            if (n_free == 0u && n) {
+                n_free = lane_starved(c.ctl, sh, A.free_list, A.my_free, need, cnt);
+                const uint32_t fav = lane_see(sh.cold[warp].fav);
+                if (fav != LN_NONE) allowed = 1u << fav;
+                if (++stalls > (1u << 24) && lane == 0) lane_error(c.ctl, sh, RDF_ERR_TIMEOUT);
+            }
+        }
+        if (n_free) stalls = 0u;
+        const uint32_t n_got = min(n, n_free), rank = __popc(need & lower);
+        const bool take = ((need >> lane) & 1u) && rank < n_got;
+        if (cnt + n_got * (NP - 1) > LN_STACK) {
+            const uint32_t k = lane_spill_calls(c.ctl, sh, A.call_list, A.my_calls, base, min(cnt, LN_STACK / 2));
+            base += k; cnt -= k;
+            if (allowed != LN_ALL && lane == 0) sh.cold[warp].fav_base -= min(sh.cold[warp].fav_base, k);
+            __syncwarp();
+        }
+        // the calls besides the first go to the stack
+        uint32_t at = base + cnt;
+        if (NP == 2) {
+            const uint32_t both = __ballot_sync(LN_ALL, take && inner == 3u);
+            at += __popc(both & lower);
+            cnt += __popc(both);
+        } else {
+            const uint32_t two = __ballot_sync(LN_ALL, take && __popc(inner) >= 2), three = __ballot_sync(LN_ALL, take && inner == 7u);
+            at += __popc(two & lower) + __popc(three & lower);
+            cnt += __popc(two) + __popc(three);
+        }
+        const bool whole = calls && inner == 0u;     // all have returned
+        if (take || whole) {
+            if (wave >= z.max_depth) lane_error(c.ctl, sh, RDF_ERR_TAG_OVERFLOW);
+            if (wave < (uint32_t)POOL_BINS - 1u) atomicAdd(&sh.calling[wave], 1u);
+            else lane_count_late(c, z, sh, wave + 1u, NP);
+        }
+        if (take) {
+            const uint32_t f = A.my_free[n_free - 1u - rank], q0 = __ffs(inner) - 1u, returned = inner ^ ((1u << NP) - 1u);
+            A.link_of[f] = link;
+            A.wave_of[f] = wave;
+            if (NP == 2) {
+                // one of them has returned: its value; neither has: the parameters, for the second call
+                A.state[f] = returned ? (wave + 1u) << 8 | returned : 0u;
+                if (inner == 2u) A.ops[f] = x[0];
+                else A.args[f] = inner == 3u ? a[0] : x[1];
+                if (inner == 3u) {
+#pragma unroll
+                    for (int k = 1; k < NA; ++k) A.args[k * cap + f] = a[k];
+                    A.my_calls[at % LN_STACK] = (uint16_t)(f | 1u << 13);
+                }
+            } else {
+                A.state[f] = returned;
+                A.wmax[f] = wave + 1u;
+#pragma unroll
+                for (int q = 0; q < NP; ++q)
+                    if ((returned >> q) & 1u) A.ops[q * cap + f] = x[q];
+                const uint32_t others = inner & (inner - 1u);
+                if (others) {
+#pragma unroll
+                    for (int k = 0; k < NA; ++k) A.args[k * cap + f] = a[k];
+                    if (others & 2u) A.my_calls[at++ % LN_STACK] = (uint16_t)(f | 1u << 13);
+                    if (others & 4u) A.my_calls[at % LN_STACK] = (uint16_t)(f | 2u << 13);
+                }
+            }
+            // on with the first one
+#pragma unroll
+            for (int k = 0; k < NA; ++k) {
+                a[k] = r[0][k];
+                if (q0 == 1u) a[k] = r[1][k];
+                if (NP > 2 && q0 == 2u) a[k] = r[NP - 1][k];
+            }
+            link = f | q0 << 13;
+            wave += 1u;
+        }
+        n_free -= n_got;
+        if (whole) {
+            wave += 1u;
+            ++fired;
+            fire(x);
+        }
+        // ---- values arrive
+        bool given = false;
+        uint32_t f = 0;
+        if (mode == LN_VALUE) {
+            mode = LN_IDLE;
+            if (link & LN_ROOT) {
+                const uint32_t to = link & ~LN_ROOT;
+                if (to < (uint32_t)c.B) c.y[to] = a[0] + p.out_imm;
+                atomicSub(&sh.live, 1u);
+            } else {
+                const uint32_t q = link >> 13;
+                f = link & LN_FRAME;
+                if (NP == 2) {
+                    (q == 0u ? A.ops : A.args)[f] = a[0];
+                    const uint32_t there = lane_exch(&A.state[f], wave << 8 | 1u << q);
+                    given = there != 0u;
+                    if (given) {
+                        x[0] = A.ops[f]; x[1] = A.args[f];
+                        wave = max(wave, there >> 8);
+                    }
+                } else {
+                    A.ops[q * cap + f] = a[0];
+                    atomicMax(&A.wmax[f], wave);
+                    const uint32_t there = lane_or(&A.state[f], 1u << q);
+                    given = (there | 1u << q) == (1u << NP) - 1u;
+                    if (given) {
+                        x[0] = A.ops[f]; x[1] = A.ops[cap + f]; x[2] = A.ops[2 * cap + f];
+                        wave = A.wmax[f];
+                    }
+                }
+                if (given) {
+                    link = A.link_of[f];
+                    ++fired;
+                    fire(x);
+                }
+            }
+        }
+        const uint32_t gives = __ballot_sync(LN_ALL, given);
+        if (gives) {                                 // frames that have done their work
+            const uint32_t g = __popc(gives);
+            if (n_free + g > LN_FREE) n_free = lane_spill_free(c.ctl, sh, A.free_list, A.my_free, n_free, 2u * LN_STEP);
+            if (n_free + g <= LN_FREE) {   // (or the call ends with an error)
+                if (given) A.my_free[n_free + __popc(gives & lower)] = (uint16_t)f;
+                n_free += g;
+            }
+        }
+        // ---- others have nothing to do
+        if (cnt >= LN_SHARE && allowed == LN_ALL) {
+            const uint32_t k = lane_see(sh.hungry) ? lane_hand_calls(sh, A.stacks, A.my_calls, base, cnt / 2u) : 0u;
+            base += k; cnt -= k;
+        }
+    }
+    __syncthreads();
+    if (sh.stop == (uint32_t)POOL_LEAVE) {
+        LaneState<NA> t{mode, {}, link, wave, n_free, base, cnt, stock, false};
+#pragma unroll
+        for (int k = 0; k < NA; ++k) t.a[k] = a[k];
+        lane_leave<NA, NP>(c, p, z, sh, smem, t);
+    }
+    // ---- counters.  Every operator that has fired had its operands but the last one parked, and its invocation made NP calls
+    const uint32_t tail = p.cont == PI_CALL ? 1u : 0u;
+    const uint32_t fired_n = __reduce_add_sync(LN_ALL, fired);
+    if (lane == 0 && fired_n) {
+        atomicAdd(&c.ctl->invocations, (unsigned long long)fired_n * (NP + tail));
+        atomicAdd(&c.ctl->store_matches, (unsigned long long)fired_n);
+        atomicAdd(&c.ctl->store_inserts, (unsigned long long)fired_n * (NP - 1));
+    }
+    const uint32_t begun = sh.begun;
+    if (tid == 0 && begun) atomicAdd(&c.ctl->invocations, (unsigned long long)begun);
+    for (uint32_t w = tid; w < (uint32_t)POOL_BINS; w += LN_THREADS) {
+        const uint32_t m = (w < 2u ? begun : 0u) + (w ? NP * sh.calling[w - 1u] : 0u) + sh.tails[w];
+        sh.waves[w] = m;
+        if (m && w && z.max_depth != LN_NONE) atomicMax(&c.ctl->max_depth, w);
+    }
+    __syncthreads();
+    pool_report(c, sh.waves, 0u, z.late_waves, z.max_calls, z.max_parked, z.fallback, t_start, &sh.scratch);
+}

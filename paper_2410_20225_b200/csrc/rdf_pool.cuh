@@ -27,6 +27,8 @@
 // fib(0..10) 0.137 -> 0.037 ms, 200 calls of tak 1.75 -> 0.80 ms (limited by the depth of the largest instance).
 // Handing calls of a busy block to idle ones through global memory was built and dropped: 200 calls of tak 0.90 -> 0.83 ms,
 // but 1024 calls of fib 0.23 -> 0.31 ms.
+// Programs of one function whose calls meet in one operator (fib and tak among them) have an executor of their own, without rounds
+// (rdf_lanes.cuh); the figures here are from before it.
 // (Included by rdf_exec.cu only: it defines kernels.)
 #pragma once
 #include "rdf_exec.h"
@@ -489,6 +491,56 @@ __device__ __noinline__ void pool_look(const DevCtx& c, const PoolSizes& z, Pool
     }
 }
 
+// The end of a block that has run its instances: its waves, and (the block that ends last) the verdict on the capacities of the call.
+// bins: tokens of the first POOL_BINS waves; max_wave: the thread's latest wave beyond them.
+__device__ __forceinline__ void pool_report(const DevCtx& c, const uint32_t* bins, uint32_t max_wave, uint32_t n_late, unsigned long long max_calls,
+                                            unsigned long long max_parked, int fallback, long long t_start, uint32_t* scratch) {
+    const uint32_t tid = threadIdx.x, T = blockDim.x, *late_waves = reinterpret_cast<const uint32_t*>(c.q[0]);
+    uint32_t w = max_wave;
+    for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += T)
+        if (bins[i]) {
+            atomicAdd(&c.ctl->wave_tokens[i], bins[i]);
+            w = max(w, i);
+        }
+    w = __reduce_max_sync(0xffffffffu, w);
+    if ((tid & 31u) == 0 && (w || tid == 0)) atomicMax(&c.ctl->waves, w + 1u);
+    if (blockIdx.x == 0 && tid == 0) c.ctl->cyc[0] = clock64() - t_start;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) *scratch = atomicAdd(&c.ctl->blocks_done.v, 1u);
+    __syncthreads();
+    if (*scratch != gridDim.x - 1u) return;
+    __threadfence();
+    // the widest wave of the call
+    uint32_t wide = 0, late = 0;
+    const uint32_t n_waves = ld_volatile_u32(&c.ctl->waves);
+    for (uint32_t i = tid; i < min(n_waves, (uint32_t)POOL_BINS); i += T) wide = max(wide, __ldcg(&c.ctl->wave_tokens[i]));
+    if (n_waves > (uint32_t)POOL_BINS)
+        for (uint32_t i = tid; i < min(n_waves - (uint32_t)POOL_BINS, n_late); i += T) {
+            const uint32_t v = __ldcg(&late_waves[i]);
+            (i + 1u < n_late ? wide : late) = max(v, i + 1u < n_late ? wide : late);
+        }
+    wide = __reduce_max_sync(0xffffffffu, wide);
+    late = __reduce_max_sync(0xffffffffu, late);
+    if ((tid & 31u) == 0) {
+        atomicMax(&c.ctl->max_wave_tokens, max(wide, late));
+        // (the last bin is a sum over waves, and an upper bound only)
+        if (c.tag_mode == RDF_TAGS_PATH && wide > c.qcap && !c.ctl->pool_exhausted) set_status(c, RDF_ERR_QUEUE_FULL);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        volatile Control* k = c.ctl;
+        k->tokens = k->invocations + (unsigned long long)c.B;
+        if (k->pool_exhausted) {
+            if (!fallback) set_status(c, RDF_ERR_QUEUE_FULL);
+        } else {
+            if (c.tag_mode == RDF_TAGS_FRAME && k->invocations > max_calls) set_status(c, RDF_ERR_FRAMES_FULL);
+            if (c.tag_mode == RDF_TAGS_PATH && k->store_inserts > max_parked) set_status(c, RDF_ERR_STORE_FULL);
+        }
+        k->forward_status = k->status;
+    }
+}
+
 __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ PoolProgram program,
                                                                              const __grid_constant__ PoolSizes z) {
     constexpr uint32_t T = POOL_THREADS;
@@ -589,55 +641,12 @@ __global__ void __launch_bounds__(POOL_THREADS, POOL_PER_SM) rdf_pool_kernel(con
         __syncthreads();
         pool_leave(c, smem, sh);
     }
-    // ---- counters, and (the block that ends last) the verdict on the capacities of the call
     if (sh.stop == 2 && tid == 0) c.ctl->pool_exhausted = 1;
     ThreadStats st;
     st.invocations = t.invocations; st.max_depth = t.max_depth;
     st.sc.inserts = t.inserts; st.sc.matches = t.matches;
     flush_stats(c, st);
-    uint32_t w = t.max_wave;
-    for (uint32_t i = tid; i < (uint32_t)POOL_BINS; i += T)
-        if (sh.waves[i]) {
-            atomicAdd(&c.ctl->wave_tokens[i], sh.waves[i]);
-            w = max(w, i);
-        }
-    w = __reduce_max_sync(0xffffffffu, w);
-    if ((tid & 31u) == 0 && (w || tid == 0)) atomicMax(&c.ctl->waves, w + 1u);
-    if (blockIdx.x == 0 && tid == 0) c.ctl->cyc[0] = clock64() - t_start;
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) sh.next_chunk = atomicAdd(&c.ctl->blocks_done.v, 1u);
-    __syncthreads();
-    if (sh.next_chunk != gridDim.x - 1u) return;
-    __threadfence();
-    // the widest wave of the call
-    uint32_t wide = 0, late = 0;
-    const uint32_t n_waves = ld_volatile_u32(&c.ctl->waves);
-    for (uint32_t i = tid; i < min(n_waves, (uint32_t)POOL_BINS); i += T) wide = max(wide, __ldcg(&c.ctl->wave_tokens[i]));
-    if (n_waves > (uint32_t)POOL_BINS)
-        for (uint32_t i = tid; i < min(n_waves - (uint32_t)POOL_BINS, t.n_late); i += T) {
-            const uint32_t v = __ldcg(&t.late_waves[i]);
-            (i + 1u < t.n_late ? wide : late) = max(v, i + 1u < t.n_late ? wide : late);
-        }
-    wide = __reduce_max_sync(0xffffffffu, wide);
-    late = __reduce_max_sync(0xffffffffu, late);
-    if ((tid & 31u) == 0) {
-        atomicMax(&c.ctl->max_wave_tokens, max(wide, late));
-        // (the last bin is a sum over waves, and an upper bound only)
-        if (c.tag_mode == RDF_TAGS_PATH && wide > c.qcap && !c.ctl->pool_exhausted) set_status(c, RDF_ERR_QUEUE_FULL);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        volatile Control* k = c.ctl;
-        k->tokens = k->invocations + (unsigned long long)c.B;
-        if (k->pool_exhausted) {
-            if (!z.fallback) set_status(c, RDF_ERR_QUEUE_FULL);
-        } else {
-            if (c.tag_mode == RDF_TAGS_FRAME && k->invocations > z.max_calls) set_status(c, RDF_ERR_FRAMES_FULL);
-            if (c.tag_mode == RDF_TAGS_PATH && k->store_inserts > z.max_parked) set_status(c, RDF_ERR_STORE_FULL);
-        }
-        k->forward_status = k->status;
-    }
+    pool_report(c, sh.waves, t.max_wave, t.n_late, z.max_calls, z.max_parked, z.fallback, t_start, &sh.next_chunk);
 }
 
 // In front of the general scheduler: what the pool kernel could not run (a block ran out of frames: recursion deeper than a

@@ -933,3 +933,93 @@ def test_first_call_of_a_graph_under_capture(mode):
         cg.replay()
         torch.cuda.synchronize()
         assert y.tolist() == [_fib_iter(int(v)) for v in x]
+
+
+# ------------------------------------------------------------ a call per thread
+def _lane_program(kind):
+    """One recursive function whose calls meet in one operator: two or three calls, one to three parameters, one or two conditions
+    (the calls behind either of them), every operator, operands and results with constants added, an operator that is a call."""
+    n_args, op = {"add": (1, "add"), "sub": (1, "sub"), "mul2": (2, "mul"), "max3": (3, "max"), "tail3": (3, "tail3"),
+                  "two": (1, "two"), "first": (1, "first")}[kind]
+    r = rdf.Function("result", 1)
+    f = rdf.Function("f", n_args)
+    x = [f.param(k) for k in range(n_args)]
+    c = f.const
+    r.ret(r.add(r.call(1, r.param(), *[r.const(k + 3) for k in range(n_args - 1)]), r.const(7 if kind == "sub" else 0)))
+    rest = [f.add(v, c(1)) for v in x[1:]][::-1]
+    a, b = f.call(1, f.sub(x[0], c(1)), *rest), f.call(1, f.sub(x[0], c(2)), *x[1:])
+    small = f.lt(x[0], c(2))
+    if op == "tail3":
+        one = c(1)
+        a, b = f.call(1, f.sub(x[0], one), x[1], x[2]), f.call(1, f.sub(x[1], one), x[2], x[0])
+        f.ret(f.if_(f.lt(x[1], x[0]), f.call(1, a, b, f.call(1, f.sub(x[2], one), x[0], x[1])), x[2]))
+    elif op == "two":
+        f.ret(f.if_(f.lt(x[0], c(1)), c(3), f.if_(f.eq(x[0], c(1)), f.add(x[0], c(4)), f.add(f.add(b, a), c(-1)))))
+    elif op == "first":
+        f.ret(f.if_(f.lt(c(1), x[0]), f.add(a, b), f.sub(x[0], c(9))))
+    else:
+        body = {"add": f.add, "sub": f.sub, "mul": f.mul, "max": f.max}[op](a, b)
+        f.ret(f.if_(small, x[-1], body))
+    return [r, f]
+
+
+@pytest.mark.parametrize("kind", ["add", "sub", "mul2", "max3", "tail3", "two", "first"])
+def test_lane_executor_against_the_general_scheduler(kind):
+    """Values and what is reported of the run (waves, calls, parked operands), from one instance to several per warp."""
+    fs = _lane_program(kind)
+    hi = 9 if kind == "tail3" else 14
+    modes = [rdf.TAGS_FRAME] + ([rdf.TAGS_PATH] if kind in ("add", "sub", "two", "first") else [])
+    for mode in modes:
+        for B in (1, 33, 700, 9000):
+            x = torch.from_numpy(np.random.default_rng(B).integers(-1, hi if B < 9000 else 8, size=B)).cuda()
+            g = rdf.Graph(fs, 0, mode)
+            g.eval_int(x, max_invocations=4_000_000)
+            _same_report(fs, 0, mode, x, g.stats()["invocations"])
+
+
+@pytest.mark.parametrize("mode", [rdf.TAGS_PATH, rdf.TAGS_FRAME])
+def test_lane_executor_when_frames_run_short(mode):
+    """Full binary recursions on every lane at once need more frames than a block has, and skewed ones run deeper than the reserve."""
+    f = rdf.Function("f", 1)
+    n, c = f.param(), f.const
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f.ret(f.if_(f.lt(n, c(1)), c(1), f.add(f.call(1, f.sub(n, c(1))), f.call(1, f.sub(n, c(1 if mode == rdf.TAGS_PATH else 30))))))
+    want = [1]
+    for v in range(1, 121):
+        want.append(want[v - 1] + (want[v - 1] if mode == rdf.TAGS_PATH else want[max(v - 30, 0)]))
+    depth, B = (16, 600) if mode == rdf.TAGS_PATH else (120, 3000)
+    g = rdf.Graph([r, f], 0, mode)
+    y, _ = g.eval_int(torch.full((B,), depth, dtype=torch.int64, device="cuda"), max_invocations=B * (2 * want[depth] - 1))
+    assert y.tolist() == [want[depth]] * B and g.stats()["invocations"] == B * (2 * want[depth] - 1)
+
+
+@pytest.mark.parametrize("mode,B", [(rdf.TAGS_FRAME, 300), (rdf.TAGS_PATH, 300)])
+def test_lane_executor_leaves_a_long_instance(mode, B):
+    """A block left over with long instances leaves calls, parked operands and frames to the general scheduler."""
+    r = rdf.Function("result", 1)
+    r.ret(r.call(1, r.param()))
+    f = rdf.Function("f", 1)
+    n, c = f.param(), f.const
+    f.ret(f.if_(f.lt(n, c(1)), n, f.sub(f.call(1, f.sub(n, c(2))), f.call(1, f.sub(n, c(1))))))
+    val, calls = {}, {}
+    for v in range(-1, 27):
+        val[v], calls[v] = (v, 1) if v < 1 else (val[v - 2] - val[v - 1], 1 + calls[v - 2] + calls[v - 1])
+    big = 26 if mode == rdf.TAGS_FRAME else 18
+    xs = np.random.default_rng(1).integers(0, 4, size=B)
+    xs[[7, B // 2]] = big
+    total = int(sum(calls[v] for v in xs))
+    g = rdf.Graph([r, f], 0, mode)
+    x = torch.from_numpy(xs).cuda()
+    for _ in range(3):
+        y, _ = g.eval_int(x, max_invocations=max(total, 200_000))
+        st = g.stats()
+        assert y.tolist() == [val[v] for v in xs]
+        assert st["invocations"] == total and st["tokens"] == total + B and st["store_inserts"] == st["store_matches"] == (total - B) // 2
+    if mode == rdf.TAGS_FRAME:
+        code = 0
+        try:
+            g.eval_int(x, max_invocations=total - 1)
+        except rdf.RdfError as e:
+            code = e.code
+        assert code == -6
