@@ -19,6 +19,7 @@
 #include "rdf_cluster.cuh"
 #include "rdf_lists.cuh"
 #include "rdf_fold.cuh"
+#include "rdf_grove.cuh"
 #include "rdf_lstm.cuh"
 #include "rdf_tc.cuh"
 
@@ -1490,6 +1491,39 @@ static cudaLaunchConfig_t il_cluster_config(cudaLaunchAttribute* at, size_t smem
     return cfg;
 }
 
+// Small batches of the TreeRNN, forward (rdf_grove.cuh), while latency is most of the call: 512 trees of H = 64 (0.14 GFLOP) 153 -> 62 us,
+// 200 of H = 300 (1.3) 438 -> 159, 500 of H = 148 (0.8) 301 -> 133, but 1500 of these (2.5) 356 -> 345 and 8000 of H = 64 (2.6) 316 -> 303:
+// the tiles of the other way come close to it there.  bf16, against tensor cores: 48 trees of H = 300 (0.3) 150 -> 88, 2000 of H = 64 (0.6)
+// 164 -> 121, but 200 of H = 300 (1.3) 177 -> 204.  From H = 32 on: fewer operand words leave most lanes of a sum idle.
+static const double GROVE_FLOPS = 2.5e9, GROVE_FLOPS_BF16 = 0.7e9;
+static bool grove_takes(const rdf_graph* g, const rdf_batch* in, const Layout& L, const ExecState* S, const DevCtx& c, GroveSizes& z) {
+    if (!g->has_rnn || g->has_lstm || L.want_grad || c.H < 32 || S->wait_cycles != 0 || (c.compute == RDF_BF16) != (L.use_tc != 0)) return false;
+    if (in->max_invocations > 0x3FFFFFFFll || c.V > 0x7FFFFFFF || 0.5 * (double)in->max_invocations * 4.0 * c.H * c.H > (L.use_tc ? GROVE_FLOPS_BF16 : GROVE_FLOPS)) return false;
+    const size_t row = (size_t)8 * c.H;                      // bytes of a column of W
+    for (z.blocks = 1; z.blocks <= (uint32_t)CLUSTER_CTAS; z.blocks *= 2) {
+        z.cols = (((uint32_t)c.H + z.blocks - 1) / z.blocks + 3) / 4 * 4;
+        if (z.cols * row <= GROVE_W_BYTES && z.cols * 8 <= (uint32_t)GROVE_THREADS) break;
+    }
+    if (z.blocks > (uint32_t)CLUSTER_CTAS) return false;
+    z.groups = (uint32_t)std::min<long long>(in->B, S->grove_clusters[z.blocks == 1 ? 0 : z.blocks == 2 ? 1 : z.blocks == 4 ? 2 : 3]);
+    if (z.groups < 1) return false;
+    z.max_calls = (uint32_t)in->max_invocations;
+    return true;
+}
+static int rdf_launch_grove(ExecState* S, const DevCtx& c, const GroveSizes& z, float* h_root, cudaStream_t stream) {
+    const size_t smem = (size_t)(z.cols + 2 * GROVE_STEP) * 8 * c.H;
+    const auto kernel = c.use_tc ? rdf_grove_kernel<true> : rdf_grove_kernel<false>;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = z.blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(z.groups * z.blocks); cfg.blockDim = dim3(8 * z.cols);
+    cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = z.blocks > 1 ? 1 : 0;
+    CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, c, z, h_root)));
+    return RDF_OK;
+}
+
 int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     (void)g;
     int dev = 0;
@@ -1549,6 +1583,21 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
         cfg.attrs = at; cfg.numAttrs = 1;
         int n = 0, m = 0;
         ok = ok && cudaOccupancyMaxActiveClusters(&n, rdf_operator_cluster_wide_kernel<CLUSTER_WIDE_CPC>, &cfg) == cudaSuccess;
+        S->grove_clusters[0] = sms;
+        for (int k = 1; k < 4; ++k) {
+            const int blocks = 1 << k, smem = (int)GROVE_W_BYTES + (44 << 10);       // (the largest configurations)
+            int fit = 0;
+            cudaLaunchConfig_t gcfg = {};
+            cudaLaunchAttribute gat[1];
+            gat[0].id = cudaLaunchAttributeClusterDimension;
+            gat[0].val.clusterDim.x = blocks; gat[0].val.clusterDim.y = 1; gat[0].val.clusterDim.z = 1;
+            gcfg.gridDim = dim3(sms / blocks * blocks); gcfg.blockDim = dim3(512); gcfg.dynamicSmemBytes = smem; gcfg.attrs = gat; gcfg.numAttrs = 1;
+            if (cudaFuncSetAttribute(rdf_grove_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                cudaOccupancyMaxActiveClusters(&fit, rdf_grove_kernel<true>, &gcfg) == cudaSuccess)
+                S->grove_clusters[k] = std::min(fit, sms / blocks);
+            else
+                cudaGetLastError();
+        }
         cfg.blockDim = dim3(CL_THREADS); cfg.dynamicSmemBytes = narrow;
         ok = ok && cudaOccupancyMaxActiveClusters(&m, rdf_operator_cluster_kernel<32, 32>, &cfg) == cudaSuccess;
         n = std::min(n, m);
@@ -1803,6 +1852,18 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                       S->wave_limit == 0 && S->probe_mode == RDF_PROBE_THREAD && in->B < (1ll << 31) &&
                       any_width &&
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B || lanes);
+    GroveSizes grove{};
+    if (fold && grove_takes(g, in, L, S, c, grove)) {
+        rdf_mark(S, 1, stream);
+        const int rc = rdf_launch_grove(S, c, grove, out->h_root, stream);
+        if (rc != RDF_OK) return rc;
+        for (int k = 2; k <= 5; ++k) rdf_mark(S, k, stream);
+        S->last_clusters = 0;
+        S->last_ctl = c.ctl;
+        S->last_stream = stream;
+        S->ran = true;
+        return RDF_OK;
+    }
     if (pool) {
         // bounded depth, one match per frame: a pool always suffices (should it not, the call ends with a status)
         bool fallback = !(g->tag_mode == RDF_TAGS_PATH && g->match.size() <= 1);

@@ -1,0 +1,324 @@
+// The forward pass of a small batch of trees by the TreeRNN, in one kernel.
+//
+//     f(v) = leaf(tok v)                      if is_leaf(v)
+//          = cell(f(child v), f(child v))     otherwise
+//
+// In a small batch every level of the recursion is a few dozen cells, and what it costs is latency: a grid barrier per level on the
+// way down (rdf_fold.cuh), one per level on the way up, and five launches.  Instances exchange nothing, so here the instances are
+// dealt out to groups, and a group is one cluster of up to eight blocks that runs its instances from their roots to their states:
+//
+//   down   block 0 of the cluster, level by level: the cells of a level are consecutive records {operand, operand}, an operand a
+//          cell's record number or a leaf's token; block barriers only.  Meanwhile the other blocks fetch their columns of W,
+//          which stay in shared memory
+//   up     level by level from the deepest, cells in steps of up to GROVE_STEP: their operand rows (states of cells through L2,
+//          embedding rows of leaves) are staged in every block of the cluster, each computes its columns, a cluster barrier ends
+//          the level.  A warp computes four columns for all cells of the step, the contraction spread over its lanes
+//
+// fp32 arithmetic throughout; with bf16 operands (bf16 models) states, embedding rows and weights are rounded to bf16 as the
+// tensor-core path rounds them, so that the products are exact.
+//
+// What bounds it: per level the latency of a record, its operand rows, the sums and the barrier; beyond that the shared-memory
+// reads of the sums, 12 of 16 bytes per lane for 128 multiply-adds.  (With one column per thread and the contraction over eight
+// lanes, 9 reads for 32, a step of eight cells of 300 units took 10 000 cycles: a 16-byte read costs a warp four cycles
+// whether its lanes read the same words or not.)
+// (Included by rdf_exec.cu only: it defines kernels.)
+#pragma once
+#include "rdf_fold.cuh"
+
+static const int GROVE_STEP = 8, GROVE_ITEMS = 64, GROVE_THREADS = 512;
+static const size_t GROVE_W_BYTES = 112 << 10;          // columns of W in a block
+static const uint32_t GROVE_LEAF = 0x80000000u;         // operand: a leaf, | token
+
+struct GroveSizes {
+    uint32_t groups, blocks;     // clusters, blocks of a cluster
+    uint32_t cols;               // columns of W per block, a multiple of four
+    uint32_t max_calls;          // invocations the caller allows
+};
+
+struct GroveShared {
+    uint2    items[2][GROVE_ITEMS];      // operands of the first cells of a level, by level parity
+    uint32_t warp_n[2][32];
+    uint32_t base;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// exclusive prefix of k (0 .. 3) over the block's threads, and the total.  Two block barriers.
+__device__ __forceinline__ uint32_t grove_scan(GroveShared& sh, uint32_t k, uint32_t& total) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, lower = (1u << lane) - 1u, n_warps = blockDim.x >> 5;
+    const uint32_t a = __ballot_sync(0xffffffffu, k & 1u), b = __ballot_sync(0xffffffffu, k & 2u);
+    if (lane == 0) sh.warp_n[0][warp] = __popc(a) + 2u * __popc(b);
+    __syncthreads();
+    const uint32_t w = lane < n_warps ? sh.warp_n[0][lane] : 0u;
+    total = __reduce_add_sync(0xffffffffu, w);
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+    __syncthreads();
+    return before + __popc(a & lower) + 2u * __popc(b & lower);
+}
+
+// Down: the group's cells, level by level, as records in c.cell_ops {operand 0, operand 1}; c.wave_marks[first record of a level] =
+// {first record, records} of the level above it.  Leaves the deepest level in sh.base, sh.n.
+__device__ __forceinline__ void grove_descend(const DevCtx& c, const GroveSizes& z, GroveShared& sh, uint32_t group) {
+    const uint32_t tid = threadIdx.x, T = blockDim.x, B = (uint32_t)c.B, mine = group < B ? (B - group + z.groups - 1) / z.groups : 0u;
+    uint2* const rec = reinterpret_cast<uint2*>(c.cell_ops);
+    uint32_t base = 0, n = 0, levels = 1, cells = 0, leaves = 0;
+    bool failed = false;
+    // places for the next level, asked for while its nodes are fetched: two for every cell (an instance has a leaf more than
+    // cells, so that a run that fits max_calls finds them)
+    auto ask = [&](uint32_t most) {
+        if (tid == 0) {
+            const uint32_t at = atomicAdd(&c.ctl->frame_count.v, most);
+            bool ok = true;
+            if ((uint64_t)at + most > z.max_calls) { set_status(c, RDF_ERR_FRAMES_FULL); ok = false; }
+            // (in token waves a level costs one on the way down and one on the way up)
+            else if (2ull * levels + 1u > c.wave_limit) { set_status(c, RDF_ERR_WAVE_LIMIT); ok = false; }
+            sh.base = ok ? at : GROVE_LEAF;
+            if (ok) c.wave_marks[at] = make_uint4(base, n, 0u, 0u);
+        }
+    };
+    {   // the roots
+        ask(mine);
+        uint32_t total = 0;
+        uint4 r = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+        auto root = [&](uint32_t i) { return fold_record(c, fold_words<false>(c, __ldg(&c.tree_root[group + i * z.groups])), 0u); };
+        for (uint32_t i0 = 0; i0 < mine; i0 += T) {          // (two passes: the places of a level are consecutive)
+            if (i0 + tid < mine) r = root(i0 + tid);
+            total += __syncthreads_count(i0 + tid < mine && (int32_t)r.x >= 0);
+        }
+        leaves = mine - total;
+        uint32_t at = sh.base;
+        failed = (at & GROVE_LEAF) != 0u;
+        base = at; n = failed ? 0u : total;
+        for (uint32_t i0 = 0; i0 < mine && !failed; i0 += T) {
+            const uint32_t i = i0 + tid;
+            if (mine > T && i < mine) r = root(i);
+            const bool cell = i < mine && (int32_t)r.x >= 0;
+            uint32_t sum;
+            const uint32_t rank = grove_scan(sh, cell, sum);
+            if (cell) __stcg(&rec[at + rank], make_uint2(r.x, r.y));               // (its two nodes, for the next level)
+            if (i < mine) c.y[group + i * z.groups] = cell ? (int64_t)(at + rank) : (int64_t)(GROVE_LEAF | r.y);
+            at += sum;
+        }
+        __syncthreads();
+    }
+    while (n) {
+        ++levels;
+        cells += n;
+        __syncthreads();
+        ask(2u * n);
+        // the children's words; how many are cells
+        uint4 l = make_uint4(0, 0, 0, 0), r = l;
+        uint32_t total = 0;
+        for (uint32_t i0 = 0; i0 < n; i0 += T) {
+            const uint32_t i = i0 + tid;
+            uint32_t k = 0;
+            if (i < n) {
+                const uint2 v = __ldcg(&rec[base + i]);
+                const NodeWords a = fold_words<true>(c, (int32_t)(c.fold_right[0] ? v.y : v.x)), b = fold_words<true>(c, (int32_t)(c.fold_right[1] ? v.y : v.x));
+                l = fold_record(c, a, 0u);
+                r = fold_record(c, b, 0u);
+                k = ((int32_t)l.x >= 0) + ((int32_t)r.x >= 0);
+            }
+            uint32_t sum;
+            const uint32_t rank = grove_scan(sh, k, sum);
+            l.w = rank;                                      // (kept where one pass is enough)
+            total += sum;
+        }
+        leaves += 2u * n - total;
+        uint32_t at = sh.base;
+        if (at & GROVE_LEAF) {
+            failed = true;
+            n = 0;
+            break;
+        }
+        const uint32_t first = at;
+        for (uint32_t i0 = 0; i0 < n; i0 += T) {
+            const uint32_t i = i0 + tid;
+            uint32_t rank = l.w, sum = 0;
+            if (n > T) {
+                uint32_t k = 0;
+                if (i < n) {
+                    const uint2 v = __ldcg(&rec[base + i]);
+                    l = fold_record(c, fold_words<false>(c, (int32_t)(c.fold_right[0] ? v.y : v.x)), 0u);
+                    r = fold_record(c, fold_words<false>(c, (int32_t)(c.fold_right[1] ? v.y : v.x)), 0u);
+                    k = ((int32_t)l.x >= 0) + ((int32_t)r.x >= 0);
+                }
+                rank = grove_scan(sh, k, sum);
+            }
+            if (i < n) {
+                uint32_t at_l = at + rank, at_r = at_l + ((int32_t)l.x >= 0);
+                if ((int32_t)l.x >= 0) __stcg(&rec[at_l], make_uint2(l.x, l.y));
+                else at_l = GROVE_LEAF | l.y;
+                if ((int32_t)r.x >= 0) __stcg(&rec[at_r], make_uint2(r.x, r.y));
+                else at_r = GROVE_LEAF | r.y;
+                __stcg(&rec[base + i], make_uint2(at_l, at_r));
+            }
+            at += sum;
+        }
+        __syncthreads();
+        if (total == 0u) break;
+        base = first; n = total;
+    }
+    if (tid == 0) {
+        // (a level that could not be entered: nothing is computed, the status says why)
+        __stcg(reinterpret_cast<uint4*>(c.q[0]) + group, make_uint4(base, n, failed ? 1u : 0u, 0u));
+        atomicAdd(&c.ctl->cells, (unsigned long long)cells);
+        atomicAdd(&c.ctl->leaves, (unsigned long long)leaves);
+        atomicMax(&c.ctl->waves, 2u * levels + 1u);
+    }
+}
+
+// v[i]: this lane's part of sum i.  Afterwards the sum of index lane % N over the warp
+template <int N>
+__device__ __forceinline__ float grove_sum(float (&v)[N], uint32_t lane) {
+#pragma unroll
+    for (int o = 16; o >= N; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+#pragma unroll
+    for (int o = N / 2; o >= 1; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < o; ++i) v[i] = (up ? v[i + o] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + o], o);
+    }
+    return v[0];
+}
+// MS cells' operand rows x times the warp's four columns w, the contraction over the lanes: lane 4 i + j has cell i, column j (the
+// first 4 MS lanes)
+template <int MS>
+__device__ __forceinline__ float grove_dot(const float4* w, const float4* x, uint32_t K4, uint32_t lane) {
+    float acc[4 * MS] = {};
+    for (uint32_t k = lane; k < K4; k += 32u) {
+        float4 a[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[j] = w[j * K4 + k];
+#pragma unroll
+        for (int i = 0; i < MS; ++i) {
+            const float4 b = x[i * K4 + k];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[4 * i + j] = fmaf(a[j].x, b.x, fmaf(a[j].y, b.y, fmaf(a[j].z, b.z, fmaf(a[j].w, b.w, acc[4 * i + j]))));
+        }
+    }
+    return grove_sum<4 * MS>(acc, lane);
+}
+
+__device__ __forceinline__ float4 grove_round(float4 v) {
+    return make_float4(__bfloat162float(__float2bfloat16(v.x)), __bfloat162float(__float2bfloat16(v.y)), __bfloat162float(__float2bfloat16(v.z)),
+                       __bfloat162float(__float2bfloat16(v.w)));
+}
+// four units of the state that an operand stands for
+template <bool BF>
+__device__ __forceinline__ float4 grove_state(const DevCtx& c, uint32_t operand, uint32_t k4) {
+    if (operand & GROVE_LEAF) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(c.E + (size_t)(operand & ~GROVE_LEAF) * c.D) + k4);
+        return BF ? grove_round(v) : v;
+    }
+    if (!BF) return ldcg4(c.arena + (size_t)operand * c.H + 4u * k4);
+    const uint2 v = __ldcg(reinterpret_cast<const uint2*>(c.arena_bf + (size_t)operand * c.Hp) + k4);
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+}
+
+template <bool BF>
+__global__ void __launch_bounds__(GROVE_THREADS, 1) rdf_grove_kernel(const __grid_constant__ DevCtx c, const __grid_constant__ GroveSizes z, float* h_root) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ GroveShared sh;
+    const uint32_t tid = threadIdx.x, T = blockDim.x, group = blockIdx.x / z.blocks, rank = z.blocks > 1 ? cluster_rank() : 0u;
+    const uint32_t H4 = c.H / 4, K4 = 2u * H4, col0 = rank * z.cols, n_cols = min(z.cols, (uint32_t)c.H > col0 ? (uint32_t)c.H - col0 : 0u);
+    float4* const w = reinterpret_cast<float4*>(dyn);
+    float4* const x = w + (size_t)z.cols * K4;           // [2][GROVE_STEP][K4]
+    const long long t_start = clock64();
+    auto meet = [&]() {
+        if (z.blocks > 1) cluster_sync_all();
+        else __syncthreads();
+    };
+    if (rank == 0) grove_descend(c, z, sh, group);
+    for (uint32_t i = tid; i < z.cols * K4; i += T) {
+        const float4 v = i / K4 >= n_cols ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(reinterpret_cast<const float4*>(c.W) + (size_t)(col0 + i / K4) * K4 + i % K4);
+        w[i] = BF ? grove_round(v) : v;
+    }
+    meet();
+    const uint32_t lane = tid & 31u, wcol = (tid >> 5) * 4u, col = wcol + (lane & 3u);       // a warp has four columns
+    const bool has_col = col < n_cols;
+    const float bias = has_col ? __ldg(&c.b[col0 + col]) : 0.f;
+    const uint2* const rec = reinterpret_cast<const uint2*>(c.cell_ops);
+    const uint4 deepest = __ldcg(reinterpret_cast<const uint4*>(c.q[0]) + group);       // (the same in all blocks of the cluster)
+    uint32_t base = deepest.x, n = deepest.y;
+    uint32_t par = 0;
+    // the words of a step's operand rows that this thread fetches (GROVE_STEP * K4, at most four per thread)
+    uint32_t my_cell[4], my_k[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t i = tid + q * T;
+        my_cell[q] = i < GROVE_STEP * K4 ? i / K4 : 0x80000000u;
+        my_k[q] = i % K4;
+    }
+    if (tid < min(n, (uint32_t)GROVE_ITEMS)) sh.items[0][tid] = __ldcg(&rec[base + tid]);
+    __syncthreads();
+    while (n) {
+        const uint4 up = __ldcg(&c.wave_marks[base]);        // {first record, records} of the level above
+        if (tid < min(up.y, (uint32_t)GROVE_ITEMS)) sh.items[par ^ 1u][tid] = __ldcg(&rec[up.x + tid]);
+        float4 next[4];
+        auto fetch = [&](uint32_t s0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t i = s0 + my_cell[q];
+                if (i >= n) continue;
+                const uint2 it = i < (uint32_t)GROVE_ITEMS ? sh.items[par][i] : __ldcg(&rec[base + i]);
+                next[q] = grove_state<BF>(c, my_k[q] < H4 ? it.x : it.y, my_k[q] < H4 ? my_k[q] : my_k[q] - H4);
+            }
+        };
+        auto stage = [&](uint32_t s0, float4* to) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (s0 + my_cell[q] < n) to[tid + q * T] = next[q];
+        };
+        fetch(0);
+        uint32_t buf = 0;
+        for (uint32_t s0 = 0; s0 < n; s0 += GROVE_STEP) {
+            float4* const xs = x + (size_t)buf * GROVE_STEP * K4;
+            stage(s0, xs);
+            __syncthreads();
+            if (s0 + GROVE_STEP < n) fetch(s0 + GROVE_STEP);
+            const uint32_t m = min(n - s0, (uint32_t)GROVE_STEP);
+            const float4* const wc = w + (size_t)wcol * K4;
+            const float v = m > 4u ? grove_dot<8>(wc, xs, K4, lane) : m > 2u ? grove_dot<4>(wc, xs, K4, lane) : grove_dot<2>(wc, xs, K4, lane);
+            if (has_col && lane / 4u < m) {                  // (m > 4: all lanes have a sum; fewer cells: the first ones)
+                const float h = tanhf(v + bias);
+                const size_t row = base + s0 + lane / 4u;
+                if (BF) c.arena_bf[row * c.Hp + col0 + col] = __float2bfloat16(h);
+                else __stcg(&c.arena[row * c.H + col0 + col], h);
+            }
+            buf ^= 1u;
+        }
+        meet();
+        base = up.x; n = up.y;
+        par ^= 1u;
+    }
+    // root states: the blocks of the cluster in turn
+    const uint32_t B = (uint32_t)c.B;
+    if (!deepest.z)
+        for (uint32_t i = rank; group + i * z.groups < B; i += z.blocks) {
+            const uint32_t b = group + i * z.groups, operand = (uint32_t)__ldcg(reinterpret_cast<const long long*>(&c.y[b]));
+            for (uint32_t k = tid; k < H4; k += T) reinterpret_cast<float4*>(h_root + (size_t)b * c.H)[k] = grove_state<BF>(c, operand, k);
+        }
+    // the group that ends last: what is reported of the call, in terms of the token waves of the graph (as rdf_fold_kernel)
+    if (rank != 0 || tid != 0) return;
+    __threadfence();
+    if (atomicAdd(&c.ctl->blocks_done.v, 1u) != z.groups - 1u) return;
+    __threadfence();
+    volatile Control* k = c.ctl;
+    const unsigned long long inv = k->cells + k->leaves;
+    if (inv > z.max_calls) set_status(c, RDF_ERR_FRAMES_FULL);
+    k->frame_count.v = (uint32_t)(c.B + inv);
+    k->call_waves = k->n_depth_waves = (k->waves - 1u) / 2u;
+    k->max_wave_tokens = max(B, (uint32_t)k->leaves);
+    k->invocations = inv; k->tokens = (unsigned long long)c.B + 2ull * inv;
+    k->store_inserts = k->store_matches = k->cells;
+    k->cyc[0] = clock64() - t_start;
+    k->forward_status = k->status;
+}

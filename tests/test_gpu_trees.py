@@ -578,3 +578,97 @@ def test_loss_head_class_counts(cell, compute, H, C):
     p["b_s"] = np.asarray(0.25 * np.arange(C) - 0.5, dtype=np.float32)
     tb = workloads.tree_batch_from_shapes([workloads.random_split_shape(rng, int(L)) for L in rng.integers(1, 30, 40)], 7, vocab=70, n_classes=C)
     check_grad({"trees": tb, "params": p}, compute, cell=cell)
+
+
+# ------------------------------------------------------------ small batches, forward
+def _batch_of(kind, B, seed):
+    """Flat trees: 'split' random splits of up to 24 leaves, 'short' one to three leaves, 'shared' both operands of every second cell
+    are the same node (an invocation each), 'chain' degenerate trees."""
+    rng = np.random.default_rng(seed)
+    root, left, right = [], [], []
+    for b in range(B):
+        L = {"split": int(rng.integers(1, 25)), "short": int(rng.integers(1, 4)), "shared": 8, "chain": 40 + b % 7}[kind]
+        base = len(left)
+        root.append(base)
+        if kind == "shared":                      # three cells in a row, each with the next one twice
+            for k in range(3):
+                left.append(base + k + 1)
+                right.append(base + k + 1)
+            left.append(-1)
+            right.append(-1)
+            continue
+        todo = [L]
+        while todo:                               # pre-order
+            n = todo.pop()
+            at = len(left)
+            left.append(-1)
+            right.append(-1)
+            if n > 1:
+                k = 1 if kind == "chain" else int(rng.integers(1, n))
+                left[at] = at + 1
+                right[at] = at + 2 * k
+                todo += [n - k, k]
+    left, right = np.array(left, dtype=np.int32), np.array(right, dtype=np.int32)
+    tok = np.where(left < 0, rng.integers(0, 37, size=left.size), -1).astype(np.int32)
+    arrays = {"tree_root": np.array(root, dtype=np.int32), "left": left, "right": right, "tok": tok, "label": np.zeros_like(tok)}
+    return {k: torch.from_numpy(v).cuda() for k, v in arrays.items()}
+
+
+def _states64(dt, p, bf16):
+    """Root states in 64 bits; bf16: states rounded as the library rounds them."""
+    left, right, tok = (dt[k].cpu().long() for k in ("left", "right", "tok"))
+    rnd = (lambda t: t.float().bfloat16().double()) if bf16 else (lambda t: t)
+    E, W, b = (p[k].double().cpu() for k in ("E", "W", "b"))
+    h = torch.zeros(left.numel(), W.shape[0], dtype=torch.float64)
+    done = left < 0
+    h[done] = rnd(E[tok[done]])
+    while not done.all():
+        i = (~done & done[left.clamp(min=0)] & done[right.clamp(min=0)]).nonzero().flatten()
+        h[i] = rnd(torch.tanh(torch.cat([h[left[i]], h[right[i]]], 1) @ W.T + b))
+        done[i] = True
+    return h[dt["tree_root"].cpu().long()]
+
+
+@pytest.mark.parametrize("compute,H", [(rdf.F32, 32), (rdf.F32, 64), (rdf.F32, 68), (rdf.F32, 132), (rdf.F32, 260), (rdf.F32, 320),
+                                       (rdf.BF16, 32), (rdf.BF16, 100), (rdf.BF16, 256), (rdf.BF16, 320)])
+@pytest.mark.parametrize("kind,B", [("split", 1), ("split", 120), ("short", 20), ("shared", 9), ("chain", 33)])
+def test_small_batch_forward(compute, H, kind, B):
+    """One kernel for the whole call against 64 bits and against the passes that larger batches go through (a wait limit selects
+    them), over the numbers of blocks per group, columns that are no multiple of a block's, and one to many cells per level."""
+    dt = _batch_of(kind, B, H + B)
+    gen = torch.Generator(device="cuda").manual_seed(H)
+    p = {"E": torch.randn(37, H, device="cuda", generator=gen) * 0.3, "W": torch.randn(H, 2 * H, device="cuda", generator=gen) / (2 * H) ** 0.5,
+         "b": torch.randn(H, device="cuda", generator=gen) * 0.2}
+    if compute == rdf.BF16:
+        p = {k: v.bfloat16().float() for k, v in p.items()}
+    inv = {"shared": B * 15}.get(kind, dt["left"].numel())
+    g, other = graph(), graph()
+    other.set_limits(wait_cycles=1 << 33)
+    got, _ = g.eval_trees(dt, p, compute, max_invocations=inv)
+    assert g.stats()["kernel_launches"] == 1
+    want, _ = other.eval_trees(dt, p, compute, max_invocations=inv)
+    a, b = g.stats(), other.stats()
+    keys = ("invocations", "tokens", "waves", "max_wave_tokens", "cells", "leaves", "store_inserts", "store_matches")
+    assert {k: a[k] for k in keys} == {k: b[k] for k in keys}
+    exact = _states64(dt, p, compute == rdf.BF16)
+    # fp32: 2 H products per sum, up to 47 cells on a path; bf16: a rounding that falls the other way (2^-9) and what follows from it
+    tol = 1e-2 if compute == rdf.BF16 else 2e-5
+    assert relerr(got.cpu().numpy(), exact.numpy()) <= tol and relerr(got.cpu().numpy(), want.double().cpu().numpy()) <= 2 * tol
+    code = 0
+    try:
+        g.eval_trees(dt, p, compute, max_invocations=inv - 1)
+    except rdf.RdfError as e:
+        code = e.code
+    assert code == -6
+
+
+def test_small_batch_forward_many_instances_per_group():
+    """More instances, and more cells on a level, than a block has threads."""
+    dt = _batch_of("short", 60000, 5)
+    p = {"E": torch.randn(37, 32, device="cuda"), "W": torch.randn(32, 64, device="cuda") / 8, "b": torch.zeros(32, device="cuda")}
+    g, other = graph(), graph()
+    other.set_limits(wait_cycles=1 << 33)
+    got, _ = g.eval_trees(dt, p)
+    assert g.stats()["kernel_launches"] == 1
+    want, _ = other.eval_trees(dt, p)
+    assert relerr(got.cpu().numpy(), want.cpu().numpy()) <= 1e-5 and g.stats()["cells"] == other.stats()["cells"]
