@@ -733,21 +733,27 @@ __global__ void __launch_bounds__(1024, 1) rdf_scheduler_kernel(const __grid_con
 
 
 // Vector operators of the interleaved execution.  A group of operators of one kind: rows xs[item][0 .. K) in shared memory,
-// outputs tanh(W[:, k0 : k0 + K] x + b).  A warp computes 16 items x 16 outputs, a thread 2 x 4 of them: its 8 lanes along the
-// items read 8 consecutive rows and its 4 lanes along the outputs 4 consecutive rows of W with 128-bit loads (row strides of
-// an odd number of 16-byte pieces: no bank conflicts, one pass each), 6 loads for 32 FMAs.  W stays in shared memory for the
-// whole kernel up to H = IL_SMEM_W_H; wider ones are read through L1.  The terms of a sum are added in index order (a Switch
-// decides on the sign of a sum over the state: another order could flip it).
+// outputs tanh(W[:, k0 : k0 + K] x + b).  A warp computes 16, 32 or 64 items x 16 outputs, a thread 2, 4 or 8 x 4 of them -- as few
+// items as cover the group, so that all warps have some.  Its 8 lanes along the items read 8 consecutive rows and its 4 lanes along
+// the outputs 4 consecutive rows of W with 128-bit loads (row strides of an odd number of 16-byte pieces: no bank conflicts).  A
+// 128-bit load takes shared memory four cycles whether lanes share words or not, so 6 loads for 32 FMAs (two items) leave a third
+// of the FMA rate, 8 for 64 half of it, 12 for 128 two thirds.  W stays in shared memory for the whole kernel up to
+// H = IL_SMEM_W_H; wider ones are read through L1.  The terms of a sum are added in index order (a Switch decides on the sign of
+// a sum over the state: another order could flip it).
+// 16 warps: with 32 a thread had 64 registers and spilled.  8192 seeds, H = 128, depth 10: two items per thread, 32 warps 2215 us; four
+// items 2080 (and 4000 seeds, H = 256, 1661 -> 1729); up to eight items, 16 warps 1917 (1299); rows fetched four at a time per warp, from
+// operands listed in shared memory, 1777.  300 seeds, depth 8: 723 -> 590; 50, H = 96: 594 -> 512.
 static const int IL_SMEM_W_H = 128;
 // One cluster of 8 blocks runs the waves of a call while they are narrow: up to IL_CLUSTER_TOKENS tokens, and tokens x H x H
 // up to IL_CLUSTER_FMA.  How wide the waves get is up to the values (the gate) and the depth limit, so the kernel looks at each
 // wave and leaves the rest of the call to the grid at the first one that is wider.  Besides its faster barrier, the acquire of a
 // grid barrier drops the block's local memory (spilled registers, label arrays) from L1 twice per wave.
-// Grid alone / this / cluster alone, us: 8 seeds, H = 16, depth 10: 523 / 335 / 327; 100, H = 128: 862 / 830 / 915; 20, H = 256,
+// Measured with 32 warps per block and two items per thread; grid alone / this / cluster alone, us: 8 seeds, H = 16, depth 10: 523 / 335 / 327; 100, H = 128: 862 / 830 / 915; 20, H = 256,
 // depth 8: 1806 / 1580 / 1586; 64 full trees, H = 128, depth 10: 1031 / 1010 / 7660; 64, H = 128, depth 18: 1636 / 1600 / 2990.
 // Where the lines lie: with tokens x H x H up to 2^24, 500 seeds, H = 100, depth 6 take 584 us (grid 488), with 2^23 20 seeds,
 // H = 256 1687; with up to 8192 tokens 3000 seeds, H = 40, depth 4 take 379 (grid 310, this 318), with 2048 600 seeds, H = 16 533
 // (grid 586, this 484).
+static const int IL_WARPS = 16, IL_THREADS = 32 * IL_WARPS;
 static const uint32_t IL_CLUSTER_TOKENS = 4096;
 static const unsigned long long IL_CLUSTER_FMA = 10ull << 20;
 __host__ __device__ inline bool il_narrow(unsigned long long tokens, int H) {
@@ -755,42 +761,51 @@ __host__ __device__ inline bool il_narrow(unsigned long long tokens, int H) {
 }
 __host__ __device__ inline int il_stride(int K) { return K + (K % 8 == 0 ? 4 : 8); }
 __host__ __device__ inline int il_out_warps(int H) { return H < 128 ? (H + 15) / 16 : 8; }
-__host__ __device__ inline int il_group_max(int H) { return 32 / il_out_warps(H) * 16; }         // items that the 32 warps cover
+__host__ __device__ inline int il_group_max(int H) { return IL_WARPS / il_out_warps(H) * 32; }   // cells of a group: four per thread
+// operand rows of a group: cells, or twice as many unary operators
+__host__ __device__ inline int il_rows_floats(int H) {
+    const int cells = il_group_max(H) * il_stride(2 * H), unary = 2 * il_group_max(H) * il_stride(H);
+    return cells > unary ? cells : unary;
+}
 static inline int interleaved_smem_bytes(int H) {
-    return (il_group_max(H) * il_stride(2 * H) + (H <= IL_SMEM_W_H ? H * il_stride(2 * H) : 0)) * (int)sizeof(float);
+    return (il_rows_floats(H) + (H <= IL_SMEM_W_H ? H * il_stride(2 * H) : 0)) * (int)sizeof(float);
 }
 
-template <bool SMEM_W>
-__device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int stride, const float* w_rows, int w_stride, int K, uint32_t out0,
-                                         uint32_t out1, int row0, int jw, int lane) {
+template <bool SMEM_W, int IT>
+__device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int stride, const float* w_rows, int w_stride, int K, const uint32_t (&out)[8], int row0,
+                                         int jw, int lane) {
     const int H = c.H, og = lane >> 3;
     const float* x0 = xs + (size_t)row0 * stride;
-    const float* x1 = x0 + 8 * stride;
     for (int j0 = jw * 16 + og; j0 < H; j0 += 128) {
         const float* wr[4];
-        float acc[2][4];
+        float acc[IT][4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int j = min(j0 + 4 * q, H - 1);                  // (a row past the last output repeats the last one: not stored)
             wr[q] = w_rows + (size_t)j * w_stride;
-            acc[0][q] = acc[1][q] = __ldg(&c.b[j]);
+            const float bias = __ldg(&c.b[j]);
+#pragma unroll
+            for (int i = 0; i < IT; ++i) acc[i][q] = bias;
         }
 #pragma unroll 2
         for (int k = 0; k < K; k += 4) {
-            const float4 xa = *reinterpret_cast<const float4*>(x0 + k), xb = *reinterpret_cast<const float4*>(x1 + k);
+            float4 x[IT];
+#pragma unroll
+            for (int i = 0; i < IT; ++i) x[i] = *reinterpret_cast<const float4*>(x0 + 8 * i * stride + k);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float4 w = SMEM_W ? *reinterpret_cast<const float4*>(wr[q] + k) : __ldg(reinterpret_cast<const float4*>(wr[q] + k));
-                acc[0][q] = fmaf(w.w, xa.w, fmaf(w.z, xa.z, fmaf(w.y, xa.y, fmaf(w.x, xa.x, acc[0][q]))));
-                acc[1][q] = fmaf(w.w, xb.w, fmaf(w.z, xb.z, fmaf(w.y, xb.y, fmaf(w.x, xb.x, acc[1][q]))));
+#pragma unroll
+                for (int i = 0; i < IT; ++i) acc[i][q] = fmaf(w.w, x[i].w, fmaf(w.z, x[i].z, fmaf(w.y, x[i].y, fmaf(w.x, x[i].x, acc[i][q]))));
             }
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int j = j0 + 4 * q;
             if (j >= H) break;
-            if (out0 < c.frame_cap) c.arena[(size_t)out0 * c.S + j] = tanhf(acc[0][q]);
-            if (out1 < c.frame_cap) c.arena[(size_t)out1 * c.S + j] = tanhf(acc[1][q]);
+#pragma unroll
+            for (int i = 0; i < IT; ++i)
+                if (out[i] < c.frame_cap) c.arena[(size_t)out[i] * c.S + j] = tanhf(acc[i][q]);
         }
     }
 }
@@ -803,12 +818,14 @@ __device__ __forceinline__ void il_group(const DevCtx& c, const float* xs, int s
 // Two grid barriers per wave (tokens | operators).  fp32, H <= INTERLEAVED_MAX_H.
 // What bounds it: the FMA and load issue of the wide waves and the latency of the narrow ones.  8192 seeds, H = 128, 44
 // waves: groups of 32 with the kinds mixed (unary operators as cells with a zero half) and tokens on the first blocks only
-// 4.24 ms, this 1.86 ms (operators 2.9 -> 1.25, tokens 1.0 -> 0.33).
+// 4.24 ms, this 1.48 ms.
 // CLUSTER: the whole grid is one cluster, whose barrier takes a fifth of the time of the grid barrier; it leaves at the first wave
 // that is not il_narrow, and the form for the whole grid, launched behind it, carries on from the queues.
 template <bool CLUSTER>
-__global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_constant__ DevCtx c) {
+__global__ void __launch_bounds__(IL_THREADS, 1) rdf_interleaved_kernel(const __grid_constant__ DevCtx c) {
     __shared__ SharedProgram sp;
+    __shared__ uint2 s_in[64 * IL_WARPS];                            // operands and results of a group's operators
+    __shared__ uint32_t s_out[64 * IL_WARPS];
     extern __shared__ __align__(16) unsigned char il_smem[];
     const uint4 from = c.ctl->il_state[0], from2 = c.ctl->il_state[1];         // (zeros unless a cluster has run waves of this call)
     // The cluster's own word that it has ended the call.  (Not the status word: a faster block may be in the first wave already and
@@ -828,7 +845,7 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
     float* xs = reinterpret_cast<float*>(il_smem);
     const bool smem_w = H <= IL_SMEM_W_H;
     const int w_stride = smem_w ? il_stride(2 * H) : 2 * H;
-    float* ws = xs + il_group_max(H) * il_stride(2 * H);
+    float* ws = xs + il_rows_floats(H);
     if (smem_w)
         for (int p = threadIdx.x; p < H * (H / 2); p += blockDim.x) {
             const int j = p / (H / 2), k = (p % (H / 2)) * 4;
@@ -878,43 +895,72 @@ __global__ void __launch_bounds__(1024, 1) rdf_interleaved_kernel(const __grid_c
             for (int k = lane; k < H; k += 32) out[k] = __ldg(&e[k]);
         }
         const uint32_t total = end[0] - done[0] + end[1] - done[1] + end[2] - done[2];
-        const uint32_t G = min((uint32_t)il_group_max(H), ((total + gridDim.x - 1) / gridDim.x + 15u) & ~15u);
-        const uint32_t g0 = G ? (end[0] - done[0] + G - 1) / G : 0u, g1 = G ? (end[1] - done[1] + G - 1) / G : 0u, g2 = G ? (end[2] - done[2] + G - 1) / G : 0u;
+        // (rows of unary operators are half as long: twice as many fit)
+        const uint32_t G1 = min(2u * il_group_max(H), ((total + gridDim.x - 1) / gridDim.x + 15u) & ~15u), G0 = min((uint32_t)il_group_max(H), G1);
+        const uint32_t g0 = G0 ? (end[0] - done[0] + G0 - 1) / G0 : 0u, g1 = G1 ? (end[1] - done[1] + G1 - 1) / G1 : 0u, g2 = G1 ? (end[2] - done[2] + G1 - 1) / G1 : 0u;
         for (uint32_t g = blockIdx.x; g < g0 + g1 + g2; g += gridDim.x) {
             const int kind = g < g0 ? 0 : g < g0 + g1 ? 1 : 2;
+            const uint32_t G = kind == 0 ? G0 : G1;
             // (no arrays by index: they would live in local memory, which the barrier's acquire has just dropped from L1)
             const uint32_t first = (kind == 0 ? done[0] : kind == 1 ? done[1] : done[2]) + (g - (kind == 0 ? 0u : kind == 1 ? g0 : g0 + g1)) * G;
             const uint32_t cnt = min(G, (kind == 0 ? end[0] : kind == 1 ? end[1] : end[2]) - first);
             const uint2* unary = kind == 2 ? c.unary_items[1] : c.unary_items[0];
             const int K = kind == 0 ? 2 * H : H, stride = il_stride(K);
             __syncthreads();                                        // (the previous group's operands are no longer read)
-            for (uint32_t i = warp; i < cnt; i += 32u) {
-                uint32_t l, r = 0u;
+            for (uint32_t i = threadIdx.x; i < cnt; i += (uint32_t)IL_THREADS) {
+                uint32_t o, l, r = 0u;
                 if (kind == 0) {
                     const CellItem it = c.cell_items[first + i];
-                    l = it.l; r = it.r;
-                } else l = unary[first + i].y;
-                const bool ok = l < c.frame_cap && r < c.frame_cap;
-                if (!ok && lane == 0) set_status(c, RDF_ERR_BAD_ARG);
-                for (int k = lane * 4; k < K; k += 128) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (ok) v = k < H ? ldcg4(c.arena + (size_t)l * c.S + k) : ldcg4(c.arena + (size_t)r * c.S + (k - H));
-                    *reinterpret_cast<float4*>(xs + (size_t)i * stride + k) = v;
+                    o = it.out; l = it.l; r = it.r;
+                } else {
+                    const uint2 it = unary[first + i];
+                    o = it.x; l = it.y;
                 }
+                if (l >= c.frame_cap || r >= c.frame_cap) {
+                    set_status(c, RDF_ERR_BAD_ARG);
+                    l = 0xFFFFFFFFu;
+                }
+                s_out[i] = o;
+                s_in[i] = make_uint2(l, r);
             }
-            // this thread's two items: rows row0 and row0 + 8 of the group
-            const int row0 = iw * 16 + (lane & 7);
-            uint32_t out[2];
+            __syncthreads();
+            // a warp's rows four at a time: their loads are in flight together
+            for (uint32_t i0 = warp; i0 < cnt; i0 += 4u * IL_WARPS)
+                for (int k = lane * 4; k < K; k += 128) {
+                    float4 v[4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t i = i0 + u * IL_WARPS;
+                        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (i >= cnt) continue;
+                        const uint2 in = s_in[i];
+                        if (in.x != 0xFFFFFFFFu) v[u] = k < H ? ldcg4(c.arena + (size_t)in.x * c.S + k) : ldcg4(c.arena + (size_t)in.y * c.S + (k - H));
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i0 + u * IL_WARPS < cnt) *reinterpret_cast<float4*>(xs + (size_t)(i0 + u * IL_WARPS) * stride + k) = v[u];
+                }
+            // this thread's items: rows row0, row0 + 8, ... of the group
+            const uint32_t n_iw = IL_WARPS / out_warps;
+            const int per_warp = cnt <= 16u * n_iw ? 16 : cnt <= 32u * n_iw ? 32 : 64, row0 = iw * per_warp + (lane & 7);
+            uint32_t out[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
                 const uint32_t at = (uint32_t)row0 + 8u * i;
-                out[i] = at >= cnt ? 0xFFFFFFFFu : kind == 0 ? c.cell_items[first + at].out : unary[first + at].x;
+                out[i] = at >= cnt || 8 * i >= per_warp ? 0xFFFFFFFFu : s_out[at];
             }
             __syncthreads();
             const int k0 = kind == 2 ? H : 0;
-            if ((uint32_t)(iw * 16) < cnt) {
-                if (smem_w) il_group<true>(c, xs, stride, ws + k0, w_stride, K, out[0], out[1], row0, jw, lane);
-                else il_group<false>(c, xs, stride, c.W + k0, w_stride, K, out[0], out[1], row0, jw, lane);
+            if ((uint32_t)(iw * per_warp) < cnt) {
+                if (smem_w) {
+                    if (per_warp == 16) il_group<true, 2>(c, xs, stride, ws + k0, w_stride, K, out, row0, jw, lane);
+                    else if (per_warp == 32) il_group<true, 4>(c, xs, stride, ws + k0, w_stride, K, out, row0, jw, lane);
+                    else il_group<true, 8>(c, xs, stride, ws + k0, w_stride, K, out, row0, jw, lane);
+                } else {
+                    if (per_warp == 16) il_group<false, 2>(c, xs, stride, c.W + k0, w_stride, K, out, row0, jw, lane);
+                    else if (per_warp == 32) il_group<false, 4>(c, xs, stride, c.W + k0, w_stride, K, out, row0, jw, lane);
+                    else il_group<false, 8>(c, xs, stride, c.W + k0, w_stride, K, out, row0, jw, lane);
+                }
             }
         }
         done_leaves = n_leaf;
@@ -1486,7 +1532,7 @@ static cudaLaunchConfig_t il_cluster_config(cudaLaunchAttribute* at, size_t smem
     cudaLaunchConfig_t cfg = {};
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CLUSTER_CTAS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(CLUSTER_CTAS); cfg.blockDim = dim3(1024);
+    cfg.gridDim = dim3(CLUSTER_CTAS); cfg.blockDim = dim3(IL_THREADS);
     cfg.dynamicSmemBytes = smem; cfg.stream = stream; cfg.attrs = at; cfg.numAttrs = 1;
     return cfg;
 }
@@ -1547,7 +1593,7 @@ int rdf_prepare_device(rdf_graph* g, ExecState* S) {
     S->lstm32_per_sm = std::min(per_sm, 2);
     const int il_smem = std::max(interleaved_smem_bytes(IL_SMEM_W_H), interleaved_smem_bytes(INTERLEAVED_MAX_H));      // the two largest configurations
     CUDA_OK(cudaFuncSetAttribute(rdf_interleaved_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, il_smem));
-    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel<false>, 1024, il_smem));
+    CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rdf_interleaved_kernel<false>, IL_THREADS, il_smem));
     if (per_sm < 1) return RDF_ERR_CUDA;
     {
         cudaLaunchAttribute at[1];
@@ -1937,7 +1983,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
             const cudaLaunchConfig_t cfg = il_cluster_config(at, (size_t)interleaved_smem_bytes(c.H), stream);
             RDF_KERNEL(S, CUDA_OK(cudaLaunchKernelEx(&cfg, rdf_interleaved_kernel<true>, c)));
         }
-        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel<false>, dim3(S->grid), dim3(1024), args,
+        RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_interleaved_kernel<false>, dim3(S->grid), dim3(IL_THREADS), args,
                                             (size_t)interleaved_smem_bytes(c.H), stream)));
     } else
         RDF_KERNEL(S, CUDA_OK(cudaLaunchCooperativeKernel((void*)rdf_scheduler_kernel, dim3(S->grid), dim3(1024), args,

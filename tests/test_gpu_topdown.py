@@ -224,3 +224,28 @@ def test_topdown_wide_waves_of_few_seeds_use_the_device():
         g.stats()
         ms.append(e[0].elapsed_time(e[1]) / 5)
     assert ms[0] < ms[1], ms
+
+
+@pytest.mark.parametrize("B,H,D", [(1, 16, 4), (40, 48, 5), (600, 112, 6), (3000, 128, 6), (700, 16, 7), (260, 256, 4), (900, 132, 3)])
+def test_group_sizes_of_the_operators(B, H, D):
+    """Two, four and eight items per thread, one to all warps along the outputs, weights in shared memory and through L1: every state is one
+    fixed expression, so the groups that an operator falls into must not show.  A seed alone and the same seed in a batch agree bit by bit."""
+    fs, r = rdf.topdown_program(D)
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    p = {"E": torch.randn(50, H, device="cuda", generator=gen), "W": torch.randn(H, 2 * H, device="cuda", generator=gen) / (2 * H) ** 0.5,
+         "b": torch.randn(H, device="cuda", generator=gen) * 0.1, "W_s": torch.randn(5, H, device="cuda", generator=gen) / H ** 0.5,
+         "b_s": torch.full((5,), 0.3, device="cuda")}
+
+    def run(tok):
+        n = tok.numel()
+        one = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+        dt = {"tree_root": torch.arange(n, dtype=torch.int32, device="cuda"), "left": one, "right": one, "tok": tok, "label": one}
+        h, _ = rdf.Graph(fs, r, rdf.TAGS_FRAME).eval_trees(dt, p, max_invocations=n * 4 * 2 ** D)
+        return h
+    tok = (torch.arange(B, device="cuda") * 7 % 50).int()
+    h = run(tok)
+    for t in (0, 7, 49):
+        rows = h[tok == t]
+        if rows.numel():
+            alone = run(torch.tensor([t], dtype=torch.int32, device="cuda"))
+            assert torch.equal(rows, alone.expand_as(rows))
