@@ -1542,8 +1542,10 @@ static cudaLaunchConfig_t il_cluster_config(cudaLaunchAttribute* at, size_t smem
 // the tiles of the other way come close to it there.  bf16, against tensor cores: 48 trees of H = 300 (0.3) 150 -> 88, 2000 of H = 64 (0.6)
 // 164 -> 121, but 200 of H = 300 (1.3) 177 -> 204.  From H = 32 on: fewer operand words leave most lanes of a sum idle.
 static const double GROVE_FLOPS = 2.5e9, GROVE_FLOPS_BF16 = 0.7e9;
-static bool grove_takes(const rdf_graph* g, const rdf_batch* in, const Layout& L, const ExecState* S, const DevCtx& c, GroveSizes& z) {
+static bool grove_takes(const rdf_graph* g, const rdf_batch* in, const Layout& L, const ExecState* S, const DevCtx& c, const float* h_root, GroveSizes& z) {
     if (!g->has_rnn || g->has_lstm || L.want_grad || c.H < 32 || S->wait_cycles != 0 || (c.compute == RDF_BF16) != (L.use_tc != 0)) return false;
+    // (rows are read and written 16 bytes at a time)
+    if (((reinterpret_cast<uintptr_t>(c.E) | reinterpret_cast<uintptr_t>(c.W) | reinterpret_cast<uintptr_t>(h_root)) & 15) != 0) return false;
     if (in->max_invocations > 0x3FFFFFFFll || c.V > 0x7FFFFFFF || 0.5 * (double)in->max_invocations * 4.0 * c.H * c.H > (L.use_tc ? GROVE_FLOPS_BF16 : GROVE_FLOPS)) return false;
     const size_t row = (size_t)8 * c.H;                      // bytes of a column of W
     for (z.blocks = 1; z.blocks <= (uint32_t)CLUSTER_CTAS; z.blocks *= 2) {
@@ -1785,7 +1787,7 @@ static const uint32_t POOL_MIN_FRAMES = 15 * POOL_THREADS / 4;   // (bodies of u
 // general scheduler is no help (one call of tak(18, 12, 6), 63 609 calls in 150 waves: 1.20 ms in waves, 0.36).
 static const long long LANE_CALLS = 100000, LANE_TAIL_CALLS = 400000;
 static bool lane_takes(const rdf_graph* g, const rdf_batch* in, const ExecState* S) {
-    if (!g->lanes || in->B >= (1ll << 30)) return false;
+    if (!g->lanes || !in->x || in->B >= (1ll << 30)) return false;      // (no argument: a program with tree operators in a function nobody calls)
     if (in->max_invocations <= LANE_CALLS || in->B >= S->grid) return true;
     return g->lane_prog.cont == PI_CALL && in->max_invocations <= LANE_TAIL_CALLS * in->B;
 }
@@ -1899,7 +1901,7 @@ int rdf_launch_forward(rdf_graph* g, const rdf_batch* in, rdf_outputs* out, char
                       any_width &&
                       (in->B >= POOL_MANY || in->max_invocations <= POOL_CALLS * in->B || lanes);
     GroveSizes grove{};
-    if (fold && grove_takes(g, in, L, S, c, grove)) {
+    if (fold && grove_takes(g, in, L, S, c, out->h_root, grove)) {
         rdf_mark(S, 1, stream);
         const int rc = rdf_launch_grove(S, c, grove, out->h_root, stream);
         if (rc != RDF_OK) return rc;

@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(LN_THREADS, 1) rdf_lanes_kernel(const __grid_c
     uint32_t allowed = LN_ALL;                   // lanes that may take calls and frames (the favoured one, if there is one)
     uint32_t room = (cap - LN_WARPS * LN_FREE0) / LN_WARPS;      // its share of the block's free frames, as last seen
     uint32_t stock = 0;                          // instances taken and not begun
-    uint32_t stalls = 0;                         // iterations without a frame, one after the other
+    uint32_t stalls = 0;                         // iterations without a frame, one after the other (0.2 us and more each)
     uint32_t fired = 0;                    // operators the lane has fired
     int      mode = LN_IDLE;
     int64_t  a[NA];
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(LN_THREADS, 1) rdf_lanes_kernel(const __grid_c
                 n_free = lane_starved(c.ctl, sh, A.free_list, A.my_free, need, cnt);
                 const uint32_t fav = lane_see(sh.cold[warp].fav);
                 if (fav != LN_NONE) allowed = 1u << fav;
-                if (++stalls > (1u << 24) && lane == 0) lane_error(c.ctl, sh, RDF_ERR_TIMEOUT);
+                if (++stalls > (1u << 28) && lane == 0) lane_error(c.ctl, sh, RDF_ERR_TIMEOUT);
             }
         }
         if (n_free) stalls = 0u;

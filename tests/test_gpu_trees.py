@@ -672,3 +672,14 @@ def test_small_batch_forward_many_instances_per_group():
     assert g.stats()["kernel_launches"] == 1
     want, _ = other.eval_trees(dt, p)
     assert relerr(got.cpu().numpy(), want.cpu().numpy()) <= 1e-5 and g.stats()["cells"] == other.stats()["cells"]
+
+
+@pytest.mark.parametrize("compute", [rdf.F32, rdf.BF16])
+def test_small_batch_forward_into_rows_at_any_address(compute):
+    """Root states go to the caller's array, which need not lie on a 16-byte boundary."""
+    dt = _batch_of("split", 20, 3)
+    p = {"E": torch.randn(37, 64, device="cuda"), "W": torch.randn(64, 128, device="cuda") / 12, "b": torch.zeros(64, device="cuda")}
+    want, _ = graph().eval_trees(dt, p, compute)
+    room = torch.zeros(20 * 64 + 1, device="cuda")
+    got, _ = graph().eval_trees(dt, p, compute, h_root=room[1:].view(20, 64))
+    assert relerr(got.cpu().numpy(), want.cpu().numpy()) <= TOL[compute]
