@@ -45,7 +45,8 @@ WORKLOAD_NAMES = {
 }
 CELL = {"treernn": "rnn", "treelstm": "lstm"}
 KERNEL_SOURCES = ["rdf_device.cuh", "rdf_exec.cu", "rdf_exec.h", "rdf_grad.cu", "rdf_internal.h", "rdf_lists.cuh", "rdf_lstm.cuh",
-                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh", "rdf_cluster.cuh", "rdf_pool.cuh", "rdf_math.cuh"]
+                  "rdf_tc.cuh", "rdf_tc_dw.cuh", "rdf_fold.cuh", "rdf_cluster.cuh", "rdf_pool.cuh", "rdf_lanes.cuh",
+                  "rdf_grove.cuh", "rdf_math.cuh"]
 
 
 def fib_iter(n):
@@ -468,10 +469,11 @@ def time_case(case, steps, warmup, flush, dist=None, e2e_steps=None, full_e2e=Fa
 
 
 # --------------------------------------------------------------------------- kernels against their rooflines
-def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
+def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload, launches=0):
     """One row per kernel (group) of the step: CUDA-event time of its phase, algorithmic bytes or flops, the
     measured peak that bounds it and the fraction reached.  Tensor peak: the burst figure for a kernel of under a
-    millisecond (it runs alone between two events on an otherwise idle device), the sustained one above that."""
+    millisecond (it runs alone between two events on an otherwise idle device), the sustained one above that.  launches: of
+    the step (a small forward batch of trees is one kernel)."""
     N = case.N
     rows = []
 
@@ -494,7 +496,7 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
 
     if case.cfg["kind"] == "fib":
         if case.store == "thread":              # (the hash store belongs to the general scheduler)
-            add("rdf_pool_kernel", "schedule", "hbm", 16.0 * len(case.cfg["x"]),
+            add("rdf_lanes_kernel", "schedule", "hbm", 16.0 * len(case.cfg["x"]),
                 "16 B per instance: argument read, result written (frames, tokens and operands stay in shared memory)")
         else:
             add("rdf_scheduler_kernel", "schedule", "hbm", 128.0 * N,
@@ -510,6 +512,9 @@ def kernel_table(case, phase_ms, pk, fp32_peak, traffic, workload):
     Hp = 64 * ((H + 63) // 64)
     lstm = case.cell == "lstm"
     mm = "tensor" if case.use_tc else "alu"
+    if launches == 1:
+        add("rdf_grove_kernel", "schedule", "alu", case.flops_fwd(), "cell contraction 2*2H*H per cell, scheduling in the same kernel")
+        return rows
     add("rdf_fold_kernel", "schedule", "hbm", N * 36.0 + C * 20.0 + Lf * 8.0,
         "per invocation: node words read, frame record and operand words written; list entry of a cell / leaf written")
     if not case.use_tc and not lstm:
@@ -571,7 +576,7 @@ def run(args):
     pk = peaks()
     fp32_peak = probe_fp32_fma_tflops()
     traffic = dram_traffic_table()
-    kernels = kernel_table(case, head["phase_ms"], pk, fp32_peak, traffic, args.workload)
+    kernels = kernel_table(case, head["phase_ms"], pk, fp32_peak, traffic, args.workload, head["stats"]["kernel_launches"])
     # ---- roofline of the dominant kernel (the phase with the largest share of the step)
     dom = max(kernels, key=lambda r: r["ms"])
     roof = {"kernel": dom["kernel"], "bound": dom["bound"], "achieved": dom["achieved"], "peak": dom["peak"], "unit": dom["unit"],
@@ -594,7 +599,7 @@ def run(args):
                     cs = Case(rdf, torch, c_k, grad)
                     n = 5 if c_k["N"] > 2_000_000 else min(args.steps, 20)
                     res = time_case(cs, n, 3, flush, e2e_steps=min(n, 5))
-                kt = kernel_table(cs, res["phase_ms"], pk, fp32_peak, traffic, k)
+                kt = kernel_table(cs, res["phase_ms"], pk, fp32_peak, traffic, k, res["stats"]["kernel_launches"])
                 top = max(kt, key=lambda r: r["ms"])
                 table.append({"workload": k, "pass": "forward+backward" if grad else "forward", "dtype": cs.dtype,
                               "invocations_per_step": c_k["N"], "ms_per_step": res["ms_per_step"], "value": res["value"],
